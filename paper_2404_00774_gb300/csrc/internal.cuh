@@ -141,8 +141,6 @@ void centroid_scores(const IndexData& ix, const void* Q, soar_dtype dt, int64_t 
 
 // ----------------------------------------------------------- mlp.cu
 int64_t mlp_param_count(int D, int H);
-void mlp_forward(const float* P, int D, int H, const float* Z, int B, bool bf16, float* A1, float* H1, float* A2,
-                 float* H2, float* y, cudaStream_t s);
 void mlp_backward(const float* P, int D, int H, const float* Z, const float* target, int B, bool bf16, float* G,
                   float* loss, cudaStream_t s, Scratch& scr);
 void mlp_adam(float* P, const float* G, float* m1, float* m2, int64_t n, int step, float lr, float b1, float b2,
