@@ -5,29 +5,16 @@
 // whose lists overflowed are rescanned exactly, spilled copies of a point
 // are dropped (Section 3.5: a spilled point's copies carry bit-identical
 // exact scores) and each query keeps its top k (Section 2.2).
-//   k <= 32   finish_queries: a warp per query, rescoring and merge fused
-//   k <= 128  query_bounds + rescore_wide: a warp per (query, partition)
-//             slot, leaving one exact list per slot for the caller's merge
+//   finish_queries  a warp per query (k <= 32, batches that fill the chip)
+//   finish_block    a block per query (k <= 128)
 #include "scan_common.cuh"
 
 namespace soar {
 
 namespace {
 
-constexpr int kWideK = kTcWideK;   // largest k of the heap mode
-constexpr int kWideList = kTcWideList;   // largest candidate list per slot in that mode
-
-// Largest L_k over each query's partitions: a lower bound of its final k-th
-// best exact score.
-__global__ void query_bounds(const int2* __restrict__ hdr, const int32_t* __restrict__ inv, int64_t nq, int t,
-                             const int32_t* __restrict__ tpq, float* __restrict__ lstar) {
-  const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (q >= nq) return;
-  const int tq = tpq ? min(max(tpq[q], 0), t) : t;
-  float best = -INFINITY;
-  for (int j = 0; j < tq; ++j) best = fmaxf(best, __int_as_float(hdr[inv[q * t + j]].x));
-  lstar[q] = best;
-}
+// Largest batch finished by a block per query when k <= 32.
+constexpr int64_t kBlockFinishMax = 4096;
 
 // Exact fp32 <q, x> of row-major row `pos` (row stride rs; k ascending, the
 // same order for every copy of a point).  fp32 rows: rs a multiple of 4.
@@ -70,130 +57,164 @@ __device__ __forceinline__ float exact_dot_rm(const float* __restrict__ q, const
 }
 
 
-// Rescoring for 32 < k <= 128 (heap mode, lists of kc <= 256 entries), a
-// warp per (query, partition) slot: the candidates whose upper bound reaches
-// the query's bound are rescored exactly and the best k kept;
-// a slot whose list overflowed is rescanned exactly over its partition into
-// a shared-memory top-k list.  The slot is rewritten best first and closed
-// by a (-inf, -1) entry when shorter than kc.
+// Finishing pass of a block per query (k <= 128).  The query's bound L* (the
+// largest L_k its finished partitions published) bounds its final k-th best
+// exact score from below; the candidates of all its lists whose upper bound
+// reaches L* are gathered in shared memory, rescored exactly a thread each,
+// sorted with the best k so far, and equal neighbours (a spilled point's
+// copies have bit-identical keys) dropped.  A partition whose list overflowed
+// is rescanned exactly by the whole block.
+// Bound: latency (a few hundred scattered 16-byte loads a query).  It replaces
+// a warp per (query, partition) list plus a k-way merge of t sorted lists by
+// a warp (k = 100, 1 024 queries of 272 lists: 870 us with its helper kernels,
+// 99 now), and takes k <= 32 too for batches that do not fill the chip
+// with a warp per query, where one warp rescanning overflowed partitions set
+// the time of a small batch (100 queries: 259 us before, 87 now).
+constexpr int kFbThreads = 128;
+constexpr int kFbKeys = 1024;                  // the best k so far and the pending candidates
+constexpr int kFbPend = kFbKeys - kTcWideK;
+constexpr int kFbUnroll = 4;                   // list entries a thread loads per round
+
 template <typename RowT>
-__global__ void __launch_bounds__(256) rescore_wide(Cand* __restrict__ cand, const int2* __restrict__ hdr, int64_t P,
-                                                    const int32_t* __restrict__ pair_vals, int t,
-                                                    const float* __restrict__ lstar, const float* __restrict__ Qf,
-                                                    int kp, const RowT* __restrict__ rows, int rs,
-                                                    const int32_t* __restrict__ ids,
-                                                    const int32_t* __restrict__ part_of_pair,
-                                                    const int64_t* __restrict__ gstart,
-                                                    const int64_t* __restrict__ part_off, int k, int kc,
-                                                    const int32_t* __restrict__ tpq) {
+__global__ void __launch_bounds__(kFbThreads) finish_block(
+    const Cand* __restrict__ cand, const int2* __restrict__ hdr, const unsigned* __restrict__ gbound,
+    const int32_t* __restrict__ inv, int t, const int32_t* __restrict__ tpq, const float* __restrict__ Qf, int kp,
+    const RowT* __restrict__ rows, int rs, const int32_t* __restrict__ ids, const int32_t* __restrict__ top,
+    const int64_t* __restrict__ part_off, int k, int kc, int64_t* __restrict__ ids_out,
+    float* __restrict__ scores_out) {
   constexpr unsigned kFull = 0xffffffffu;
-  constexpr int R = kWideList / 32;       // candidates per lane
-  constexpr int U = kWideK / 32;          // top-k entries per lane
-  __shared__ Cand top_s[8][kWideK];
-  const int64_t e = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;   // uniform within a warp
-  const int lane = threadIdx.x & 31;
-  if (e >= P) return;
-  const int64_t q = pair_vals[e] / t;
-  const int j = pair_vals[e] - (int)(q * t);
-  if (tpq && j >= min(max(tpq[q], 0), t)) return;
-  const int2 h = hdr[e];
-  const int cnt = min(h.y & 0x7fffffff, kc);
-  const bool ovf = h.y < 0;
-  const float bound = lstar[q];
+  constexpr int T = kFbThreads;
+  __shared__ uint64_t buf[kFbKeys];            // [0, best) ascending distinct keys
+  __shared__ int32_t pend[kFbPend];            // row positions
+  __shared__ int32_t pre_s[T], e_s[T], warp_s[32];
+  __shared__ unsigned ovf_s[T / 32];
+  __shared__ int fill_s;
+  const int64_t q = blockIdx.x;
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  const int tq = tpq ? min(max(tpq[q], 0), t) : t;
+  const float lstar = key_float(gbound[q]);
   const float* qv = Qf + q * (int64_t)kp;
-  Cand* slot = cand + e * (int64_t)kc;
-  if (!ovf) {
-    float v[R];
-    int id[R];
+  int best = 0;                                // uniform
+  if (tid == 0) fill_s = 0;
+  __syncthreads();
+  // the pending rows rescored and merged into the best k (all threads; fill_s visible)
+  const auto flush = [&]() {
+    const int n = fill_s;
+    if (n == 0) return;
+    for (int i = tid; i < n; i += T) {
+      const int32_t pos = pend[i];
+      buf[best + i] = rank_key(exact_dot_rm(qv, rows, rs, pos), (uint32_t)ids[pos]);
+    }
+    int N = 2;
+    while (N < best + n) N <<= 1;
+    for (int i = best + n + tid; i < N; i += T) buf[i] = ~0ull;
+    __syncthreads();
+    if (tid == 0) fill_s = 0;
+    for (int size = 2; size <= N; size <<= 1)
+      for (int stride = size >> 1; stride > 0; stride >>= 1) {
+        for (int i = tid; i < N / 2; i += T) {
+          const int a = 2 * i - (i & (stride - 1)), b = a + stride;
+          const uint64_t x = buf[a], y = buf[b];
+          if ((x > y) == ((a & size) == 0)) {
+            buf[a] = y;
+            buf[b] = x;
+          }
+        }
+        __syncthreads();
+      }
+    // distinct keys move down, chunk by chunk (a key never moves up, and the
+    // entry before a chunk is read before anything is written there)
+    int m = 0;
+    for (int base = 0; base < N && m < k; base += T) {
+      const int i = base + tid;
+      const uint64_t x = i < N ? buf[i] : ~0ull, y = (i > 0 && i < N) ? buf[i - 1] : ~0ull;
+      const int take = (x != ~0ull && (i == 0 || x != y)) ? 1 : 0;
+      int total;
+      const int r = m + block_exclusive_scan<int>(take, warp_s, total);   // (synchronises: every read is done)
+      if (take && r < k) buf[r] = x;
+      m += total;
+      __syncthreads();
+    }
+    best = min(m, k);
+  };
+  for (int j0 = 0; j0 < tq; j0 += T) {
+    const int j = j0 + tid;
+    int e_l = 0, cnt_l = 0;
+    bool ovf_l = false;
+    if (j < tq) {
+      e_l = inv[q * t + j];
+      const int hy = hdr[e_l].y;
+      ovf_l = hy < 0;
+      cnt_l = ovf_l ? 0 : min(hy & 0x7fffffff, kc);
+    }
+    int total;
+    const int ex = block_exclusive_scan<int>(cnt_l, warp_s, total);
+    pre_s[tid] = ex;
+    e_s[tid] = e_l;
+    const unsigned ob = __ballot_sync(kFull, ovf_l);
+    if (lane == 0) ovf_s[w] = ob;
+    __syncthreads();
+    for (int base = 0; base < total; base += T * kFbUnroll) {
+      if (fill_s + T * kFbUnroll > kFbPend) flush();     // (fill_s last written before a barrier: uniform)
+      bool keep[kFbUnroll];
+      int32_t pos[kFbUnroll];
 #pragma unroll
-    for (int r = 0; r < R; ++r) {
-      const int idx = lane + 32 * r;
-      v[r] = -INFINITY;
-      id[r] = -1;
-      if (idx < cnt) {
-        const Cand c = slot[idx];
-        if (c.s >= bound) {
-          v[r] = exact_dot_rm(qv, rows, rs, c.id);
-          id[r] = ids[c.id];
+      for (int u = 0; u < kFbUnroll; ++u) {
+        const int f = base + u * T + tid;
+        keep[u] = false;
+        pos[u] = 0;
+        if (f < total) {
+          int lo = 0;                           // the last list that starts at or before f: the one holding entry f
+#pragma unroll
+          for (int step = T / 2; step > 0; step >>= 1)
+            if (pre_s[lo + step] <= f) lo += step;
+          const Cand c = cand[(int64_t)e_s[lo] * kc + (f - pre_s[lo])];
+          keep[u] = c.s >= lstar;
+          pos[u] = c.id;
         }
       }
-    }
-    __syncwarp();
-    int out = 0;
-    for (; out < k; ++out) {
-      float bs = v[0];
-      int bid = id[0], br = 0;
+      __syncthreads();                          // every thread has read fill_s
 #pragma unroll
-      for (int r = 1; r < R; ++r)
-        if (better(v[r], id[r], bs, bid)) { bs = v[r]; bid = id[r]; br = r; }
-      float ws = bs;
-      int wid = bid, wl = lane;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const float os = __shfl_xor_sync(kFull, ws, o);
-        const int oid = __shfl_xor_sync(kFull, wid, o);
-        const int ol = __shfl_xor_sync(kFull, wl, o);
-        if (better(os, oid, ws, wid) || (os == ws && oid == wid && ol < wl)) { ws = os; wid = oid; wl = ol; }
+      for (int u = 0; u < kFbUnroll; ++u) {
+        const unsigned kb = __ballot_sync(kFull, keep[u]);
+        int at = 0;
+        if (lane == 0 && kb) at = atomicAdd(&fill_s, __popc(kb));
+        at = __shfl_sync(kFull, at, 0);
+        if (keep[u]) pend[at + __popc(kb & ((1u << lane) - 1u))] = pos[u];
       }
-      if (wid == -1) break;                  // every candidate taken
-      if (lane == wl) {
-#pragma unroll
-        for (int r = 0; r < R; ++r)
-          if (r == br) { v[r] = -INFINITY; id[r] = -1; }
-      }
-      if (lane == 0) slot[out] = Cand{ws, wid};
+      __syncthreads();
     }
-    if (lane == 0 && out < kc) slot[out] = Cand{-INFINITY, -1};
-    return;
+    // partitions whose lists overflowed: rescanned exactly
+    for (int word = 0; word < T / 32; ++word)
+      for (unsigned bits = ovf_s[word]; bits; bits &= bits - 1) {
+        const int p = top[q * t + j0 + 32 * word + __ffs(bits) - 1];
+        const int64_t r1 = part_off[p + 1];
+        for (int64_t r0 = part_off[p]; r0 < r1; r0 += T) {
+          if (best < k || fill_s + T > kFbPend) flush();   // early rows fill the best k, then only better ones wait
+          const uint64_t thr = best == k ? buf[k - 1] : ~0ull;
+          __syncthreads();
+          const int64_t r = r0 + tid;
+          const bool in = r < r1 && rank_key(exact_dot_rm(qv, rows, rs, r), (uint32_t)ids[r]) < thr;
+          const unsigned kb = __ballot_sync(kFull, in);
+          int at = 0;
+          if (lane == 0 && kb) at = atomicAdd(&fill_s, __popc(kb));
+          at = __shfl_sync(kFull, at, 0);
+          if (in) pend[at + __popc(kb & ((1u << lane) - 1u))] = (int32_t)r;
+          __syncthreads();
+        }
+      }
+    __syncthreads();                            // pre_s, e_s and ovf_s are rewritten next
   }
-  // overflow: exact rescan of the partition
-  Cand* L = top_s[threadIdx.x >> 5];
-  for (int i = lane; i < k; i += 32) L[i] = Cand{-INFINITY, -1};
-  __syncwarp();
-  const int p = part_of_pair[e];
-  const int64_t r0 = part_off[p];
-  const int64_t nrows = part_off[p + 1] - part_off[p];
-  for (int64_t base = 0; base < nrows; base += 32) {
-    const int64_t r = base + lane;
-    float v = -INFINITY;
-    int rid = -1;
-    if (r < nrows) {
-      v = exact_dot_rm(qv, rows, rs, r0 + r);
-      rid = ids[r0 + r];
-    }
-    unsigned ball = __ballot_sync(kFull, r < nrows && better(v, rid, L[k - 1].s, L[k - 1].id));
-    while (ball) {
-      const int src = __ffs(ball) - 1;
-      ball &= ball - 1;
-      const float vs = __shfl_sync(kFull, v, src);
-      const int is = __shfl_sync(kFull, rid, src);
-      if (!better(vs, is, L[k - 1].s, L[k - 1].id)) continue;   // same answer in every lane
-      int nb = 0;                                              // entries better than (vs, is)
-      for (int i = lane; i < k; i += 32) nb += better(L[i].s, L[i].id, vs, is) ? 1 : 0;
-      nb = __reduce_add_sync(kFull, nb);
-      Cand tmp[U];
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const int i = lane + 32 * u;
-        if (i >= nb && i < k - 1) tmp[u] = L[i];
-      }
-      __syncwarp();
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const int i = lane + 32 * u;
-        if (i >= nb && i < k - 1) L[i + 1] = tmp[u];
-      }
-      __syncwarp();
-      if (lane == 0) L[nb] = Cand{vs, is};
-      __syncwarp();
-    }
+  flush();
+  for (int i = tid; i < k; i += T) {
+    const bool have = i < best;
+    ids_out[q * k + i] = have ? (int64_t)(uint32_t)(buf[i] & 0xffffffffu) : -1;
+    scores_out[q * k + i] = have ? key_float(~(uint32_t)(buf[i] >> 32)) : -INFINITY;
   }
-  for (int i = lane; i < k; i += 32) slot[i] = L[i];
-  if (lane == 0 && k < kc) slot[k] = Cand{-INFINITY, -1};
 }
 
 // Finishing pass for k <= 32, a warp per query: the query's bound L* (the
-// largest L_k of its partitions) bounds its final k-th best exact score from
+// largest L_k its finished partitions published) bounds its final k-th best exact score from
 // below; every candidate whose upper bound reaches L* (and beats the current
 // k-th best) is rescored exactly, and every partition whose list overflowed
 // is rescanned exactly.  The exact results go into a lane-distributed sorted
@@ -202,9 +223,9 @@ __global__ void __launch_bounds__(256) rescore_wide(Cand* __restrict__ cand, con
 // query's ids / scores, padded with -1 / -inf.
 template <typename RowT>
 __global__ void __launch_bounds__(256) finish_queries(
-    const Cand* __restrict__ cand, const int2* __restrict__ hdr, const int32_t* __restrict__ inv, int64_t nq, int t,
-    const int32_t* __restrict__ tpq, const float* __restrict__ Qf, int kp, const RowT* __restrict__ rows, int rs,
-    const int32_t* __restrict__ ids, const int32_t* __restrict__ top, const int64_t* __restrict__ gstart,
+    const Cand* __restrict__ cand, const int2* __restrict__ hdr, const unsigned* __restrict__ gbound,
+    const int32_t* __restrict__ inv, int64_t nq, int t, const int32_t* __restrict__ tpq, const float* __restrict__ Qf,
+    int kp, const RowT* __restrict__ rows, int rs, const int32_t* __restrict__ ids, const int32_t* __restrict__ top,
     const int64_t* __restrict__ part_off, int k, int kc, int64_t* __restrict__ ids_out,
     float* __restrict__ scores_out) {
   constexpr unsigned kFull = 0xffffffffu;
@@ -214,10 +235,7 @@ __global__ void __launch_bounds__(256) finish_queries(
   const int lane = threadIdx.x & 31;
   if (q >= nq) return;
   const int tq = tpq ? min(max(tpq[q], 0), t) : t;
-  float lstar = -INFINITY;
-  for (int j = lane; j < tq; j += 32) lstar = fmaxf(lstar, __int_as_float(hdr[inv[q * t + j]].x));
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) lstar = fmaxf(lstar, __shfl_xor_sync(kFull, lstar, o));
+  const float lstar = key_float(gbound[q]);
   const float* qv = Qf + q * (int64_t)kp;
   uint64_t mine = ~0ull;          // lane j < k: the j-th best key so far (empty: after every real key)
   uint64_t thr = ~0ull;           // the k-th best key
@@ -323,49 +341,26 @@ __global__ void __launch_bounds__(256) finish_queries(
   }
 }
 
-
-// partition of every sorted pair (for the overflow rescans)
-__global__ void pair_partitions(const int32_t* __restrict__ top, const int32_t* __restrict__ pair_vals, int64_t P,
-                                int32_t* __restrict__ part) {
-  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e < P) part[e] = top[pair_vals[e]];
-}
-
 }  // namespace
 
-void finish_tc_queries(const IndexData& ix, const Cand* lists, const int2* hdr, const int32_t* inv, int64_t nq,
-                       int t, const int32_t* tpq, const float* Qf, const int32_t* top, int k, int kc,
-                       int64_t* ids_out, float* scores_out, cudaStream_t s) {
-  if (ix.dtype == SOAR_F32)
-    finish_queries<float><<<ceil_div(nq * 32, 256), 256, 0, s>>>(lists, hdr, inv, nq, t, tpq, Qf, ix.tc_kp,
-                                                                 static_cast<const float*>(ix.vectors), ix.row_stride,
-                                                                 ix.ids, top, ix.tc_gstart, ix.offsets, k, kc,
-                                                                 ids_out, scores_out);
-  else
-    finish_queries<__nv_bfloat16><<<ceil_div(nq * 32, 256), 256, 0, s>>>(
-        lists, hdr, inv, nq, t, tpq, Qf, ix.tc_kp, static_cast<const __nv_bfloat16*>(ix.vectors), ix.row_stride,
-        ix.ids, top, ix.tc_gstart, ix.offsets, k, kc, ids_out, scores_out);
-  SOAR_LAUNCHED();
-}
-
-void rescore_tc_wide(const IndexData& ix, Cand* lists, const int2* hdr, const int32_t* inv,
-                     const int32_t* pair_vals, int64_t nq, int t, const int32_t* tpq, const float* Qf,
-                     const int32_t* top, int k, int kc, cudaStream_t s, Scratch& scr) {
-  const int64_t P = nq * t;
-  float* lstar = scr.get<float>(nq);
-  query_bounds<<<ceil_div(nq, 256), 256, 0, s>>>(hdr, inv, nq, t, tpq, lstar);
-  SOAR_LAUNCHED();
-  int32_t* part = scr.get<int32_t>(P);
-  pair_partitions<<<ceil_div(P, 256), 256, 0, s>>>(top, pair_vals, P, part);
-  SOAR_LAUNCHED();
-  if (ix.dtype == SOAR_F32)
-    rescore_wide<float><<<ceil_div(P * 32, 256), 256, 0, s>>>(lists, hdr, P, pair_vals, t, lstar, Qf, ix.tc_kp,
-                                                              static_cast<const float*>(ix.vectors), ix.row_stride,
-                                                              ix.ids, part, ix.tc_gstart, ix.offsets, k, kc, tpq);
-  else
-    rescore_wide<__nv_bfloat16><<<ceil_div(P * 32, 256), 256, 0, s>>>(
-        lists, hdr, P, pair_vals, t, lstar, Qf, ix.tc_kp, static_cast<const __nv_bfloat16*>(ix.vectors),
-        ix.row_stride, ix.ids, part, ix.tc_gstart, ix.offsets, k, kc, tpq);
+void finish_tc_queries(const IndexData& ix, const Cand* lists, const int2* hdr, const unsigned* gbound,
+                       const int32_t* inv, int64_t nq, int t, const int32_t* tpq, const float* Qf,
+                       const int32_t* top, int k, int kc, int64_t* ids_out, float* scores_out, cudaStream_t s) {
+  const auto launch = [&](auto row) {
+    using RowT = decltype(row);
+    const RowT* rows = static_cast<const RowT*>(ix.vectors);
+    // a warp per query once that fills the chip; a block per query below that and for k > 32
+    if (k <= 32 && nq > kBlockFinishMax)
+      finish_queries<RowT><<<ceil_div(nq * 32, 256), 256, 0, s>>>(lists, hdr, gbound, inv, nq, t, tpq, Qf, ix.tc_kp,
+                                                                  rows, ix.row_stride, ix.ids, top, ix.offsets, k, kc,
+                                                                  ids_out, scores_out);
+    else
+      finish_block<RowT><<<(unsigned)nq, kFbThreads, 0, s>>>(lists, hdr, gbound, inv, t, tpq, Qf, ix.tc_kp, rows,
+                                                             ix.row_stride, ix.ids, top, ix.offsets, k, kc, ids_out,
+                                                             scores_out);
+  };
+  if (ix.dtype == SOAR_F32) launch(float{});
+  else launch(__nv_bfloat16{});
   SOAR_LAUNCHED();
 }
 

@@ -55,28 +55,24 @@ constexpr int kTcWideK = 128;
 constexpr int kTcWideList = 256;
 
 // Finishing of the tensor-core scan (finish_tc.cu), on the scan's candidate
-// lists [nq * t][kc] and headers [nq * t] (L_k, count | overflow << 31):
-// for k <= 32 the exact top k of every query into ids_out / scores_out;
-// for k <= 128 every pair slot's list rescored exactly in place (best
-// first, an id of -1 closing a shorter list) for the caller's merge.
-void finish_tc_queries(const IndexData& ix, const Cand* lists, const int2* hdr, const int32_t* inv, int64_t nq,
-                       int t, const int32_t* tpq, const float* Qf, const int32_t* top, int k, int kc,
-                       int64_t* ids_out, float* scores_out, cudaStream_t s);
-void rescore_tc_wide(const IndexData& ix, Cand* lists, const int2* hdr, const int32_t* inv,
-                     const int32_t* pair_vals, int64_t nq, int t, const int32_t* tpq, const float* Qf,
-                     const int32_t* top, int k, int kc, cudaStream_t s, Scratch& scr);
+// lists [nq * t][kc], headers [nq * t] (L_k, count | overflow << 31) and the
+// queries' bounds [nq] (ordered key of the largest L_k): the exact top k
+// (k <= 128) of every query into ids_out / scores_out.
+void finish_tc_queries(const IndexData& ix, const Cand* lists, const int2* hdr, const unsigned* gbound,
+                       const int32_t* inv, int64_t nq, int t, const int32_t* tpq, const float* Qf,
+                       const int32_t* top, int k, int kc, int64_t* ids_out, float* scores_out, cudaStream_t s);
 
-// Tensor-core scan (scan_tc.cu) of a fp32 index (rows in the core-matrix
-// layout of tc.cuh, queries as fp32 rows of tc_kp columns): screening on the
-// tensor cores, then exact rescoring.  For k <= 32 it also merges: the
-// final top k of every query goes to ids_out / scores_out and it returns
-// true.  Otherwise it leaves in `lists` one list of scan_tc_list_len(k)
-// (exact score, id) entries per pair slot, best first, an id of -1 closing
-// a shorter list, for the caller's merge, and returns false.
+// Tensor-core scan (scan_tc.cu) of a full-vector index (rows in the
+// core-matrix layout of tc.cuh, queries as fp32 rows of tc_kp columns):
+// screening on the tensor cores, then exact rescoring; the final top k of
+// every query goes to ids_out / scores_out.  counter: zero; hdr [nq * t]:
+// cleared headers of the grouped pairs; gbound [nq]: the ordered key of -inf;
+// lists: room for scan_tc_list_len(k) candidates a pair.
 // k <= scan_tc_max_k(ix) (at most 128).
-bool scan_tc_search(const IndexData& ix, const IvfWork& work, int max_items, const float* Qf, const float* qnorm,
+void scan_tc_search(const IndexData& ix, const IvfWork& work, int max_items, const float* Qf, const float* qnorm,
                     const int32_t* top, const int32_t* inv, const int32_t* tpq, int64_t nq, int t, int k,
-                    Cand* lists, int* err, int64_t* ids_out, float* scores_out, cudaStream_t s, Scratch& scr);
+                    Cand* lists, int* counter, int2* hdr, unsigned* gbound, int* err, int64_t* ids_out,
+                    float* scores_out, cudaStream_t s, Scratch& scr);
 int scan_tc_max_k(const IndexData& ix);
 // Candidate-list length per pair slot of the group-maxima scan (scan_gm.cu),
 // which takes k <= 16 when its shared memory fits the row width.

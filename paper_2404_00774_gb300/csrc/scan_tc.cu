@@ -29,8 +29,7 @@
 //     below, and
 //   * the rows with s~ + delta >= L_k (up to kCand, pruned as a_k rises);
 //     a row outside that set cannot be in the top k.
-// No row is rescored here.  The finishing kernels of finish_tc.cu
-// (finish_queries for k <= 32; rescore_wide and the merge for k > 32) later
+// No row is rescored here.  The finishing kernels of finish_tc.cu later
 // take, per query, the largest L_k over its partitions, rescore exactly the
 // candidates whose upper bound reaches it and rescan exactly any partition
 // whose candidate list overflowed, so the results equal those of an exact
@@ -586,20 +585,6 @@ void launch_scan_tc(int k, int grid, size_t smem, cudaStream_t s, const TcParams
   SOAR_LAUNCHED();
 }
 
-
-__global__ void fill_u32(unsigned* __restrict__ a, int64_t n, unsigned v) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) a[i] = v;
-}
-
-// Every pair slot's header before the scan: bound -inf, no candidates, so
-// that a slot the scan never wrote (a CTA that gave up a wait) is read by the
-// finishing kernels as an empty list.
-__global__ void clear_headers(int2* __restrict__ hdr, int64_t n) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) hdr[i] = make_int2(__float_as_int(-INFINITY), 0);
-}
-
 std::atomic<long long> g_wait_limit{0};
 
 }  // namespace
@@ -615,45 +600,31 @@ int scan_tc_max_k(const IndexData& ix) {
 
 int scan_tc_list_len(int k) { return list_len_for(k); }
 
-bool scan_tc_search(const IndexData& ix, const IvfWork& work, int max_items, const float* Qf, const float* qnorm,
+void scan_tc_search(const IndexData& ix, const IvfWork& work, int max_items, const float* Qf, const float* qnorm,
                     const int32_t* top, const int32_t* inv, const int32_t* tpq, int64_t nq, int t, int k,
-                    Cand* lists, int* err, int64_t* ids_out, float* scores_out, cudaStream_t s, Scratch& scr) {
+                    Cand* lists, int* counter, int2* hdr, unsigned* gbound, int* err, int64_t* ids_out,
+                    float* scores_out, cudaStream_t s, Scratch& scr) {
   const int es = ix.dtype == SOAR_F32 ? 4 : 2;
   const int stages = pick_stages(ix.tc_kp, k, es);
   if (stages < 2 || k > kWideK) fail(SOAR_EUNSUPPORTED, "tensor-core scan: k too large");
   const int kc = list_len_for(k);
-  const int64_t P = nq * t;
-  int2* hdr = scr.get<int2>(P);
-  clear_headers<<<ceil_div(P, 256), 256, 0, s>>>(hdr, P);
-  SOAR_LAUNCHED();
   const long long lim = g_wait_limit.load();
-  TcParams prm{work, ix.tc_rows, ix.tc_gstart, ix.tc_pmax, Qf, qnorm, ix.tc_kp, delta_scale(ix.tc_kp, es), k, kc,
-               stages, lim > 0 ? lim : tc::kWaitLimit, nullptr, err, nullptr, lists, hdr};
-  prm.gbound = scr.get<unsigned>(nq);
-  fill_u32<<<ceil_div(nq, 256), 256, 0, s>>>(prm.gbound, nq, 0x007fffffu);   // ordered key of -inf
-  SOAR_LAUNCHED();
-  prm.counter = scr.get<int>(1);
-  SOAR_CUDA(cudaMemsetAsync(prm.counter, 0, sizeof(int), s));
+  const TcParams prm{work, ix.tc_rows, ix.tc_gstart, ix.tc_pmax, Qf, qnorm, ix.tc_kp, delta_scale(ix.tc_kp, es), k,
+                     kc, stages, lim > 0 ? lim : tc::kWaitLimit, counter, err, gbound, lists, hdr};
   const size_t smem = smem_bytes(ix.tc_kp, k, stages, es);
   const int grid = std::max(1, std::min(max_items, num_sms()));
   stage_mark(s, "scan", true);
   if (scan_gm_usable(ix, k))
-    scan_gm_launch(ix, work, grid, Qf, qnorm, nq, k, prm.dscale, prm.wait_limit, prm.counter, err, prm.gbound,
-                   lists, hdr, s, scr);
+    scan_gm_launch(ix, work, grid, Qf, qnorm, nq, k, prm.dscale, prm.wait_limit, counter, err, gbound, lists, hdr, s,
+                   scr);
   else if (es == 4)
     launch_scan_tc<float>(k, grid, smem, s, prm);
   else
     launch_scan_tc<__nv_bfloat16>(k, grid, smem, s, prm);
   stage_mark(s, "scan", false);
   stage_mark(s, "rescore", true);
-  if (k <= kCand) {
-    finish_tc_queries(ix, lists, hdr, inv, nq, t, tpq, Qf, top, k, kc, ids_out, scores_out, s);
-    stage_mark(s, "rescore", false);
-    return true;
-  }
-  rescore_tc_wide(ix, lists, hdr, inv, work.pair_vals, nq, t, tpq, Qf, top, k, kc, s, scr);
+  finish_tc_queries(ix, lists, hdr, gbound, inv, nq, t, tpq, Qf, top, k, kc, ids_out, scores_out, s);
   stage_mark(s, "rescore", false);
-  return false;
 }
 
 }  // namespace soar

@@ -40,3 +40,64 @@ def test_mlp_gradients_at_tile_edges(soar, B, d_in, hidden):
     tol = 2.0 ** -24 * (d_in + 4 * hidden + 2 * B + 40)
     for got, w, s in zip((y, loss[0], G), want, scale):
         assert ((got.cpu().double() - w).abs() <= tol * s).all()
+
+
+def _index(soar, n, d, c, seed, dtype=torch.float32, copies=0):
+    """(X, C, A, index): random unit rows (the first `copies` of them equal) under random rows as centroids."""
+    g = torch.Generator().manual_seed(seed)
+    X = torch.nn.functional.normalize(torch.randn(n, d, generator=g), dim=1)
+    X[:copies] = X[0]
+    X = X.to(dtype)
+    C = X.float()[torch.randperm(n, generator=g)[:c]].contiguous()
+    A = soar.soar_assign(X.cuda(), C.cuda(), 1.0, 1)
+    return X, C, A, soar.soar_index_build(X.cuda(), C.cuda(), A)
+
+
+def _check_search(soar, X, C, A, ix, Q, k, t, tpq=None, sample=40):
+    """A sample of the batch against every probed row scored in fp64; an id may differ where scores tie."""
+    ids, sc = soar.soar_search(ix, Q.cuda(), k, t, None if tpq is None else tpq.cuda())
+    top = soar.soar_select_partitions(ix, Q.cuda(), t).cpu()
+    A, Xd = A.cpu(), X.double()
+    for q in torch.linspace(0, Q.shape[0] - 1, min(sample, Q.shape[0])).long().tolist():
+        m = t if tpq is None else int(tpq[q].clamp(0, t))
+        in_union = torch.isin(A, top[q, :m].to(A.dtype)).any(1)
+        full = torch.where(in_union, Xd @ Q[q].double(), torch.tensor(-float("inf"), dtype=torch.float64))
+        want, at = full.sort(descending=True, stable=True)
+        have = min(k, int(in_union.sum()))
+        got_i, got_s = ids[q].cpu(), sc[q].cpu().double()
+        assert (got_i[have:] == -1).all() and torch.isinf(got_s[have:]).all()
+        assert torch.allclose(got_s[:have], want[:have], rtol=0, atol=1e-5)
+        assert torch.allclose(full[got_i[:have]], want[:have], rtol=0, atol=1e-5)
+        assert got_i[:have].unique().numel() == have
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("nq,k,t,copies", [
+    (1, 1, 30, 0),          # one query, one result
+    (60, 33, 60, 0),        # smallest k of the wide lists
+    (40, 128, 200, 0),      # more lists than a block has threads, largest k
+    (50, 100, 60, 700),     # tied rows overflow the lists: rescans by the block
+    (50, 10, 60, 700),
+    (4200, 10, 4, 700),     # rescans by a warp (large batches)
+    (4096, 3, 3, 0), (4097, 3, 3, 0),   # both sides of the block / warp line
+])
+def test_finishing_of_small_and_wide_searches(soar, dtype, nq, k, t, copies):
+    X, C, A, ix = _index(soar, 9000, 24, 260, 3, dtype, copies)
+    g = torch.Generator().manual_seed(nq)
+    Q = torch.nn.functional.normalize(torch.randn(nq, 24, generator=g), dim=1)
+    if copies:
+        Q[::2] = X[0].float() + 0.05 * Q[::2]
+    tpq = torch.randint(-2, t + 3, (nq,), generator=g).int()     # values outside [0, t] are clamped
+    for counts in (None, tpq):
+        _check_search(soar, X, C, A, ix, Q, k, t, counts)
+    ix.close()
+
+
+@pytest.mark.parametrize("c", [8191, 8192, 9000])
+def test_grouping_past_one_scan_block(soar, c):
+    X, C, A, ix = _index(soar, 20_000, 16, c, 5)
+    g = torch.Generator().manual_seed(c)
+    Q = torch.nn.functional.normalize(torch.randn(5000, 16, generator=g), dim=1)
+    _check_search(soar, X, C, A, ix, Q, 10, 8)
+    _check_search(soar, X, C, A, ix, Q, 10, 8, torch.randint(0, 9, (5000,), generator=g).int())
+    ix.close()
