@@ -103,12 +103,13 @@ void pq_train(const void* X, soar_dtype dt, int64_t n, int32_t d, const float* C
 void pq_encode_index(IndexData& ix, const void* X, soar_dtype dt, cudaStream_t s, Scratch& scr);
 void free_index(IndexData& ix);
 
-// A flat index over fx.n rows (fx.vectors, fx.dtype, fx.row_stride, fx.d and
-// fx.c = ceil(n / chunk) set by the caller; chunk a multiple of 8): chunk p
-// holds rows [p * chunk, (p + 1) * chunk) with their ids, plus the
-// tensor-core layout of the rows; every array is taken from `scr`.  Lets the
-// partition scan serve as an exact brute force.
-void build_flat_tc(IndexData& fx, int64_t chunk, cudaStream_t s, Scratch& scr);
+// A flat index over the fx.n rows X [n][d] (fx.vectors, fx.dtype, fx.row_stride,
+// fx.d and fx.c = ceil(n / chunk) set by the caller; chunk a multiple of 8):
+// chunk p holds rows [p * chunk, (p + 1) * chunk) with their ids, plus the
+// tensor-core layout of the rows; every array is taken from `scr`.  vec (not
+// null: where fx.vectors is not X itself) receives the rows padded to
+// fx.row_stride.  Lets the partition scan serve as an exact brute force.
+void build_flat_tc(IndexData& fx, const void* X, void* vec, int64_t chunk, cudaStream_t s, Scratch& scr);
 
 // index_io.cu: the index's device arrays to / from a file (format in index_io.cu).
 void save_index(const IndexData& ix, const char* path, cudaStream_t s);

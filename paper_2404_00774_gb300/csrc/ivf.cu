@@ -86,59 +86,113 @@ __global__ void group_counts(const int64_t* __restrict__ off, int c, int64_t* __
   cnt[p] = p < c ? (off[p + 1] - off[p] + 7) / 8 : 0;
 }
 
-// Partition p's rows -> 8-row groups in the core-matrix layout (tc.cuh): with
-// E = 16 / sizeof(T) elements per 16-byte row chunk, element k of padded row
-// i goes to group gstart[p] + i/8, element (k/E)*8E + (i%8)*E + k%E.
-template <typename T>
-__global__ void fill_tc_rows(const T* __restrict__ rows, int row_stride, int d, const int64_t* __restrict__ off,
-                             const int32_t* __restrict__ ids, const int64_t* __restrict__ gstart, int kp,
-                             T* __restrict__ out, int32_t* __restrict__ out_ids) {
+// One 16-byte chunk (E elements from k0 on, zeros past d) of a row of X.
+template <typename T, bool Vec>
+__device__ __forceinline__ uint4 row_chunk(const T* __restrict__ x, int k0, int d) {
   constexpr int E = 16 / (int)sizeof(T);
-  const int p = blockIdx.x;
-  const int64_t r0 = off[p];
-  const int size = (int)(off[p + 1] - r0);
-  const int64_t g0 = gstart[p];
-  const int padded = (int)(gstart[p + 1] - g0) * 8;
-  for (int64_t idx = threadIdx.x; idx < (int64_t)padded * kp; idx += blockDim.x) {
-    const int i = (int)(idx / kp), k = (int)(idx % kp);
-    const T v = (i < size && k < d) ? rows[(r0 + i) * row_stride + k] : T(0.f);
-    out[(g0 + i / 8) * (int64_t)(8 * kp) + (k / E) * (8 * E) + (i % 8) * E + (k % E)] = v;
-  }
-  for (int i = threadIdx.x; i < padded; i += blockDim.x) out_ids[g0 * 8 + i] = i < size ? ids[r0 + i] : -1;
-}
-
-// ||x|| of every padded row (warp per row).
-template <typename T>
-__global__ void tc_row_norms(const T* __restrict__ tc_rows, int64_t nrows_padded, int kp, float* __restrict__ norms) {
-  constexpr int E = 16 / (int)sizeof(T);
-  const int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  if (r >= nrows_padded) return;
-  const T* g = tc_rows + (r / 8) * (int64_t)(8 * kp) + (r % 8) * E;
-  float acc = 0.f;
-  for (int k = lane; k < kp; k += 32) {
-    const float v = load_elem(g, (k / E) * (8 * E) + (k % E));
-    acc = fmaf(v, v, acc);
-  }
-  acc = warp_sum(acc);
-  if (lane == 0) norms[r] = sqrtf(acc);
-}
-
-// Largest row norm of every partition (block per partition).
-__global__ void partition_max_norm(const float* __restrict__ norms, const int64_t* __restrict__ gstart,
-                                   float* __restrict__ pmax) {
-  const int p = blockIdx.x;
-  float mx = 0.f;
-  for (int64_t r = gstart[p] * 8 + threadIdx.x; r < gstart[p + 1] * 8; r += blockDim.x) mx = fmaxf(mx, norms[r]);
+  if constexpr (Vec) {
+    return k0 < d ? __ldg(reinterpret_cast<const uint4*>(x + k0)) : make_uint4(0u, 0u, 0u, 0u);
+  } else {
+    union { T e[E]; uint4 v; } u;
+    u.v = make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-  __shared__ float wm[32];
-  if ((threadIdx.x & 31) == 0) wm[threadIdx.x >> 5] = mx;
+    for (int i = 0; i < E; ++i)
+      if (k0 + i < d) u.e[i] = x[k0 + i];
+    return u.v;
+  }
+}
+template <typename T>
+__device__ __forceinline__ float chunk_square(uint4 v) {
+  const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+  float s = 0.f;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    if constexpr (sizeof(T) == 4) {
+      const float a = __uint_as_float(w[i]);
+      s = fmaf(a, a, s);
+    } else {
+      const float a = __uint_as_float(w[i] << 16), b = __uint_as_float(w[i] & 0xffff0000u);
+      s = fmaf(b, b, fmaf(a, a, s));
+    }
+  }
+  return s;
+}
+
+// Partition p's rows in one pass over X: the row-major copy (vec [rows][vstride],
+// unless null), the 8-row groups of the core-matrix layout (tc.cuh: with E = 16 /
+// sizeof(T) elements per 16-byte chunk, element k of padded row i goes to group
+// gstart[p] + i/8, element (k/E)*8E + (i%8)*E + k%E), their ids (-1 on padding),
+// ||x|| of every padded row (0 on padding) and the partition's largest ||x||
+// (pmax, zero before the launch).  ids null: row r of X is row r.
+// A warp takes a group: lane = (row lane % 8, chunk lane / 8 of four), so that a
+// store fills 512 consecutive bytes of the group and a load takes 64 bytes of
+// each row.  Bound: HBM (X read once, both copies written once).  Blocks are
+// (partition, slice of its groups): a flat index has 19 partitions of 65 536 rows,
+// which a block each left 133 of 152 SMs idle (1.18 M x 100 fp32: 3 840 us, 309
+// for the norms; now 171 together); an index of 2 000 partitions took
+// 1 211 (gather) + 991 (this layout) + 615 us (norms) for 2.37 M rows, now 637.
+constexpr int kPackWarps = 8;
+template <typename T, bool Vec>
+__global__ void __launch_bounds__(32 * kPackWarps) pack_partitions(
+    const T* __restrict__ X, int d, const int64_t* __restrict__ off, const int32_t* __restrict__ ids,
+    const int64_t* __restrict__ gstart, int kp, T* __restrict__ tc, int32_t* __restrict__ tc_ids,
+    float* __restrict__ norms, float* __restrict__ pmax, T* __restrict__ vec, int vstride) {
+  constexpr int E = 16 / (int)sizeof(T);
+  __shared__ float wm[kPackWarps];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, i = lane & 7, c0 = lane >> 3;
+  const int p = blockIdx.x;
+  const int64_t r0 = off[p], r1 = off[p + 1], g0 = gstart[p], g1 = gstart[p + 1];
+  float mx = 0.f;
+  for (int64_t g = g0 + (int64_t)blockIdx.y * kPackWarps + w; g < g1; g += (int64_t)gridDim.y * kPackWarps) {
+    const int64_t r = r0 + (g - g0) * 8 + i;
+    const bool in = r < r1;
+    const int32_t id = in ? (ids ? ids[r] : (int32_t)r) : -1;
+    const T* x = X + (int64_t)(in ? id : 0) * d;
+    uint4* out = reinterpret_cast<uint4*>(tc + g * 8 * kp);
+    float ss = 0.f;
+#pragma unroll 4
+    for (int c = c0; c < kp / E; c += 4) {
+      const uint4 v = in ? row_chunk<T, Vec>(x, c * E, d) : make_uint4(0u, 0u, 0u, 0u);
+      out[c * 8 + i] = v;
+      if (vec && in && c * E < vstride) *reinterpret_cast<uint4*>(vec + r * vstride + c * E) = v;
+      ss += chunk_square<T>(v);
+    }
+    ss += __shfl_xor_sync(0xffffffffu, ss, 8);
+    ss += __shfl_xor_sync(0xffffffffu, ss, 16);
+    const float nrm = sqrtf(ss);
+    mx = fmaxf(mx, nrm);
+    if (lane < 8) {
+      norms[g * 8 + i] = nrm;
+      tc_ids[g * 8 + i] = id;
+    }
+  }
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  if (lane == 0) wm[w] = mx;
   __syncthreads();
   if (threadIdx.x == 0) {
-    for (int w = 1; w < (int)(blockDim.x >> 5); ++w) mx = fmaxf(mx, wm[w]);
-    pmax[p] = mx;
+    for (int u = 1; u < kPackWarps; ++u) mx = fmaxf(mx, wm[u]);
+    atomicMax(reinterpret_cast<int*>(pmax + p), __float_as_int(mx));   // (mx >= 0: ordered like its bits)
   }
+}
+
+// Launches pack_partitions for the index's row type; about 64 groups a block.
+void pack_index(const IndexData& ix, const void* X, const int32_t* ids, void* vec, cudaStream_t s) {
+  SOAR_CUDA(cudaMemsetAsync(ix.tc_pmax, 0, sizeof(float) * ix.c, s));
+  const int64_t each = (ix.tc_groups + ix.c - 1) / ix.c;
+  const dim3 grid(ix.c, (unsigned)std::min<int64_t>(65535, std::max<int64_t>(1, (each + 63) / 64)));
+  const auto launch = [&](auto elem) {
+    using T = decltype(elem);
+    // whole 16-byte chunks: rows that start on 16 bytes and end with one
+    const bool aligned = (ix.d * sizeof(T)) % 16 == 0 && (reinterpret_cast<uintptr_t>(X) & 15u) == 0;
+    auto kern = aligned ? pack_partitions<T, true> : pack_partitions<T, false>;
+    kern<<<grid, 32 * kPackWarps, 0, s>>>(static_cast<const T*>(X), ix.d, ix.offsets, ids, ix.tc_gstart, ix.tc_kp,
+                                          static_cast<T*>(ix.tc_rows), ix.tc_ids, ix.tc_norms, ix.tc_pmax,
+                                          static_cast<T*>(vec), ix.row_stride);
+  };
+  if (ix.dtype == SOAR_F32) launch(float{});
+  else launch(__nv_bfloat16{});
+  SOAR_LAUNCHED();
 }
 
 __global__ void chunk_offsets(int64_t n, int64_t chunk, int c, int64_t* __restrict__ off,
@@ -147,7 +201,7 @@ __global__ void chunk_offsets(int64_t n, int64_t chunk, int c, int64_t* __restri
   if (p > c) return;
   const int64_t r = min(n, (int64_t)p * chunk);
   off[p] = r;
-  gstart[p] = (int64_t)p * (chunk / 8);     // every chunk but the last is a whole number of groups
+  gstart[p] = p < c ? (int64_t)p * (chunk / 8) : (n + 7) / 8;     // every chunk but the last is a whole number of groups
   if (p < c) order[p] = p;
 }
 
@@ -158,7 +212,7 @@ __global__ void iota_i32(int32_t* __restrict__ a, int64_t n) {
 
 }  // namespace
 
-void build_flat_tc(IndexData& fx, int64_t chunk, cudaStream_t s, Scratch& scr) {
+void build_flat_tc(IndexData& fx, const void* X, void* vec, int64_t chunk, cudaStream_t s, Scratch& scr) {
   const int64_t n = fx.n;
   const int c = fx.c, d = fx.d;
   const size_t esz = fx.dtype == SOAR_F32 ? 4 : 2;
@@ -169,11 +223,8 @@ void build_flat_tc(IndexData& fx, int64_t chunk, cudaStream_t s, Scratch& scr) {
   fx.part_order = scr.get<int32_t>(c);
   chunk_offsets<<<ceil_div((int64_t)c + 1, 256), 256, 0, s>>>(n, chunk, c, fx.offsets, fx.tc_gstart, fx.part_order);
   SOAR_LAUNCHED();
-  // the last chunk's group count: its rows rounded up to 8
-  const int64_t groups = (int64_t)(c - 1) * (chunk / 8) + (n - (int64_t)(c - 1) * chunk + 7) / 8;
-  fx.tc_groups = groups;
-  SOAR_CUDA(cudaMemcpyAsync(fx.tc_gstart + c, &groups, sizeof(int64_t), cudaMemcpyHostToDevice, s));
-  SOAR_CUDA(cudaStreamSynchronize(s));   // the host value above must not go out of scope before the copy
+  fx.tc_groups = (n + 7) / 8;
+  const int64_t groups = fx.tc_groups;
   fx.ids = scr.get<int32_t>(n);
   iota_i32<<<ceil_div(n, 256), 256, 0, s>>>(fx.ids, n);
   SOAR_LAUNCHED();
@@ -181,23 +232,7 @@ void build_flat_tc(IndexData& fx, int64_t chunk, cudaStream_t s, Scratch& scr) {
   fx.tc_ids = scr.get<int32_t>((size_t)groups * 8);
   fx.tc_norms = scr.get<float>((size_t)groups * 8);
   fx.tc_pmax = scr.get<float>(c);
-  if (fx.dtype == SOAR_F32) {
-    fill_tc_rows<float><<<c, 1024, 0, s>>>(static_cast<const float*>(fx.vectors), fx.row_stride, d, fx.offsets, fx.ids,
-                                          fx.tc_gstart, fx.tc_kp, static_cast<float*>(fx.tc_rows), fx.tc_ids);
-    SOAR_LAUNCHED();
-    tc_row_norms<float><<<ceil_div(groups * 8 * 32, 256), 256, 0, s>>>(static_cast<const float*>(fx.tc_rows),
-                                                                       groups * 8, fx.tc_kp, fx.tc_norms);
-  } else {
-    fill_tc_rows<__nv_bfloat16><<<c, 1024, 0, s>>>(static_cast<const __nv_bfloat16*>(fx.vectors), fx.row_stride, d,
-                                                   fx.offsets, fx.ids, fx.tc_gstart, fx.tc_kp,
-                                                  static_cast<__nv_bfloat16*>(fx.tc_rows), fx.tc_ids);
-    SOAR_LAUNCHED();
-    tc_row_norms<__nv_bfloat16><<<ceil_div(groups * 8 * 32, 256), 256, 0, s>>>(
-        static_cast<const __nv_bfloat16*>(fx.tc_rows), groups * 8, fx.tc_kp, fx.tc_norms);
-  }
-  SOAR_LAUNCHED();
-  partition_max_norm<<<c, 256, 0, s>>>(fx.tc_norms, fx.tc_gstart, fx.tc_pmax);
-  SOAR_LAUNCHED();
+  pack_index(fx, X, nullptr, vec, s);
 }
 
 void quantize_fp8(const void* V, soar_dtype dt, int64_t m, int32_t d, uint8_t* codes, int32_t code_stride,
@@ -248,18 +283,17 @@ void build_index(IndexData& ix, const void* X, soar_dtype dt, const float* C, co
   const int32_t* vs = in_tmp ? vals2 : vals;
   segment_offsets(ks, rows, c, ix.offsets, s);
   SOAR_CUDA(cudaMemcpyAsync(ix.ids, vs, sizeof(int32_t) * rows, cudaMemcpyDeviceToDevice, s));
+  if (ix.mode == SOAR_SCORE_F32) {
+    dev_alloc((void**)&ix.tc_gstart, sizeof(int64_t) * (c + 1));
+    group_counts<<<ceil_div((int64_t)c + 1, 256), 256, 0, s>>>(ix.offsets, c, ix.tc_gstart);
+    SOAR_LAUNCHED();
+    exclusive_scan_i64(ix.tc_gstart, ix.tc_gstart, (int64_t)c + 1, s, scr);
+  }
 
   // vector rows, 16-byte aligned
   if (ix.mode == SOAR_SCORE_F32) {
     ix.row_stride = (int)(((d * esz + 15) / 16) * 16 / esz);
-    dev_alloc(&ix.vectors, esz * (size_t)rows * ix.row_stride);
-    if (dt == SOAR_F32)
-      gather_rows<float><<<(unsigned)rows, 128, 0, s>>>(static_cast<const float*>(X), d, vs, rows, ix.row_stride,
-                                                        static_cast<float*>(ix.vectors));
-    else
-      gather_rows<__nv_bfloat16><<<(unsigned)rows, 128, 0, s>>>(static_cast<const __nv_bfloat16*>(X), d, vs, rows,
-                                                                ix.row_stride, static_cast<__nv_bfloat16*>(ix.vectors));
-    SOAR_LAUNCHED();
+    dev_alloc(&ix.vectors, esz * (size_t)rows * ix.row_stride);   // filled with the tensor-core copy below
   } else if (ix.mode == SOAR_SCORE_FP8) {
     ix.code_stride = (d + 15) / 16 * 16;
     ix.row_stride = ix.code_stride;
@@ -321,8 +355,11 @@ void build_index(IndexData& ix, const void* X, soar_dtype dt, const float* C, co
   SOAR_CUDA(cudaStreamSynchronize(s));
   if (hbad & 1) fail(SOAR_EINVAL, "soar_index_build: an assignment lies outside [0, c)");
   if (hbad & 2) fail(SOAR_EINVAL, "soar_index_build: a point is assigned twice to one partition");
-  int64_t mx = 0;
-  for (int p = 0; p < c; ++p) mx = std::max(mx, off[p + 1] - off[p]);
+  int64_t mx = 0, groups = 0;
+  for (int p = 0; p < c; ++p) {
+    mx = std::max(mx, off[p + 1] - off[p]);
+    groups += (off[p + 1] - off[p] + 7) / 8;
+  }
   ix.max_partition = mx;
 
   // partitions ordered by size, largest first (ties by id): the search hands
@@ -342,36 +379,12 @@ void build_index(IndexData& ix, const void* X, soar_dtype dt, const float* C, co
   if (ix.mode == SOAR_SCORE_F32) {
     const int kstep = dt == SOAR_F32 ? 8 : 16;
     ix.tc_kp = (d + kstep - 1) / kstep * kstep;
-    dev_alloc((void**)&ix.tc_gstart, sizeof(int64_t) * (c + 1));
-    group_counts<<<ceil_div((int64_t)c + 1, 256), 256, 0, s>>>(ix.offsets, c, ix.tc_gstart);
-    SOAR_LAUNCHED();
-    exclusive_scan_i64(ix.tc_gstart, ix.tc_gstart, (int64_t)c + 1, s, scr);
-    int64_t groups = 0;
-    SOAR_CUDA(cudaMemcpyAsync(&groups, ix.tc_gstart + c, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-    SOAR_CUDA(cudaStreamSynchronize(s));
     ix.tc_groups = groups;
     dev_alloc(&ix.tc_rows, esz * (size_t)groups * 8 * ix.tc_kp);
     dev_alloc((void**)&ix.tc_ids, sizeof(int32_t) * (size_t)groups * 8);
     dev_alloc((void**)&ix.tc_norms, sizeof(float) * (size_t)groups * 8);
-    if (dt == SOAR_F32) {
-      fill_tc_rows<float><<<c, 256, 0, s>>>(static_cast<const float*>(ix.vectors), ix.row_stride, d, ix.offsets,
-                                            ix.ids, ix.tc_gstart, ix.tc_kp, static_cast<float*>(ix.tc_rows),
-                                            ix.tc_ids);
-      SOAR_LAUNCHED();
-      tc_row_norms<float><<<ceil_div(groups * 8 * 32, 256), 256, 0, s>>>(static_cast<const float*>(ix.tc_rows),
-                                                                         groups * 8, ix.tc_kp, ix.tc_norms);
-    } else {
-      fill_tc_rows<__nv_bfloat16><<<c, 256, 0, s>>>(static_cast<const __nv_bfloat16*>(ix.vectors), ix.row_stride, d,
-                                                    ix.offsets, ix.ids, ix.tc_gstart, ix.tc_kp,
-                                                    static_cast<__nv_bfloat16*>(ix.tc_rows), ix.tc_ids);
-      SOAR_LAUNCHED();
-      tc_row_norms<__nv_bfloat16><<<ceil_div(groups * 8 * 32, 256), 256, 0, s>>>(
-          static_cast<const __nv_bfloat16*>(ix.tc_rows), groups * 8, ix.tc_kp, ix.tc_norms);
-    }
-    SOAR_LAUNCHED();
     dev_alloc((void**)&ix.tc_pmax, sizeof(float) * c);
-    partition_max_norm<<<c, 256, 0, s>>>(ix.tc_norms, ix.tc_gstart, ix.tc_pmax);
-    SOAR_LAUNCHED();
+    pack_index(ix, X, ix.ids, ix.vectors, s);
   }
   // fp32 centroid scores: the codebook packed for the tensor-core selection
   if (ix.mode != SOAR_SCORE_FP8 && select_tc_fits((d + 7) / 8 * 8)) {

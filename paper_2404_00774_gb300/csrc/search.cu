@@ -1176,15 +1176,10 @@ void exact_mips(const void* X, soar_dtype xdt, int64_t n, int32_t d, const void*
                 int32_t k, int64_t* ids_out, float* scores_out, cudaStream_t s, Scratch& scr) {
   const size_t esz = xdt == SOAR_F32 ? 4 : 2;
   const int stride = (int)(((d * esz + 15) / 16) * 16 / esz);
-  const void* rows = X;
-  if (stride != d || (reinterpret_cast<uintptr_t>(X) & 15u)) {
-    // padded copy so every row starts on a 16-byte boundary
-    void* pad = scr.get<unsigned char>(esz * (size_t)n * stride);
-    SOAR_CUDA(cudaMemcpy2DAsync(pad, esz * stride, X, esz * d, esz * d, n, cudaMemcpyDeviceToDevice, s));
-    if (stride != d)
-      SOAR_CUDA(cudaMemset2DAsync(static_cast<unsigned char*>(pad) + esz * d, esz * stride, 0, esz * (stride - d), n, s));
-    rows = pad;
-  }
+  const bool padded = stride != d || (reinterpret_cast<uintptr_t>(X) & 15u);
+  // where rows do not start on 16-byte boundaries, a padded copy of them
+  void* pad = padded ? scr.get<unsigned char>(esz * (size_t)n * stride) : nullptr;
+  const void* rows = padded ? pad : X;
   // Tensor-core path: the rows become a flat index of 65 536-row chunks that
   // every query probes, so the partition scan (tensor-core screening with
   // exact fp32 finishing) returns the exact top k of all rows.
@@ -1202,7 +1197,7 @@ void exact_mips(const void* X, soar_dtype xdt, int64_t n, int32_t d, const void*
     const int kstep = xdt == SOAR_F32 ? 8 : 16;
     fx.tc_kp = (d + kstep - 1) / kstep * kstep;
     if (k <= scan_tc_max_k(fx)) {
-      build_flat_tc(fx, kChunkRows, s, scr);
+      build_flat_tc(fx, X, pad, kChunkRows, s, scr);
       const int c = fx.c, len = scan_tc_list_len(k);
       const size_t qesz = qdt == SOAR_F32 ? 4 : 2;
       // queries in batches whose candidate lists stay within about 1 GB
@@ -1225,6 +1220,11 @@ void exact_mips(const void* X, soar_dtype xdt, int64_t n, int32_t d, const void*
       }
       return;
     }
+  }
+  if (padded) {
+    SOAR_CUDA(cudaMemcpy2DAsync(pad, esz * stride, X, esz * d, esz * d, n, cudaMemcpyDeviceToDevice, s));
+    if (stride != d)
+      SOAR_CUDA(cudaMemset2DAsync(static_cast<unsigned char*>(pad) + esz * d, esz * stride, 0, esz * (stride - d), n, s));
   }
   // float query rows as wide as the expanded data rows
   const int qstride = stride;

@@ -101,3 +101,25 @@ def test_grouping_past_one_scan_block(soar, c):
     _check_search(soar, X, C, A, ix, Q, 10, 8)
     _check_search(soar, X, C, A, ix, Q, 10, 8, torch.randint(0, 9, (5000,), generator=g).int())
     ix.close()
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("n,d,shift", [(7, 5, 0), (8, 8, 0), (9, 8, 1), (1000, 33, 3), (700, 96, 0), (65_541, 24, 1)])
+def test_row_copies_of_odd_and_unaligned_rows(soar, dtype, n, d, shift):
+    g = torch.Generator().manual_seed(n)
+    flat = torch.randn(n * d + shift, generator=g).to(dtype).cuda()
+    X = flat[shift:].view(n, d)                                  # rows that need not start on 16 bytes
+    Q = torch.randn(37, d, generator=g).cuda()
+    c = max(2, n // 50)
+    C = X[:c].float().contiguous()
+    A = soar.soar_assign(X, C, 1.0, 1)
+    ix = soar.soar_index_build(X, C, A)
+    rows = ix.vectors()
+    assert torch.equal(rows[:, :d], X[ix.ids().long()]) and not rows[:, d:].any()
+    k = min(10, n)
+    full = Q.double() @ X.double().T
+    want = full.topk(k, 1)[0]
+    for ids, sc in (soar.soar_search(ix, Q, k, c), soar.soar_exact_mips(X, Q, k)):
+        assert torch.allclose(sc.double(), want, rtol=1e-5, atol=1e-4)
+        assert torch.allclose(full.gather(1, ids), want, rtol=1e-5, atol=1e-4)
+    ix.close()
