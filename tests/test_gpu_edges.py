@@ -123,3 +123,26 @@ def test_row_copies_of_odd_and_unaligned_rows(soar, dtype, n, d, shift):
         assert torch.allclose(sc.double(), want, rtol=1e-5, atol=1e-4)
         assert torch.allclose(full.gather(1, ids), want, rtol=1e-5, atol=1e-4)
     ix.close()
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("d,big", [(3, 0.0), (130, 0.0), (130, 2e38)])
+def test_centroid_means_of_every_cluster_size(soar, dtype, d, big):
+    """Clusters of 1 to 140 rows (every remainder of the summation's batches); `big` makes fp32 sums overflow."""
+    g = torch.Generator().manual_seed(d)
+    sizes = torch.arange(1, 141)
+    c = sizes.numel()
+    centre = 1000.0 * torch.arange(1, c + 1)[:, None] * torch.nn.functional.one_hot(torch.arange(c) % d, d)
+    own = torch.repeat_interleave(torch.arange(c), sizes)
+    X = (centre[own] + torch.randn(own.numel(), d, generator=g)).to(dtype)
+    if big:                                        # one more cluster far away whose sums exceed fp32
+        far = torch.full((40, d), big).to(dtype)
+        X, own, c = torch.cat([X, far]), torch.cat([own, torch.full((40,), c)]), c + 1
+    first = torch.tensor([int((own == j).nonzero()[0]) for j in range(c)]).int()
+    C = soar.soar_train_centroids(X.cuda(), c, 1, first.cuda()).cpu()
+    a = soar.soar_assign(X.cuda(), X.float()[first.long()].contiguous().cuda(), 0.0, 0).cpu()[:, 0].long()
+    for j in range(c):
+        rows = X[a == j].double()
+        if len(rows):
+            want = rows.mean(0).float()
+            assert ((C[j] - want).abs() <= 2.0 ** -23 * want.abs()).all(), j
