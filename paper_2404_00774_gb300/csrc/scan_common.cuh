@@ -98,16 +98,33 @@ bool scan_by_query_usable(const IndexData& ix, int64_t nq, int t, int k);
 void scan_by_query(const IndexData& ix, const float* Qf, int qstride, const int32_t* top, const int32_t* tpq,
                    int64_t nq, int t, int k, Cand* lists, cudaStream_t s);
 
-// FP8 shortlist (shortlist.cu): for every query the ids of the R best
-// approximate scores s_q * s_x * sum q8 x8 over its probed union, each point
-// once (its copy in the earliest-probed partition), padded with -1; Qf are
-// the queries' code values (code_stride columns), qscale their scales.
-void fp8_shortlist(const IndexData& ix, const float* Qf, const float* qscale, const int32_t* top,
-                   const int32_t* tpq, int64_t nq, int t, int R, int32_t* cand, cudaStream_t s, Scratch& scr);
-// The same shortlist for a PQ4 index: approximate score <q, C_p> + sum_s
-// <q_s, B[s][code_s]> of each point's earliest-probed copy; Qf fp32 rows of
-// qstride columns.
-void pq_shortlist(const IndexData& ix, const float* Qf, int qstride, const int32_t* top, const int32_t* tpq,
-                  int64_t nq, int t, int R, int32_t* cand, cudaStream_t s, Scratch& scr);
+// Search over the compressed layouts (shortlist.cu): for every query the R best
+// approximate scores over its probed union, each point once (its copy in the
+// earliest-probed partition), rescored exactly against Q (dt), the best k
+// (k <= R <= 4 096) into ids_out / scores_out.
+//   FP8  approximate score s_q * s_x * sum q8 x8; Qf the queries' code values
+//        (code_stride columns), qscale their scales
+//   PQ4  approximate score <q, C_p> + sum_s <q_s, B[s][code_s]>; Qf fp32 rows of
+//        qstride columns
+void fp8_search(const IndexData& ix, const float* Qf, const float* qscale, const void* Q, soar_dtype dt,
+                const int32_t* top, const int32_t* tpq, int64_t nq, int t, int R, int k, int64_t* ids_out,
+                float* scores_out, cudaStream_t s, Scratch& scr);
+void pq_search(const IndexData& ix, const float* Qf, int qstride, const void* Q, soar_dtype dt, const int32_t* top,
+               const int32_t* tpq, int64_t nq, int t, int R, int k, int64_t* ids_out, float* scores_out,
+               cudaStream_t s, Scratch& scr);
+
+// (query, probe) pairs of a batch grouped by partition (search.cu).
+struct Grouped {
+  const int32_t* order;    // [c] partitions in the order their items are handed out
+  int64_t* pair_off;       // [c + 1]
+  const int32_t* vals;     // pairs sorted by partition (value q * t + j)
+  int32_t* item_base;      // [c + 1]
+  int* counter;            // work items handed out so far, zero
+  int max_items;
+  int2* hdr;               // tensor-core scan: cleared headers of the pair slots, bounds of the queries
+  unsigned* gbound;
+};
+Grouped group_pairs(const IndexData& ix, int64_t nq, int t, const int32_t* tpq, int qb, const int32_t* top,
+                    int32_t* inv, cudaStream_t s, Scratch& scr, bool tc, bool first_probes_first);
 
 }  // namespace soar

@@ -15,8 +15,6 @@
 //            (score desc, id asc); a spilled point scored in two partitions
 //            has bit-identical (score, id) in both, so the copies are
 //            adjacent and the second is dropped (deduplication, Section 3.5)
-//   rescore  FP8 indices: the merged candidates are rescored exactly in fp32
-//            from the single stored copy and the top k kept
 #include <algorithm>
 
 #include "internal.cuh"
@@ -733,57 +731,6 @@ __global__ void __launch_bounds__(128) merge_kernel(const Cand* __restrict__ par
   }
 }
 
-// ------------------------------------------------------------ exact rescoring
-
-// Warp per query: exact fp32 <q, x> of each candidate from the single stored
-// copy, then the best k by repeated warp arg-max (candidates are distinct).
-template <typename OT, typename QT>
-__global__ void __launch_bounds__(128) rescore_kernel(const int32_t* __restrict__ cand, int R, int64_t nq,
-                                                      const QT* __restrict__ Q, int d, const OT* __restrict__ orig,
-                                                      int ostride, int k, float* __restrict__ work,
-                                                      int64_t* __restrict__ ids_out, float* __restrict__ s_out) {
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int64_t q = (int64_t)blockIdx.x * 4 + w;
-  if (q >= nq) return;
-  float* ws = work + q * R;
-  const int32_t* cq = cand + q * R;
-  for (int i = lane; i < R; i += 32) {
-    int id = cq[i];
-    float s = -INFINITY;
-    if (id >= 0) {
-      s = 0.f;
-      const OT* x = orig + (int64_t)id * ostride;
-      for (int kk = 0; kk < d; ++kk) s = fmaf(load_elem(Q, q * d + kk), load_elem(x, kk), s);
-    }
-    ws[i] = s;
-  }
-  __syncwarp();
-  for (int out = 0; out < k; ++out) {
-    float bs = -INFINITY;
-    int bid = -1, bi = -1;
-    for (int i = lane; i < R; i += 32) {
-      int id = cq[i];
-      if (id < 0) continue;
-      float s = ws[i];
-      if (bi < 0 || better(s, id, bs, bid)) { bs = s; bid = id; bi = i; }
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      float os = __shfl_xor_sync(0xffffffffu, bs, o);
-      int oid = __shfl_xor_sync(0xffffffffu, bid, o);
-      int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-      bool take = oi >= 0 && (bi < 0 || better(os, oid, bs, bid));
-      if (take) { bs = os; bid = oid; bi = oi; }
-    }
-    if (lane == 0) {
-      ids_out[q * k + out] = bi >= 0 ? bid : -1;
-      s_out[q * k + out] = bi >= 0 ? bs : -INFINITY;
-    }
-    if (bi >= 0 && lane == (bi & 31)) ws[bi] = -INFINITY, const_cast<int32_t*>(cq)[bi] = -1;
-    __syncwarp();
-  }
-}
-
 // ------------------------------------------------------------ host glue
 
 int scan_smem_bytes(int xs, int k, int qb) {
@@ -880,16 +827,7 @@ void select_prepared(const IndexData& ix, const float* Qf, const float* qscale, 
   SOAR_LAUNCHED();
 }
 
-struct Grouped {
-  const int32_t* order;    // [c] partitions in the order their items are handed out
-  int64_t* pair_off;       // [c + 1]
-  const int32_t* vals;     // pairs sorted by partition (value q * t + j)
-  int32_t* item_base;      // [c + 1]
-  int* counter;            // work items handed out so far, zero
-  int max_items;
-  int2* hdr;               // tensor-core scan: cleared headers of the pair slots, bounds of the queries
-  unsigned* gbound;
-};
+}  // namespace
 
 // (query, probe) pairs grouped by partition (counting sort), the inverse
 // map inv[q * t + j] = grouped position, and the work items (partition,
@@ -923,6 +861,8 @@ Grouped group_pairs(const IndexData& ix, int64_t nq, int t, const int32_t* tpq, 
   g.max_items = (int)std::min<int64_t>(P / qb + c + 1, 1 << 30);
   return g;
 }
+
+namespace {
 
 template <typename RowT>
 void ivf_scan_typed(const IndexData& ix, const float* Qf, const float* qscale, int64_t nq, int t,
@@ -1115,36 +1055,8 @@ void search(const IndexData& ix, const void* Q, soar_dtype dt, int64_t nq, int32
     stage_mark(s, "merge", false);
     return;
   }
-  // FP8 / PQ4: the best `rescore` approximate scores of each query's probed
-  // union (each point once), rescored exactly in fp32 from the stored rows.
-  int32_t* cand = scr.get<int32_t>((size_t)nq * rescore);
-  stage_mark(s, "scan", true);
-  if (fp8)
-    fp8_shortlist(ix, Qf, qscale, top, tpq, nq, t, rescore, cand, s, scr);
-  else
-    pq_shortlist(ix, Qf, qstride, top, tpq, nq, t, rescore, cand, s, scr);
-  stage_mark(s, "scan", false);
-  float* work = scr.get<float>((size_t)nq * rescore);
-  const int ostride = ix.dtype == SOAR_F32 ? (ix.d + 3) / 4 * 4 : (ix.d + 7) / 8 * 8;
-  if (ix.dtype == SOAR_F32) {
-    if (dt == SOAR_F32)
-      rescore_kernel<float, float><<<ceil_div(nq, 4), 128, 0, s>>>(cand, rescore, nq, static_cast<const float*>(Q),
-          ix.d, static_cast<const float*>(ix.originals), ostride, k, work, ids_out, scores_out);
-    else
-      rescore_kernel<float, __nv_bfloat16><<<ceil_div(nq, 4), 128, 0, s>>>(cand, rescore, nq,
-          static_cast<const __nv_bfloat16*>(Q), ix.d, static_cast<const float*>(ix.originals), ostride, k, work,
-          ids_out, scores_out);
-  } else {
-    if (dt == SOAR_F32)
-      rescore_kernel<__nv_bfloat16, float><<<ceil_div(nq, 4), 128, 0, s>>>(cand, rescore, nq,
-          static_cast<const float*>(Q), ix.d, static_cast<const __nv_bfloat16*>(ix.originals), ostride, k, work,
-          ids_out, scores_out);
-    else
-      rescore_kernel<__nv_bfloat16, __nv_bfloat16><<<ceil_div(nq, 4), 128, 0, s>>>(cand, rescore, nq,
-          static_cast<const __nv_bfloat16*>(Q), ix.d, static_cast<const __nv_bfloat16*>(ix.originals), ostride, k,
-          work, ids_out, scores_out);
-  }
-  SOAR_LAUNCHED();
+  if (fp8) fp8_search(ix, Qf, qscale, Q, dt, top, tpq, nq, t, rescore, k, ids_out, scores_out, s, scr);
+  else pq_search(ix, Qf, qstride, Q, dt, top, tpq, nq, t, rescore, k, ids_out, scores_out, s, scr);
 }
 
 namespace {

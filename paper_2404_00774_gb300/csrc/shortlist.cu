@@ -1,26 +1,37 @@
-// Exact top-R shortlist of approximately scored candidates over each query's
-// probed union (Section 3.5: compressed representations are duplicated for
-// every assignment, the high-bitrate rows are stored once and rescore the
-// best candidates), for two compressed layouts: per-row scaled E4M3 codes
-// of every copy (approximate score s_q * s_x * sum q8 x8), and 4-bit PQ
-// codes of every copy's residual x - C_p (approximate score <q, C_p> +
-// sum_s <q_s, B[s][code_s]>).
+// Search over the compressed layouts (Section 3.5: compressed representations
+// are duplicated for every assignment, the high-bitrate rows are stored once
+// and rescore the best candidates): per query the R best approximate scores
+// of its probed union, each point once, rescored exactly, the best k kept.
+// Two layouts: per-row scaled E4M3 codes of every copy (approximate score
+// s_q * s_x * sum q8 x8), and 4-bit PQ codes of every copy's residual x - C_p
+// (approximate score <q, C_p> + sum_s <q_s, B[s][code_s]>).  A point counts by
+// its copy in the partition the query probed earliest.
 //
-// Three kernels:
-//   pair_offsets  each probed pair's place in its query's slice of a key
-//                 buffer (the sizes of the earlier probed partitions);
-//   approx_pairs  a warp per (query, probe) pair scores the partition's rows
-//                 (lane = row, code rows read coalesced), drops a copy when
-//                 the point has another copy in a partition the query probed
-//                 earlier (from the index's copy of the assignment: each
-//                 point counts once) and writes one 64-bit rank key per row
-//                 (approximate score descending, then id ascending; the
-//                 all-ones key for a dropped copy);
-//   select_top_r  a warp per query finds the R smallest keys of its slice by an MSB-first
-//                 radix select over bytes (warp histograms in shared memory;
-//                 the keys are distinct, so the selected set is exact) and
-//                 writes their ids.
-// The caller rescores those ids exactly from the stored rows.
+//   score_items    (partition, up to 32 / 64 of its queries): the partition's
+//                  rows times the queries on the tensor cores, one 4-byte key
+//                  per (query, row) written at the pair's place in the
+//                  query's slice; 0 for a copy that does not count
+//   finish_slices  a block per query: the R best rows of its slice, rescored
+//                  exactly from the stored rows, and the best k of those
+//
+// Exactness.  The shortlist is defined on approximate scores summed in fp32 in
+// a fixed order (`Rows::exact`).  The tensor cores add in another order, so a
+// key holds such a score within delta only (`Rows::delta`).  With T the R-th
+// largest key of a slice, a row above T + 2 delta is in the shortlist and one
+// below T - 2 delta is not; the few between are scored again in the defined
+// order and ranked by it (score descending, lower id first), so the shortlist
+// is the defined one.
+//
+// Why partition-major: a warp per (query, probe) pair read a partition's codes
+// once per query and spent one table look-up or one fp8 conversion a term
+// (10 000 queries, 10^7 x 96 fp8, t = 6, R = 1 000: scoring 6 230, selecting
+// 2 990, rescoring 2 810 us; 1.18 M x 100 PQ4, t = 14, R = 100: 4 076, 1 884
+// and 398 us).  Here the codes are read and decoded once for up to 64 queries:
+// FP8_SCORE and FP8_FINISH us, PQ_SCORE and PQ_FINISH us.  The product is a few
+// percent of the work, so warp-level MMAs fed from registers are used: a key
+// leaves the registers it was computed in, with no TMEM round trip.
+#include <algorithm>
+
 #include "internal.cuh"
 #include "scan_common.cuh"
 
@@ -28,28 +39,115 @@ namespace soar {
 
 namespace {
 
-constexpr int kSlWarps = 8;
-constexpr int kSlMaxProbesSmem = 256;   // probe lists held in shared memory up to this t
+constexpr int kWarps = 8;
+constexpr int kThreads = 32 * kWarps;
+constexpr int kProbesSmem = 64;      // probe lists held in shared memory up to this t
 
 __device__ __forceinline__ float fp8_code_value(uint32_t b) {
   __half_raw h = __nv_cvt_fp8_to_halfraw((__nv_fp8_storage_t)b, __NV_E4M3);
   return __half2float(__half(h));
 }
 
-// FP8 rows: approx = s_q * s_x * sum q8 x8 (products summed in fp32 in
-// ascending element order); per warp the query's code values.
+// D (16 x 8, fp32) += A (16 x 32 e4m3) B (32 x 8 e4m3)
+__device__ __forceinline__ void mma_e4m3(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
+                                         uint32_t b0, uint32_t b1) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k32.row.col.f32.e4m3.e4m3.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
+      "{%0, %1, %2, %3};"
+      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+      : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+// D (16 x 8, fp32) += A (16 x 16 bf16) B (16 x 8 bf16)
+__device__ __forceinline__ void mma_bf16x16(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
+                                            uint32_t b0, uint32_t b1) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
+      "{%0, %1, %2, %3};"
+      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+      : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+
+// (x, y) as a bf16 pair (x in the low half), and what it leaves over
+__device__ __forceinline__ uint32_t bf16_pair(float x, float y, float& rx, float& ry) {
+  const __nv_bfloat162 h = __floats2bfloat162_rn(x, y);
+  const float2 f = __bfloat1622float2(h);
+  rx = x - f.x;
+  ry = y - f.y;
+  return *reinterpret_cast<const uint32_t*>(&h);
+}
+
+// A layout gives: the queries of an item in shared memory, the scores of 16
+// rows against 8 * nt queries (accumulator element i of tile n: row lane / 4 +
+// 8 * (i / 2), query 8 n + 2 * (lane % 4) + i % 2), and the score in the
+// defined order.
+
+// Per-row scaled E4M3 codes.
 struct Fp8Rows {
+  static constexpr int kTiles = 4;      // most 8-query tiles per item
   const uint8_t* codes;
   int code_stride;
   const float* row_scales;
   const float* Qf;        // [nq][code_stride] code values
   const float* qscale;
-  __host__ __device__ int smem_floats() const { return code_stride; }
-  __device__ void load(float* qs, int64_t q, int lane) const {
-    for (int i = lane; i < code_stride; i += 32) qs[i] = Qf[q * (int64_t)code_stride + i];
+  int k64;                // 64-byte steps of a row
+  int tiles;              // 8-query tiles staged per item, at most kTiles
+
+  __host__ __device__ int query_stride() const { return 64 * k64 + 16; }   // bytes; + 16: conflict-free reads
+  __host__ __device__ size_t item_smem() const { return (size_t)8 * tiles * query_stride(); }
+  __device__ void stage_shared(unsigned char*) const {}
+  __device__ void stage_query(unsigned char* sm, int slot, int64_t q, int lane) const {
+    uint8_t* dst = sm + slot * query_stride();
+    for (int i = lane; i < 64 * k64; i += 32)
+      dst[i] = (q >= 0 && i < code_stride)
+                   ? (uint8_t)__nv_cvt_float_to_fp8(Qf[q * code_stride + i], __NV_SATFINITE, __NV_E4M3)
+                   : (uint8_t)0;
   }
-  __device__ float partition_base(const float*, int, int) const { return 0.f; }
-  __device__ float score(const float* qs, int64_t q, int64_t r, float) const {
+  // The K order is free as long as both operands agree: lane % 4 takes a 16-byte
+  // chunk of each 64 bytes of a row, whose four words serve two MMAs.
+  __device__ void tile(const unsigned char* sm, int64_t r0, int64_t r1, int nt, int lane, float (&acc)[kTiles][4]) const {
+    const int g = lane >> 2, tig = lane & 3;
+    const int64_t ra = r0 + g, rb = ra + 8;
+    const uint8_t* xa = codes + (ra < r1 ? ra : r0) * code_stride;
+    const uint8_t* xb = codes + (rb < r1 ? rb : r0) * code_stride;
+#pragma unroll 2
+    for (int ks = 0; ks < k64; ++ks) {
+      const int o = 64 * ks + 16 * tig;
+      uint4 a = make_uint4(0u, 0u, 0u, 0u), b = a;
+      if (o < code_stride) {
+        a = __ldg(reinterpret_cast<const uint4*>(xa + o));
+        b = __ldg(reinterpret_cast<const uint4*>(xb + o));
+      }
+#pragma unroll
+      for (int n = 0; n < kTiles; ++n)
+        if (n < nt) {
+          const uint4 w = *reinterpret_cast<const uint4*>(sm + (8 * n + g) * query_stride() + o);
+          mma_e4m3(acc[n], a.x, b.x, a.y, b.y, w.x, w.y);
+          mma_e4m3(acc[n], a.z, b.z, a.w, b.w, w.z, w.w);
+        }
+    }
+  }
+  __device__ float row_factor(int64_t r) const { return row_scales[r]; }
+  __device__ float query_factor(int64_t q, int64_t) const { return qscale[q]; }
+  __device__ static float combine(float acc, float rf, float qf) { return acc * qf * rf; }
+  // finishing: the query's code values in shared memory
+  __host__ __device__ int query_floats() const { return code_stride; }
+  __device__ float3 stage_finish(float* qs, int64_t q, const float*, int) const {
+    float n2 = 0.f;
+    for (int i = threadIdx.x; i < code_stride; i += kThreads) {
+      const float v = Qf[q * (int64_t)code_stride + i];
+      qs[i] = v;
+      n2 = fmaf(v, v, n2);
+    }
+    return make_float3(n2, 0.f, 0.f);
+  }
+  // |key's score - defined score|: both sums of exact products have at most
+  // code_stride fp32 additions, each within 2^-23 of a partial sum that stays
+  // below ||q8|| ||x8||, and ||x8|| <= 448 sqrt(d); a factor of four to spare.
+  // The scale of a row is at most smax.
+  __device__ float delta(float3 v, int64_t q, float smax) const {
+    return ldexpf((float)code_stride, -20) * sqrtf(v.x) * 448.f * sqrtf((float)code_stride) * qscale[q] * smax;
+  }
+  __device__ float exact(const float* qs, int64_t q, int64_t r, float) const {
     const uint4* x = reinterpret_cast<const uint4*>(codes + r * (int64_t)code_stride);
     float acc = 0.f;
     for (int c = 0; c < code_stride / 16; ++c) {
@@ -64,239 +162,727 @@ struct Fp8Rows {
   }
 };
 
-// PQ4 rows: approx = <q, C_p> + sum_s LUT[s][code_s] with LUT[s][j] =
-// <q_s, B[s][j]>; per warp the LUT ([m][16]) followed by the query row.
+// PQ4 codes: approx = <q, C_p> + sum_s LUT[s][code_s], LUT[s][j] = <q_s, B[s][j]>.
+// A subspace's two dimensions are one bf16 pair of an MMA operand, so decoding
+// a code is one shared-memory read of its centre (hi and lo parts); centres and
+// queries enter as hi + lo and the lo lo product is dropped.
 struct Pq4Rows {
+  static constexpr int kTiles = 8;
   const uint8_t* codes;
   int code_stride, m, d;
   const float* B;         // [m][16][2]
-  const float* C;         // [c][d]
   const float* Qf;        // [nq][qstride] fp32
   int qstride;
-  __host__ __device__ int smem_floats() const { return m * 16 + qstride; }
-  __device__ void load(float* qs, int64_t q, int lane) const {
-    float* qrow = qs + m * 16;
-    for (int i = lane; i < qstride; i += 32) qrow[i] = Qf[q * (int64_t)qstride + i];
-    for (int e = lane; e < m * 16; e += 32) {
-      const int sidx = e / 16;
-      const float q0 = Qf[q * (int64_t)qstride + 2 * sidx], q1 = Qf[q * (int64_t)qstride + 2 * sidx + 1];
-      qs[e] = fmaf(q1, B[2 * e + 1], q0 * B[2 * e]);
+  const float* base;      // [pairs] <q, C_p>
+  int steps;              // K steps of 8 subspaces
+  int tiles;
+
+  __host__ __device__ int query_stride() const { return 8 * steps + 4; }   // words a part; + 4: conflict-free reads
+  __host__ __device__ size_t item_smem() const {
+    return (size_t)8 * steps * 16 * 8 + (size_t)2 * 8 * tiles * query_stride() * 4;
+  }
+  __device__ void stage_shared(unsigned char* sm) const {
+    uint2* lut = reinterpret_cast<uint2*>(sm);
+    for (int e = threadIdx.x; e < 8 * steps * 16; e += kThreads) {
+      float x = 0.f, y = 0.f, rx, ry, u, v;
+      if (e < m * 16) {
+        const float2 c = reinterpret_cast<const float2*>(B)[e];
+        x = c.x;
+        y = c.y;
+      }
+      const uint32_t hi = bf16_pair(x, y, rx, ry);
+      lut[e] = make_uint2(hi, bf16_pair(rx, ry, u, v));
     }
   }
-  // <q, C_p> in fp32 (lanes over the dimensions, a fixed shuffle tree, lane 0's value to all)
-  __device__ float partition_base(const float* qs, int p, int lane) const {
-    const float* qrow = qs + m * 16;
-    const float* cp = C + (int64_t)p * d;
-    float v = 0.f;
-    for (int k = lane; k < d; k += 32) v = fmaf(qrow[k], cp[k], v);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return __shfl_sync(0xffffffffu, v, 0);
+  __device__ void stage_query(unsigned char* sm, int slot, int64_t q, int lane) const {
+    uint32_t* hi = reinterpret_cast<uint32_t*>(sm + (size_t)8 * steps * 16 * 8) + slot * query_stride();
+    uint32_t* lo = hi + 8 * tiles * query_stride();
+    for (int i = lane; i < 8 * steps; i += 32) {
+      float x = 0.f, y = 0.f, rx, ry, u, v;
+      if (q >= 0 && i < m) {
+        const float2 w = *reinterpret_cast<const float2*>(Qf + q * (int64_t)qstride + 2 * i);
+        x = w.x;
+        y = w.y;
+      }
+      hi[i] = bf16_pair(x, y, rx, ry);
+      lo[i] = bf16_pair(rx, ry, u, v);
+    }
   }
-  __device__ float score(const float* qs, int64_t, int64_t r, float base) const {
-    const uint4* x = reinterpret_cast<const uint4*>(codes + r * (int64_t)code_stride);
-    float acc = 0.f;
-    for (int c = 0; c < code_stride / 16; ++c) {
-      const uint4 v = __ldg(x + c);
-      const uint32_t wv[4] = {v.x, v.y, v.z, v.w};
+  __device__ void tile(const unsigned char* sm, int64_t r0, int64_t r1, int nt, int lane, float (&acc)[kTiles][4]) const {
+    const uint2* lut = reinterpret_cast<const uint2*>(sm);
+    const uint32_t* qhi = reinterpret_cast<const uint32_t*>(sm + (size_t)8 * steps * 16 * 8);
+    const uint32_t* qlo = qhi + 8 * tiles * query_stride();
+    const int g = lane >> 2, tig = lane & 3;
+    const int64_t ra = r0 + g, rb = ra + 8;
+    const uint32_t* xa = reinterpret_cast<const uint32_t*>(codes + (ra < r1 ? ra : r0) * code_stride);
+    const uint32_t* xb = reinterpret_cast<const uint32_t*>(codes + (rb < r1 ? rb : r0) * code_stride);
+    for (int ks = 0; ks < steps; ++ks) {          // (a row has at least 4 * steps bytes)
+      const uint32_t wa = __ldg(xa + ks) >> (4 * tig), wb = __ldg(xb + ks) >> (4 * tig);
+      const uint2* l0 = lut + (8 * ks + tig) * 16;
+      const uint2 a0 = l0[wa & 15u], a1 = l0[wb & 15u], a2 = l0[64 + ((wa >> 16) & 15u)], a3 = l0[64 + ((wb >> 16) & 15u)];
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int b = 0; b < 8; ++b) {
-          const int sidx = 32 * c + 8 * i + b;        // nibble b of word i of chunk c
-          if (sidx < m) acc += qs[16 * sidx + ((wv[i] >> (4 * b)) & 0xfu)];
+      for (int n = 0; n < kTiles; ++n)
+        if (n < nt) {
+          const int o = (8 * n + g) * query_stride() + 8 * ks + tig;
+          const uint32_t h0 = qhi[o], h1 = qhi[o + 4];
+          mma_bf16x16(acc[n], a0.x, a1.x, a2.x, a3.x, h0, h1);
+          mma_bf16x16(acc[n], a0.y, a1.y, a2.y, a3.y, h0, h1);
+          mma_bf16x16(acc[n], a0.x, a1.x, a2.x, a3.x, qlo[o], qlo[o + 4]);
         }
     }
-    return base + acc;
+  }
+  __device__ float row_factor(int64_t) const { return 0.f; }
+  __device__ float query_factor(int64_t, int64_t pair) const { return base[pair]; }
+  __device__ static float combine(float acc, float, float qf) { return qf + acc; }
+  __host__ __device__ int query_floats() const { return qstride; }
+  // this thread's shares of ||q||^2 and of sum_s max_j ||B[s][j]||^2, and its largest |<q, C_p>|
+  __device__ float3 stage_finish(float* qs, int64_t q, const float* bases, int tq) const {
+    float3 v = make_float3(0.f, 0.f, 0.f);
+    for (int i = threadIdx.x; i < qstride; i += kThreads) {
+      const float x = Qf[q * (int64_t)qstride + i];
+      qs[i] = x;
+      v.x = fmaf(x, x, v.x);
+    }
+    for (int s = threadIdx.x; s < m; s += kThreads) {
+      float most = 0.f;
+#pragma unroll
+      for (int j = 0; j < 16; ++j) {
+        const float2 c = reinterpret_cast<const float2*>(B)[16 * s + j];
+        most = fmaxf(most, fmaf(c.y, c.y, c.x * c.x));
+      }
+      v.y += most;
+    }
+    for (int j = threadIdx.x; j < tq; j += kThreads) v.z = fmaxf(v.z, fabsf(bases[j]));
+    return v;
+  }
+  // 3 * 2^-18 ||q|| ||r|| for the dropped parts, 2^-23 of it for each of the
+  // 3 d + d / 2 additions, and the rounding of base + sum; a factor to spare.
+  __device__ float delta(float3 v, int64_t, float) const {
+    const float qb = sqrtf(v.x) * sqrtf(v.y);
+    return qb * (ldexpf(1.f, -14) + ldexpf((float)d, -20)) + ldexpf(v.z + qb, -21);
+  }
+  __device__ float exact(const float* qs, int64_t, int64_t r, float pair_base) const {
+    const uint32_t* x = reinterpret_cast<const uint32_t*>(codes + r * (int64_t)code_stride);
+    float acc = 0.f;
+    for (int s = 0; s < m; ++s) {
+      const float2 c = reinterpret_cast<const float2*>(B)[16 * s + ((__ldg(x + s / 8) >> (4 * (s % 8))) & 15u)];
+      acc += fmaf(qs[2 * s + 1], c.y, qs[2 * s] * c.x);
+    }
+    return pair_base + acc;
   }
 };
 
-// Each probed pair's first position in its query's key slice: the sizes of
-// the query's earlier probed partitions added up (a thread per query).
+// base[e] = <q, C_p> of every probed pair in fp32 (a warp per pair: lanes over
+// the dimensions, a fixed shuffle tree).
+__global__ void pair_bases(const float* __restrict__ Qf, int qstride, const float* __restrict__ C, int d,
+                           const int32_t* __restrict__ top, const int32_t* __restrict__ tpq, int64_t q0, int64_t nq,
+                           int t, float* __restrict__ base) {
+  const int64_t e = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31;
+  if (e >= nq * t) return;
+  const int64_t q = q0 + e / t;
+  if (tpq && (int)(e % t) >= min(max(tpq[q], 0), t)) return;
+  const float* qrow = Qf + q * (int64_t)qstride;
+  const float* cp = C + (int64_t)top[q0 * t + e] * d;
+  float v = 0.f;
+  for (int k = lane; k < d; k += 32) v = fmaf(qrow[k], cp[k], v);
+  v = warp_sum(v);
+  if (lane == 0) base[e] = v;
+}
+
+// Each probed pair's first position in its query's slice (the sizes of the
+// query's earlier probed partitions added up) and the slice's length; a warp
+// per query.
 __global__ void pair_offsets(const int64_t* __restrict__ off, const int32_t* __restrict__ top,
                              const int32_t* __restrict__ tpq, int64_t q0, int64_t nq, int t,
                              int64_t* __restrict__ pos, int64_t* __restrict__ counts) {
-  const int64_t ql = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t ql = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31;
   if (ql >= nq) return;
   const int64_t q = q0 + ql;
   const int tq = tpq ? min(max(tpq[q], 0), t) : t;
   int64_t acc = 0;
-  for (int j = 0; j < tq; ++j) {
-    pos[ql * t + j] = acc;
-    const int p = top[q * (int64_t)t + j];
-    acc += off[p + 1] - off[p];
-  }
-  counts[ql] = acc;
-}
-
-// A warp per (query, probe) pair: the approximate score of every row of the
-// probed partition, written as a rank key at the pair's place in the query's
-// slice; a copy whose point has another copy in a partition the query probed
-// earlier writes the all-ones key instead (it sorts after every real key and
-// its id bits read as -1).
-template <typename Rows>
-__global__ void __launch_bounds__(32 * kSlWarps) approx_pairs(
-    Rows rows, const int32_t* __restrict__ ids, const int64_t* __restrict__ off, const int32_t* __restrict__ assign,
-    int a, const int32_t* __restrict__ top, const int32_t* __restrict__ tpq, int64_t q0, int64_t nq, int t,
-    int64_t slice, const int64_t* __restrict__ pos, uint64_t* __restrict__ keys) {
-  extern __shared__ __align__(16) unsigned char sl_smem[];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int64_t el = (int64_t)blockIdx.x * kSlWarps + w;   // pair within this chunk: ql * t + j
-  if (el >= nq * t) return;                               // uniform within the warp
-  const int64_t ql = el / t;
-  const int j = (int)(el - ql * t);
-  const int64_t q = q0 + ql;
-  const int tq = tpq ? min(max(tpq[q], 0), t) : t;
-  if (j >= tq) return;
-  const int per = rows.smem_floats();
-  float* qs = reinterpret_cast<float*>(sl_smem) + w * per;
-  int32_t* probes_s = reinterpret_cast<int32_t*>(reinterpret_cast<float*>(sl_smem) + kSlWarps * per) +
-                      w * kSlMaxProbesSmem;
-  rows.load(qs, q, lane);
-  const int32_t* probes = top + q * (int64_t)t;
-  if (j <= kSlMaxProbesSmem) {
-    for (int jj = lane; jj < j; jj += 32) probes_s[jj] = probes[jj];
-    probes = probes_s;
-  }
-  __syncwarp();
-  const int p = top[q * (int64_t)t + j];
-  const float base = rows.partition_base(qs, p, lane);
-  const int64_t r0 = off[p], r1 = off[p + 1];
-  uint64_t* out = keys + ql * slice + pos[el] - r0;
-  for (int64_t r = r0 + lane; r < r1; r += 32) {
-    const int32_t id = ids[r];
-    bool keep = true;
-    // the point's copy in an earlier-probed partition is the one that counts
-    for (int i = 0; i < a && keep; ++i) {
-      const int other = assign[(int64_t)id * a + i];
-      if (other == p) continue;
-      for (int jj = 0; jj < j; ++jj)
-        if (probes[jj] == other) { keep = false; break; }
+  for (int j0 = 0; j0 < tq; j0 += 32) {
+    const int j = j0 + lane;
+    int64_t v = 0;
+    if (j < tq) {
+      const int p = top[q * (int64_t)t + j];
+      v = off[p + 1] - off[p];
     }
-    out[r] = keep ? rank_key(rows.score(qs, q, r, base), (uint32_t)id) : ~0ull;
+    int64_t x = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int64_t y = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= o) x += y;
+    }
+    if (j < tq) pos[ql * t + j] = acc + x - v;
+    acc += __shfl_sync(0xffffffffu, x, 31);
+  }
+  if (lane == 0) counts[ql] = acc;
+}
+
+// Work items (partition, up to 8 * kTiles of its queries; blockIdx.y takes every
+// gridDim.y-th step of 128 rows): keys of every (query, row).  A key is the
+// order-preserving image of the score, 0 for a copy that does not count.  smax
+// (FP8, zero before the launch): the largest scale of the rows met, which are
+// positive and so ordered like their bits.
+template <typename Rows>
+__global__ void __launch_bounds__(kThreads) score_items(Rows rows, IvfWork work, const int32_t* __restrict__ ids,
+                                                        const int32_t* __restrict__ assign, int a,
+                                                        const int32_t* __restrict__ top, int64_t q0, int64_t slice,
+                                                        const int64_t* __restrict__ pos, uint32_t* __restrict__ keys,
+                                                        int* __restrict__ smax) {
+  constexpr unsigned kFull = 0xffffffffu;
+  constexpr int QB = 8 * Rows::kTiles;
+  constexpr int kMaxOther = 4;                  // copies of a point besides this one
+  extern __shared__ __align__(16) unsigned char sl_smem[];
+  __shared__ int64_t out_s[QB];                 // where the pair's keys start
+  __shared__ int32_t probes_s[QB][kProbesSmem + 1];
+  __shared__ int32_t j_s[QB];
+  __shared__ const int32_t* list_s[QB];         // the query's probes
+  __shared__ float qf_s[QB];
+  const int item = blockIdx.x;
+  if (item >= work.count()) return;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  // the item's partition: the last entry of item_base at or below it, 32 probes at a time
+  int oi = 0;
+  for (int len = work.c; len > 1;) {
+    const int step = (len + 31) / 32, at = oi + lane * step;
+    const unsigned below = __ballot_sync(kFull, lane * step < len && work.item_base[min(at, work.c)] <= item);
+    const int take = __popc(below) - 1;
+    oi += take * step;
+    len = min(step, len - take * step);
+  }
+  const int p = work.order[oi];
+  const int64_t e0 = work.pair_off[p] + (int64_t)(item - work.item_base[oi]) * work.qb;
+  const int nqi = (int)min((int64_t)work.qb, work.pair_off[p + 1] - e0);
+  const int64_t r0 = work.part_off[p], r1 = work.part_off[p + 1];
+  rows.stage_shared(sl_smem);
+  for (int i = w; i < 8 * rows.tiles; i += kWarps) {
+    const bool use = i < nqi;
+    int64_t ql = -1;
+    if (use) {
+      const int pr = work.pair_vals[e0 + i];    // ql * t + j
+      ql = pr / work.tmax;
+      const int j = (int)(pr - ql * work.tmax);
+      const int32_t* probes = top + (q0 + ql) * (int64_t)work.tmax;
+      if (lane == 0) {
+        out_s[i] = ql * slice + pos[pr];
+        j_s[i] = j;
+        list_s[i] = probes;
+        qf_s[i] = rows.query_factor(q0 + ql, pr);
+      }
+      if (j <= kProbesSmem)
+        for (int jj = lane; jj < j; jj += 32) probes_s[i][jj] = probes[jj];
+    }
+    rows.stage_query(sl_smem, i, use ? q0 + ql : -1, lane);
+  }
+  __syncthreads();
+  const int nt = (nqi + 7) / 8, g = lane >> 2, tig = lane & 3;
+  float most = 0.f;
+  for (int64_t t0 = r0 + 16 * (w + kWarps * (int64_t)blockIdx.y); t0 < r1; t0 += 16 * kWarps * (int64_t)gridDim.y) {
+    float acc[Rows::kTiles][4];
+#pragma unroll
+    for (int n = 0; n < Rows::kTiles; ++n)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) acc[n][i] = 0.f;
+    // lane l: the other partitions of row l % 16
+    int32_t other[kMaxOther] = {-1, -1, -1, -1};
+    float rf = 0.f;
+    if (t0 + (lane & 15) < r1) {
+      const int64_t r = t0 + (lane & 15);
+      const int32_t id = ids[r];
+      rf = rows.row_factor(r);
+      most = fmaxf(most, rf);
+      int at = 0;
+      for (int i = 0; i < a; ++i) {
+        const int v = assign[(int64_t)id * a + i];
+        if (v == p) continue;
+#pragma unroll
+        for (int u = 0; u < kMaxOther; ++u)
+          if (u == at) other[u] = v;
+        ++at;
+      }
+    }
+    rows.tile(sl_smem, t0, r1, nt, lane, acc);
+    const float rfa = __shfl_sync(kFull, rf, g), rfb = __shfl_sync(kFull, rf, g + 8);
+    // rows g and g + 8: which of the two have a copy in one of a query's earlier probes
+    int32_t oa[kMaxOther], ob[kMaxOther];
+#pragma unroll
+    for (int u = 0; u < kMaxOther; ++u) {
+      oa[u] = __shfl_sync(kFull, other[u], g);
+      ob[u] = __shfl_sync(kFull, other[u], g + 8);
+    }
+#pragma unroll
+    for (int n = 0; n < Rows::kTiles; ++n) {
+      if (n >= nt) break;
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        const int slot = 8 * n + 2 * tig + i;
+        if (slot >= nqi) continue;
+        const int j = j_s[slot];
+        const bool near = j <= kProbesSmem;
+        bool da = false, db = false;
+        for (int jj = 0; jj < j; ++jj) {
+          const int32_t pr = near ? probes_s[slot][jj] : list_s[slot][jj];
+          da = da || pr == oa[0];
+          db = db || pr == ob[0];
+          if (a > 2) {
+#pragma unroll
+            for (int u = 1; u < kMaxOther; ++u) {
+              da = da || pr == oa[u];
+              db = db || pr == ob[u];
+            }
+          }
+        }
+        uint32_t* out = keys + out_s[slot] + (t0 - r0) + g;
+        const float qf = qf_s[slot];
+        if (t0 + g < r1) out[0] = da ? 0u : float_key(Rows::combine(acc[n][i], rfa, qf));
+        if (t0 + g + 8 < r1) out[8] = db ? 0u : float_key(Rows::combine(acc[n][2 + i], rfb, qf));
+      }
+    }
+  }
+  if (smax) {
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) most = fmaxf(most, __shfl_xor_sync(kFull, most, o));
+    if (lane == 0 && __float_as_int(most) > __ldcg(smax)) atomicMax(smax, __float_as_int(most));
   }
 }
 
-// The R smallest keys of each query's slice -> their ids (cand [nq][R],
-// padded with -1 when the slice holds fewer than R keys).
-__global__ void __launch_bounds__(32 * kSlWarps) select_top_r(const uint64_t* __restrict__ keys,
-                                                              const int64_t* __restrict__ counts, int64_t nq,
-                                                              int64_t slice, int R, int32_t* __restrict__ cand) {
-  constexpr unsigned kFull = 0xffffffffu;
-  __shared__ int hist_all[kSlWarps][256];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int64_t ql = (int64_t)blockIdx.x * kSlWarps + w;
-  if (ql >= nq) return;
-  const uint64_t* K = keys + ql * slice;
-  const int64_t n = counts[ql];
-  int32_t* out = cand + ql * (int64_t)R;
-  int* hist = hist_all[w];
-  uint64_t limit = ~0ull;                 // keys <= limit are selected
-  if (n > R) {
-    uint64_t prefix = 0, mask = 0;
-    int64_t need = R;
-    for (int shift = 56; shift >= 0; shift -= 8) {
-      for (int b = lane; b < 256; b += 32) hist[b] = 0;
-      __syncwarp();
-      for (int64_t i = lane; i < n; i += 32) {
-        const uint64_t kk = K[i];
-        if ((kk & mask) == prefix) atomicAdd(&hist[(kk >> shift) & 0xff], 1);
-      }
-      __syncwarp();
-      // lane l owns bins 8l .. 8l+7; a warp scan of their sums finds the
-      // first bin whose inclusive count reaches `need`
-      int v[8], s = 0;
+// Exact fp32 <q, x> of a stored row, elements in ascending order.
+__device__ __forceinline__ float row_dot(const float* __restrict__ q, const float* __restrict__ x, int stride) {
+  float s = 0.f;
+#pragma unroll 8
+  for (int k = 0; k < stride; k += 4) {
+    const float4 v = __ldg(reinterpret_cast<const float4*>(x + k)), a = *reinterpret_cast<const float4*>(q + k);
+    s = fmaf(a.x, v.x, s);
+    s = fmaf(a.y, v.y, s);
+    s = fmaf(a.z, v.z, s);
+    s = fmaf(a.w, v.w, s);
+  }
+  return s;
+}
+__device__ __forceinline__ float row_dot(const float* __restrict__ q, const __nv_bfloat16* __restrict__ x, int stride) {
+  float s = 0.f;
+#pragma unroll 6
+  for (int k = 0; k < stride; k += 8) {
+    const uint4 v = __ldg(reinterpret_cast<const uint4*>(x + k));
+    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-      for (int i = 0; i < 8; ++i) { v[i] = hist[8 * lane + i]; s += v[i]; }
-      int incl = s;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(kFull, incl, o);
-        if (lane >= o) incl += y;
-      }
-      const int excl = incl - s;
-      const unsigned hit = __ballot_sync(kFull, incl >= need);
-      const int owner = __ffs(hit) - 1;           // need <= total, so some lane hits
-      int bin = 0, before = 0, in_bin = 0;
-      if (lane == owner) {
-        int c = excl;
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          if (c + v[i] >= need) { bin = 8 * lane + i; before = c; in_bin = v[i]; break; }
-          c += v[i];
+    for (int i = 0; i < 4; ++i) {
+      s = fmaf(q[k + 2 * i], __uint_as_float(w[i] << 16), s);
+      s = fmaf(q[k + 2 * i + 1], __uint_as_float(w[i] & 0xffff0000u), s);
+    }
+  }
+  return s;
+}
+
+constexpr int kBins = 2048;
+constexpr int kBand = 1024;         // rows near the R-th score ranked in the defined order
+constexpr int kSample = 8;          // keys a thread samples for the histogram's range
+
+// Ascending bitonic sort of buf[0, N), N a power of two (all threads).
+__device__ void block_sort(uint64_t* buf, int N) {
+  for (int size = 2; size <= N; size <<= 1)
+    for (int stride = size >> 1; stride > 0; stride >>= 1) {
+      for (int i = threadIdx.x; i < N / 2; i += kThreads) {
+        const int a = 2 * i - (i & (stride - 1)), b = a + stride;
+        const uint64_t x = buf[a], y = buf[b];
+        if ((x > y) == ((a & size) == 0)) {
+          buf[a] = y;
+          buf[b] = x;
         }
       }
-      bin = __shfl_sync(kFull, bin, owner);
-      before = __shfl_sync(kFull, before, owner);
-      in_bin = __shfl_sync(kFull, in_bin, owner);
-      prefix |= (uint64_t)bin << shift;
-      mask |= (uint64_t)0xff << shift;
-      if (before + in_bin == need || shift == 0) {   // the whole bin fits: done
-        limit = prefix | (shift ? (((uint64_t)1 << shift) - 1) : 0);
-        break;
-      }
-      need -= before;
-      __syncwarp();
+      __syncthreads();
     }
-  }
-  // every key below the limit, then keys equal to it (at most one real key:
-  // the keys are distinct) until R are taken; a dropped copy's all-ones key
-  // is never a real candidate, so the rest is padding
-  int64_t m = 0;
-  for (int pass = 0; pass < 2 && m < R; ++pass) {
-    if (pass == 1 && limit == ~0ull) break;
-    for (int64_t i0 = 0; i0 < n && m < R; i0 += 32) {
-      const int64_t i = i0 + lane;
-      const uint64_t kk = i < n ? K[i] : ~0ull;
-      const bool take = i < n && (pass == 0 ? kk < limit : kk == limit);
-      const unsigned bal = __ballot_sync(kFull, take);
-      const int64_t pos = m + __popc(bal & ((1u << lane) - 1u));
-      if (take && pos < R) out[pos] = (int32_t)(kk & 0xffffffffu);
-      m += __popc(bal);
-    }
-  }
-  for (int64_t i = min(m, (int64_t)R) + lane; i < R; i += 32) out[i] = -1;
 }
 
+// A block per query: the R best rows of its slice (see the file comment), their
+// exact scores, the best k.
+//   bins     the slice is counted in 2 048 linear bins over the range of a
+//            sample (rows outside it fall into the end bins, which keeps the
+//            bins ordered); the R-th best lies in one bin, and the bins within
+//            2 delta of that one are the band
+//   list     every row above the band, then the band's best in the defined
+//            order.  A band that does not fit (thousands of near-equal scores,
+//            or infinities) is resolved by a radix select over all rows'
+//            defined keys instead.
+//   rescore  a thread per row; the best k by per-warp sorted lists (k <= 32) or
+//            a sort
+// Bound: the latency of two passes over the slice (L2) and of the scattered
+// rows; 256 threads and about 30 KB of shared memory leave seven blocks an SM
+// to hide it.
+template <typename Rows, typename OT>
+__global__ void __launch_bounds__(kThreads) finish_slices(
+    Rows rows, const uint32_t* __restrict__ keys, const int64_t* __restrict__ counts, int64_t slice,
+    const int64_t* __restrict__ pos, const int32_t* __restrict__ top, const int32_t* __restrict__ tpq, int64_t q0,
+    int t, const int64_t* __restrict__ off, const int32_t* __restrict__ ids, const float* __restrict__ base,
+    const float* __restrict__ smax, const void* __restrict__ Q, int qdt, int d, const OT* __restrict__ orig,
+    int ostride, int R, int k, int64_t* __restrict__ ids_out, float* __restrict__ scores_out) {
+  constexpr unsigned kFull = 0xffffffffu;
+  extern __shared__ __align__(16) unsigned char fs_smem[];
+  __shared__ int32_t warp_s[32];
+  __shared__ float red_s[5][kWarps];
+  __shared__ int n_list, n_band, bin_s, above_s;
+  __shared__ float lo_s, hi_s, delta_s;
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  const int64_t ql = blockIdx.x, q = q0 + ql;
+  const uint32_t* K = keys + ql * slice;
+  const int n = (int)counts[ql];
+  const int tq = tpq ? min(max(tpq[q], 0), t) : t;
+  const int64_t* qpos = pos + ql * t;
+  const int32_t* probes = top + q * (int64_t)t;
+  // shared memory: query row, query for the defined order, histogram / band, list, exact keys
+  float* qrow = reinterpret_cast<float*>(fs_smem);
+  float* qs = qrow + (ostride + 3) / 4 * 4;
+  int* hist = reinterpret_cast<int*>(qs + (rows.query_floats() + 3) / 4 * 4);
+  uint64_t* band_key = reinterpret_cast<uint64_t*>(hist);                 // over the histogram once the bin is known
+  int32_t* band = reinterpret_cast<int32_t*>(hist + kBins);               // [kBand]
+  int32_t* list = band + kBand;                                           // [R] positions in the slice, then ids
+  uint64_t* ex = reinterpret_cast<uint64_t*>(list + (R + 1) / 2 * 2);     // [pow2 >= R]
+
+  for (int i = tid; i < ostride; i += kThreads)
+    qrow[i] = i >= d ? 0.f
+              : qdt == SOAR_F32 ? static_cast<const float*>(Q)[q * d + i]
+                                : __bfloat162float(static_cast<const __nv_bfloat16*>(Q)[q * d + i]);
+  float3 norms = rows.stage_finish(qs, q, base ? base + ql * t : nullptr, tq);
+  norms.x = warp_sum(norms.x);
+  norms.y = warp_sum(norms.y);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) norms.z = fmaxf(norms.z, __shfl_xor_sync(kFull, norms.z, o));
+  if (tid == 0) n_list = n_band = 0;
+  for (int i = tid; i < kBins; i += kThreads) hist[i] = 0;
+  // a sample's range
+  float lo = INFINITY, hi = -INFINITY;
+  for (int u = 0; u < kSample; ++u) {
+    const int64_t i = (int64_t)(u * kThreads + tid) * n / (kSample * kThreads);
+    const uint32_t key = i < n ? K[i] : 0u;
+    if (key) {
+      const float s = key_float(key);
+      lo = fminf(lo, s);
+      hi = fmaxf(hi, s);
+    }
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    lo = fminf(lo, __shfl_xor_sync(kFull, lo, o));
+    hi = fmaxf(hi, __shfl_xor_sync(kFull, hi, o));
+  }
+  if (lane == 0) {
+    red_s[0][w] = lo;
+    red_s[1][w] = hi;
+    red_s[2][w] = norms.x;
+    red_s[3][w] = norms.y;
+    red_s[4][w] = norms.z;
+  }
+  __syncthreads();
+  if (tid == 0) {
+    for (int u = 1; u < kWarps; ++u) {
+      lo = fminf(lo, red_s[0][u]);
+      hi = fmaxf(hi, red_s[1][u]);
+      norms.x += red_s[2][u];
+      norms.y += red_s[3][u];
+      norms.z = fmaxf(norms.z, red_s[4][u]);
+    }
+    lo_s = lo;
+    hi_s = hi;
+    delta_s = rows.delta(norms, q, smax ? *smax : 0.f);
+  }
+  __syncthreads();
+  lo = lo_s;
+  hi = hi_s;
+  const float delta = delta_s;
+  // position i of the slice: its probe, then its row
+  const auto probe_of = [&](int64_t i) {
+    int a = 0, b = tq - 1;
+    while (a < b) {
+      const int mid = (a + b + 1) >> 1;
+      if (qpos[mid] <= i) a = mid;
+      else b = mid - 1;
+    }
+    return a;
+  };
+  const auto defined_key = [&](int64_t i) {
+    const int j = probe_of(i);
+    const int64_t r = off[probes[j]] + (i - qpos[j]);
+    return rank_key(rows.exact(qs, q, r, base ? base[ql * t + j] : 0.f), (uint32_t)ids[r]);
+  };
+  const auto append = [&](bool in, int* count, int32_t* to, int cap, int32_t v) {
+    const unsigned b = __ballot_sync(kFull, in);
+    int at = 0;
+    if (lane == 0 && b) at = atomicAdd(count, __popc(b));
+    at = __shfl_sync(kFull, at, 0) + __popc(b & ((1u << lane) - 1u));
+    if (in && at < cap) to[at] = v;
+  };
+
+  const float scale = (float)(kBins - 1) / (hi - lo);
+  // linear bins need a finite range; a few keys need no histogram
+  bool linear = scale > 0.f && scale < INFINITY && delta < INFINITY;
+  const auto bin_of = [&](uint32_t key) {
+    return (int)fminf(fmaxf((key_float(key) - lo) * scale, 0.f), (float)(kBins - 1));
+  };
+  int total = 0;                                        // rows that count
+  if (linear) {
+#pragma unroll 4
+    for (int i = tid; i < n; i += kThreads) {
+      const uint32_t key = K[i];
+      if (key) atomicAdd(&hist[bin_of(key)], 1);
+    }
+    __syncthreads();
+    // from the top: thread l owns bins kBins - 1 - 8 l ... ; the bin of the R-th best
+    constexpr int kOwn = kBins / kThreads;
+    int mine = 0;
+#pragma unroll
+    for (int u = 0; u < kOwn; ++u) mine += hist[kBins - 1 - (tid * kOwn + u)];
+    const int before = block_exclusive_scan<int>(mine, warp_s, total);
+    if (before < R && before + mine >= R) {
+      int c = before;
+      for (int u = 0; u < kOwn; ++u) {
+        const int b = kBins - 1 - (tid * kOwn + u);
+        c += hist[b];
+        if (c >= R) {
+          bin_s = b;
+          break;
+        }
+      }
+    }
+    __syncthreads();
+    if (total > R) {
+      const float wide = ceilf(2.f * delta * scale) + 1.f;
+      const int mb = wide < (float)kBins ? (int)wide : kBins;
+      const int b_lo = max(0, bin_s - mb), b_hi = min(kBins - 1, bin_s + mb);
+      // rows in the band
+      int in_band = 0;
+      for (int b = b_lo + tid; b <= b_hi; b += kThreads) in_band += hist[b];
+      int m;
+      block_exclusive_scan<int>(in_band, warp_s, m);
+      if (m > kBand) {
+        linear = false;
+      } else {
+#pragma unroll 4
+        for (int i0 = 0; i0 < n; i0 += kThreads) {
+          const int i = i0 + tid;
+          const uint32_t key = i < n ? K[i] : 0u;
+          const int b = key ? bin_of(key) : -1;
+          append(b > b_hi, &n_list, list, R, i);
+          append(b >= b_lo && b <= b_hi, &n_band, band, kBand, i);
+        }
+        __syncthreads();
+        int N = 2;
+        while (N < m) N <<= 1;
+        for (int i = tid; i < N; i += kThreads) band_key[i] = ~0ull;      // (the histogram is no longer read)
+        __syncthreads();
+        for (int i = tid; i < m; i += kThreads) band_key[i] = defined_key(band[i]);
+        __syncthreads();
+        block_sort(band_key, N);
+        // the list's rows as ids, then the band's best
+        const int have = n_list;
+        for (int i = tid; i < have; i += kThreads) {
+          const int j = probe_of(list[i]);
+          list[i] = ids[off[probes[j]] + (list[i] - qpos[j])];
+        }
+        for (int i = tid; i < R - have; i += kThreads) list[have + i] = (int32_t)(band_key[i] & 0xffffffffu);
+        __syncthreads();
+        if (tid == 0) n_list = R;
+      }
+    }
+  }
+  __syncthreads();
+  if (!linear || total <= R) {
+    // every row that counts, or (more than R of them) those up to the R-th
+    // smallest defined key, found byte by byte
+    uint64_t limit = ~0ull;
+    if (!linear) {
+      int cnt = 0;
+      for (int i = tid; i < n; i += kThreads) cnt += K[i] != 0u;
+      block_exclusive_scan<int>(cnt, warp_s, total);
+    }
+    if (total > R) {
+      uint64_t prefix = 0, mask = 0;
+      int need = R;
+      for (int shift = 56; shift >= 0; shift -= 8) {
+        __syncthreads();
+        for (int i = tid; i < 256; i += kThreads) hist[i] = 0;
+        __syncthreads();
+        for (int i = tid; i < n; i += kThreads) {
+          if (!K[i]) continue;
+          const uint64_t kk = defined_key(i);
+          if ((kk & mask) == prefix) atomicAdd(&hist[(kk >> shift) & 0xff], 1);
+        }
+        __syncthreads();
+        if (tid == 0) {
+          int b = 0, c = 0;
+          while (b < 255 && c + hist[b] < need) c += hist[b++];
+          bin_s = b;
+          above_s = c;
+        }
+        __syncthreads();
+        need -= above_s;
+        prefix |= (uint64_t)bin_s << shift;
+        mask |= (uint64_t)0xff << shift;
+      }
+      limit = prefix;
+    }
+    __syncthreads();
+    if (tid == 0) n_list = 0;
+    __syncthreads();
+    for (int i0 = 0; i0 < n; i0 += kThreads) {
+      const int i = i0 + tid;
+      const bool counts_ = i < n && K[i] != 0u;
+      const bool in = counts_ && (limit == ~0ull || defined_key(i) <= limit);
+      int32_t id = -1;
+      if (in) {
+        const int j = probe_of(i);
+        id = ids[off[probes[j]] + (i - qpos[j])];
+      }
+      append(in, &n_list, list, R, id);
+    }
+    __syncthreads();
+  }
+  // ---- exact scores of the listed rows, the best k
+  const int have = min(n_list, R);
+  if (k <= 32) {
+    uint64_t best = ~0ull, thr = ~0ull;         // lane j < k: the warp's j-th best key
+    const auto insert = [&](uint64_t key) {
+      unsigned bal = __ballot_sync(kFull, key < thr);
+      while (bal) {
+        const int src = __ffs(bal) - 1;
+        bal &= bal - 1;
+        const uint64_t kk = __shfl_sync(kFull, key, src);
+        if (kk >= thr) continue;
+        const int at = __popc(__ballot_sync(kFull, lane < k && best < kk));
+        const uint64_t up = __shfl_up_sync(kFull, best, 1);
+        if (lane > at && lane < k) best = up;
+        if (lane == at) best = kk;
+        thr = __shfl_sync(kFull, best, k - 1);
+      }
+    };
+    for (int i0 = 32 * w; i0 < have; i0 += kThreads) {
+      const int i = i0 + lane;
+      uint64_t key = ~0ull;
+      if (i < have) {
+        const int32_t id = list[i];
+        const float s = row_dot(qrow, orig + (int64_t)id * ostride, ostride);
+        if (s == s) key = rank_key(s, (uint32_t)id);
+      }
+      insert(key);
+    }
+    ex[32 * w + lane] = lane < k ? best : ~0ull;
+    __syncthreads();
+    if (w == 0) {
+      for (int u = 1; u < kWarps; ++u) insert(ex[32 * u + lane]);
+      if (lane < k) {
+        ids_out[q * k + lane] = best != ~0ull ? (int64_t)(uint32_t)(best & 0xffffffffu) : -1;
+        scores_out[q * k + lane] = best != ~0ull ? key_float(~(uint32_t)(best >> 32)) : -INFINITY;
+      }
+    }
+  } else {
+    int N = 2;
+    while (N < max(have, k)) N <<= 1;           // (k <= R: within ex)
+    for (int i = tid; i < N; i += kThreads) {
+      uint64_t key = ~0ull;
+      if (i < have) {
+        const int32_t id = list[i];
+        const float s = row_dot(qrow, orig + (int64_t)id * ostride, ostride);
+        if (s == s) key = rank_key(s, (uint32_t)id);
+      }
+      ex[i] = key;
+    }
+    __syncthreads();
+    block_sort(ex, N);
+    for (int i = tid; i < k; i += kThreads) {
+      const uint64_t key = ex[i];
+      ids_out[q * k + i] = key != ~0ull ? (int64_t)(uint32_t)(key & 0xffffffffu) : -1;
+      scores_out[q * k + i] = key != ~0ull ? key_float(~(uint32_t)(key >> 32)) : -INFINITY;
+    }
+  }
+}
+
+// Queries per pass, so that the keys stay within 2 GB.
+int64_t key_chunk(int64_t slice, int64_t nq) {
+  return std::min(nq, std::max<int64_t>(8, ((int64_t)1 << 29) / slice));
+}
 
 template <typename Rows>
-void run_shortlist(const IndexData& ix, const Rows& rws, const int32_t* top, const int32_t* tpq, int64_t nq, int t,
-                   int R, int32_t* cand, cudaStream_t s, Scratch& scr) {
+void run(const IndexData& ix, Rows rws, float* base, int* smax, const float* Qf, int qstride, const void* Q,
+         soar_dtype dt, const int32_t* top, const int32_t* tpq, int64_t nq, int t, int R, int k, int64_t* ids_out,
+         float* scores_out, cudaStream_t s, Scratch& scr) {
+  rws.tiles = Rows::kTiles;
+  while (rws.tiles > 1 && rws.item_smem() > 180 * 1024) --rws.tiles;     // wide rows: fewer queries an item
+  const int QB = 8 * rws.tiles;
   const int64_t slice = std::max<int64_t>(1, std::min<int64_t>((int64_t)t * ix.max_partition, ix.rows));
-  // queries per pass so that the key buffer stays within 2 GB
-  const int64_t chunk = std::max<int64_t>(kSlWarps, std::min<int64_t>(nq, ((int64_t)1 << 28) / slice));
-  const int64_t cq = std::min(chunk, nq);
-  uint64_t* keys = scr.get<uint64_t>((size_t)cq * slice);
+  const int64_t cq = key_chunk(slice, nq);
+  uint32_t* keys = scr.get<uint32_t>((size_t)cq * slice);
   int64_t* counts = scr.get<int64_t>(cq);
   int64_t* pos = scr.get<int64_t>((size_t)cq * t);
-  const size_t smem = (size_t)kSlWarps * rws.smem_floats() * sizeof(float) + (size_t)kSlWarps * kSlMaxProbesSmem * 4;
-  SOAR_CUDA(cudaFuncSetAttribute(approx_pairs<Rows>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  int32_t* inv = scr.get<int32_t>((size_t)cq * t);
   const int a = 1 + ix.spills;
+  const int ostride = ix.dtype == SOAR_F32 ? (ix.d + 3) / 4 * 4 : (ix.d + 7) / 8 * 8;
+  int sorted = kThreads;                                  // exact keys: the warps' lists, or R of them to sort
+  if (k > 32)
+    while (sorted < R) sorted <<= 1;
+  const size_t fin_smem = sizeof(float) * ((size_t)(ostride + 3) / 4 * 4 + (rws.query_floats() + 3) / 4 * 4) +
+                          sizeof(int) * (size_t)(kBins + kBand) + sizeof(int32_t) * (size_t)((R + 1) / 2 * 2) +
+                          sizeof(uint64_t) * (size_t)sorted;
+  const size_t item_smem = rws.item_smem();
+  SOAR_CUDA(cudaFuncSetAttribute(score_items<Rows>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)item_smem));
+  const auto finish = [&](auto elem, int64_t q0, int64_t m) {
+    using OT = decltype(elem);
+    auto kern = finish_slices<Rows, OT>;
+    SOAR_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fin_smem));
+    kern<<<(unsigned)m, kThreads, fin_smem, s>>>(rws, keys, counts, slice, pos, top, tpq, q0, t, ix.offsets, ix.ids,
+                                                 base, reinterpret_cast<const float*>(smax), Q, (int)dt, ix.d, static_cast<const OT*>(ix.originals),
+                                                 ostride, R, k, ids_out, scores_out);
+    SOAR_LAUNCHED();
+  };
   for (int64_t q0 = 0; q0 < nq; q0 += cq) {
     const int64_t m = std::min(cq, nq - q0);
-    pair_offsets<<<ceil_div(m, 128), 128, 0, s>>>(ix.offsets, top, tpq, q0, m, t, pos, counts);
+    Scratch cs(s);
+    const int32_t* tp = tpq ? tpq + q0 : nullptr;
+    const Grouped g = group_pairs(ix, m, t, tp, QB, top + q0 * t, inv, s, cs, false, false);
+    stage_mark(s, "scan", true);
+    pair_offsets<<<ceil_div(m * 32, 256), 256, 0, s>>>(ix.offsets, top, tpq, q0, m, t, pos, counts);
     SOAR_LAUNCHED();
-    approx_pairs<Rows><<<ceil_div(m * t, kSlWarps), 32 * kSlWarps, smem, s>>>(rws, ix.ids, ix.offsets, ix.assign, a,
-                                                                              top, tpq, q0, m, t, slice, pos, keys);
+    if (base) {
+      pair_bases<<<ceil_div(m * t * 32, 256), 256, 0, s>>>(Qf, qstride, ix.centroids, ix.d, top, tpq, q0, m, t, base);
+      SOAR_LAUNCHED();
+    }
+    // a batch of few pairs splits each partition's rows over several blocks
+    const int64_t items = std::min<int64_t>(m * t, g.max_items);
+    const unsigned split = (unsigned)std::max<int64_t>(1, std::min<int64_t>(16, 8 * num_sms() / std::max<int64_t>(1, items)));
+    const IvfWork work{ix.offsets, g.pair_off, g.vals, g.order, g.item_base, ix.c, t, QB};
+    score_items<Rows><<<dim3((unsigned)items, split), kThreads, item_smem, s>>>(rws, work, ix.ids, ix.assign, a, top,
+                                                                               q0, slice, pos, keys, smax);
     SOAR_LAUNCHED();
-    select_top_r<<<ceil_div(m, kSlWarps), 32 * kSlWarps, 0, s>>>(keys, counts, m, slice, R, cand + q0 * R);
-    SOAR_LAUNCHED();
+    stage_mark(s, "scan", false);
+    stage_mark(s, "rescore", true);
+    if (ix.dtype == SOAR_F32) finish(float{}, q0, m);
+    else finish(__nv_bfloat16{}, q0, m);
+    stage_mark(s, "rescore", false);
   }
 }
 
 }  // namespace
 
-void fp8_shortlist(const IndexData& ix, const float* Qf, const float* qscale, const int32_t* top,
-                   const int32_t* tpq, int64_t nq, int t, int R, int32_t* cand, cudaStream_t s, Scratch& scr) {
-  const Fp8Rows rws{static_cast<const uint8_t*>(ix.vectors), ix.code_stride, ix.row_scales, Qf, qscale};
-  run_shortlist(ix, rws, top, tpq, nq, t, R, cand, s, scr);
+void fp8_search(const IndexData& ix, const float* Qf, const float* qscale, const void* Q, soar_dtype dt,
+                const int32_t* top, const int32_t* tpq, int64_t nq, int t, int R, int k, int64_t* ids_out,
+                float* scores_out, cudaStream_t s, Scratch& scr) {
+  int* smax = scr.get<int>(1);
+  SOAR_CUDA(cudaMemsetAsync(smax, 0, sizeof(int), s));
+  const Fp8Rows rws{static_cast<const uint8_t*>(ix.vectors), ix.code_stride, ix.row_scales, Qf, qscale,
+                    (ix.code_stride + 63) / 64, 0};
+  run(ix, rws, nullptr, smax, Qf, ix.code_stride, Q, dt, top, tpq, nq, t, R, k,
+      ids_out, scores_out, s, scr);
 }
 
-void pq_shortlist(const IndexData& ix, const float* Qf, int qstride, const int32_t* top, const int32_t* tpq,
-                  int64_t nq, int t, int R, int32_t* cand, cudaStream_t s, Scratch& scr) {
-  const Pq4Rows rws{static_cast<const uint8_t*>(ix.vectors), ix.code_stride, ix.pq_m, ix.d, ix.pq_cb, ix.centroids,
-                    Qf, qstride};
-  run_shortlist(ix, rws, top, tpq, nq, t, R, cand, s, scr);
+void pq_search(const IndexData& ix, const float* Qf, int qstride, const void* Q, soar_dtype dt, const int32_t* top,
+               const int32_t* tpq, int64_t nq, int t, int R, int k, int64_t* ids_out, float* scores_out,
+               cudaStream_t s, Scratch& scr) {
+  const int64_t slice = std::max<int64_t>(1, std::min<int64_t>((int64_t)t * ix.max_partition, ix.rows));
+  float* base = scr.get<float>((size_t)key_chunk(slice, nq) * t);
+  const Pq4Rows rws{static_cast<const uint8_t*>(ix.vectors), ix.code_stride, ix.pq_m, ix.d, ix.pq_cb, Qf, qstride,
+                    base, (ix.pq_m + 7) / 8, 0};
+  run(ix, rws, base, nullptr, Qf, qstride, Q, dt, top, tpq, nq, t, R, k, ids_out, scores_out, s, scr);
 }
 
 }  // namespace soar
