@@ -167,7 +167,7 @@ struct Fp8Rows {
 // a code is one shared-memory read of its centre (hi and lo parts); centres and
 // queries enter as hi + lo and the lo lo product is dropped.
 struct Pq4Rows {
-  static constexpr int kTiles = 8;
+  static constexpr int kTiles = 4;      // (eight took 122 registers: two blocks an SM, 1 346 us)
   const uint8_t* codes;
   int code_stride, m, d;
   const float* B;         // [m][16][2]
@@ -177,9 +177,10 @@ struct Pq4Rows {
   int steps;              // K steps of 8 subspaces
   int tiles;
 
-  __host__ __device__ int query_stride() const { return 8 * steps + 4; }   // words a part; + 4: conflict-free reads
+  // a query's K step holds, for each lane % 4, its four operand words (hi, hi + 4 pairs on, lo, lo + 4 pairs on)
+  __host__ __device__ int query_stride() const { return 64 * steps + 16; }   // bytes; + 16: conflict-free reads
   __host__ __device__ size_t item_smem() const {
-    return (size_t)8 * steps * 16 * 8 + (size_t)2 * 8 * tiles * query_stride() * 4;
+    return (size_t)8 * steps * 16 * 8 + (size_t)8 * tiles * query_stride();
   }
   __device__ void stage_shared(unsigned char* sm) const {
     uint2* lut = reinterpret_cast<uint2*>(sm);
@@ -195,8 +196,7 @@ struct Pq4Rows {
     }
   }
   __device__ void stage_query(unsigned char* sm, int slot, int64_t q, int lane) const {
-    uint32_t* hi = reinterpret_cast<uint32_t*>(sm + (size_t)8 * steps * 16 * 8) + slot * query_stride();
-    uint32_t* lo = hi + 8 * tiles * query_stride();
+    uint32_t* dst = reinterpret_cast<uint32_t*>(sm + (size_t)8 * steps * 16 * 8 + slot * query_stride());
     for (int i = lane; i < 8 * steps; i += 32) {
       float x = 0.f, y = 0.f, rx, ry, u, v;
       if (q >= 0 && i < m) {
@@ -204,18 +204,19 @@ struct Pq4Rows {
         x = w.x;
         y = w.y;
       }
-      hi[i] = bf16_pair(x, y, rx, ry);
-      lo[i] = bf16_pair(rx, ry, u, v);
+      uint32_t* at = dst + 16 * (i / 8) + 4 * (i % 4) + (i / 4) % 2;
+      at[0] = bf16_pair(x, y, rx, ry);
+      at[2] = bf16_pair(rx, ry, u, v);
     }
   }
   __device__ void tile(const unsigned char* sm, int64_t r0, int64_t r1, int nt, int lane, float (&acc)[kTiles][4]) const {
     const uint2* lut = reinterpret_cast<const uint2*>(sm);
-    const uint32_t* qhi = reinterpret_cast<const uint32_t*>(sm + (size_t)8 * steps * 16 * 8);
-    const uint32_t* qlo = qhi + 8 * tiles * query_stride();
+    const unsigned char* qw = sm + (size_t)8 * steps * 16 * 8 + (lane >> 2) * query_stride() + 16 * (lane & 3);
     const int g = lane >> 2, tig = lane & 3;
     const int64_t ra = r0 + g, rb = ra + 8;
     const uint32_t* xa = reinterpret_cast<const uint32_t*>(codes + (ra < r1 ? ra : r0) * code_stride);
     const uint32_t* xb = reinterpret_cast<const uint32_t*>(codes + (rb < r1 ? rb : r0) * code_stride);
+#pragma unroll 2
     for (int ks = 0; ks < steps; ++ks) {          // (a row has at least 4 * steps bytes)
       const uint32_t wa = __ldg(xa + ks) >> (4 * tig), wb = __ldg(xb + ks) >> (4 * tig);
       const uint2* l0 = lut + (8 * ks + tig) * 16;
@@ -223,11 +224,10 @@ struct Pq4Rows {
 #pragma unroll
       for (int n = 0; n < kTiles; ++n)
         if (n < nt) {
-          const int o = (8 * n + g) * query_stride() + 8 * ks + tig;
-          const uint32_t h0 = qhi[o], h1 = qhi[o + 4];
-          mma_bf16x16(acc[n], a0.x, a1.x, a2.x, a3.x, h0, h1);
-          mma_bf16x16(acc[n], a0.y, a1.y, a2.y, a3.y, h0, h1);
-          mma_bf16x16(acc[n], a0.x, a1.x, a2.x, a3.x, qlo[o], qlo[o + 4]);
+          const uint4 v = *reinterpret_cast<const uint4*>(qw + 8 * n * query_stride() + 64 * ks);
+          mma_bf16x16(acc[n], a0.x, a1.x, a2.x, a3.x, v.x, v.y);
+          mma_bf16x16(acc[n], a0.y, a1.y, a2.y, a3.y, v.x, v.y);
+          mma_bf16x16(acc[n], a0.x, a1.x, a2.x, a3.x, v.z, v.w);
         }
     }
   }
@@ -380,30 +380,50 @@ __global__ void __launch_bounds__(kThreads) score_items(Rows rows, IvfWork work,
   __syncthreads();
   const int nt = (nqi + 7) / 8, g = lane >> 2, tig = lane & 3;
   float most = 0.f;
-  for (int64_t t0 = r0 + 16 * (w + kWarps * (int64_t)blockIdx.y); t0 < r1; t0 += 16 * kWarps * (int64_t)gridDim.y) {
+  const int64_t step = 16 * kWarps * (int64_t)gridDim.y;
+  int64_t t0 = r0 + 16 * (w + kWarps * (int64_t)blockIdx.y);
+  const auto fetch_id = [&](int64_t tile) { return tile + (lane & 15) < r1 ? ids[tile + (lane & 15)] : -1; };
+  int32_t id = fetch_id(t0), next_id = fetch_id(t0 + step), next_other = -1;
+  float next_rf = 0.f;
+  const auto fetch_row = [&](int64_t tile) {      // of the rows whose ids are in `id`
+    next_other = -1;
+    next_rf = 0.f;
+    if (id < 0) return;
+    next_rf = rows.row_factor(tile + (lane & 15));
+    if (a == 2) {
+      const int2 v = __ldg(reinterpret_cast<const int2*>(assign) + id);
+      next_other = v.x == p ? v.y : v.x;
+    }
+  };
+  fetch_row(t0);
+  for (; t0 < r1; t0 += step) {
     float acc[Rows::kTiles][4];
 #pragma unroll
     for (int n = 0; n < Rows::kTiles; ++n)
 #pragma unroll
       for (int i = 0; i < 4; ++i) acc[n][i] = 0.f;
     // lane l: the other partitions of row l % 16
-    int32_t other[kMaxOther] = {-1, -1, -1, -1};
-    float rf = 0.f;
-    if (t0 + (lane & 15) < r1) {
-      const int64_t r = t0 + (lane & 15);
-      const int32_t id = ids[r];
-      rf = rows.row_factor(r);
-      most = fmaxf(most, rf);
-      int at = 0;
-      for (int i = 0; i < a; ++i) {
-        const int v = assign[(int64_t)id * a + i];
-        if (v == p) continue;
+    int32_t other[kMaxOther] = {next_other, -1, -1, -1};
+    const float rf = next_rf;
+    most = fmaxf(most, rf);
+    if (a > 2) {
+      other[0] = -1;
+      if (id >= 0) {
+        int at = 0;
+        for (int i = 0; i < a; ++i) {
+          const int v = assign[(int64_t)id * a + i];
+          if (v == p) continue;
 #pragma unroll
-        for (int u = 0; u < kMaxOther; ++u)
-          if (u == at) other[u] = v;
-        ++at;
+          for (int u = 0; u < kMaxOther; ++u)
+            if (u == at) other[u] = v;
+          ++at;
+        }
       }
     }
+    // the next step's assignments and the ids of the step after it are on their way during this one
+    id = next_id;
+    fetch_row(t0 + step);
+    next_id = fetch_id(t0 + 2 * step);
     rows.tile(sl_smem, t0, r1, nt, lane, acc);
     const float rfa = __shfl_sync(kFull, rf, g), rfb = __shfl_sync(kFull, rf, g + 8);
     // rows g and g + 8: which of the two have a copy in one of a query's earlier probes
@@ -479,7 +499,11 @@ __device__ __forceinline__ float row_dot(const float* __restrict__ q, const __nv
 
 constexpr int kBins = 2048;
 constexpr int kBand = 1024;         // rows near the R-th score ranked in the defined order
-constexpr int kSample = 8;          // keys a thread samples for the histogram's range
+constexpr int kSample = 8;          // keys a thread samples
+
+// Rows of a slice kept in shared memory: those at or above a bound that a
+// sample puts somewhat below the R-th best.
+__host__ __device__ inline int kept_rows(int R) { return 2 * R + 1024; }
 
 // Ascending bitonic sort of buf[0, N), N a power of two (all threads).
 __device__ void block_sort(uint64_t* buf, int N) {
@@ -499,19 +523,20 @@ __device__ void block_sort(uint64_t* buf, int N) {
 
 // A block per query: the R best rows of its slice (see the file comment), their
 // exact scores, the best k.
-//   bins     the slice is counted in 2 048 linear bins over the range of a
-//            sample (rows outside it fall into the end bins, which keeps the
-//            bins ordered); the R-th best lies in one bin, and the bins within
-//            2 delta of that one are the band
+//   keep     2 048 sampled keys put a bound somewhat below the R-th best; the
+//            rows at or above it go to shared memory in one pass over the slice
+//            (where the sample misleads, the passes below run over the slice)
+//   bins     the kept rows are counted in 2 048 linear bins (keys outside their
+//            range fall into the end bins, which keeps the bins ordered); the
+//            R-th best lies in one bin, and the bins within 2 delta of that
+//            one are the band
 //   list     every row above the band, then the band's best in the defined
 //            order.  A band that does not fit (thousands of near-equal scores,
 //            or infinities) is resolved by a radix select over all rows'
 //            defined keys instead.
 //   rescore  a thread per row; the best k by per-warp sorted lists (k <= 32) or
 //            a sort
-// Bound: the latency of two passes over the slice (L2) and of the scattered
-// rows; 256 threads and about 30 KB of shared memory leave seven blocks an SM
-// to hide it.
+// Bound: the latency of one pass over the slice and of the scattered rows.
 template <typename Rows, typename OT>
 __global__ void __launch_bounds__(kThreads) finish_slices(
     Rows rows, const uint32_t* __restrict__ keys, const int64_t* __restrict__ counts, int64_t slice,
@@ -523,7 +548,7 @@ __global__ void __launch_bounds__(kThreads) finish_slices(
   extern __shared__ __align__(16) unsigned char fs_smem[];
   __shared__ int32_t warp_s[32];
   __shared__ float red_s[5][kWarps];
-  __shared__ int n_list, n_band, bin_s, above_s;
+  __shared__ int n_list, n_band, n_kept, bin_s, above_s;
   __shared__ float lo_s, hi_s, delta_s;
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   const int64_t ql = blockIdx.x, q = q0 + ql;
@@ -532,14 +557,18 @@ __global__ void __launch_bounds__(kThreads) finish_slices(
   const int tq = tpq ? min(max(tpq[q], 0), t) : t;
   const int64_t* qpos = pos + ql * t;
   const int32_t* probes = top + q * (int64_t)t;
-  // shared memory: query row, query for the defined order, histogram / band, list, exact keys
+  // shared memory: query row, query for the defined order, histogram / band
+  // keys, band, list, kept rows / exact keys
+  const int cap = kept_rows(R);
   float* qrow = reinterpret_cast<float*>(fs_smem);
   float* qs = qrow + (ostride + 3) / 4 * 4;
   int* hist = reinterpret_cast<int*>(qs + (rows.query_floats() + 3) / 4 * 4);
   uint64_t* band_key = reinterpret_cast<uint64_t*>(hist);                 // over the histogram once the bin is known
   int32_t* band = reinterpret_cast<int32_t*>(hist + kBins);               // [kBand]
   int32_t* list = band + kBand;                                           // [R] positions in the slice, then ids
-  uint64_t* ex = reinterpret_cast<uint64_t*>(list + (R + 1) / 2 * 2);     // [pow2 >= R]
+  uint32_t* kept = reinterpret_cast<uint32_t*>(list + (R + 1) / 2 * 2);   // [cap] keys
+  int32_t* kept_at = reinterpret_cast<int32_t*>(kept + cap);              // [cap] positions
+  uint64_t* ex = reinterpret_cast<uint64_t*>(kept);                       // [pow2 >= R] once the list is known
 
   for (int i = tid; i < ostride; i += kThreads)
     qrow[i] = i >= d ? 0.f
@@ -550,19 +579,21 @@ __global__ void __launch_bounds__(kThreads) finish_slices(
   norms.y = warp_sum(norms.y);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) norms.z = fmaxf(norms.z, __shfl_xor_sync(kFull, norms.z, o));
-  if (tid == 0) n_list = n_band = 0;
-  for (int i = tid; i < kBins; i += kThreads) hist[i] = 0;
-  // a sample's range
+  if (tid == 0) n_list = n_band = n_kept = 0;
+  // a sample and its range
+  uint32_t sample[kSample];
   float lo = INFINITY, hi = -INFINITY;
+#pragma unroll
   for (int u = 0; u < kSample; ++u) {
     const int64_t i = (int64_t)(u * kThreads + tid) * n / (kSample * kThreads);
-    const uint32_t key = i < n ? K[i] : 0u;
-    if (key) {
-      const float s = key_float(key);
-      lo = fminf(lo, s);
-      hi = fmaxf(hi, s);
-    }
+    sample[u] = i < n ? K[i] : 0u;
   }
+#pragma unroll
+  for (int u = 0; u < kSample; ++u)
+    if (sample[u]) {
+      lo = fminf(lo, key_float(sample[u]));
+      hi = fmaxf(hi, key_float(sample[u]));
+    }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
     lo = fminf(lo, __shfl_xor_sync(kFull, lo, o));
@@ -615,88 +646,137 @@ __global__ void __launch_bounds__(kThreads) finish_slices(
     if (in && at < cap) to[at] = v;
   };
 
-  const float scale = (float)(kBins - 1) / (hi - lo);
-  // linear bins need a finite range; a few keys need no histogram
-  bool linear = scale > 0.f && scale < INFINITY && delta < INFINITY;
+  // kBins linear bins of [lo, hi]; false where the range is not a finite interval
+  float scale = 0.f;
+  const auto set_bins = [&]() {
+    scale = (float)(kBins - 1) / (hi - lo);
+    for (int i = tid; i < kBins; i += kThreads) hist[i] = 0;
+    __syncthreads();
+    return scale > 0.f && scale < INFINITY && delta < INFINITY;
+  };
   const auto bin_of = [&](uint32_t key) {
     return (int)fminf(fmaxf((key_float(key) - lo) * scale, 0.f), (float)(kBins - 1));
   };
-  int total = 0;                                        // rows that count
-  if (linear) {
-#pragma unroll 4
-    for (int i = tid; i < n; i += kThreads) {
-      const uint32_t key = K[i];
-      if (key) atomicAdd(&hist[bin_of(key)], 1);
-    }
-    __syncthreads();
-    // from the top: thread l owns bins kBins - 1 - 8 l ... ; the bin of the R-th best
+  // counted rows, and bin_s = the bin that holds the want-th best of them
+  const auto find_bin = [&](int want) {
     constexpr int kOwn = kBins / kThreads;
-    int mine = 0;
+    __syncthreads();
+    int mine = 0, all;
 #pragma unroll
     for (int u = 0; u < kOwn; ++u) mine += hist[kBins - 1 - (tid * kOwn + u)];
-    const int before = block_exclusive_scan<int>(mine, warp_s, total);
-    if (before < R && before + mine >= R) {
-      int c = before;
+    int c = block_exclusive_scan<int>(mine, warp_s, all);
+    if (c < want && c + mine >= want)
       for (int u = 0; u < kOwn; ++u) {
         const int b = kBins - 1 - (tid * kOwn + u);
         c += hist[b];
-        if (c >= R) {
+        if (c >= want) {
           bin_s = b;
           break;
         }
       }
+    __syncthreads();
+    return all;
+  };
+  // The list from `count` rows (key_at, pos_at), all rows of the slice that
+  // count or (open) all at or above lo; false where it cannot tell.
+  const auto choose = [&](int count, auto key_at, auto pos_at, bool open) {
+    if (!set_bins()) return false;
+    for (int i = tid; i < count; i += kThreads) {
+      const uint32_t key = key_at(i);
+      if (key) atomicAdd(&hist[bin_of(key)], 1);
+    }
+    const int all = find_bin(R);
+    if (all <= R) return false;
+    const float wide = ceilf(2.f * delta * scale) + 1.f;
+    const int mb = wide < (float)kBins ? (int)wide : kBins;
+    if (open && bin_s < mb) return false;                                // rows below lo might be in the band
+    const int b_lo = max(0, bin_s - mb), b_hi = min(kBins - 1, bin_s + mb);
+    int in_band = 0, m;
+    for (int b = b_lo + tid; b <= b_hi; b += kThreads) in_band += hist[b];
+    block_exclusive_scan<int>(in_band, warp_s, m);
+    if (m > kBand) return false;
+    for (int i0 = 0; i0 < count; i0 += kThreads) {
+      const int i = i0 + tid;
+      const uint32_t key = i < count ? key_at(i) : 0u;
+      const int b = key ? bin_of(key) : -1;
+      if (!__any_sync(kFull, b >= b_lo)) continue;
+      append(b > b_hi, &n_list, list, R, b > b_hi ? pos_at(i) : 0);
+      append(b >= b_lo && b <= b_hi, &n_band, band, kBand, b >= b_lo ? pos_at(i) : 0);
     }
     __syncthreads();
-    if (total > R) {
-      const float wide = ceilf(2.f * delta * scale) + 1.f;
-      const int mb = wide < (float)kBins ? (int)wide : kBins;
-      const int b_lo = max(0, bin_s - mb), b_hi = min(kBins - 1, bin_s + mb);
-      // rows in the band
-      int in_band = 0;
-      for (int b = b_lo + tid; b <= b_hi; b += kThreads) in_band += hist[b];
-      int m;
-      block_exclusive_scan<int>(in_band, warp_s, m);
-      if (m > kBand) {
-        linear = false;
-      } else {
-#pragma unroll 4
-        for (int i0 = 0; i0 < n; i0 += kThreads) {
-          const int i = i0 + tid;
-          const uint32_t key = i < n ? K[i] : 0u;
-          const int b = key ? bin_of(key) : -1;
-          append(b > b_hi, &n_list, list, R, i);
-          append(b >= b_lo && b <= b_hi, &n_band, band, kBand, i);
-        }
-        __syncthreads();
-        int N = 2;
-        while (N < m) N <<= 1;
-        for (int i = tid; i < N; i += kThreads) band_key[i] = ~0ull;      // (the histogram is no longer read)
-        __syncthreads();
-        for (int i = tid; i < m; i += kThreads) band_key[i] = defined_key(band[i]);
-        __syncthreads();
-        block_sort(band_key, N);
-        // the list's rows as ids, then the band's best
-        const int have = n_list;
-        for (int i = tid; i < have; i += kThreads) {
-          const int j = probe_of(list[i]);
-          list[i] = ids[off[probes[j]] + (list[i] - qpos[j])];
-        }
-        for (int i = tid; i < R - have; i += kThreads) list[have + i] = (int32_t)(band_key[i] & 0xffffffffu);
-        __syncthreads();
-        if (tid == 0) n_list = R;
+    int N = 2;
+    while (N < m) N <<= 1;
+    for (int i = tid; i < N; i += kThreads) band_key[i] = i < m ? defined_key(band[i]) : ~0ull;   // (bins: no longer read)
+    __syncthreads();
+    block_sort(band_key, N);
+    // the list's rows as ids, then the band's best
+    const int have = n_list;
+    for (int i = tid; i < have; i += kThreads) {
+      const int j = probe_of(list[i]);
+      list[i] = ids[off[probes[j]] + (list[i] - qpos[j])];
+    }
+    for (int i = tid; i < R - have; i += kThreads) list[have + i] = (int32_t)(band_key[i] & 0xffffffffu);
+    __syncthreads();
+    if (tid == 0) n_list = R;
+    return true;
+  };
+
+  uint32_t floor_key = 1u;                              // every row that counts
+  bool finite = n <= cap || set_bins();
+  if (n > cap && finite) {
+#pragma unroll
+    for (int u = 0; u < kSample; ++u)
+      if (sample[u]) atomicAdd(&hist[bin_of(sample[u])], 1);
+    const float expect = (float)R * (kSample * kThreads) / (float)n;
+    const int want = (int)(1.25f * expect + 4.f * sqrtf(expect) + 8.f);
+    if (find_bin(want) > want) floor_key = max(1u, float_key(lo + (float)(bin_s - 1) / scale));
+  }
+  // one pass: four keys a load (slices start on 16 bytes)
+  const auto keep = [&](uint32_t key, int i) {
+    if (key >= floor_key) {
+      const int at = atomicAdd(&n_kept, 1);
+      if (at < cap) {
+        kept[at] = key;
+        kept_at[at] = i;
       }
     }
+  };
+  if (finite) {
+#pragma unroll 4
+    for (int i = 4 * tid; i + 3 < n; i += 4 * kThreads) {
+      const uint4 v = __ldg(reinterpret_cast<const uint4*>(K + i));
+      keep(v.x, i);
+      keep(v.y, i + 1);
+      keep(v.z, i + 2);
+      keep(v.w, i + 3);
+    }
+    if (tid < n % 4) keep(K[n / 4 * 4 + tid], n / 4 * 4 + tid);
   }
   __syncthreads();
-  if (!linear || total <= R) {
+  const int m_kept = n_kept;
+  bool done = false, few = false;                       // few: every row that counts is kept, and at most R are
+  if (finite && m_kept <= cap) {
+    if (floor_key == 1u && m_kept <= R) {
+      few = true;
+    } else if (m_kept > R) {
+      if (floor_key > 1u) lo = key_float(floor_key);
+      done = choose(m_kept, [&](int i) { return kept[i]; }, [&](int i) { return kept_at[i]; }, floor_key > 1u);
+    }
+  }
+  if (!done && !few) {
+    __syncthreads();
+    if (tid == 0) n_list = n_band = 0;
+    lo = lo_s;
+    done = choose(n, [&](int i) { return K[i]; }, [&](int i) { return i; }, false);
+  }
+  __syncthreads();
+  if (!done) {
     // every row that counts, or (more than R of them) those up to the R-th
     // smallest defined key, found byte by byte
     uint64_t limit = ~0ull;
-    if (!linear) {
-      int cnt = 0;
-      for (int i = tid; i < n; i += kThreads) cnt += K[i] != 0u;
-      block_exclusive_scan<int>(cnt, warp_s, total);
-    }
+    int cnt = 0, total;
+    for (int i = tid; i < n; i += kThreads) cnt += K[i] != 0u;
+    block_exclusive_scan<int>(cnt, warp_s, total);
     if (total > R) {
       uint64_t prefix = 0, mask = 0;
       int need = R;
@@ -798,9 +878,29 @@ __global__ void __launch_bounds__(kThreads) finish_slices(
   }
 }
 
-// Queries per pass, so that the keys stay within 2 GB.
-int64_t key_chunk(int64_t slice, int64_t nq) {
-  return std::min(nq, std::max<int64_t>(8, ((int64_t)1 << 29) / slice));
+// Keys a query may need, a multiple of four (slices are read 16 bytes at a time).
+int64_t slice_rows(const IndexData& ix, int t) {
+  return (std::max<int64_t>(1, std::min<int64_t>((int64_t)t * ix.max_partition, ix.rows)) + 3) / 4 * 4;
+}
+// Queries per pass, so that the keys stay within `most` entries.
+int64_t key_chunk(int64_t slice, int64_t nq, int64_t most) {
+  return std::min(nq, std::max<int64_t>(8, most / slice));
+}
+// Room for the keys of as many queries as 4 GB hold, or 2 GB where the device
+// has no more: a slice is sized for the largest partitions and mostly a third
+// full, and a batch in two passes reads its partitions twice.
+uint32_t* key_room(int64_t slice, int64_t nq, int64_t& cq, Scratch& scr) {
+  cq = key_chunk(slice, nq, (int64_t)1 << 30);
+  const int64_t less = key_chunk(slice, nq, (int64_t)1 << 29);
+  if (cq == less) return scr.get<uint32_t>((size_t)cq * slice);
+  try {
+    return scr.get<uint32_t>((size_t)cq * slice);
+  } catch (const Error& e) {
+    if (e.status != SOAR_ENOMEM) throw;
+    cudaGetLastError();                       // clear the failed allocation
+  }
+  cq = less;
+  return scr.get<uint32_t>((size_t)cq * slice);
 }
 
 template <typename Rows>
@@ -810,9 +910,9 @@ void run(const IndexData& ix, Rows rws, float* base, int* smax, const float* Qf,
   rws.tiles = Rows::kTiles;
   while (rws.tiles > 1 && rws.item_smem() > 180 * 1024) --rws.tiles;     // wide rows: fewer queries an item
   const int QB = 8 * rws.tiles;
-  const int64_t slice = std::max<int64_t>(1, std::min<int64_t>((int64_t)t * ix.max_partition, ix.rows));
-  const int64_t cq = key_chunk(slice, nq);
-  uint32_t* keys = scr.get<uint32_t>((size_t)cq * slice);
+  const int64_t slice = slice_rows(ix, t);
+  int64_t cq;
+  uint32_t* keys = key_room(slice, nq, cq, scr);
   int64_t* counts = scr.get<int64_t>(cq);
   int64_t* pos = scr.get<int64_t>((size_t)cq * t);
   int32_t* inv = scr.get<int32_t>((size_t)cq * t);
@@ -823,7 +923,7 @@ void run(const IndexData& ix, Rows rws, float* base, int* smax, const float* Qf,
     while (sorted < R) sorted <<= 1;
   const size_t fin_smem = sizeof(float) * ((size_t)(ostride + 3) / 4 * 4 + (rws.query_floats() + 3) / 4 * 4) +
                           sizeof(int) * (size_t)(kBins + kBand) + sizeof(int32_t) * (size_t)((R + 1) / 2 * 2) +
-                          sizeof(uint64_t) * (size_t)sorted;
+                          std::max(sizeof(uint64_t) * (size_t)kept_rows(R), sizeof(uint64_t) * (size_t)sorted);
   const size_t item_smem = rws.item_smem();
   SOAR_CUDA(cudaFuncSetAttribute(score_items<Rows>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)item_smem));
   const auto finish = [&](auto elem, int64_t q0, int64_t m) {
@@ -878,8 +978,8 @@ void fp8_search(const IndexData& ix, const float* Qf, const float* qscale, const
 void pq_search(const IndexData& ix, const float* Qf, int qstride, const void* Q, soar_dtype dt, const int32_t* top,
                const int32_t* tpq, int64_t nq, int t, int R, int k, int64_t* ids_out, float* scores_out,
                cudaStream_t s, Scratch& scr) {
-  const int64_t slice = std::max<int64_t>(1, std::min<int64_t>((int64_t)t * ix.max_partition, ix.rows));
-  float* base = scr.get<float>((size_t)key_chunk(slice, nq) * t);
+  const int64_t slice = slice_rows(ix, t);
+  float* base = scr.get<float>((size_t)key_chunk(slice, nq, (int64_t)1 << 30) * t);
   const Pq4Rows rws{static_cast<const uint8_t*>(ix.vectors), ix.code_stride, ix.pq_m, ix.d, ix.pq_cb, Qf, qstride,
                     base, (ix.pq_m + 7) / 8, 0};
   run(ix, rws, base, nullptr, Qf, qstride, Q, dt, top, tpq, nq, t, R, k, ids_out, scores_out, s, scr);
