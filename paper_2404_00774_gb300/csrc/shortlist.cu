@@ -41,7 +41,6 @@ namespace {
 
 constexpr int kWarps = 8;
 constexpr int kThreads = 32 * kWarps;
-constexpr int kProbesSmem = 64;      // probe lists held in shared memory up to this t
 
 __device__ __forceinline__ float fp8_code_value(uint32_t b) {
   __half_raw h = __nv_cvt_fp8_to_halfraw((__nv_fp8_storage_t)b, __NV_E4M3);
@@ -141,11 +140,12 @@ struct Fp8Rows {
     return make_float3(n2, 0.f, 0.f);
   }
   // |key's score - defined score|: both sums of exact products have at most
-  // code_stride fp32 additions, each within 2^-23 of a partial sum that stays
-  // below ||q8|| ||x8||, and ||x8|| <= 448 sqrt(d); a factor of four to spare.
+  // code_stride fp32 additions, off by 2^-24 (defined order) and at most 2^-23
+  // (tensor cores; measured 2^-23 over a whole sum) of a partial sum that stays
+  // below ||q8|| ||x8||, and ||x8|| <= 448 sqrt(d); the rest covers the scaling.
   // The scale of a row is at most smax.
   __device__ float delta(float3 v, int64_t q, float smax) const {
-    return ldexpf((float)code_stride, -20) * sqrtf(v.x) * 448.f * sqrtf((float)code_stride) * qscale[q] * smax;
+    return ldexpf((float)code_stride, -22) * sqrtf(v.x) * 448.f * sqrtf((float)code_stride) * qscale[q] * smax;
   }
   __device__ float exact(const float* qs, int64_t q, int64_t r, float) const {
     const uint4* x = reinterpret_cast<const uint4*>(codes + r * (int64_t)code_stride);
@@ -321,7 +321,35 @@ __global__ void pair_offsets(const int64_t* __restrict__ off, const int32_t* __r
   if (lane == 0) counts[ql] = acc;
 }
 
-// Work items (partition, up to 8 * kTiles of its queries; blockIdx.y takes every
+// Which of an item's queries probed a partition before this one: a hash table
+// in shared memory from partition to a mask of the item's query slots, so that a
+// row looks its point's other partitions up once for all queries (comparing each
+// query's earlier probes row by row was two thirds of the scoring's
+// instructions).  kHashMost entries at most; an item with more (large t) compares.
+constexpr int kHashSize = 2048, kHashMost = 1024;
+struct ProbeMasks {
+  int32_t key[kHashSize];
+  uint32_t mask[kHashSize];
+  __device__ static int at(int32_t p) { return (int)(((uint32_t)p * 2654435769u) >> 21); }   // 11 bits
+  __device__ void add(int32_t p, uint32_t bit) {
+    for (int h = at(p);; h = (h + 1) & (kHashSize - 1)) {
+      const int32_t old = atomicCAS(&key[h], -1, p);
+      if (old == -1 || old == p) {
+        atomicOr(&mask[h], bit);
+        return;
+      }
+    }
+  }
+  __device__ uint32_t find(int32_t p) const {
+    for (int h = at(p);; h = (h + 1) & (kHashSize - 1)) {
+      const int32_t k = key[h];
+      if (k == p) return mask[h];
+      if (k == -1) return 0u;
+    }
+  }
+};
+
+// Work items (partition, up to 32 of its queries; blockIdx.y takes every
 // gridDim.y-th step of 128 rows): keys of every (query, row).  A key is the
 // order-preserving image of the score, 0 for a copy that does not count.  smax
 // (FP8, zero before the launch): the largest scale of the rows met, which are
@@ -334,13 +362,14 @@ __global__ void __launch_bounds__(kThreads) score_items(Rows rows, IvfWork work,
                                                         int* __restrict__ smax) {
   constexpr unsigned kFull = 0xffffffffu;
   constexpr int QB = 8 * Rows::kTiles;
-  constexpr int kMaxOther = 4;                  // copies of a point besides this one
+  static_assert(QB <= 32, "a mask word holds the item's queries");
   extern __shared__ __align__(16) unsigned char sl_smem[];
-  __shared__ int64_t out_s[QB];                 // where the pair's keys start
-  __shared__ int32_t probes_s[QB][kProbesSmem + 1];
-  __shared__ int32_t j_s[QB];
+  __shared__ uint32_t* out_s[QB];               // where the pair's keys start
   __shared__ const int32_t* list_s[QB];         // the query's probes
+  __shared__ int32_t j_s[QB];                   // how many of them come before this partition
   __shared__ float qf_s[QB];
+  __shared__ ProbeMasks masks;
+  __shared__ int earlier_s;
   const int item = blockIdx.x;
   if (item >= work.count()) return;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -357,7 +386,15 @@ __global__ void __launch_bounds__(kThreads) score_items(Rows rows, IvfWork work,
   const int64_t e0 = work.pair_off[p] + (int64_t)(item - work.item_base[oi]) * work.qb;
   const int nqi = (int)min((int64_t)work.qb, work.pair_off[p + 1] - e0);
   const int64_t r0 = work.part_off[p], r1 = work.part_off[p + 1];
+  const int nrows = (int)(r1 - r0);
   rows.stage_shared(sl_smem);
+  if (a > 1)
+    for (int i = threadIdx.x; i < kHashSize; i += kThreads) {
+      masks.key[i] = -1;
+      masks.mask[i] = 0u;
+    }
+  if (threadIdx.x == 0) earlier_s = 0;
+  __syncthreads();
   for (int i = w; i < 8 * rows.tiles; i += kWarps) {
     const bool use = i < nqi;
     int64_t ql = -1;
@@ -365,74 +402,79 @@ __global__ void __launch_bounds__(kThreads) score_items(Rows rows, IvfWork work,
       const int pr = work.pair_vals[e0 + i];    // ql * t + j
       ql = pr / work.tmax;
       const int j = (int)(pr - ql * work.tmax);
-      const int32_t* probes = top + (q0 + ql) * (int64_t)work.tmax;
       if (lane == 0) {
-        out_s[i] = ql * slice + pos[pr];
+        out_s[i] = keys + ql * slice + pos[pr];
+        list_s[i] = top + (q0 + ql) * (int64_t)work.tmax;
         j_s[i] = j;
-        list_s[i] = probes;
         qf_s[i] = rows.query_factor(q0 + ql, pr);
+        atomicAdd(&earlier_s, min(j, kHashMost + 1));
       }
-      if (j <= kProbesSmem)
-        for (int jj = lane; jj < j; jj += 32) probes_s[i][jj] = probes[jj];
     }
     rows.stage_query(sl_smem, i, use ? q0 + ql : -1, lane);
   }
   __syncthreads();
+  const bool hashed = earlier_s <= kHashMost;
+  if (a > 1 && hashed) {
+    for (int i = w; i < nqi; i += kWarps)
+      for (int jj = lane; jj < j_s[i]; jj += 32) masks.add(list_s[i][jj], 1u << i);
+    __syncthreads();
+  }
   const int nt = (nqi + 7) / 8, g = lane >> 2, tig = lane & 3;
+  // the item's queries whose earlier probes hold the row's point
+  const auto dropped = [&](int32_t o) -> uint32_t {
+    if (hashed) return masks.find(o);
+    uint32_t m = 0u;
+    for (int i = 0; i < nqi; ++i)
+      for (int jj = 0; jj < j_s[i]; ++jj)
+        if (list_s[i][jj] == o) {
+          m |= 1u << i;
+          break;
+        }
+    return m;
+  };
   float most = 0.f;
-  const int64_t step = 16 * kWarps * (int64_t)gridDim.y;
-  int64_t t0 = r0 + 16 * (w + kWarps * (int64_t)blockIdx.y);
-  const auto fetch_id = [&](int64_t tile) { return tile + (lane & 15) < r1 ? ids[tile + (lane & 15)] : -1; };
-  int32_t id = fetch_id(t0), next_id = fetch_id(t0 + step), next_other = -1;
+  const int step = 16 * kWarps * (int)gridDim.y;
+  int t0 = 16 * (w + kWarps * (int)blockIdx.y);
+  const int32_t* pids = ids + r0;
+  const auto fetch_id = [&](int tile) { return tile + (lane & 15) < nrows ? pids[tile + (lane & 15)] : -1; };
+  int32_t id = fetch_id(t0), next_id = fetch_id(t0 + step);
+  int2 next_assign = make_int2(-1, -1);
   float next_rf = 0.f;
-  const auto fetch_row = [&](int64_t tile) {      // of the rows whose ids are in `id`
-    next_other = -1;
+  const auto fetch_row = [&](int tile) {        // of the rows whose ids are in `id`
     next_rf = 0.f;
     if (id < 0) return;
-    next_rf = rows.row_factor(tile + (lane & 15));
-    if (a == 2) {
-      const int2 v = __ldg(reinterpret_cast<const int2*>(assign) + id);
-      next_other = v.x == p ? v.y : v.x;
-    }
+    next_rf = rows.row_factor(r0 + tile + (lane & 15));
+    if (a == 2) next_assign = __ldg(reinterpret_cast<const int2*>(assign) + id);
   };
   fetch_row(t0);
-  for (; t0 < r1; t0 += step) {
+  for (; t0 < nrows; t0 += step) {
     float acc[Rows::kTiles][4];
 #pragma unroll
     for (int n = 0; n < Rows::kTiles; ++n)
 #pragma unroll
       for (int i = 0; i < 4; ++i) acc[n][i] = 0.f;
-    // lane l: the other partitions of row l % 16
-    int32_t other[kMaxOther] = {next_other, -1, -1, -1};
     const float rf = next_rf;
-    most = fmaxf(most, rf);
-    if (a > 2) {
-      other[0] = -1;
-      if (id >= 0) {
-        int at = 0;
-        for (int i = 0; i < a; ++i) {
-          const int v = assign[(int64_t)id * a + i];
-          if (v == p) continue;
-#pragma unroll
-          for (int u = 0; u < kMaxOther; ++u)
-            if (u == at) other[u] = v;
-          ++at;
-        }
-      }
-    }
+    const int2 as = next_assign;
+    const int32_t id_now = id;
     // the next step's assignments and the ids of the step after it are on their way during this one
     id = next_id;
     fetch_row(t0 + step);
     next_id = fetch_id(t0 + 2 * step);
-    rows.tile(sl_smem, t0, r1, nt, lane, acc);
-    const float rfa = __shfl_sync(kFull, rf, g), rfb = __shfl_sync(kFull, rf, g + 8);
-    // rows g and g + 8: which of the two have a copy in one of a query's earlier probes
-    int32_t oa[kMaxOther], ob[kMaxOther];
-#pragma unroll
-    for (int u = 0; u < kMaxOther; ++u) {
-      oa[u] = __shfl_sync(kFull, other[u], g);
-      ob[u] = __shfl_sync(kFull, other[u], g + 8);
+    most = fmaxf(most, rf);
+    // lane l: the queries for which row l % 16 does not count
+    uint32_t drop = 0u;
+    if (a == 2) {
+      if (id_now >= 0) drop = dropped(as.x == p ? as.y : as.x);
+    } else if (a > 2 && id_now >= 0) {
+      for (int i = 0; i < a; ++i) {
+        const int v = assign[(int64_t)id_now * a + i];
+        if (v != p) drop |= dropped(v);
+      }
     }
+    rows.tile(sl_smem, r0 + t0, r1, nt, lane, acc);
+    const float rfa = __shfl_sync(kFull, rf, g), rfb = __shfl_sync(kFull, rf, g + 8);
+    const uint32_t da = __shfl_sync(kFull, drop, g) >> (2 * tig), db = __shfl_sync(kFull, drop, g + 8) >> (2 * tig);
+    const bool ina = t0 + g < nrows, inb = t0 + g + 8 < nrows;
 #pragma unroll
     for (int n = 0; n < Rows::kTiles; ++n) {
       if (n >= nt) break;
@@ -440,25 +482,10 @@ __global__ void __launch_bounds__(kThreads) score_items(Rows rows, IvfWork work,
       for (int i = 0; i < 2; ++i) {
         const int slot = 8 * n + 2 * tig + i;
         if (slot >= nqi) continue;
-        const int j = j_s[slot];
-        const bool near = j <= kProbesSmem;
-        bool da = false, db = false;
-        for (int jj = 0; jj < j; ++jj) {
-          const int32_t pr = near ? probes_s[slot][jj] : list_s[slot][jj];
-          da = da || pr == oa[0];
-          db = db || pr == ob[0];
-          if (a > 2) {
-#pragma unroll
-            for (int u = 1; u < kMaxOther; ++u) {
-              da = da || pr == oa[u];
-              db = db || pr == ob[u];
-            }
-          }
-        }
-        uint32_t* out = keys + out_s[slot] + (t0 - r0) + g;
+        uint32_t* out = out_s[slot] + (t0 + g);
         const float qf = qf_s[slot];
-        if (t0 + g < r1) out[0] = da ? 0u : float_key(Rows::combine(acc[n][i], rfa, qf));
-        if (t0 + g + 8 < r1) out[8] = db ? 0u : float_key(Rows::combine(acc[n][2 + i], rfb, qf));
+        if (ina) out[0] = (da >> (8 * n + i)) & 1u ? 0u : float_key(Rows::combine(acc[n][i], rfa, qf));
+        if (inb) out[8] = (db >> (8 * n + i)) & 1u ? 0u : float_key(Rows::combine(acc[n][2 + i], rfb, qf));
       }
     }
   }
@@ -487,12 +514,15 @@ __device__ __forceinline__ float row_dot(const float* __restrict__ q, const __nv
 #pragma unroll 6
   for (int k = 0; k < stride; k += 8) {
     const uint4 v = __ldg(reinterpret_cast<const uint4*>(x + k));
-    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      s = fmaf(q[k + 2 * i], __uint_as_float(w[i] << 16), s);
-      s = fmaf(q[k + 2 * i + 1], __uint_as_float(w[i] & 0xffff0000u), s);
-    }
+    const float4 a = *reinterpret_cast<const float4*>(q + k), b = *reinterpret_cast<const float4*>(q + k + 4);
+    s = fmaf(a.x, __uint_as_float(v.x << 16), s);
+    s = fmaf(a.y, __uint_as_float(v.x & 0xffff0000u), s);
+    s = fmaf(a.z, __uint_as_float(v.y << 16), s);
+    s = fmaf(a.w, __uint_as_float(v.y & 0xffff0000u), s);
+    s = fmaf(b.x, __uint_as_float(v.z << 16), s);
+    s = fmaf(b.y, __uint_as_float(v.z & 0xffff0000u), s);
+    s = fmaf(b.z, __uint_as_float(v.w << 16), s);
+    s = fmaf(b.w, __uint_as_float(v.w & 0xffff0000u), s);
   }
   return s;
 }
@@ -731,26 +761,44 @@ __global__ void __launch_bounds__(kThreads) finish_slices(
     const int want = (int)(1.25f * expect + 4.f * sqrtf(expect) + 8.f);
     if (find_bin(want) > want) floor_key = max(1u, float_key(lo + (float)(bin_s - 1) / scale));
   }
-  // one pass: four keys a load (slices start on 16 bytes)
-  const auto keep = [&](uint32_t key, int i) {
-    if (key >= floor_key) {
-      const int at = atomicAdd(&n_kept, 1);
-      if (at < cap) {
-        kept[at] = key;
-        kept_at[at] = i;
-      }
-    }
-  };
+  // one pass: four keys a load (slices start on 16 bytes), one counter step a warp and load
   if (finite) {
-#pragma unroll 4
-    for (int i = 4 * tid; i + 3 < n; i += 4 * kThreads) {
-      const uint4 v = __ldg(reinterpret_cast<const uint4*>(K + i));
-      keep(v.x, i);
-      keep(v.y, i + 1);
-      keep(v.z, i + 2);
-      keep(v.w, i + 3);
+    const int n4 = n / 4;
+#pragma unroll 2
+    for (int i0 = 32 * w; i0 <= n4; i0 += kThreads) {
+      const int i = i0 + lane;
+      uint4 v = make_uint4(0u, 0u, 0u, 0u);
+      if (i < n4) {
+        v = __ldg(reinterpret_cast<const uint4*>(K) + i);
+      } else if (i == n4) {                             // the last one to three keys
+        if (n % 4 > 0) v.x = K[4 * i];
+        if (n % 4 > 1) v.y = K[4 * i + 1];
+        if (n % 4 > 2) v.z = K[4 * i + 2];
+      }
+      const uint32_t key[4] = {v.x, v.y, v.z, v.w};
+      int mine = 0;
+#pragma unroll
+      for (int u = 0; u < 4; ++u) mine += key[u] >= floor_key ? 1 : 0;
+      if (!__any_sync(kFull, mine)) continue;
+      int incl = mine;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(kFull, incl, o);
+        if (lane >= o) incl += y;
+      }
+      int at = 0;
+      if (lane == 31) at = atomicAdd(&n_kept, incl);
+      at = __shfl_sync(kFull, at, 31) + incl - mine;
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (key[u] >= floor_key) {
+          if (at < cap) {
+            kept[at] = key[u];
+            kept_at[at] = 4 * i + u;
+          }
+          ++at;
+        }
     }
-    if (tid < n % 4) keep(K[n / 4 * 4 + tid], n / 4 * 4 + tid);
   }
   __syncthreads();
   const int m_kept = n_kept;
