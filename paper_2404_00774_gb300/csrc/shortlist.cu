@@ -27,7 +27,7 @@
 // (10 000 queries, 10^7 x 96 fp8, t = 6, R = 1 000: scoring 6 230, selecting
 // 2 990, rescoring 2 810 us; 1.18 M x 100 PQ4, t = 14, R = 100: 4 076, 1 884
 // and 398 us).  Here the codes are read and decoded once for up to 64 queries:
-// FP8_SCORE and FP8_FINISH us, PQ_SCORE and PQ_FINISH us.  The product is a few
+// 763 and 988 us, 756 and 567 us.  The product is a few
 // percent of the work, so warp-level MMAs fed from registers are used: a key
 // leaves the registers it was computed in, with no TMEM round trip.
 #include <algorithm>
@@ -66,6 +66,11 @@ __device__ __forceinline__ void mma_bf16x16(float (&c)[4], uint32_t a0, uint32_t
       : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+
 // (x, y) as a bf16 pair (x in the low half), and what it leaves over
 __device__ __forceinline__ uint32_t bf16_pair(float x, float y, float& rx, float& ry) {
   const __nv_bfloat162 h = __floats2bfloat162_rn(x, y);
@@ -75,10 +80,13 @@ __device__ __forceinline__ uint32_t bf16_pair(float x, float y, float& rx, float
   return *reinterpret_cast<const uint32_t*>(&h);
 }
 
-// A layout gives: the queries of an item in shared memory, the scores of 16
-// rows against 8 * nt queries (accumulator element i of tile n: row lane / 4 +
-// 8 * (i / 2), query 8 n + 2 * (lane % 4) + i % 2), and the score in the
-// defined order.
+// A layout gives: the queries of an item in shared memory, a fragment of 16
+// rows' codes, its product with 8 * nt queries (accumulator element i of tile n:
+// row lane / 4 + 8 * (i / 2), query 8 n + 2 * (lane % 4) + i % 2), and the score
+// in the defined order.
+struct Frag {
+  uint4 a[2], b[2];
+};
 
 // Per-row scaled E4M3 codes.
 struct Fp8Rows {
@@ -102,26 +110,31 @@ struct Fp8Rows {
                    : (uint8_t)0;
   }
   // The K order is free as long as both operands agree: lane % 4 takes a 16-byte
-  // chunk of each 64 bytes of a row, whose four words serve two MMAs.
-  __device__ void tile(const unsigned char* sm, int64_t r0, int64_t r1, int nt, int lane, float (&acc)[kTiles][4]) const {
-    const int g = lane >> 2, tig = lane & 3;
-    const int64_t ra = r0 + g, rb = ra + 8;
-    const uint8_t* xa = codes + (ra < r1 ? ra : r0) * code_stride;
-    const uint8_t* xb = codes + (rb < r1 ? rb : r0) * code_stride;
-#pragma unroll 2
-    for (int ks = 0; ks < k64; ++ks) {
-      const int o = 64 * ks + 16 * tig;
-      uint4 a = make_uint4(0u, 0u, 0u, 0u), b = a;
+  // chunk of each 64 bytes of a row, whose four words serve two MMAs.  A fragment
+  // is two such steps of rows lane / 4 and lane / 4 + 8.
+  __host__ __device__ int fragments() const { return (k64 + 1) / 2; }
+  __device__ void load(Frag& f, const uint8_t* xa, const uint8_t* xb, int part, int lane) const {
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const int o = 64 * (2 * part + u) + 16 * (lane & 3);
+      f.a[u] = f.b[u] = make_uint4(0u, 0u, 0u, 0u);
       if (o < code_stride) {
-        a = __ldg(reinterpret_cast<const uint4*>(xa + o));
-        b = __ldg(reinterpret_cast<const uint4*>(xb + o));
+        f.a[u] = __ldg(reinterpret_cast<const uint4*>(xa + o));
+        f.b[u] = __ldg(reinterpret_cast<const uint4*>(xb + o));
       }
+    }
+  }
+  __device__ void multiply(const unsigned char* sm, const Frag& f, int part, int nt, int lane, float (&acc)[kTiles][4]) const {
+    const unsigned char* qw = sm + (lane >> 2) * query_stride() + 16 * (lane & 3) + 128 * part;
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      if (2 * part + u >= k64) break;
 #pragma unroll
       for (int n = 0; n < kTiles; ++n)
         if (n < nt) {
-          const uint4 w = *reinterpret_cast<const uint4*>(sm + (8 * n + g) * query_stride() + o);
-          mma_e4m3(acc[n], a.x, b.x, a.y, b.y, w.x, w.y);
-          mma_e4m3(acc[n], a.z, b.z, a.w, b.w, w.z, w.w);
+          const uint4 w = *reinterpret_cast<const uint4*>(qw + 8 * n * query_stride() + 64 * u);
+          mma_e4m3(acc[n], f.a[u].x, f.b[u].x, f.a[u].y, f.b[u].y, w.x, w.y);
+          mma_e4m3(acc[n], f.a[u].z, f.b[u].z, f.a[u].w, f.b[u].w, w.z, w.w);
         }
     }
   }
@@ -209,17 +222,30 @@ struct Pq4Rows {
       at[2] = bf16_pair(rx, ry, u, v);
     }
   }
-  __device__ void tile(const unsigned char* sm, int64_t r0, int64_t r1, int nt, int lane, float (&acc)[kTiles][4]) const {
-    const uint2* lut = reinterpret_cast<const uint2*>(sm);
-    const unsigned char* qw = sm + (size_t)8 * steps * 16 * 8 + (lane >> 2) * query_stride() + 16 * (lane & 3);
-    const int g = lane >> 2, tig = lane & 3;
-    const int64_t ra = r0 + g, rb = ra + 8;
-    const uint32_t* xa = reinterpret_cast<const uint32_t*>(codes + (ra < r1 ? ra : r0) * code_stride);
-    const uint32_t* xb = reinterpret_cast<const uint32_t*>(codes + (rb < r1 ? rb : r0) * code_stride);
-#pragma unroll 2
-    for (int ks = 0; ks < steps; ++ks) {          // (a row has at least 4 * steps bytes)
-      const uint32_t wa = __ldg(xa + ks) >> (4 * tig), wb = __ldg(xb + ks) >> (4 * tig);
-      const uint2* l0 = lut + (8 * ks + tig) * 16;
+  // A fragment is 32 code bytes (eight K steps) of rows lane / 4 and lane / 4 + 8.
+  __host__ __device__ int fragments() const { return (steps + 7) / 8; }
+  __device__ void load(Frag& f, const uint8_t* xa, const uint8_t* xb, int part, int) const {
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const int o = 32 * part + 16 * u;
+      f.a[u] = f.b[u] = make_uint4(0u, 0u, 0u, 0u);
+      if (o < code_stride) {
+        f.a[u] = __ldg(reinterpret_cast<const uint4*>(xa + o));
+        f.b[u] = __ldg(reinterpret_cast<const uint4*>(xb + o));
+      }
+    }
+  }
+  __device__ void multiply(const unsigned char* sm, const Frag& f, int part, int nt, int lane, float (&acc)[kTiles][4]) const {
+    const uint2* lut = reinterpret_cast<const uint2*>(sm) + (lane & 3) * 16 + 1024 * part;
+    const unsigned char* qw = sm + (size_t)8 * steps * 16 * 8 + (lane >> 2) * query_stride() + 16 * (lane & 3) + 512 * part;
+    const int sh = 4 * (lane & 3);
+#pragma unroll
+    for (int ks = 0; ks < 8; ++ks) {
+      if (8 * part + ks >= steps) break;
+      const uint4 ca = f.a[ks / 4], cb = f.b[ks / 4];
+      const uint32_t wa = (ks % 4 == 0 ? ca.x : ks % 4 == 1 ? ca.y : ks % 4 == 2 ? ca.z : ca.w) >> sh;
+      const uint32_t wb = (ks % 4 == 0 ? cb.x : ks % 4 == 1 ? cb.y : ks % 4 == 2 ? cb.z : cb.w) >> sh;
+      const uint2* l0 = lut + 128 * ks;
       const uint2 a0 = l0[wa & 15u], a1 = l0[wb & 15u], a2 = l0[64 + ((wa >> 16) & 15u)], a3 = l0[64 + ((wb >> 16) & 15u)];
 #pragma unroll
       for (int n = 0; n < kTiles; ++n)
@@ -355,7 +381,7 @@ struct ProbeMasks {
 // (FP8, zero before the launch): the largest scale of the rows met, which are
 // positive and so ordered like their bits.
 template <typename Rows>
-__global__ void __launch_bounds__(kThreads) score_items(Rows rows, IvfWork work, const int32_t* __restrict__ ids,
+__global__ void __launch_bounds__(kThreads, 3) score_items(Rows rows, IvfWork work, const int32_t* __restrict__ ids,
                                                         const int32_t* __restrict__ assign, int a,
                                                         const int32_t* __restrict__ top, int64_t q0, int64_t slice,
                                                         const int64_t* __restrict__ pos, uint32_t* __restrict__ keys,
@@ -368,6 +394,7 @@ __global__ void __launch_bounds__(kThreads) score_items(Rows rows, IvfWork work,
   __shared__ const int32_t* list_s[QB];         // the query's probes
   __shared__ int32_t j_s[QB];                   // how many of them come before this partition
   __shared__ float qf_s[QB];
+  __shared__ int64_t q_s[QB];
   __shared__ ProbeMasks masks;
   __shared__ int earlier_s;
   const int item = blockIdx.x;
@@ -395,23 +422,25 @@ __global__ void __launch_bounds__(kThreads) score_items(Rows rows, IvfWork work,
     }
   if (threadIdx.x == 0) earlier_s = 0;
   __syncthreads();
-  for (int i = w; i < 8 * rows.tiles; i += kWarps) {
-    const bool use = i < nqi;
-    int64_t ql = -1;
-    if (use) {
+  if (threadIdx.x < QB) {                       // a thread per query slot
+    const int i = threadIdx.x;
+    int64_t q = -1;
+    if (i < nqi) {
       const int pr = work.pair_vals[e0 + i];    // ql * t + j
-      ql = pr / work.tmax;
+      const int64_t ql = pr / work.tmax;
       const int j = (int)(pr - ql * work.tmax);
-      if (lane == 0) {
-        out_s[i] = keys + ql * slice + pos[pr];
-        list_s[i] = top + (q0 + ql) * (int64_t)work.tmax;
-        j_s[i] = j;
-        qf_s[i] = rows.query_factor(q0 + ql, pr);
-        atomicAdd(&earlier_s, min(j, kHashMost + 1));
-      }
+      q = q0 + ql;
+      out_s[i] = keys + ql * slice + pos[pr];
+      list_s[i] = top + q * (int64_t)work.tmax;
+      j_s[i] = j;
+      qf_s[i] = rows.query_factor(q, pr);
+      atomicAdd(&earlier_s, min(j, kHashMost + 1));
     }
-    rows.stage_query(sl_smem, i, use ? q0 + ql : -1, lane);
+    q_s[i] = q;
   }
+  __syncthreads();
+#pragma unroll 4
+  for (int i = w; i < 8 * rows.tiles; i += kWarps) rows.stage_query(sl_smem, i, q_s[i], lane);
   __syncthreads();
   const bool hashed = earlier_s <= kHashMost;
   if (a > 1 && hashed) {
@@ -447,6 +476,9 @@ __global__ void __launch_bounds__(kThreads) score_items(Rows rows, IvfWork work,
     if (a == 2) next_assign = __ldg(reinterpret_cast<const int2*>(assign) + id);
   };
   fetch_row(t0);
+  // rows past the end read the partition's first row instead
+  const auto row_codes = [&](int r) { return rows.codes + (r0 + (r < nrows ? r : 0)) * rows.code_stride; };
+  const int parts = rows.fragments();
   for (; t0 < nrows; t0 += step) {
     float acc[Rows::kTiles][4];
 #pragma unroll
@@ -460,6 +492,8 @@ __global__ void __launch_bounds__(kThreads) score_items(Rows rows, IvfWork work,
     id = next_id;
     fetch_row(t0 + step);
     next_id = fetch_id(t0 + 2 * step);
+    Frag f;
+    rows.load(f, row_codes(t0 + g), row_codes(t0 + g + 8), 0, lane);
     most = fmaxf(most, rf);
     // lane l: the queries for which row l % 16 does not count
     uint32_t drop = 0u;
@@ -471,7 +505,11 @@ __global__ void __launch_bounds__(kThreads) score_items(Rows rows, IvfWork work,
         if (v != p) drop |= dropped(v);
       }
     }
-    rows.tile(sl_smem, r0 + t0, r1, nt, lane, acc);
+    rows.multiply(sl_smem, f, 0, nt, lane, acc);
+    for (int part = 1; part < parts; ++part) {                  // wide rows
+      rows.load(f, row_codes(t0 + g), row_codes(t0 + g + 8), part, lane);
+      rows.multiply(sl_smem, f, part, nt, lane, acc);
+    }
     const float rfa = __shfl_sync(kFull, rf, g), rfb = __shfl_sync(kFull, rf, g + 8);
     const uint32_t da = __shfl_sync(kFull, drop, g) >> (2 * tig), db = __shfl_sync(kFull, drop, g + 8) >> (2 * tig);
     const bool ina = t0 + g < nrows, inb = t0 + g + 8 < nrows;
@@ -496,33 +534,53 @@ __global__ void __launch_bounds__(kThreads) score_items(Rows rows, IvfWork work,
   }
 }
 
-// Exact fp32 <q, x> of a stored row, elements in ascending order.
-__device__ __forceinline__ float row_dot(const float* __restrict__ q, const float* __restrict__ x, int stride) {
-  float s = 0.f;
-#pragma unroll 8
-  for (int k = 0; k < stride; k += 4) {
-    const float4 v = __ldg(reinterpret_cast<const float4*>(x + k)), a = *reinterpret_cast<const float4*>(q + k);
-    s = fmaf(a.x, v.x, s);
-    s = fmaf(a.y, v.y, s);
-    s = fmaf(a.z, v.z, s);
-    s = fmaf(a.w, v.w, s);
-  }
-  return s;
+// One 16-byte chunk of a stored row, elements in ascending order.
+__device__ __forceinline__ float chunk_dot(const float* q, uint4 v, float s, float) {
+  const float4 a = *reinterpret_cast<const float4*>(q);
+  s = fmaf(a.x, __uint_as_float(v.x), s);
+  s = fmaf(a.y, __uint_as_float(v.y), s);
+  s = fmaf(a.z, __uint_as_float(v.z), s);
+  return fmaf(a.w, __uint_as_float(v.w), s);
 }
-__device__ __forceinline__ float row_dot(const float* __restrict__ q, const __nv_bfloat16* __restrict__ x, int stride) {
+__device__ __forceinline__ float chunk_dot(const float* q, uint4 v, float s, __nv_bfloat16) {
+  const float4 a = *reinterpret_cast<const float4*>(q), b = *reinterpret_cast<const float4*>(q + 4);
+  s = fmaf(a.x, __uint_as_float(v.x << 16), s);
+  s = fmaf(a.y, __uint_as_float(v.x & 0xffff0000u), s);
+  s = fmaf(a.z, __uint_as_float(v.y << 16), s);
+  s = fmaf(a.w, __uint_as_float(v.y & 0xffff0000u), s);
+  s = fmaf(b.x, __uint_as_float(v.z << 16), s);
+  s = fmaf(b.y, __uint_as_float(v.z & 0xffff0000u), s);
+  s = fmaf(b.z, __uint_as_float(v.w << 16), s);
+  return fmaf(b.w, __uint_as_float(v.w & 0xffff0000u), s);
+}
+
+// Exact fp32 <q, x> of 32 stored rows, lane l's row l (id < 0: none), each sum
+// in ascending order by its lane.  The rows pass through shared memory nine
+// 16-byte chunks at a time, copied by the whole warp so that a row's bytes are
+// read together: a lane reading its own row touches 32 lines an instruction
+// (10^7 rows of 192 bytes: 1 150 of 1 654 us, about 480 staged).  Nine chunks a row also
+// keep the lanes' 16-byte reads on distinct banks.
+constexpr int kRowChunks = 9;
+template <typename OT>
+__device__ float warp_rows_dot(const float* q, const OT* __restrict__ rows, int stride, int32_t id, uint4* buf, int lane) {
+  constexpr unsigned kFull = 0xffffffffu;
+  constexpr int E = 16 / (int)sizeof(OT);
+  const int chunks = stride / E, blocks = (chunks + kRowChunks - 1) / kRowChunks, per = (chunks + blocks - 1) / blocks;
+  const int many = 32 - __clz(__ballot_sync(kFull, id >= 0));      // rows up to the last one there is
   float s = 0.f;
-#pragma unroll 6
-  for (int k = 0; k < stride; k += 8) {
-    const uint4 v = __ldg(reinterpret_cast<const uint4*>(x + k));
-    const float4 a = *reinterpret_cast<const float4*>(q + k), b = *reinterpret_cast<const float4*>(q + k + 4);
-    s = fmaf(a.x, __uint_as_float(v.x << 16), s);
-    s = fmaf(a.y, __uint_as_float(v.x & 0xffff0000u), s);
-    s = fmaf(a.z, __uint_as_float(v.y << 16), s);
-    s = fmaf(a.w, __uint_as_float(v.y & 0xffff0000u), s);
-    s = fmaf(b.x, __uint_as_float(v.z << 16), s);
-    s = fmaf(b.y, __uint_as_float(v.z & 0xffff0000u), s);
-    s = fmaf(b.z, __uint_as_float(v.w << 16), s);
-    s = fmaf(b.w, __uint_as_float(v.w & 0xffff0000u), s);
+  for (int c0 = 0; c0 < chunks; c0 += per) {
+    const int m = min(per, chunks - c0);
+    __syncwarp();
+    for (int i0 = 0; i0 < many * m; i0 += 32) {
+      const int i = i0 + lane, r = i / m, c = i - r * m;
+      const int32_t rid = __shfl_sync(kFull, id, r & 31);
+      if (r < many && rid >= 0)
+        cp_async16(buf + r * kRowChunks + c, reinterpret_cast<const uint4*>(rows + (int64_t)rid * stride) + c0 + c);
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncwarp();
+    if (id >= 0)
+      for (int c = 0; c < m; ++c) s = chunk_dot(q + (c0 + c) * E, buf[lane * kRowChunks + c], s, OT());
   }
   return s;
 }
@@ -530,6 +588,7 @@ __device__ __forceinline__ float row_dot(const float* __restrict__ q, const __nv
 constexpr int kBins = 2048;
 constexpr int kBand = 1024;         // rows near the R-th score ranked in the defined order
 constexpr int kSample = 8;          // keys a thread samples
+constexpr int kProbeTable = 64;     // probes looked up in shared memory up to this t
 
 // Rows of a slice kept in shared memory: those at or above a bound that a
 // sample puts somewhat below the R-th best.
@@ -573,13 +632,15 @@ __global__ void __launch_bounds__(kThreads) finish_slices(
     const int64_t* __restrict__ pos, const int32_t* __restrict__ top, const int32_t* __restrict__ tpq, int64_t q0,
     int t, const int64_t* __restrict__ off, const int32_t* __restrict__ ids, const float* __restrict__ base,
     const float* __restrict__ smax, const void* __restrict__ Q, int qdt, int d, const OT* __restrict__ orig,
-    int ostride, int R, int k, int64_t* __restrict__ ids_out, float* __restrict__ scores_out) {
+    int ostride, int R, int k, int stage_at, int64_t* __restrict__ ids_out, float* __restrict__ scores_out) {
   constexpr unsigned kFull = 0xffffffffu;
   extern __shared__ __align__(16) unsigned char fs_smem[];
   __shared__ int32_t warp_s[32];
   __shared__ float red_s[5][kWarps];
   __shared__ int n_list, n_band, n_kept, bin_s, above_s;
   __shared__ float lo_s, hi_s, delta_s;
+  __shared__ int at_s[kProbeTable];             // where the probes' rows start in the slice
+  __shared__ int64_t row_s[kProbeTable];        // and the index row of the slice's position 0 in that probe
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   const int64_t ql = blockIdx.x, q = q0 + ql;
   const uint32_t* K = keys + ql * slice;
@@ -596,9 +657,13 @@ __global__ void __launch_bounds__(kThreads) finish_slices(
   uint64_t* band_key = reinterpret_cast<uint64_t*>(hist);                 // over the histogram once the bin is known
   int32_t* band = reinterpret_cast<int32_t*>(hist + kBins);               // [kBand]
   int32_t* list = band + kBand;                                           // [R] positions in the slice, then ids
-  uint32_t* kept = reinterpret_cast<uint32_t*>(list + (R + 1) / 2 * 2);   // [cap] keys
+  uint32_t* kept = reinterpret_cast<uint32_t*>(
+      fs_smem + (reinterpret_cast<unsigned char*>(list + (R + 1) / 2 * 2) - fs_smem + 15) / 16 * 16);   // [cap] keys
   int32_t* kept_at = reinterpret_cast<int32_t*>(kept + cap);              // [cap] positions
-  uint64_t* ex = reinterpret_cast<uint64_t*>(kept);                       // [pow2 >= R] once the list is known
+  // once the list is known: the exact keys and a warp's staged rows (over each
+  // other for k <= 32, where the keys are the warps' few best)
+  uint64_t* ex = reinterpret_cast<uint64_t*>(kept);                       // [sorted]
+  uint4* stage = reinterpret_cast<uint4*>(fs_smem + stage_at) + 32 * kRowChunks * w;
 
   for (int i = tid; i < ostride; i += kThreads)
     qrow[i] = i >= d ? 0.f
@@ -610,6 +675,10 @@ __global__ void __launch_bounds__(kThreads) finish_slices(
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) norms.z = fmaxf(norms.z, __shfl_xor_sync(kFull, norms.z, o));
   if (tid == 0) n_list = n_band = n_kept = 0;
+  if (tid < tq && tid < kProbeTable) {
+    at_s[tid] = (int)qpos[tid];
+    row_s[tid] = off[probes[tid]] - qpos[tid];
+  }
   // a sample and its range
   uint32_t sample[kSample];
   float lo = INFINITY, hi = -INFINITY;
@@ -653,19 +722,21 @@ __global__ void __launch_bounds__(kThreads) finish_slices(
   lo = lo_s;
   hi = hi_s;
   const float delta = delta_s;
-  // position i of the slice: its probe, then its row
-  const auto probe_of = [&](int64_t i) {
+  // position i of the slice: its probe, its row
+  const bool table = tq <= kProbeTable;
+  const auto probe_of = [&](int i) {
     int a = 0, b = tq - 1;
     while (a < b) {
       const int mid = (a + b + 1) >> 1;
-      if (qpos[mid] <= i) a = mid;
+      if ((table ? at_s[mid] : (int)qpos[mid]) <= i) a = mid;
       else b = mid - 1;
     }
     return a;
   };
-  const auto defined_key = [&](int64_t i) {
+  const auto row_of = [&](int i, int j) { return table ? row_s[j] + i : off[probes[j]] - qpos[j] + i; };
+  const auto defined_key = [&](int i) {
     const int j = probe_of(i);
-    const int64_t r = off[probes[j]] + (i - qpos[j]);
+    const int64_t r = row_of(i, j);
     return rank_key(rows.exact(qs, q, r, base ? base[ql * t + j] : 0.f), (uint32_t)ids[r]);
   };
   const auto append = [&](bool in, int* count, int32_t* to, int cap, int32_t v) {
@@ -742,8 +813,7 @@ __global__ void __launch_bounds__(kThreads) finish_slices(
     // the list's rows as ids, then the band's best
     const int have = n_list;
     for (int i = tid; i < have; i += kThreads) {
-      const int j = probe_of(list[i]);
-      list[i] = ids[off[probes[j]] + (list[i] - qpos[j])];
+      list[i] = ids[row_of(list[i], probe_of(list[i]))];
     }
     for (int i = tid; i < R - have; i += kThreads) list[have + i] = (int32_t)(band_key[i] & 0xffffffffu);
     __syncthreads();
@@ -859,10 +929,7 @@ __global__ void __launch_bounds__(kThreads) finish_slices(
       const bool counts_ = i < n && K[i] != 0u;
       const bool in = counts_ && (limit == ~0ull || defined_key(i) <= limit);
       int32_t id = -1;
-      if (in) {
-        const int j = probe_of(i);
-        id = ids[off[probes[j]] + (i - qpos[j])];
-      }
+      if (in) id = ids[row_of(i, probe_of(i))];
       append(in, &n_list, list, R, id);
     }
     __syncthreads();
@@ -887,14 +954,11 @@ __global__ void __launch_bounds__(kThreads) finish_slices(
     };
     for (int i0 = 32 * w; i0 < have; i0 += kThreads) {
       const int i = i0 + lane;
-      uint64_t key = ~0ull;
-      if (i < have) {
-        const int32_t id = list[i];
-        const float s = row_dot(qrow, orig + (int64_t)id * ostride, ostride);
-        if (s == s) key = rank_key(s, (uint32_t)id);
-      }
-      insert(key);
+      const int32_t id = i < have ? list[i] : -1;
+      const float s = warp_rows_dot(qrow, orig, ostride, id, stage, lane);
+      insert(id >= 0 && s == s ? rank_key(s, (uint32_t)id) : ~0ull);
     }
+    __syncthreads();                              // (the staged rows lie over ex)
     ex[32 * w + lane] = lane < k ? best : ~0ull;
     __syncthreads();
     if (w == 0) {
@@ -907,14 +971,11 @@ __global__ void __launch_bounds__(kThreads) finish_slices(
   } else {
     int N = 2;
     while (N < max(have, k)) N <<= 1;           // (k <= R: within ex)
-    for (int i = tid; i < N; i += kThreads) {
-      uint64_t key = ~0ull;
-      if (i < have) {
-        const int32_t id = list[i];
-        const float s = row_dot(qrow, orig + (int64_t)id * ostride, ostride);
-        if (s == s) key = rank_key(s, (uint32_t)id);
-      }
-      ex[i] = key;
+    for (int i0 = 32 * w; i0 < N; i0 += kThreads) {
+      const int i = i0 + lane;
+      const int32_t id = i < have ? list[i] : -1;
+      const float s = warp_rows_dot(qrow, orig, ostride, id, stage, lane);
+      if (i < N) ex[i] = id >= 0 && s == s ? rank_key(s, (uint32_t)id) : ~0ull;
     }
     __syncthreads();
     block_sort(ex, N);
@@ -969,9 +1030,12 @@ void run(const IndexData& ix, Rows rws, float* base, int* smax, const float* Qf,
   int sorted = kThreads;                                  // exact keys: the warps' lists, or R of them to sort
   if (k > 32)
     while (sorted < R) sorted <<= 1;
-  const size_t fin_smem = sizeof(float) * ((size_t)(ostride + 3) / 4 * 4 + (rws.query_floats() + 3) / 4 * 4) +
-                          sizeof(int) * (size_t)(kBins + kBand) + sizeof(int32_t) * (size_t)((R + 1) / 2 * 2) +
-                          std::max(sizeof(uint64_t) * (size_t)kept_rows(R), sizeof(uint64_t) * (size_t)sorted);
+  const auto up = [](size_t b) { return (b + 15) / 16 * 16; };
+  const size_t kept_at = up(sizeof(float) * ((size_t)(ostride + 3) / 4 * 4 + (rws.query_floats() + 3) / 4 * 4) +
+                            sizeof(int) * (size_t)(kBins + kBand) + sizeof(int32_t) * (size_t)((R + 1) / 2 * 2));
+  const size_t stage_at = kept_at + (k > 32 ? up(sizeof(uint64_t) * (size_t)sorted) : 0);
+  const size_t fin_smem = std::max(kept_at + sizeof(uint64_t) * (size_t)std::max(kept_rows(R), sorted),
+                                   stage_at + sizeof(uint4) * 32 * kRowChunks * kWarps);
   const size_t item_smem = rws.item_smem();
   SOAR_CUDA(cudaFuncSetAttribute(score_items<Rows>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)item_smem));
   const auto finish = [&](auto elem, int64_t q0, int64_t m) {
@@ -980,7 +1044,7 @@ void run(const IndexData& ix, Rows rws, float* base, int* smax, const float* Qf,
     SOAR_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fin_smem));
     kern<<<(unsigned)m, kThreads, fin_smem, s>>>(rws, keys, counts, slice, pos, top, tpq, q0, t, ix.offsets, ix.ids,
                                                  base, reinterpret_cast<const float*>(smax), Q, (int)dt, ix.d, static_cast<const OT*>(ix.originals),
-                                                 ostride, R, k, ids_out, scores_out);
+                                                 ostride, R, k, (int)stage_at, ids_out, scores_out);
     SOAR_LAUNCHED();
   };
   for (int64_t q0 = 0; q0 < nq; q0 += cq) {
