@@ -1,37 +1,46 @@
 // Primary and first spilled assignment on the 5th-generation tensor cores.
 //
-// One persistent CTA per SM takes tiles of 128 points.  The tile's points
-// (and, for the spill, their unit residuals r_hat = (x - C[pi(x)]) / ||x - C[pi(x)]||)
-// form the A operands in shared memory (fp32 rows in the K-major core-matrix
-// layout of tc.cuh, staged by cp.async); the codebook, packed once per pass
-// in that layout as B tiles of N = 256 centroids (128 for the spill) split
-// into 8-column K steps, streams through a deep shared-memory ring of those
-// K steps, copied by cp.async.bulk (it stays in L2: every CTA reads all of
-// it, each CTA starting at its own tile).  Per K step one thread issues the
-// kind::tf32 MMA X.C^T (and R.C^T for the spill) into a double-buffered TMEM
-// accumulator; a wide N keeps the MMAs compute-bound rather than bound by
-// re-reading the A tile from shared memory.  Eight epilogue warps read the
-// scores back, one point per TMEM lane and half of the tile's columns per
-// warp, and evaluate the expanded loss of Theorem 3.1
+// One persistent CTA per SM takes items of points whose rows form two A operands
+// of 128 rows in shared memory (fp32 in the K-major core-matrix layout of
+// tc.cuh, staged by cp.async): for the primary assignment two blocks of 128
+// points, for the spill 128 points and their unit residuals r_hat = (x -
+// C[pi(x)]) / ||x - C[pi(x)]|| (one A operand where rows are too wide for two).
+// The codebook, packed once per pass in that layout as B tiles of 128
+// centroids split into 8-column K steps, streams through a shared-memory ring
+// of those K steps, copied by cp.async.bulk (it stays in L2: every CTA reads
+// all of it, each starting at its own tile); every B tile serves both A
+// operands, which halves that traffic.  Per K step one thread issues the
+// kind::tf32 MMAs into a double-buffered TMEM accumulator.  Eight epilogue
+// warps read the scores back, one point per TMEM lane (the spill: two warps a
+// lane, half of the tile's columns each), and evaluate the expanded loss of
+// Theorem 3.1
 //     L(c') = ||c'||^2 - 2<x, c'> + lambda (<x, r_hat> - <c', r_hat>)^2
 // (||x||^2 dropped: constant per point; lambda term absent for the primary).
 //
-// Rigorous screening.  kind::tf32 truncates each operand to 10 mantissa bits,
-// so |<a, b>~ - <a, b>| < 2^-9 ||a|| ||b|| (fp32 accumulation is far below
-// that).  With a factor-2 margin the screened loss of a pair is within
-//     delta = 2^-7 ||x|| ||c'|| + lambda e (2 |t~| + e),  e = 2^-8 ||c'||,
-// (t~ = <x, r_hat> - <c', r_hat>~) plus a small fp32 rounding allowance of the
-// exact loss.  Per point the epilogue keeps the kList smallest lower bounds
-// L~ - delta and the smallest upper bound U = min(L~ + delta); the true
-// minimiser has lower bound <= U, so it is among the kept candidates unless
-// more than kList lower bounds reach U (the point is then flagged and its
-// refine pass scores every centroid).  Centroids the point is already
-// assigned to are excluded (the spill reading of Section 3.3).  The refine
-// kernel decides among the candidates with the direct form
-// ||x - c'||^2 + lambda <x - c', r_hat>^2, lower index on ties.
+// Rigorous screening.  Both operands are rounded to the nearest tf32 value
+// before the MMA (an error of 2^-11 each; the hardware would truncate, 2^-10), so
+// |<a, b>~ - <a, b>| < 2^-10 (1 + 2^-12) ||a|| ||b||, and the fp32 accumulation
+// adds at most 2^-16 ||a|| ||b||.  The screened loss of a pair is within
+//     delta = 2^-9 (1 + 2^-4) ||x|| ||c'|| + lambda e (2 |t~| + e),
+//     e = 2^-10 (1 + 2^-4) ||c'||,
+// (t~ = <x, r_hat> - <c', r_hat>~) plus an allowance for the fp32 rounding of the
+// loss and of the exact decision.  Per point the epilogue keeps the smallest
+// upper bound U = min(L~ + delta) so far and the pairs with L~ - delta <= U; the
+// true minimiser is among them unless more than the list holds are (the point
+// is then flagged and its refine pass scores every centroid).  Centroids the
+// point is already assigned to are excluded.  A point with one candidate left
+// is decided; the others are queued, and the refine kernel decides among the
+// candidates with the direct form ||x - c'||^2 + lambda <x - c', r_hat>^2, lower
+// index on ties.
+//
+// Bound of the primary: the epilogue's issue slots and the codebook stream from
+// L2 (tf32 floor 0.51 ms for 1.18 M x 100 against 2 000 centroids).  Keeping the
+// sixteen smallest lower bounds sorted cost 37 of 47 instructions a pair (5.9 ms
+// a pass, the spill 6.8); most pairs are now dismissed eight at a time by a
+// maximum that the TMEM load computes: 1.84 ms, the spill 3.82.
 //
 // Warp roles: 0 = bulk-copy producer, 1 = TMEM owner and MMA issuer,
-// 2..5 = epilogue and A-operand loaders.  Every mbarrier wait is bounded;
+// 2 = gate, 3..10 = epilogue and A-operand loaders.  Every mbarrier wait is bounded;
 // on expiry the CTA raises *err, stops, waits (bounded) for its copies and
 // MMAs in flight, frees its TMEM and returns.
 #include <type_traits>
@@ -43,25 +52,30 @@ namespace soar {
 
 namespace {
 
-constexpr int kTM = 128;       // points per tile (MMA M)
-constexpr int kEpi = 256;      // epilogue threads (8 warps: 4 lane quarters x 2 column halves)
+constexpr int kTM = 128;       // rows of an A operand (MMA M)
+constexpr int kN = 128;        // centroids of a B tile (MMA N): two operands x two buffers fill the 512 TMEM columns
+constexpr int kEpi = 256;      // epilogue threads (8 warps: 4 lane quarters x 2)
 constexpr int kThr = 96 + kEpi;   // producer, MMA issuer, gate, epilogue
 constexpr int kStagesMax = 8;
 constexpr int kStageBytes = 32768;   // codebook stage: 32 KB keeps bulk copies near full L2 bandwidth
-constexpr int kList = 16;      // candidates kept per point
-// parking area: a tile's 16 screened bounds per epilogue thread, overlaid at
-// the end by the merge area (two lists of kList plus two scalars per point)
-constexpr int kPark = 16 * kEpi > 2 * kList * kTM + 2 * kTM ? 16 * kEpi : 2 * kList * kTM + 2 * kTM;
+constexpr int kSteps = kStageBytes / (kN * 32);   // K steps per codebook stage
+constexpr int kList = 16;      // candidates handed to the refine per point
 
-// B tile width per pass: both fill the 512 TMEM columns with two buffers.
-__host__ __device__ constexpr int tile_n(int ndir) { return ndir ? 128 : 256; }
+// v rounded to the nearest value with 10 explicit mantissa bits (ties away from
+// zero); infinities and NaNs pass through.
+__device__ __forceinline__ float round_tf32(float v) {
+  uint32_t u = __float_as_uint(v);
+  if ((u & 0x7f800000u) == 0x7f800000u) return v;
+  u = (u + 0x1000u) & 0xffffe000u;
+  return __uint_as_float(u);
+}
 
 template <typename XT>
 struct AsgParams {
   const XT* X;
   int64_t n;
   int d, kp;
-  const float* Cc;        // [ctiles][kp / 8][N][8] packed codebook (padding rows: zeros, +inf norm)
+  const float* Cc;        // [ctiles][kp / 8][kN][8] packed codebook (padding rows: zeros, +inf norm)
   const float* tmax;      // [ctiles] largest ||c|| of each B tile
   const float* C;         // [c][d] row-major
   int c, ctiles;
@@ -70,7 +84,7 @@ struct AsgParams {
   const float* inv_rn;    // [n][4] 1 / ||x - C[pi(x)]|| (0 for a zero residual)
   float lambda;
   int stages;
-  int* counter;
+  int cap;                // candidates an epilogue thread holds
   int* err;
   int32_t* cand;          // [n][kList] candidate centroids, -1 padded
   int32_t* ovf;           // [n] 1 when the candidates are not conclusive
@@ -82,31 +96,31 @@ struct AsgParams {
 __device__ __forceinline__ float ld(const float* p) { return __ldg(p); }
 __device__ __forceinline__ float ld(const __nv_bfloat16* p) { return __bfloat162float(*p); }
 
-template <int NDIR, typename XT>
+// OPS = A operands: 2 (primary: two blocks of points; spill: points and
+// residuals) or, for the primary only, 1.
+template <int NDIR, int OPS, typename XT>
 __global__ void __launch_bounds__(kThr, 1) assign_tc_kernel(AsgParams<XT> P) {
-  constexpr int N = tile_n(NDIR);
-  constexpr uint32_t kW = (1 + NDIR) * N;       // TMEM columns per accumulator buffer
-  constexpr int kHalf = N / 2;                  // columns per epilogue thread and tile
-  constexpr int G = kStageBytes / (N * 32);     // K steps per codebook stage
+  constexpr bool kSplit = NDIR > 0 || OPS == 1;    // two epilogue threads a point, half of the columns each
+  constexpr int kPts = kSplit ? kTM : 2 * kTM;  // points per item
+  constexpr int kCols = kSplit ? kN / 2 : kN;   // columns per epilogue thread and tile
+  constexpr uint32_t kW = OPS * kN;             // TMEM columns per accumulator buffer
   // the no-swizzle operand layout needs 16-byte alignment only
   extern __shared__ __align__(128) unsigned char smem_raw[];
   unsigned char* base = reinterpret_cast<unsigned char*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~uintptr_t(127));
   const int kp = P.kp, S = P.stages, ksteps = kp / 8;
-  const int nch = (ksteps + G - 1) / G;         // stages per B tile
+  const int nch = (ksteps + kSteps - 1) / kSteps;   // stages per B tile
   const uint32_t sbo = (uint32_t)kp * 32u;
   const uint32_t a_bytes = (uint32_t)kTM * kp * 4u;
-  float* sX = reinterpret_cast<float*>(base);
-  float* sR = reinterpret_cast<float*>(base + a_bytes);                       // spill only
-  unsigned char* sB = base + (1 + NDIR) * (size_t)a_bytes;
-  float* lb_s = reinterpret_cast<float*>(sB + (size_t)S * kStageBytes);      // [16][kEpi] parked bounds
-  // merge area, overlaid on the parking area once every tile is done
-  float* mlb_s = lb_s;                                                       // [kList][kTM]
-  int* mid_s = reinterpret_cast<int*>(mlb_s + kList * kTM);                 // [kList][kTM]
-  float* mu_s = reinterpret_cast<float*>(mid_s + kList * kTM);              // [kTM] U of the second half
+  unsigned char* sA = base;                                                  // OPS operands
+  unsigned char* sB = base + (size_t)OPS * a_bytes;
+  float* list_lb = reinterpret_cast<float*>(sB + (size_t)S * kStageBytes);   // [cap][kEpi]
+  int* list_id = reinterpret_cast<int*>(list_lb + P.cap * kEpi);             // [cap][kEpi]
+  float* nx_s = reinterpret_cast<float*>(list_id + P.cap * kEpi);            // [kEpi] ||x||
+  float* mu_s = nx_s + kEpi;                                                // [kTM] U of the second half
   float* mev_s = mu_s + kTM;                                                // [kTM]
-  float* nx_s = lb_s + kPark;                                               // [kTM] ||x||
-  float* xr_s = nx_s + kTM;                                                 // [kTM] <x, r_hat>
+  int* mcnt_s = reinterpret_cast<int*>(mev_s + kTM);                        // [kTM]
+  float* xr_s = reinterpret_cast<float*>(mcnt_s + kTM);                     // [kTM] <x, r_hat>
   float* rn_s = xr_s + kTM;                                                 // [kTM] 1 or 0 (zero residual)
   int* prior_s = reinterpret_cast<int*>(rn_s + kTM);                        // [kTM]
   uint64_t* bars = reinterpret_cast<uint64_t*>(prior_s + kTM);
@@ -136,19 +150,21 @@ __global__ void __launch_bounds__(kThr, 1) assign_tc_kernel(AsgParams<XT> P) {
   __syncthreads();
   tc::fence_after_sync();
   const uint32_t tmem = tmem_base_s;
-  const uint32_t idesc = tc::idesc_tf32(kTM, N);
+  const uint32_t idesc = tc::idesc_tf32(kTM, kN);
   volatile int* abort_v = &abort_s;
   auto give_up = [&]() {
     if (atomicExch(&abort_s, 1) == 0) atomicExch(P.err, 1);
   };
-  // epilogue thread: TMEM lane quarter q = warp % 4 (point row m), column half hh
+  // epilogue thread: TMEM lane 32 (warp % 4) + lane = row m of an operand; hh: its
+  // operand (two blocks of points) or its half of the columns
   const int m = 32 * (warp & 3) + lane;
   const int hh = (warp - 3) >> 2;
-  const int et = threadIdx.x - 96;              // epilogue thread index (parking column)
+  const int mp = kSplit ? m : m + kTM * hh;     // point within the item
+  const int et = threadIdx.x - 96;              // epilogue thread index (list column)
 
   // static schedule: items blockIdx.x, blockIdx.x + gridDim.x, ... so that the
   // producer can stream the codebook across item boundaries
-  const int ntiles_pts = (int)((P.n + kTM - 1) / kTM);
+  const int ntiles_pts = (int)((P.n + kPts - 1) / kPts);
   const int nitems = ntiles_pts > (int)blockIdx.x ? (ntiles_pts - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
   // each CTA sweeps the codebook from its own starting tile, so that the SMs
   // do not all read the same L2 lines at the same moment
@@ -165,10 +181,10 @@ __global__ void __launch_bounds__(kThr, 1) assign_tc_kernel(AsgParams<XT> P) {
           for (int g = 0; g < nch; ++g, ++C) {
             const uint32_t s = C % S, ph = (C / S) & 1;
             if (!tc::bar_wait(empty(s), ph ^ 1, abort_v)) { give_up(); stop = true; break; }
-            const int k0 = g * G, kn = min(G, ksteps - k0);
-            const uint32_t bytes = (uint32_t)kn * N * 32;
+            const int k0 = g * kSteps, kn = min(kSteps, ksteps - k0);
+            const uint32_t bytes = (uint32_t)kn * kN * 32;
             tc::bar_arrive_expect_tx(full(s), bytes);
-            tc::bulk_copy_g2s(tc::smem_u32(sB) + s * kStageBytes, P.Cc + ((int64_t)ti * ksteps + k0) * N * 8,
+            tc::bulk_copy_g2s(tc::smem_u32(sB) + s * kStageBytes, P.Cc + ((int64_t)ti * ksteps + k0) * kN * 8,
                               bytes, full(s));
             issued_s = (int)(C + 1);
           }
@@ -180,19 +196,19 @@ __global__ void __launch_bounds__(kThr, 1) assign_tc_kernel(AsgParams<XT> P) {
     for (int it = 0; it < nitems; ++it) {
       if (tc::named_bar_or(3, kThr - 32, *abort_v != 0)) break;   // (also ends the previous item)
       const int item = (int)blockIdx.x + it * (int)gridDim.x;
-      const int64_t p = (int64_t)item * kTM + m;
+      const int64_t p = (int64_t)item * kPts + mp;
       const bool active = warp >= 3 && p < P.n;
 
-      // ---- A operands (first-half epilogue warps): the tile's points and
-      // unit residuals, each row closed by (-1/2, -1/2) in columns d, d+1
-      // against the codebook's (hi, lo) split of ||c||^2
-      if (warp >= 3 && hh == 0) {
-        float* xrow = sX + (m >> 3) * (kp * 8) + (m & 7) * 4;
-        float* rrow = sR + (m >> 3) * (kp * 8) + (m & 7) * 4;
+      // ---- A operands: a thread stages one row, rounded to tf32 and closed by
+      // (-1/2, -1/2) in columns d, d + 1 against the codebook's (hi, lo) split of
+      // ||c||^2; with residuals, the second half of the threads stages those
+      if (warp >= 3 && (OPS == 2 || hh == 0)) {
+        const bool resid = NDIR > 0 && hh == 1;
+        float* row = reinterpret_cast<float*>(sA + (size_t)(OPS == 2 ? hh : 0) * a_bytes) + (m >> 3) * (kp * 8) + (m & 7) * 4;
         float inv = 0.f;
         int prior = -1;
         const float* cr = nullptr;
-        if (NDIR > 0 && active) {
+        if (resid && active) {
           prior = P.assign[p * P.astride];
           inv = P.inv_rn[p * 4];
           cr = P.C + (int64_t)prior * P.d;
@@ -202,19 +218,18 @@ __global__ void __launch_bounds__(kThr, 1) assign_tc_kernel(AsgParams<XT> P) {
         const int d4 = vec ? P.d / 4 : 0;               // 16-byte chunks staged by cp.async
         if (vec && active) {
           const float* xsrc = reinterpret_cast<const float*>(P.X) + p * P.d;
-          for (int k4 = 0; k4 < d4; ++k4) tc::cp_async16(tc::smem_u32(xrow + k4 * 32), xsrc + 4 * k4);
-          if (NDIR > 0)
-            for (int k4 = 0; k4 < d4; ++k4) tc::cp_async16(tc::smem_u32(rrow + k4 * 32), cr + 4 * k4);
+          for (int k4 = 0; k4 < d4; ++k4) tc::cp_async16(tc::smem_u32(row + k4 * 32), xsrc + 4 * k4);
         }
         tc::cp_async_wait_all();
+#pragma unroll 4
         for (int k4 = 0; k4 < kp / 4; ++k4) {
-          float xv[4], rv[4], cv[4] = {0.f, 0.f, 0.f, 0.f};
+          float xv[4], cv[4] = {0.f, 0.f, 0.f, 0.f};
           if (k4 < d4) {
             if (active) {
-              const float4 a = *reinterpret_cast<const float4*>(xrow + k4 * 32);
+              const float4 a = *reinterpret_cast<const float4*>(row + k4 * 32);
               xv[0] = a.x; xv[1] = a.y; xv[2] = a.z; xv[3] = a.w;
-              if (NDIR > 0) {
-                const float4 b = *reinterpret_cast<const float4*>(rrow + k4 * 32);
+              if (resid) {
+                const float4 b = __ldg(reinterpret_cast<const float4*>(cr + 4 * k4));
                 cv[0] = b.x; cv[1] = b.y; cv[2] = b.z; cv[3] = b.w;
               }
             } else {
@@ -225,26 +240,31 @@ __global__ void __launch_bounds__(kThr, 1) assign_tc_kernel(AsgParams<XT> P) {
             for (int u = 0; u < 4; ++u) {
               const int k = 4 * k4 + u;
               xv[u] = (active && k < P.d) ? ld(P.X + p * P.d + k) : 0.f;
-              if (NDIR > 0) cv[u] = (active && k < P.d) ? __ldg(cr + k) : 0.f;
+              if (resid) cv[u] = (active && k < P.d) ? __ldg(cr + k) : 0.f;
             }
           }
+          float av[4];
 #pragma unroll
           for (int u = 0; u < 4; ++u) {
-            ss = fmaf(xv[u], xv[u], ss);
-            if (NDIR > 0) {
-              rv[u] = (xv[u] - cv[u]) * inv;
-              xd = fmaf(xv[u], rv[u], xd);
-            }
             const int k = 4 * k4 + u;
-            if (k == P.d || k == P.d + 1) xv[u] = -0.5f;
+            if (resid) {
+              const float rv = (xv[u] - cv[u]) * inv;
+              xd = fmaf(xv[u], rv, xd);
+              av[u] = round_tf32(rv);
+            } else {
+              ss = fmaf(xv[u], xv[u], ss);
+              av[u] = (k == P.d || k == P.d + 1) ? -0.5f : round_tf32(xv[u]);
+            }
           }
-          *reinterpret_cast<float4*>(xrow + k4 * 32) = make_float4(xv[0], xv[1], xv[2], xv[3]);
-          if (NDIR > 0) *reinterpret_cast<float4*>(rrow + k4 * 32) = make_float4(rv[0], rv[1], rv[2], rv[3]);
+          *reinterpret_cast<float4*>(row + k4 * 32) = make_float4(av[0], av[1], av[2], av[3]);
         }
-        nx_s[m] = sqrtf(ss);
-        xr_s[m] = xd;                                  // <x, r_hat> of the stored (fp32) r_hat
-        rn_s[m] = inv > 0.f ? 1.f : 0.f;
-        prior_s[m] = prior;
+        if (resid) {
+          xr_s[m] = xd;                                  // <x, r_hat> of the fp32 r_hat
+          rn_s[m] = inv > 0.f ? 1.f : 0.f;
+          prior_s[m] = prior;
+        } else {
+          nx_s[mp] = sqrtf(ss);
+        }
         tc::fence_async_smem();
       }
       asm volatile("bar.sync 3, %0;" ::"n"(kThr - 32) : "memory");
@@ -263,14 +283,14 @@ __global__ void __launch_bounds__(kThr, 1) assign_tc_kernel(AsgParams<XT> P) {
             if (lane == 0) {
               const uint32_t C = chunk_ctr + i * nch + g, s = C % S;
               tc::fence_after_sync();
-              const int k0 = g * G, kn = min(G, ksteps - k0);
+              const int k0 = g * kSteps, kn = min(kSteps, ksteps - k0);
               for (int jj = 0; jj < kn; ++jj) {
                 const int j = k0 + jj;
-                const uint64_t bd = tc::smem_desc(tc::smem_u32(sB) + s * kStageBytes + jj * N * 32, 128, 256);
-                tc::mma_tf32(tmem + b * kW, tc::smem_desc(tc::smem_u32(sX) + j * 256, 128, sbo), bd, idesc, j > 0);
-                if (NDIR > 0)
-                  tc::mma_tf32(tmem + b * kW + N, tc::smem_desc(tc::smem_u32(sR) + j * 256, 128, sbo), bd, idesc,
-                               j > 0);
+                const uint64_t bd = tc::smem_desc(tc::smem_u32(sB) + s * kStageBytes + jj * kN * 32, 128, 256);
+#pragma unroll
+                for (int o = 0; o < OPS; ++o)
+                  tc::mma_tf32(tmem + b * kW + o * kN,
+                               tc::smem_desc(tc::smem_u32(sA) + o * a_bytes + j * 256, 128, sbo), bd, idesc, j > 0);
               }
               tc::mma_commit(empty(s));              // the stage is free once these MMAs completed
             }
@@ -301,14 +321,14 @@ __global__ void __launch_bounds__(kThr, 1) assign_tc_kernel(AsgParams<XT> P) {
           }
         }
       } else {
-        // ---- epilogue: kHalf of each B tile's N columns per thread
-        float lbs[kList];
-        int ids[kList];
-#pragma unroll
-        for (int j = 0; j < kList; ++j) { lbs[j] = INFINITY; ids[j] = -1; }
-        float U = INFINITY, ev = INFINITY;
-        const float nx = nx_s[m], xr = xr_s[m], er0 = ldexpf(rn_s[m], -8);
-        const int prior = prior_s[m];
+        // ---- epilogue: kCols of each B tile's columns per thread
+        float* lbs = list_lb + et;                     // [cap] lower bounds and ids of the candidates so far
+        int* ids = list_id + et;
+        int cnt = 0;
+        float U = INFINITY, ev = INFINITY;             // ev: the smallest lower bound the list had no room for
+        const float nx = nx_s[mp], nx2 = nx * nx;
+        const float xr = NDIR > 0 ? xr_s[m] : 0.f, er0 = NDIR > 0 ? ldexpf(rn_s[m], -10) * 1.0625f : 0.f;
+        const int prior = NDIR > 0 ? prior_s[m] : -1;
         const float lam = P.lambda;
         for (int i = 0; i < P.ctiles; ++i) {
           const uint32_t T = tile_ctr + i, b = T & 1, tph = (T >> 1) & 1;
@@ -319,73 +339,83 @@ __global__ void __launch_bounds__(kThr, 1) assign_tc_kernel(AsgParams<XT> P) {
           const int ti = (i + rot) % P.ctiles;
           const float cmax = __ldg(P.tmax + ti), c2max = cmax * cmax;
           const float e = er0 * cmax;
-          float dlc = fmaf(ldexpf(nx, -7), cmax, ldexpf(fmaf(nx, cmax, c2max), -14));
+          float dlc = fmaf(ldexpf(nx, -9) * 1.0625f, cmax, ldexpf(fmaf(nx, cmax, c2max), -14) + ldexpf(nx2, -16));
           if (NDIR > 0) dlc = fmaf(lam * e, e, fmaf(ldexpf(lam, -14), (nx + cmax) * (nx + cmax), dlc));
           const float two_le = 2.f * lam * e;
 #pragma unroll 1
-          for (int rd = 0; rd < kHalf / 32 && ok; ++rd) {
-            const int col0 = hh * kHalf + 32 * rd;
-            uint32_t rx[32], rr[32];
-            const uint32_t taddr = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + b * kW + col0;
-            tc::tmem_ld32(taddr, rx);
-            if (NDIR > 0) tc::tmem_ld32(taddr + N, rr);
-            tc::tmem_ld_wait();
-            const int cbase = ti * N + col0;
-            const int jskip = (NDIR > 0) ? prior - cbase : -1;       // the point's own centroid
+          for (int rd = 0; rd < kCols / 32 && ok; ++rd) {
+            const int col0 = (kSplit ? hh * kCols : 0) + 32 * rd;
+            const uint32_t taddr = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + b * kW +
+                                   (!kSplit && OPS == 2 ? hh * kN : 0) + col0;
+            const int cbase = ti * kN + col0;
+            float v[32];                               // primary: <x, c> - ||c||^2 / 2; spill: lower bounds
+            uint32_t gm = 0u;                          // groups of eight columns that hold a candidate
+            if constexpr (NDIR == 0) {
+              uint32_t rx[32];
+              float g[4];
 #pragma unroll
-            for (int h2 = 0; h2 < 2; ++h2) {
-              const float worst0 = lbs[kList - 1];
-              uint32_t mask = 0;
-              // four interleaved partial minima keep the dependency chains
-              // short; padded centroid rows carry ||c||^2 = +inf, so their
-              // loss is +inf and they drop out without a test
-              float um[4] = {INFINITY, INFINITY, INFINITY, INFINITY};
-              float evp[4] = {INFINITY, INFINITY, INFINITY, INFINITY};
+              for (int q8 = 0; q8 < 4; ++q8) tc::tmem_ld8_max(taddr + 8 * q8, rx + 8 * q8, g[q8]);
+              tc::tmem_ld_wait();
+              // (padded centroids carry ||c||^2 = +inf: their product is -inf)
+              U = fminf(U, fmaf(-2.f, fmaxf(fmaxf(g[0], g[1]), fmaxf(g[2], g[3])), dlc));
+              const float cut = -0.5f * (U + dlc);     // L~ - delta <= U
 #pragma unroll
-              for (int j2 = 0; j2 < 16; ++j2) {
-                const int j = 16 * h2 + j2;
-                float L = -2.f * __uint_as_float(rx[j]);
-                float lb, ub;
-                if constexpr (NDIR > 0) {
-                  const float t = xr - __uint_as_float(rr[j]);
-                  L = fmaf(lam * t, t, L);
-                  const float dl = fmaf(two_le, fabsf(t), dlc);
-                  lb = j == jskip ? INFINITY : L - dl;
-                  ub = j == jskip ? INFINITY : L + dl;
-                } else {
-                  lb = L - dlc;
-                  ub = L;                                   // + dlc once per round
-                }
-                um[j2 & 3] = fminf(um[j2 & 3], ub);
-                const bool in = lb < worst0;
-                evp[j2 & 3] = in ? evp[j2 & 3] : fminf(evp[j2 & 3], lb);
-                if (in) {
-                  mask |= 1u << j2;
-                  lb_s[j2 * kEpi + et] = lb;
-                }
+              for (int q8 = 0; q8 < 4; ++q8) gm |= (g[q8] >= cut ? 1u : 0u) << q8;
+#pragma unroll
+              for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(rx[j]);
+            } else {
+              uint32_t rx[32], rr[32];
+              tc::tmem_ld32(taddr, rx);
+              tc::tmem_ld32(taddr + kN, rr);
+              tc::tmem_ld_wait();
+              float um[4] = {INFINITY, INFINITY, INFINITY, INFINITY}, lm[4] = {INFINITY, INFINITY, INFINITY, INFINITY};
+              const int jskip = prior - cbase;         // the point's own centroid
+              if (__any_sync(0xffffffffu, (unsigned)jskip < 32u)) {
+#pragma unroll
+                for (int j = 0; j < 32; ++j)
+                  if (j == jskip) rx[j] = 0xff800000u;   // -inf: an infinite loss
               }
-              float umin = fminf(fminf(um[0], um[1]), fminf(um[2], um[3]));
-              if constexpr (NDIR == 0) umin += dlc;
-              ev = fminf(ev, fminf(fminf(evp[0], evp[1]), fminf(evp[2], evp[3])));
-              U = fminf(U, umin);
-              for (; mask; mask &= mask - 1) {
-                const int j2 = __ffs(mask) - 1;
-                float v = lb_s[j2 * kEpi + et];
-                if (!(v < lbs[kList - 1])) {
-                  ev = fminf(ev, v);
-                  continue;
-                }
-                ev = fminf(ev, lbs[kList - 1]);
-                int id = cbase + 16 * h2 + j2;
 #pragma unroll
-                for (int q = 0; q < kList; ++q) {
-                  if (v < lbs[q]) {
-                    const float tv = lbs[q];
-                    const int tid2 = ids[q];
-                    lbs[q] = v;
-                    ids[q] = id;
-                    v = tv;
-                    id = tid2;
+              for (int j = 0; j < 32; ++j) {
+                const float t = xr - __uint_as_float(rr[j]);
+                const float L = fmaf(lam * t, t, -2.f * __uint_as_float(rx[j]));
+                const float dl = fmaf(two_le, fabsf(t), dlc);
+                v[j] = L - dl;
+                um[j & 3] = fminf(um[j & 3], L + dl);
+                lm[j >> 3] = fminf(lm[j >> 3], v[j]);
+              }
+              U = fminf(U, fminf(fminf(um[0], um[1]), fminf(um[2], um[3])));
+#pragma unroll
+              for (int q8 = 0; q8 < 4; ++q8) gm |= (lm[q8] <= U ? 1u : 0u) << q8;
+            }
+            // one trip per surviving group of the lane with the most of them
+            while (__any_sync(0xffffffffu, gm != 0u)) {
+              const int q8 = gm ? __ffs(gm) - 1 : 0;
+              const bool on = gm != 0u;
+              gm &= gm - 1u;
+#pragma unroll
+              for (int u = 0; u < 8; ++u) {
+                const float w = q8 < 2 ? (q8 == 0 ? v[u] : v[8 + u]) : (q8 == 2 ? v[16 + u] : v[24 + u]);
+                const float lb = NDIR == 0 ? fmaf(-2.f, w, -dlc) : w;
+                if (on && lb <= U && lb < INFINITY) {
+                  if (cnt == P.cap) {                  // candidates that fell behind make room
+                    int k = 0;
+                    for (int j = 0; j < cnt; ++j) {
+                      const float o = lbs[j * kEpi];
+                      if (o <= U) {
+                        lbs[k * kEpi] = o;
+                        ids[k * kEpi] = ids[j * kEpi];
+                        ++k;
+                      }
+                    }
+                    cnt = k;
+                  }
+                  if (cnt < P.cap) {
+                    lbs[cnt * kEpi] = lb;
+                    ids[cnt * kEpi] = cbase + 8 * q8 + u;
+                    ++cnt;
+                  } else {
+                    ev = fminf(ev, lb);
                   }
                 }
               }
@@ -396,51 +426,36 @@ __global__ void __launch_bounds__(kThr, 1) assign_tc_kernel(AsgParams<XT> P) {
           if (lane == 0) tc::bar_arrive(tempty(b));
           if (!ok) break;
         }
-        // merge the two column halves of each point (the merge area overlays
-        // the parking area: every epilogue thread must be past its tiles)
-        asm volatile("bar.sync 1, %0;" ::"n"(kEpi) : "memory");
-        if (hh == 1) {
-#pragma unroll
-          for (int q = 0; q < kList; ++q) {
-            mlb_s[q * kTM + m] = lbs[q];
-            mid_s[q * kTM + m] = ids[q];
+        if constexpr (kSplit) {                        // the second half's bounds and count for the first
+          if (hh == 1) {
+            mu_s[m] = U;
+            mev_s[m] = ev;
+            mcnt_s[m] = cnt;
           }
-          mu_s[m] = U;
-          mev_s[m] = ev;
+          asm volatile("bar.sync 1, %0;" ::"n"(kEpi) : "memory");
         }
-        asm volatile("bar.sync 1, %0;" ::"n"(kEpi) : "memory");
-        if (hh == 0 && active && !abort_s) {
-          U = fminf(U, mu_s[m]);
-          ev = fminf(ev, mev_s[m]);
-          for (int q2 = 0; q2 < kList; ++q2) {
-            float v = mlb_s[q2 * kTM + m];
-            int id = mid_s[q2 * kTM + m];
-            if (!(v < lbs[kList - 1])) {
-              ev = fminf(ev, v);
-              continue;
-            }
-            ev = fminf(ev, lbs[kList - 1]);
-#pragma unroll
-            for (int q = 0; q < kList; ++q) {
-              if (v < lbs[q] || (v == lbs[q] && id < ids[q])) {
-                const float tv = lbs[q];
-                const int ti2 = ids[q];
-                lbs[q] = v;
-                ids[q] = id;
-                v = tv;
-                id = ti2;
-              }
+        if ((!kSplit || hh == 0) && active && !abort_s) {
+          int other = 0;
+          if constexpr (kSplit) {
+            U = fminf(U, mu_s[m]);
+            ev = fminf(ev, mev_s[m]);
+            other = mcnt_s[m];
+          }
+          int ncand = 0, only = -1;
+          int32_t* cand = P.cand + p * kList;
+          for (int j = 0; j < cnt + other; ++j) {
+            const int at = j < cnt ? j * kEpi : (j - cnt) * kEpi + kTM;    // (et + kTM: the second half's list)
+            if (lbs[at] <= U) {
+              only = ids[at];
+              if (ncand < kList) cand[ncand] = only;
+              ++ncand;
             }
           }
-          int ncand = 0;
-#pragma unroll
-          for (int q = 0; q < kList; ++q) ncand += lbs[q] <= U ? 1 : 0;
-          const bool over = ev <= U;
+          const bool over = ev <= U || ncand > kList;
           if (ncand == 1 && !over) {
-            P.assign[p * P.astride + NDIR] = ids[0];   // the bounds leave one centroid: decided
+            P.assign[p * P.astride + NDIR] = only;     // the bounds leave one centroid: decided
           } else {
-#pragma unroll
-            for (int q = 0; q < kList; ++q) P.cand[p * kList + q] = lbs[q] <= U ? ids[q] : -1;
+            for (int q = ncand; q < kList; ++q) cand[q] = -1;
             P.ovf[p] = over ? 1 : 0;
           }
           // queue the undecided points for the direct-form refine (one atomic per warp)
@@ -490,39 +505,39 @@ __global__ void codebook_norms(const float* __restrict__ C, int c, int d, float*
   }
 }
 
-// Codebook as B tiles of N rows, each split into K steps of 8 columns stored
+// Codebook as B tiles of kN rows, each split into K steps of 8 columns stored
 // contiguously in the core-matrix layout of tc.cuh (8-row groups 256 bytes
-// apart): rows padded to ctiles * N and columns to kp with zeros, except
-// columns d and d + 1 holding ||c||^2 split into its tf32 part and the
-// remainder (the MMA then adds -||c||^2 / 2 to <x, c> at full fp32 accuracy);
+// apart), rounded to tf32: rows padded to ctiles * kN and columns to kp with
+// zeros, except columns d and d + 1 holding ||c||^2 split into its tf32 part and
+// the remainder (the MMA then adds -||c||^2 / 2 to <x, c> at full fp32 accuracy);
 // padding rows hold +inf there.
 __global__ void pack_codebook(const float* __restrict__ C, const float* __restrict__ n2, int c, int d, int kp,
-                              int N, int rows_pad, float* __restrict__ out) {
+                              int rows_pad, float* __restrict__ out) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= (int64_t)rows_pad * kp) return;
   const int r = (int)(i / kp), k = (int)(i % kp);
   float v = 0.f;
   if (r < c) {
     if (k < d) {
-      v = C[(int64_t)r * d + k];
+      v = round_tf32(C[(int64_t)r * d + k]);
     } else if (k <= d + 1) {
       const float hi = __uint_as_float(__float_as_uint(n2[r]) & 0xffffe000u);   // tf32 truncation
-      v = k == d ? hi : n2[r] - hi;
+      v = k == d ? hi : round_tf32(n2[r] - hi);
     }
   } else if (k == d) {
     v = INFINITY;           // padding rows: infinite loss for every point
   }
-  const int ti = r / N, rr = r % N, j = k >> 3, kk = k & 7;
-  out[((int64_t)ti * (kp / 8) + j) * N * 8 + (rr >> 3) * 64 + (kk >> 2) * 32 + (rr & 7) * 4 + (kk & 3)] = v;
+  const int ti = r / kN, rr = r % kN, j = k >> 3, kk = k & 7;
+  out[((int64_t)ti * (kp / 8) + j) * kN * 8 + (rr >> 3) * 64 + (kk >> 2) * 32 + (rr & 7) * 4 + (kk & 3)] = v;
 }
 
-// Largest ||c|| of each N-centroid tile (warp per tile).
-__global__ void tile_max_norms(const float* __restrict__ n1, int c, int N, int ctiles, float* __restrict__ tmax) {
+// Largest ||c|| of each tile (warp per tile).
+__global__ void tile_max_norms(const float* __restrict__ n1, int c, int ctiles, float* __restrict__ tmax) {
   const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (w >= ctiles) return;
   float v = 0.f;
-  for (int j = lane; j < N; j += 32) {
-    const int r = w * N + j;
+  for (int j = lane; j < kN; j += 32) {
+    const int r = w * kN + j;
     if (r < c) v = fmaxf(v, n1[r]);
   }
 #pragma unroll
@@ -608,59 +623,66 @@ __global__ void refine_list(const XT* __restrict__ X, int d, const float* __rest
   }
 }
 
-size_t smem_for(int kp, int ndir, int s) {
-  return 128 + (size_t)(1 + ndir) * kTM * kp * 4 + (size_t)s * kStageBytes + (size_t)kPark * 4 +
-         (size_t)4 * kTM * 4 + (size_t)(2 * s + 4) * 8;
+size_t smem_for(int kp, int ops, int s, int cap) {
+  return 128 + (size_t)ops * kTM * kp * 4 + (size_t)s * kStageBytes + (size_t)cap * kEpi * 8 + (size_t)kEpi * 4 +
+         (size_t)6 * kTM * 4 + (size_t)(2 * s + 4) * 8;
 }
 
 // K of the MMAs: d columns plus the two norm columns, a multiple of 8
 int kp_for(int d) { return (d + 2 + 7) / 8 * 8; }
 
-int stages_for(int kp, int ndir) {
-  for (int s = kStagesMax; s >= 2; --s)
-    if (smem_for(kp, ndir, s) <= 227 * 1024 - 256) return s;   // room for the static shared variables
-  return 0;
+// A operands, codebook stages and list length that fit: two operands before one
+// (half the codebook traffic), long lists before deep rings.
+struct Shape {
+  int ops = 0, stages = 0, cap = 0;
+};
+Shape shape_for(int kp, int ndir) {
+  for (int ops = 2; ops >= (ndir ? 2 : 1); --ops)
+    for (int cap : {16, 8})
+      for (int s = kStagesMax; s >= 2; --s)
+        if (smem_for(kp, ops, s, cap) <= 227 * 1024 - 256) return Shape{ops, s, cap};   // room for the static shared variables
+  return Shape{};
 }
 
 }  // namespace
 
-bool assign_tc_supported(int d, int ndir) { return ndir <= 1 && stages_for(kp_for(d), ndir) >= 2; }
+bool assign_tc_supported(int d, int ndir) { return ndir <= 1 && shape_for(kp_for(d), ndir).ops > 0; }
 
 template <typename XT>
 void assign_tc_pass(const XT* X, int64_t n, int d, const float* C, int c, int ndir, int32_t* assign, int astride,
                     const float* inv_rn, float lambda, cudaStream_t s, Scratch& scr) {
   const int kp = kp_for(d);
-  const int stages = stages_for(kp, ndir);
-  if (ndir > 1 || stages < 2) fail(SOAR_EUNSUPPORTED, "tensor-core assignment: unsupported shape");
-  const int N = tile_n(ndir);
-  const int ctiles = (c + N - 1) / N;
-  float* Cc = scr.get<float>((size_t)ctiles * N * kp);
+  const Shape sh = shape_for(kp, ndir);
+  if (ndir > 1 || sh.ops == 0) fail(SOAR_EUNSUPPORTED, "tensor-core assignment: unsupported shape");
+  const int ctiles = (c + kN - 1) / kN;
+  float* Cc = scr.get<float>((size_t)ctiles * kN * kp);
   float* n2 = scr.get<float>(c);
   float* n1 = scr.get<float>(c);
   float* tmax = scr.get<float>(ctiles);
   codebook_norms<<<ceil_div((int64_t)c * 32, 256), 256, 0, s>>>(C, c, d, n2, n1);
   SOAR_LAUNCHED();
-  pack_codebook<<<ceil_div((int64_t)ctiles * N * kp, 256), 256, 0, s>>>(C, n2, c, d, kp, N, ctiles * N, Cc);
+  pack_codebook<<<ceil_div((int64_t)ctiles * kN * kp, 256), 256, 0, s>>>(C, n2, c, d, kp, ctiles * kN, Cc);
   SOAR_LAUNCHED();
-  tile_max_norms<<<ceil_div((int64_t)ctiles * 32, 256), 256, 0, s>>>(n1, c, N, ctiles, tmax);
+  tile_max_norms<<<ceil_div((int64_t)ctiles * 32, 256), 256, 0, s>>>(n1, c, ctiles, tmax);
   SOAR_LAUNCHED();
   int32_t* cand = scr.get<int32_t>((size_t)n * kList);
   int32_t* ovf = scr.get<int32_t>(n);
   int32_t* queue = scr.get<int32_t>(n);
-  int* counter = scr.get<int>(2);            // work items, queued points
-  SOAR_CUDA(cudaMemsetAsync(counter, 0, 2 * sizeof(int), s));
+  int* qcount = scr.get<int>(1);             // queued points
+  SOAR_CUDA(cudaMemsetAsync(qcount, 0, sizeof(int), s));
   const int vec = std::is_same<XT, float>::value && d % 4 == 0 && reinterpret_cast<uintptr_t>(X) % 16 == 0 &&
                   reinterpret_cast<uintptr_t>(C) % 16 == 0;
-  AsgParams<XT> prm{X, n, d, kp, Cc, tmax, C, c, ctiles, assign, astride, inv_rn, lambda, stages,
-                    counter, device_error_word(), cand, ovf, queue, counter + 1, vec};
-  const size_t smem = smem_for(kp, ndir, stages);
-  auto kern = ndir == 0 ? assign_tc_kernel<0, XT> : assign_tc_kernel<1, XT>;
+  AsgParams<XT> prm{X, n, d, kp, Cc, tmax, C, c, ctiles, assign, astride, inv_rn, lambda, sh.stages,
+                    sh.cap, device_error_word(), cand, ovf, queue, qcount, vec};
+  const size_t smem = smem_for(kp, sh.ops, sh.stages, sh.cap);
+  auto kern = ndir == 0 ? (sh.ops == 2 ? assign_tc_kernel<0, 2, XT> : assign_tc_kernel<0, 1, XT>)
+                        : assign_tc_kernel<1, 2, XT>;
   SOAR_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  const int grid = (int)std::min<int64_t>((n + kTM - 1) / kTM, num_sms());
+  const int pts = ndir == 0 && sh.ops == 2 ? 2 * kTM : kTM;
+  const int grid = (int)std::min<int64_t>((n + pts - 1) / pts, num_sms());
   kern<<<grid, kThr, smem, s>>>(prm);
   SOAR_LAUNCHED();
-  refine_list<XT><<<num_sms() * 8, 256, 0, s>>>(X, d, C, c, assign, astride, ndir, lambda, cand, ovf, queue,
-                                                  counter + 1);
+  refine_list<XT><<<num_sms() * 8, 256, 0, s>>>(X, d, C, c, assign, astride, ndir, lambda, cand, ovf, queue, qcount);
   SOAR_LAUNCHED();
 }
 
