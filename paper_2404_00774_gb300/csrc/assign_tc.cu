@@ -325,7 +325,8 @@ __global__ void __launch_bounds__(kThr, 1) assign_tc_kernel(AsgParams<XT> P) {
         float* lbs = list_lb + et;                     // [cap] lower bounds and ids of the candidates so far
         int* ids = list_id + et;
         int cnt = 0;
-        float U = INFINITY, ev = INFINITY;             // ev: the smallest lower bound the list had no room for
+        float U = INFINITY, packed = INFINITY;         // packed: U when the list was last cleared of stale entries
+        float ev = INFINITY;                           // the smallest lower bound the list had no room for
         const float nx = nx_s[mp], nx2 = nx * nx;
         const float xr = NDIR > 0 ? xr_s[m] : 0.f, er0 = NDIR > 0 ? ldexpf(rn_s[m], -10) * 1.0625f : 0.f;
         const int prior = NDIR > 0 ? prior_s[m] : -1;
@@ -388,6 +389,9 @@ __global__ void __launch_bounds__(kThr, 1) assign_tc_kernel(AsgParams<XT> P) {
 #pragma unroll
               for (int q8 = 0; q8 < 4; ++q8) gm |= (lm[q8] <= U ? 1u : 0u) << q8;
             }
+            // an idle row (past the last point) is zero: it would be near all
+            // centroids of equal norm at once, and its warp's time the whole pass's
+            if (!active) gm = 0u;
             // one trip per surviving group of the lane with the most of them
             while (__any_sync(0xffffffffu, gm != 0u)) {
               const int q8 = gm ? __ffs(gm) - 1 : 0;
@@ -398,7 +402,8 @@ __global__ void __launch_bounds__(kThr, 1) assign_tc_kernel(AsgParams<XT> P) {
                 const float w = q8 < 2 ? (q8 == 0 ? v[u] : v[8 + u]) : (q8 == 2 ? v[16 + u] : v[24 + u]);
                 const float lb = NDIR == 0 ? fmaf(-2.f, w, -dlc) : w;
                 if (on && lb <= U && lb < INFINITY) {
-                  if (cnt == P.cap) {                  // candidates that fell behind make room
+                  if (cnt == P.cap && U < packed) {    // candidates that fell behind make room, once per fall of U
+                    packed = U;
                     int k = 0;
                     for (int j = 0; j < cnt; ++j) {
                       const float o = lbs[j * kEpi];

@@ -146,3 +146,99 @@ def test_centroid_means_of_every_cluster_size(soar, dtype, d, big):
         if len(rows):
             want = rows.mean(0).float()
             assert ((C[j] - want).abs() <= 2.0 ** -23 * want.abs()).all(), j
+
+
+def _fp8_rows(V):
+    scale = V.abs().amax(1, keepdim=True) / 448
+    scale = torch.where(scale > 0, scale, torch.ones_like(scale))
+    return (V / scale).to(torch.float8_e4m3fn).double() * scale.double()
+
+
+@pytest.mark.parametrize("mode", ["fp8", "pq4"])
+@pytest.mark.parametrize("d,c,t,R,copies", [
+    (16, 60, 3, 1, 0), (34, 60, 4, 33, 0),       # one row kept; lists past a warp
+    (300, 60, 4, 100, 0),                        # rows wider than one register fragment
+    (24, 300, 250, 100, 0),                      # more earlier probes than the hash table takes
+    (24, 60, 6, 700, 3000),                      # thousands of equal scores at the threshold
+    (24, 60, 60, 4096, 0),                       # the largest shortlist
+])
+def test_shortlists_at_their_limits(soar, mode, d, c, t, R, copies):
+    g = torch.Generator().manual_seed(d + c)
+    n, nq = 8000, 40
+    X = torch.nn.functional.normalize(torch.randn(n, d, generator=g), dim=1)
+    X[1000:1000 + copies] = X[0]
+    Q = torch.nn.functional.normalize(torch.randn(nq, d, generator=g), dim=1)
+    if copies:
+        Q[::2] = X[0] + 0.3 * Q[::2]
+    C = X[torch.randperm(1000, generator=g)[:c]].contiguous()
+    A = soar.soar_assign(X.cuda(), C.cuda(), 1.0, 1)
+    if mode == "fp8":
+        ix = soar.soar_index_build(X.cuda(), C.cuda(), A, mode=soar.SOAR_SCORE_FP8)
+        approx = _fp8_rows(Q) @ _fp8_rows(X).T
+        approx = approx[:, :, None].expand(-1, -1, 2)
+    else:
+        B = 0.3 * torch.randn(d // 2, 16, 2, generator=g)
+        ix = soar.soar_index_build_pq(X.cuda(), C.cuda(), A, B.cuda())
+        copies_hat = []
+        for col in range(2):
+            base = C[A[:, col].cpu().long()]
+            r = (X - base).view(n, -1, 2)
+            code = ((r[:, :, None] - B[None]) ** 2).sum(3).argmin(2)
+            copies_hat.append(base + B[torch.arange(d // 2)[None], code].reshape(n, d))
+        approx = torch.stack([Q.double() @ h.double().T for h in copies_hat], 2)
+    top = soar.soar_select_partitions(ix, Q.cuda(), t).cpu().long()
+    A = A.cpu().long()
+    k = min(R, 1024)
+    ids, sc = soar.soar_search(ix, Q.cuda(), k, t, rescore=R)
+    full = Q.double() @ X.double().T
+    for q in range(nq):
+        place = torch.full((c,), 10 ** 6).scatter_(0, top[q], torch.arange(t))
+        first = place[A].argmin(1)                                   # the copy in the earliest-probed partition
+        s = approx[q].gather(1, first[:, None])[:, 0]
+        inside = (place[A] < 10 ** 6).any(1)
+        s = torch.where(inside, s, torch.tensor(-float("inf"), dtype=torch.float64))
+        order = s.sort(descending=True, stable=True)[1]
+        short = order[: min(R, int(inside.sum()))]
+        got = ids[q].cpu()
+        got = got[got >= 0]
+        assert got.unique().numel() == got.numel() == min(k, short.numel())
+        # fp32 sums of d products: a score may change places only within this of the R-th
+        slack = d * 2.0 ** -21
+        assert (s[got] >= s[short[-1]] - slack).all()
+        sure = short[s[short] > s[short[-1]] + slack] if short.numel() == R else short
+        if sure.numel() == short.numel():
+            want = full[q, short].sort(descending=True)[0][:k]
+            assert torch.allclose(full[q, got], want, rtol=0, atol=1e-5)
+        if k == short.numel():
+            assert torch.isin(sure, got).all()
+        if copies and q % 2 == 0 and mode == "fp8":                  # equal scores: the lower ids are kept
+            tied = s[got] == s[0]
+            kept = got[tied].sort()[0]
+            all_tied = torch.nonzero(s == s[0])[:, 0]
+            assert torch.equal(kept, all_tied[: kept.numel()])
+    ix.close()
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("d,c,n", [(5, 2, 1), (100, 129, 255), (100, 128, 257), (126, 300, 300), (134, 257, 700),
+                                   (142, 257, 300), (278, 130, 200), (64, 3000, 513)])
+def test_assignment_shapes(soar, dtype, d, c, n):
+    """Ragged point blocks and codebook tiles; rows too wide for long lists (126..134) and for two operands (142..278)."""
+    g = torch.Generator().manual_seed(d + c)
+    X = torch.randn(n, d, generator=g).to(dtype)
+    C = torch.randn(c, d, generator=g)
+    if c > 2000:                                    # dozens of near-equal centroids to a point: full lists, rescans
+        C = C[:40].repeat_interleave(c // 40, 0)
+        C = C + 1e-4 * torch.randn(C.shape, generator=g)
+    A = soar.soar_assign(X.cuda(), C.cuda(), 1.5, 1).cpu().long()
+    x, cc = X.double(), C.double()
+    dist = torch.cdist(x, cc, compute_mode="donot_use_mm_for_euclid_dist") ** 2
+    first = A[:, 0]
+    got = dist.gather(1, first[:, None])[:, 0]
+    assert (got <= dist.min(1)[0] * (1 + 1e-5)).all()
+    r = x - cc[first]
+    r = r / r.norm(dim=1, keepdim=True).clamp(min=1e-30)
+    loss = dist + 1.5 * ((x * r).sum(1, keepdim=True) - r @ cc.T) ** 2
+    loss.scatter_(1, first[:, None], float("inf"))
+    assert (first != A[:, 1]).all()
+    assert (loss.gather(1, A[:, 1:])[:, 0] <= loss.min(1)[0] * (1 + 1e-5)).all()
