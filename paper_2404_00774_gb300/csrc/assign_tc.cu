@@ -82,6 +82,8 @@ struct AsgParams {
   int32_t* assign;        // [n][astride]: column 0 = primary (read by the spill pass); decided points written
   int astride;
   const float* inv_rn;    // [n][4] 1 / ||x - C[pi(x)]|| (0 for a zero residual)
+  const float* n2;        // [c] ||c||^2
+  int seeded;             // primary: column 0 of assign holds a centroid of every point to start from
   float lambda;
   int stages;
   int cap;                // candidates an epilogue thread holds
@@ -117,7 +119,8 @@ __global__ void __launch_bounds__(kThr, 1) assign_tc_kernel(AsgParams<XT> P) {
   float* list_lb = reinterpret_cast<float*>(sB + (size_t)S * kStageBytes);   // [cap][kEpi]
   int* list_id = reinterpret_cast<int*>(list_lb + P.cap * kEpi);             // [cap][kEpi]
   float* nx_s = reinterpret_cast<float*>(list_id + P.cap * kEpi);            // [kEpi] ||x||
-  float* mu_s = nx_s + kEpi;                                                // [kTM] U of the second half
+  float* seed_s = nx_s + kEpi;                                              // [kEpi] U to start from
+  float* mu_s = seed_s + kEpi;                                              // [kTM] U of the second half
   float* mev_s = mu_s + kTM;                                                // [kTM]
   int* mcnt_s = reinterpret_cast<int*>(mev_s + kTM);                        // [kTM]
   float* xr_s = reinterpret_cast<float*>(mcnt_s + kTM);                     // [kTM] <x, r_hat>
@@ -213,6 +216,11 @@ __global__ void __launch_bounds__(kThr, 1) assign_tc_kernel(AsgParams<XT> P) {
           inv = P.inv_rn[p * 4];
           cr = P.C + (int64_t)prior * P.d;
         }
+        const bool seed = NDIR == 0 && P.seeded != 0;
+        if (seed && active) {
+          prior = P.assign[p * P.astride];
+          cr = P.C + (int64_t)prior * P.d;
+        }
         float ss = 0.f, xd = 0.f;
         const bool vec = std::is_same<XT, float>::value && P.vec;
         const int d4 = vec ? P.d / 4 : 0;               // 16-byte chunks staged by cp.async
@@ -228,7 +236,7 @@ __global__ void __launch_bounds__(kThr, 1) assign_tc_kernel(AsgParams<XT> P) {
             if (active) {
               const float4 a = *reinterpret_cast<const float4*>(row + k4 * 32);
               xv[0] = a.x; xv[1] = a.y; xv[2] = a.z; xv[3] = a.w;
-              if (resid) {
+              if (resid || seed) {
                 const float4 b = __ldg(reinterpret_cast<const float4*>(cr + 4 * k4));
                 cv[0] = b.x; cv[1] = b.y; cv[2] = b.z; cv[3] = b.w;
               }
@@ -240,7 +248,7 @@ __global__ void __launch_bounds__(kThr, 1) assign_tc_kernel(AsgParams<XT> P) {
             for (int u = 0; u < 4; ++u) {
               const int k = 4 * k4 + u;
               xv[u] = (active && k < P.d) ? ld(P.X + p * P.d + k) : 0.f;
-              if (resid) cv[u] = (active && k < P.d) ? __ldg(cr + k) : 0.f;
+              if (resid || seed) cv[u] = (active && k < P.d) ? __ldg(cr + k) : 0.f;
             }
           }
           float av[4];
@@ -253,6 +261,7 @@ __global__ void __launch_bounds__(kThr, 1) assign_tc_kernel(AsgParams<XT> P) {
               av[u] = round_tf32(rv);
             } else {
               ss = fmaf(xv[u], xv[u], ss);
+              if (seed) xd = fmaf(xv[u], cv[u], xd);
               av[u] = (k == P.d || k == P.d + 1) ? -0.5f : round_tf32(xv[u]);
             }
           }
@@ -263,7 +272,12 @@ __global__ void __launch_bounds__(kThr, 1) assign_tc_kernel(AsgParams<XT> P) {
           rn_s[m] = inv > 0.f ? 1.f : 0.f;
           prior_s[m] = prior;
         } else {
-          nx_s[mp] = sqrtf(ss);
+          const float nx = sqrtf(ss);
+          nx_s[mp] = nx;
+          if (seed) {                                    // an upper bound of the loss of the point's centroid so far
+            const float c2 = active ? __ldg(P.n2 + prior) : 0.f;
+            seed_s[mp] = fmaf(-2.f, xd, c2) + ldexpf(fmaf(nx, sqrtf(c2), c2), -14) + ldexpf(ss, -16);
+          }
         }
         tc::fence_async_smem();
       }
@@ -327,6 +341,7 @@ __global__ void __launch_bounds__(kThr, 1) assign_tc_kernel(AsgParams<XT> P) {
         int cnt = 0;
         float U = INFINITY, packed = INFINITY;         // packed: U when the list was last cleared of stale entries
         float ev = INFINITY;                           // the smallest lower bound the list had no room for
+        if (NDIR == 0 && P.seeded) U = seed_s[mp];
         const float nx = nx_s[mp], nx2 = nx * nx;
         const float xr = NDIR > 0 ? xr_s[m] : 0.f, er0 = NDIR > 0 ? ldexpf(rn_s[m], -10) * 1.0625f : 0.f;
         const int prior = NDIR > 0 ? prior_s[m] : -1;
@@ -343,12 +358,12 @@ __global__ void __launch_bounds__(kThr, 1) assign_tc_kernel(AsgParams<XT> P) {
           float dlc = fmaf(ldexpf(nx, -9) * 1.0625f, cmax, ldexpf(fmaf(nx, cmax, c2max), -14) + ldexpf(nx2, -16));
           if (NDIR > 0) dlc = fmaf(lam * e, e, fmaf(ldexpf(lam, -14), (nx + cmax) * (nx + cmax), dlc));
           const float two_le = 2.f * lam * e;
+          const uint32_t tbase = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + b * kW +
+                                 (kSplit ? hh * kCols : hh * kN);
 #pragma unroll 1
           for (int rd = 0; rd < kCols / 32 && ok; ++rd) {
-            const int col0 = (kSplit ? hh * kCols : 0) + 32 * rd;
-            const uint32_t taddr = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + b * kW +
-                                   (!kSplit && OPS == 2 ? hh * kN : 0) + col0;
-            const int cbase = ti * kN + col0;
+            const uint32_t taddr = tbase + 32 * rd;
+            const int cbase = ti * kN + (kSplit ? hh * kCols : 0) + 32 * rd;
             float v[32];                               // primary: <x, c> - ||c||^2 / 2; spill: lower bounds
             uint32_t gm = 0u;                          // groups of eight columns that hold a candidate
             if constexpr (NDIR == 0) {
@@ -357,13 +372,13 @@ __global__ void __launch_bounds__(kThr, 1) assign_tc_kernel(AsgParams<XT> P) {
 #pragma unroll
               for (int q8 = 0; q8 < 4; ++q8) tc::tmem_ld8_max(taddr + 8 * q8, rx + 8 * q8, g[q8]);
               tc::tmem_ld_wait();
+#pragma unroll
+              for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(rx[j]);
               // (padded centroids carry ||c||^2 = +inf: their product is -inf)
               U = fminf(U, fmaf(-2.f, fmaxf(fmaxf(g[0], g[1]), fmaxf(g[2], g[3])), dlc));
               const float cut = -0.5f * (U + dlc);     // L~ - delta <= U
 #pragma unroll
               for (int q8 = 0; q8 < 4; ++q8) gm |= (g[q8] >= cut ? 1u : 0u) << q8;
-#pragma unroll
-              for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(rx[j]);
             } else {
               uint32_t rx[32], rr[32];
               tc::tmem_ld32(taddr, rx);
@@ -392,19 +407,35 @@ __global__ void __launch_bounds__(kThr, 1) assign_tc_kernel(AsgParams<XT> P) {
             // an idle row (past the last point) is zero: it would be near all
             // centroids of equal norm at once, and its warp's time the whole pass's
             if (!active) gm = 0u;
-            // one trip per surviving group of the lane with the most of them
+            // one trip per surviving group of the lane with the most of them, in it
+            // one per candidate (kept small: this code unrolled over the rounds ran
+            // at half the speed, short of instructions)
             while (__any_sync(0xffffffffu, gm != 0u)) {
-              const int q8 = gm ? __ffs(gm) - 1 : 0;
-              const bool on = gm != 0u;
+              const int q8 = __ffs(gm) - 1;            // -1: this lane has none left
               gm &= gm - 1u;
+              float w[8];
+              uint32_t em = 0u;
 #pragma unroll
               for (int u = 0; u < 8; ++u) {
-                const float w = q8 < 2 ? (q8 == 0 ? v[u] : v[8 + u]) : (q8 == 2 ? v[16 + u] : v[24 + u]);
-                const float lb = NDIR == 0 ? fmaf(-2.f, w, -dlc) : w;
-                if (on && lb <= U && lb < INFINITY) {
+                const float lo = q8 & 1 ? v[8 + u] : v[u], hi = q8 & 1 ? v[24 + u] : v[16 + u];
+                w[u] = q8 & 2 ? hi : lo;
+                if (NDIR == 0) w[u] = fmaf(-2.f, w[u], -dlc);
+                em |= (w[u] <= U ? 1u : 0u) << u;
+              }
+              if (q8 < 0) em = 0u;
+              while (__any_sync(0xffffffffu, em != 0u)) {
+                const int u = __ffs(em) - 1;
+                em &= em - 1u;
+                const float a0 = u & 1 ? w[1] : w[0], a1 = u & 1 ? w[3] : w[2], a2 = u & 1 ? w[5] : w[4],
+                            a3 = u & 1 ? w[7] : w[6];
+                const float b0 = u & 2 ? a1 : a0, b1 = u & 2 ? a3 : a2;
+                const float lb = u & 4 ? b1 : b0;
+                const bool take = u >= 0 && lb < INFINITY;
+                if (__any_sync(0xffffffffu, take && cnt == P.cap && U < packed)) {
                   if (cnt == P.cap && U < packed) {    // candidates that fell behind make room, once per fall of U
                     packed = U;
                     int k = 0;
+#pragma unroll 1
                     for (int j = 0; j < cnt; ++j) {
                       const float o = lbs[j * kEpi];
                       if (o <= U) {
@@ -415,14 +446,14 @@ __global__ void __launch_bounds__(kThr, 1) assign_tc_kernel(AsgParams<XT> P) {
                     }
                     cnt = k;
                   }
-                  if (cnt < P.cap) {
-                    lbs[cnt * kEpi] = lb;
-                    ids[cnt * kEpi] = cbase + 8 * q8 + u;
-                    ++cnt;
-                  } else {
-                    ev = fminf(ev, lb);
-                  }
                 }
+                const bool room = cnt < P.cap;
+                if (take && room) {
+                  lbs[cnt * kEpi] = lb;
+                  ids[cnt * kEpi] = cbase + 8 * q8 + u;
+                }
+                if (take && !room) ev = fminf(ev, lb);
+                cnt += take && room ? 1 : 0;
               }
             }
           }
@@ -629,7 +660,7 @@ __global__ void refine_list(const XT* __restrict__ X, int d, const float* __rest
 }
 
 size_t smem_for(int kp, int ops, int s, int cap) {
-  return 128 + (size_t)ops * kTM * kp * 4 + (size_t)s * kStageBytes + (size_t)cap * kEpi * 8 + (size_t)kEpi * 4 +
+  return 128 + (size_t)ops * kTM * kp * 4 + (size_t)s * kStageBytes + (size_t)cap * kEpi * 8 + (size_t)2 * kEpi * 4 +
          (size_t)6 * kTM * 4 + (size_t)(2 * s + 4) * 8;
 }
 
@@ -655,7 +686,7 @@ bool assign_tc_supported(int d, int ndir) { return ndir <= 1 && shape_for(kp_for
 
 template <typename XT>
 void assign_tc_pass(const XT* X, int64_t n, int d, const float* C, int c, int ndir, int32_t* assign, int astride,
-                    const float* inv_rn, float lambda, cudaStream_t s, Scratch& scr) {
+                    const float* inv_rn, float lambda, bool seeded, cudaStream_t s, Scratch& scr) {
   const int kp = kp_for(d);
   const Shape sh = shape_for(kp, ndir);
   if (ndir > 1 || sh.ops == 0) fail(SOAR_EUNSUPPORTED, "tensor-core assignment: unsupported shape");
@@ -677,7 +708,7 @@ void assign_tc_pass(const XT* X, int64_t n, int d, const float* C, int c, int nd
   SOAR_CUDA(cudaMemsetAsync(qcount, 0, sizeof(int), s));
   const int vec = std::is_same<XT, float>::value && d % 4 == 0 && reinterpret_cast<uintptr_t>(X) % 16 == 0 &&
                   reinterpret_cast<uintptr_t>(C) % 16 == 0;
-  AsgParams<XT> prm{X, n, d, kp, Cc, tmax, C, c, ctiles, assign, astride, inv_rn, lambda, sh.stages,
+  AsgParams<XT> prm{X, n, d, kp, Cc, tmax, C, c, ctiles, assign, astride, inv_rn, n2, seeded, lambda, sh.stages,
                     sh.cap, device_error_word(), cand, ovf, queue, qcount, vec};
   const size_t smem = smem_for(kp, sh.ops, sh.stages, sh.cap);
   auto kern = ndir == 0 ? (sh.ops == 2 ? assign_tc_kernel<0, 2, XT> : assign_tc_kernel<0, 1, XT>)
@@ -692,8 +723,8 @@ void assign_tc_pass(const XT* X, int64_t n, int d, const float* C, int c, int nd
 }
 
 template void assign_tc_pass<float>(const float*, int64_t, int, const float*, int, int, int32_t*, int, const float*,
-                                    float, cudaStream_t, Scratch&);
+                                    float, bool, cudaStream_t, Scratch&);
 template void assign_tc_pass<__nv_bfloat16>(const __nv_bfloat16*, int64_t, int, const float*, int, int, int32_t*,
-                                            int, const float*, float, cudaStream_t, Scratch&);
+                                            int, const float*, float, bool, cudaStream_t, Scratch&);
 
 }  // namespace soar
