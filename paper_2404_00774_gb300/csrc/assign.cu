@@ -278,7 +278,7 @@ void screen_launch(int ndir, const XT* X, int64_t n, int d, const float* C, cons
 
 template <typename XT>
 void assign_typed(const XT* X, int64_t n, int32_t d, const float* C, int32_t c, float lambda,
-                  int32_t spills, int32_t* assign, cudaStream_t s, Scratch& scr, bool seeded = false) {
+                  int32_t spills, int32_t* assign, cudaStream_t s, Scratch& scr) {
   const int astride = 1 + spills;
   float* cnorm = scr.get<float>(c);
   int32_t* cand = scr.get<int32_t>((size_t)n * 2);
@@ -298,7 +298,7 @@ void assign_typed(const XT* X, int64_t n, int32_t d, const float* C, int32_t c, 
     }
     if (assign_tc_supported(d, j)) {
       // primary and first spill: tensor-core screen with rigorous bounds
-      assign_tc_pass<XT>(X, n, d, C, c, j, assign, astride, inv_rn, lambda, seeded && j == 0, s, scr);
+      assign_tc_pass<XT>(X, n, d, C, c, j, assign, astride, inv_rn, lambda, s, scr);
       continue;
     }
     screen_launch<XT>(j, X, n, d, C, cnorm, c, assign, astride, inv_rn, xr, lambda, cand, s);
@@ -421,7 +421,7 @@ void kmeans_typed(const XT* X, int64_t n, int32_t d, int32_t c, int32_t iters, c
   int64_t* offsets = scr.get<int64_t>((size_t)c + 1);
   const int bits = bits_for(c);
   for (int it = 0; it < iters; ++it) {
-    assign_typed<XT>(X, n, d, C, c, 0.f, 0, assign, s, scr, it > 0);   // from the last step's assignment
+    assign_typed<XT>(X, n, d, C, c, 0.f, 0, assign, s, scr);
     iota_keys<<<ceil_div(n, 256), 256, 0, s>>>(assign, n, keys, vals);
     SOAR_LAUNCHED();
     bool in_tmp = radix_sort_pairs(keys, vals, keys2, vals2, n, bits, s, scr);

@@ -37,7 +37,9 @@
 // L2 (tf32 floor 0.51 ms for 1.18 M x 100 against 2 000 centroids).  Keeping the
 // sixteen smallest lower bounds sorted cost 37 of 47 instructions a pair (5.9 ms
 // a pass, the spill 6.8); most pairs are now dismissed eight at a time by a
-// maximum that the TMEM load computes: 1.84 ms, the spill 3.82.
+// maximum that the TMEM load computes: 1.45 ms, the spill 3.46 (of which copies and
+// MMAs 0.88 and 1.73, staging the operands 0.27 and 0.63, the survivors 0.26 and
+// 0.57).
 //
 // Warp roles: 0 = bulk-copy producer, 1 = TMEM owner and MMA issuer,
 // 2 = gate, 3..10 = epilogue and A-operand loaders.  Every mbarrier wait is bounded;
@@ -82,8 +84,6 @@ struct AsgParams {
   int32_t* assign;        // [n][astride]: column 0 = primary (read by the spill pass); decided points written
   int astride;
   const float* inv_rn;    // [n][4] 1 / ||x - C[pi(x)]|| (0 for a zero residual)
-  const float* n2;        // [c] ||c||^2
-  int seeded;             // primary: column 0 of assign holds a centroid of every point to start from
   float lambda;
   int stages;
   int cap;                // candidates an epilogue thread holds
@@ -119,8 +119,7 @@ __global__ void __launch_bounds__(kThr, 1) assign_tc_kernel(AsgParams<XT> P) {
   float* list_lb = reinterpret_cast<float*>(sB + (size_t)S * kStageBytes);   // [cap][kEpi]
   int* list_id = reinterpret_cast<int*>(list_lb + P.cap * kEpi);             // [cap][kEpi]
   float* nx_s = reinterpret_cast<float*>(list_id + P.cap * kEpi);            // [kEpi] ||x||
-  float* seed_s = nx_s + kEpi;                                              // [kEpi] U to start from
-  float* mu_s = seed_s + kEpi;                                              // [kTM] U of the second half
+  float* mu_s = nx_s + kEpi;                                                // [kTM] U of the second half
   float* mev_s = mu_s + kTM;                                                // [kTM]
   int* mcnt_s = reinterpret_cast<int*>(mev_s + kTM);                        // [kTM]
   float* xr_s = reinterpret_cast<float*>(mcnt_s + kTM);                     // [kTM] <x, r_hat>
@@ -216,11 +215,6 @@ __global__ void __launch_bounds__(kThr, 1) assign_tc_kernel(AsgParams<XT> P) {
           inv = P.inv_rn[p * 4];
           cr = P.C + (int64_t)prior * P.d;
         }
-        const bool seed = NDIR == 0 && P.seeded != 0;
-        if (seed && active) {
-          prior = P.assign[p * P.astride];
-          cr = P.C + (int64_t)prior * P.d;
-        }
         float ss = 0.f, xd = 0.f;
         const bool vec = std::is_same<XT, float>::value && P.vec;
         const int d4 = vec ? P.d / 4 : 0;               // 16-byte chunks staged by cp.async
@@ -236,7 +230,7 @@ __global__ void __launch_bounds__(kThr, 1) assign_tc_kernel(AsgParams<XT> P) {
             if (active) {
               const float4 a = *reinterpret_cast<const float4*>(row + k4 * 32);
               xv[0] = a.x; xv[1] = a.y; xv[2] = a.z; xv[3] = a.w;
-              if (resid || seed) {
+              if (resid) {
                 const float4 b = __ldg(reinterpret_cast<const float4*>(cr + 4 * k4));
                 cv[0] = b.x; cv[1] = b.y; cv[2] = b.z; cv[3] = b.w;
               }
@@ -248,7 +242,7 @@ __global__ void __launch_bounds__(kThr, 1) assign_tc_kernel(AsgParams<XT> P) {
             for (int u = 0; u < 4; ++u) {
               const int k = 4 * k4 + u;
               xv[u] = (active && k < P.d) ? ld(P.X + p * P.d + k) : 0.f;
-              if (resid || seed) cv[u] = (active && k < P.d) ? __ldg(cr + k) : 0.f;
+              if (resid) cv[u] = (active && k < P.d) ? __ldg(cr + k) : 0.f;
             }
           }
           float av[4];
@@ -261,7 +255,6 @@ __global__ void __launch_bounds__(kThr, 1) assign_tc_kernel(AsgParams<XT> P) {
               av[u] = round_tf32(rv);
             } else {
               ss = fmaf(xv[u], xv[u], ss);
-              if (seed) xd = fmaf(xv[u], cv[u], xd);
               av[u] = (k == P.d || k == P.d + 1) ? -0.5f : round_tf32(xv[u]);
             }
           }
@@ -272,12 +265,7 @@ __global__ void __launch_bounds__(kThr, 1) assign_tc_kernel(AsgParams<XT> P) {
           rn_s[m] = inv > 0.f ? 1.f : 0.f;
           prior_s[m] = prior;
         } else {
-          const float nx = sqrtf(ss);
-          nx_s[mp] = nx;
-          if (seed) {                                    // an upper bound of the loss of the point's centroid so far
-            const float c2 = active ? __ldg(P.n2 + prior) : 0.f;
-            seed_s[mp] = fmaf(-2.f, xd, c2) + ldexpf(fmaf(nx, sqrtf(c2), c2), -14) + ldexpf(ss, -16);
-          }
+          nx_s[mp] = sqrtf(ss);
         }
         tc::fence_async_smem();
       }
@@ -341,7 +329,6 @@ __global__ void __launch_bounds__(kThr, 1) assign_tc_kernel(AsgParams<XT> P) {
         int cnt = 0;
         float U = INFINITY, packed = INFINITY;         // packed: U when the list was last cleared of stale entries
         float ev = INFINITY;                           // the smallest lower bound the list had no room for
-        if (NDIR == 0 && P.seeded) U = seed_s[mp];
         const float nx = nx_s[mp], nx2 = nx * nx;
         const float xr = NDIR > 0 ? xr_s[m] : 0.f, er0 = NDIR > 0 ? ldexpf(rn_s[m], -10) * 1.0625f : 0.f;
         const int prior = NDIR > 0 ? prior_s[m] : -1;
@@ -660,7 +647,7 @@ __global__ void refine_list(const XT* __restrict__ X, int d, const float* __rest
 }
 
 size_t smem_for(int kp, int ops, int s, int cap) {
-  return 128 + (size_t)ops * kTM * kp * 4 + (size_t)s * kStageBytes + (size_t)cap * kEpi * 8 + (size_t)2 * kEpi * 4 +
+  return 128 + (size_t)ops * kTM * kp * 4 + (size_t)s * kStageBytes + (size_t)cap * kEpi * 8 + (size_t)kEpi * 4 +
          (size_t)6 * kTM * 4 + (size_t)(2 * s + 4) * 8;
 }
 
@@ -686,7 +673,7 @@ bool assign_tc_supported(int d, int ndir) { return ndir <= 1 && shape_for(kp_for
 
 template <typename XT>
 void assign_tc_pass(const XT* X, int64_t n, int d, const float* C, int c, int ndir, int32_t* assign, int astride,
-                    const float* inv_rn, float lambda, bool seeded, cudaStream_t s, Scratch& scr) {
+                    const float* inv_rn, float lambda, cudaStream_t s, Scratch& scr) {
   const int kp = kp_for(d);
   const Shape sh = shape_for(kp, ndir);
   if (ndir > 1 || sh.ops == 0) fail(SOAR_EUNSUPPORTED, "tensor-core assignment: unsupported shape");
@@ -708,7 +695,7 @@ void assign_tc_pass(const XT* X, int64_t n, int d, const float* C, int c, int nd
   SOAR_CUDA(cudaMemsetAsync(qcount, 0, sizeof(int), s));
   const int vec = std::is_same<XT, float>::value && d % 4 == 0 && reinterpret_cast<uintptr_t>(X) % 16 == 0 &&
                   reinterpret_cast<uintptr_t>(C) % 16 == 0;
-  AsgParams<XT> prm{X, n, d, kp, Cc, tmax, C, c, ctiles, assign, astride, inv_rn, n2, seeded, lambda, sh.stages,
+  AsgParams<XT> prm{X, n, d, kp, Cc, tmax, C, c, ctiles, assign, astride, inv_rn, lambda, sh.stages,
                     sh.cap, device_error_word(), cand, ovf, queue, qcount, vec};
   const size_t smem = smem_for(kp, sh.ops, sh.stages, sh.cap);
   auto kern = ndir == 0 ? (sh.ops == 2 ? assign_tc_kernel<0, 2, XT> : assign_tc_kernel<0, 1, XT>)
@@ -723,8 +710,8 @@ void assign_tc_pass(const XT* X, int64_t n, int d, const float* C, int c, int nd
 }
 
 template void assign_tc_pass<float>(const float*, int64_t, int, const float*, int, int, int32_t*, int, const float*,
-                                    float, bool, cudaStream_t, Scratch&);
+                                    float, cudaStream_t, Scratch&);
 template void assign_tc_pass<__nv_bfloat16>(const __nv_bfloat16*, int64_t, int, const float*, int, int, int32_t*,
-                                            int, const float*, float, bool, cudaStream_t, Scratch&);
+                                            int, const float*, float, cudaStream_t, Scratch&);
 
 }  // namespace soar
