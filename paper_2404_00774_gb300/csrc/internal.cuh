@@ -129,8 +129,9 @@ void pack_select_codebook(const IndexData& ix, float* out, cudaStream_t s);
 bool select_tc_usable(const IndexData& ix, const float* Qf, int qstride, int t);
 // top [nq][t] (and top_s, if not null): each query's t best centroids by
 // inner product, best first, lower id on ties; fp32 queries Qf [nq][qstride].
+// With scratch, batches that do not fill the chip are split over the codebook too.
 void select_tc(const IndexData& ix, const float* Qf, int64_t nq, int qstride, int t, int32_t* top, float* top_s,
-               cudaStream_t s);
+               cudaStream_t s, Scratch* scr);
 
 // ----------------------------------------------------------- search.cu
 

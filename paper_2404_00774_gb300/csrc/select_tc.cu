@@ -33,6 +33,8 @@
 // Every mbarrier wait is bounded (about a second); on expiry the CTA raises
 // *err, stops, waits (bounded) for its copies and MMAs in flight, frees its
 // TMEM and returns.
+#include <algorithm>
+
 #include "internal.cuh"
 #include "tc.cuh"
 
@@ -83,10 +85,17 @@ struct SelParams {
   int qstride, d, kp;
   const float* cb;    // packed codebook
   int c, tiles, t;
-  int32_t* top;       // [nq][t]
-  float* top_s;       // [nq][t] or null
+  int32_t* top;       // [nq][t], or with parts > 1 [nq][parts][t]
+  float* top_s;       // same layout, or null
   int* err;           // set to 1 when a wait expired
+  int per;            // (query block, codebook tile) units per CTA
+  int parts;          // lists per query
 };
+
+// Units are numbered query block by query block; CTA i takes units [i * per, (i
+// + 1) * per), which may cut through query blocks: list `part` of a query comes
+// from the part-th CTA that meets its block.
+__host__ __device__ inline int first_cta(int qb, int tiles, int per) { return (int)((int64_t)qb * tiles / per); }
 
 template <int TMAX>
 __global__ void __launch_bounds__(kThreads, 1) select_tc_kernel(SelParams P) {
@@ -134,9 +143,30 @@ __global__ void __launch_bounds__(kThreads, 1) select_tc_kernel(SelParams P) {
   auto give_up = [&]() {
     if (atomicExch(&abort_s, 1) == 0) atomicExch(P.err, 1);
   };
-  const int64_t q0 = (int64_t)blockIdx.x * kM;
-  const int nqb = (int)min((int64_t)kM, P.nq - q0);
   const int m = 32 * (warp & 3) + lane;   // epilogue: query slot = TMEM lane
+  const int64_t units = (P.nq + kM - 1) / kM * ntiles;
+  const int64_t u0 = (int64_t)blockIdx.x * P.per, u1 = min(units, u0 + P.per);
+  const int total = (int)(u1 - u0);       // tiles this CTA streams
+
+  if (warp == 0) {
+    // ---- producer: one bulk copy per codebook tile (hi and lo together), across query blocks
+    if (lane == 0) {
+      for (int i = 0; i < total; ++i) {
+        const uint32_t s = i % kStages, ph = (i / kStages) & 1;
+        if (!tc::bar_wait(empty(s), ph ^ 1, abort_v)) { give_up(); break; }
+        tc::bar_arrive_expect_tx(full(s), b_bytes);
+        tc::bulk_copy_g2s(tc::smem_u32(sB) + s * b_bytes, P.cb + (u0 + i) % ntiles * (int64_t)(b_bytes / 4), b_bytes,
+                          full(s));
+        issued_s = i + 1;
+      }
+    }
+  } else {
+  int done = 0;                           // tiles of earlier query blocks
+  for (int64_t u = u0; u < u1;) {         // left together, by the barrier below
+  const int qb = (int)(u / ntiles), tile0 = (int)(u % ntiles);
+  const int count = (int)min((int64_t)(ntiles - tile0), u1 - u);
+  const int64_t q0 = (int64_t)qb * kM;
+  const int nqb = (int)min((int64_t)kM, P.nq - q0);
 
   // ---- queries -> hi / lo A operands (rows past the batch are zero); the
   // row's loads go out 16 at a time so that their latencies overlap
@@ -170,24 +200,15 @@ __global__ void __launch_bounds__(kThreads, 1) select_tc_kernel(SelParams P) {
     }
     tc::fence_async_smem();
   }
-  if (warp > 0) asm volatile("bar.sync 3, %0;" ::"n"(kThreads - 32) : "memory");
+  // (every thread but the producer's: a block's queries are staged, and the MMAs
+  // of the block before, whose last tile the epilogue has read, are done)
+  if (tc::named_bar_or(3, kThreads - 32, *abort_v != 0)) break;
 
-  if (warp == 0) {
-    // ---- producer: one bulk copy per codebook tile (hi and lo together)
-    if (lane == 0) {
-      for (int i = 0; i < ntiles; ++i) {
-        const uint32_t s = i % kStages, ph = (i / kStages) & 1;
-        if (!tc::bar_wait(empty(s), ph ^ 1, abort_v)) { give_up(); break; }
-        tc::bar_arrive_expect_tx(full(s), b_bytes);
-        tc::bulk_copy_g2s(tc::smem_u32(sB) + s * b_bytes, P.cb + (int64_t)i * (b_bytes / 4), b_bytes, full(s));
-        issued_s = i + 1;
-      }
-    }
-  } else if (warp == 1) {
+  if (warp == 1) {
     // ---- MMA issuer: three tf32 passes per tile into TMEM buffer i % 2
     const uint32_t idesc = tc::idesc_tf32(kM, kN);
-    int committed = 0;
-    for (int i = 0; i < ntiles; ++i) {
+    int committed = done;
+    for (int i = done; i < done + count; ++i) {
       if (tc::named_bar_or(2, 64, false)) break;
       const uint32_t s = i % kStages, b = i & 1;
       if (lane == 0) {
@@ -211,7 +232,7 @@ __global__ void __launch_bounds__(kThreads, 1) select_tc_kernel(SelParams P) {
   } else if (warp == 2) {
     // ---- gate: waits for each tile's stage and TMEM buffer, then releases
     // the MMA issuer
-    for (int i = 0; i < ntiles; ++i) {
+    for (int i = done; i < done + count; ++i) {
       const uint32_t s = i % kStages, ph = (i / kStages) & 1, b = i & 1, tph = (i >> 1) & 1;
       int ok = 1;
       if (lane == 0) {
@@ -235,7 +256,7 @@ __global__ void __launch_bounds__(kThreads, 1) select_tc_kernel(SelParams P) {
 #pragma unroll
     for (int j = 0; j < TMAX; ++j) { ts[j] = j < lead ? INFINITY : -INFINITY; ti[j] = -1; }
     float cut = -INFINITY;                           // the t-th best score (-inf until t are held)
-    for (int i = 0; i < ntiles; ++i) {
+    for (int i = done; i < done + count; ++i) {
       const uint32_t b = i & 1, tph = (i >> 1) & 1;
       const bool ok = tc::bar_wait(tfull(b), tph, abort_v);
       if (!ok) give_up();
@@ -251,7 +272,7 @@ __global__ void __launch_bounds__(kThreads, 1) select_tc_kernel(SelParams P) {
       __syncwarp();
       if (lane == 0) tc::bar_arrive(tempty(b));
       if (!ok) break;
-      const int col0 = i * kN;
+      const int col0 = (tile0 + i - done) * kN;
       const int nvalid = min(kN, P.c - col0);
 #pragma unroll
       for (int ch = 0; ch < kN / kChunk; ++ch) {
@@ -291,18 +312,22 @@ __global__ void __launch_bounds__(kThreads, 1) select_tc_kernel(SelParams P) {
       }
     }
     if (active && !abort_s) {
-      const int64_t q = q0 + m;
+      const int64_t q = (q0 + m) * P.parts + ((int)blockIdx.x - first_cta(qb, ntiles, P.per));
 #pragma unroll
       for (int j = 0; j < TMAX; ++j) {
         if (j >= lead) {
           // an entry stays empty only when fewer than t scores exceed -inf
-          // (NaN or -inf rows):
-          // keep the ids valid partitions all the same
-          P.top[q * t + j - lead] = ti[j] >= 0 ? ti[j] : j - lead;
+          // (NaN or -inf rows, or a part with fewer centroids): the merge drops
+          // it; a whole list keeps valid partitions all the same
+          P.top[q * t + j - lead] = ti[j] >= 0 || P.parts > 1 ? ti[j] : j - lead;
           if (P.top_s) P.top_s[q * t + j - lead] = ts[j];
         }
       }
     }
+  }
+  done += count;
+  u += count;
+  }
   }
 
   // ---- teardown: after an abort, let copies and MMAs in flight land first
@@ -320,6 +345,49 @@ __global__ void __launch_bounds__(kThreads, 1) select_tc_kernel(SelParams P) {
   __syncthreads();
   tc::fence_after_sync();
   if (warp == 1) tc::tmem_dealloc(tmem, 2 * kN);
+}
+
+// The t best of a query's part lists, a warp per query (score descending, lower
+// id first, the order the parts were kept in).
+__global__ void __launch_bounds__(256) merge_parts(const int32_t* __restrict__ ids, const float* __restrict__ scores,
+                                                   int64_t nq, int tiles, int per, int parts, int t,
+                                                   int32_t* __restrict__ top, float* __restrict__ top_s) {
+  constexpr unsigned kFull = 0xffffffffu;
+  const int64_t q = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31;
+  if (q >= nq) return;
+  const int qb = (int)(q / kM);
+  const int n = (int)(((int64_t)(qb + 1) * tiles - 1) / per) - first_cta(qb, tiles, per) + 1;
+  // every part is sorted: the 32 smallest of two sorted lists are the lane-wise
+  // minima of one and the other reversed, a bitonic sequence that five exchanges
+  // sort; four parts are loaded together
+  constexpr int kAhead = 4;
+  uint64_t mine = ~0ull;                         // lane j: the j-th best key
+  for (int r0 = 0; r0 < n; r0 += kAhead) {
+    uint64_t key[kAhead];
+#pragma unroll
+    for (int u = 0; u < kAhead; ++u) {
+      const int64_t at = (q * parts + r0 + u) * t + lane;
+      const int32_t id = r0 + u < n && lane < t ? ids[at] : -1;
+      key[u] = id >= 0 ? rank_key(scores[at], (uint32_t)id) : ~0ull;
+    }
+#pragma unroll
+    for (int u = 0; u < kAhead; ++u) {
+      const uint64_t r = __shfl_sync(kFull, key[u], 31 - lane);
+      uint64_t c = r < mine ? r : mine;
+#pragma unroll
+      for (int j = 16; j > 0; j >>= 1) {
+        const uint64_t o = __shfl_xor_sync(kFull, c, j);
+        c = (lane & j) == 0 ? (o < c ? o : c) : (o > c ? o : c);
+      }
+      mine = c;
+    }
+  }
+  if (lane < t) {
+    const bool have = mine != ~0ull;
+    top[q * t + lane] = have ? (int32_t)(mine & 0xffffffffu) : lane;
+    if (top_s) top_s[q * t + lane] = have ? key_float(~(uint32_t)(mine >> 32)) : -INFINITY;
+  }
 }
 
 size_t select_smem_bytes(int kp) {
@@ -342,16 +410,44 @@ bool select_tc_usable(const IndexData& ix, const float* Qf, int qstride, int t) 
          (reinterpret_cast<uintptr_t>(Qf) & 15u) == 0;
 }
 
+// A CTA per 128 queries leaves SMs idle unless the batch has a multiple of 152
+// such blocks (79 for 10 000 queries, 1 for a single one), so the (query block,
+// codebook tile) units of smaller batches are dealt out evenly and the parts
+// merged by a warp per query.  Each part stages its queries and starts its bound
+// afresh, which pays from about forty tiles a CTA on (10 000 queries, t = 5,
+// against 10 000 centroids, 82 tiles a CTA: 289 -> 186 us with the merge; against
+// 2 000, 17 tiles: 80 + 18 against 87), or where most SMs have nothing else to do
+// (one query against 2 000: 67 -> 17 us), with at least two tiles a CTA.
 void select_tc(const IndexData& ix, const float* Qf, int64_t nq, int qstride, int t, int32_t* top, float* top_s,
-               cudaStream_t s) {
+               cudaStream_t s, Scratch* scr) {
   SOAR_REQUIRE(select_tc_usable(ix, Qf, qstride, t), "tensor-core selection not applicable");
   if (nq == 0) return;
-  SelParams P{Qf, nq, qstride, ix.d, ix.sel_kp, ix.sel_cb, ix.c, ix.sel_tiles, t, top, top_s, device_error_word()};
+  const int64_t blocks = (nq + kM - 1) / kM, units = blocks * ix.sel_tiles;
+  int64_t per = ix.sel_tiles;
+  if (scr && blocks < 2 * num_sms()) {
+    const int64_t even = std::max<int64_t>(std::min(2, ix.sel_tiles), (units + num_sms() - 1) / num_sms());
+    if (even >= 40 || blocks <= num_sms() / 4) per = std::min<int64_t>(per, even);
+  }
+  int parts = 1;
+  if (per != ix.sel_tiles)
+    for (int64_t qb = 0; qb < blocks; ++qb)
+      parts = std::max(parts, (int)(((qb + 1) * ix.sel_tiles - 1) / per) - first_cta((int)qb, ix.sel_tiles, (int)per) + 1);
+  if (parts == 1) per = ix.sel_tiles;
+  SelParams P{Qf, nq, qstride, ix.d, ix.sel_kp, ix.sel_cb, ix.c, ix.sel_tiles, t, top, top_s, device_error_word(),
+              (int)per, parts};
+  if (parts > 1) {
+    P.top = scr->get<int32_t>((size_t)nq * parts * t * 2);
+    P.top_s = reinterpret_cast<float*>(P.top + (size_t)nq * parts * t);
+  }
   const size_t smem = select_smem_bytes(ix.sel_kp);
   auto kern = t <= 16 ? select_tc_kernel<16> : select_tc_kernel<32>;
   SOAR_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  kern<<<ceil_div(nq, kM), kThreads, smem, s>>>(P);
+  kern<<<(unsigned)((units + per - 1) / per), kThreads, smem, s>>>(P);
   SOAR_LAUNCHED();
+  if (parts > 1) {
+    merge_parts<<<ceil_div(nq * 32, 256), 256, 0, s>>>(P.top, P.top_s, nq, ix.sel_tiles, (int)per, parts, t, top, top_s);
+    SOAR_LAUNCHED();
+  }
 }
 
 }  // namespace soar

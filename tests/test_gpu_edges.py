@@ -242,3 +242,24 @@ def test_assignment_shapes(soar, dtype, d, c, n):
     loss.scatter_(1, first[:, None], float("inf"))
     assert (first != A[:, 1]).all()
     assert (loss.gather(1, A[:, 1:])[:, 0] <= loss.min(1)[0] * (1 + 1e-5)).all()
+
+
+@pytest.mark.parametrize("nq,c,t", [(1, 130, 32), (1, 5300, 7), (129, 700, 17), (300, 9000, 16)])
+def test_selection_split_over_the_codebook(soar, nq, c, t):
+    """Parts that cut through query blocks, with three equal centroids among them."""
+    g = torch.Generator().manual_seed(c)
+    C = torch.randn(c, 40, generator=g)
+    C[c // 2] = C[c - 1] = C[3]
+    X = torch.randn(c, 40, generator=g)
+    A = torch.arange(c).int()[:, None].contiguous()
+    ix = soar.soar_index_build(X.cuda(), C.cuda(), A.cuda())
+    Q = torch.randn(nq, 40, generator=g)
+    Q[0] = C[3]
+    top, sc = soar.soar_select_partitions(ix, Q.cuda(), t, with_scores=True)
+    full = Q.double() @ C.double().T
+    want = full.topk(t, 1)[0]
+    assert torch.allclose(sc.cpu().double(), want, rtol=1e-5, atol=1e-4)
+    assert torch.allclose(full.gather(1, top.cpu().long()), want, rtol=1e-5, atol=1e-4)
+    assert all(top[q].unique().numel() == t for q in range(nq))
+    assert top[0, :3].tolist() == [3, c // 2, c - 1]          # equal scores: the lower id first
+    ix.close()
