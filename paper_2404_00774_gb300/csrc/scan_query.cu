@@ -19,6 +19,8 @@
 // spilled point (its exact score and id are identical).  Every probed pair
 // reads its rows once; a warp per pair keeps the whole GPU busy even for a
 // batch of a few queries.
+#include <algorithm>
+
 #include "internal.cuh"
 #include "scan_common.cuh"
 
@@ -108,20 +110,27 @@ __device__ __forceinline__ uint64_t merge_block(uint64_t mine, uint64_t key, uin
   return mine;
 }
 
-template <typename T>
+// Bound: HBM and the bytes in flight.  kAhead: 16-byte chunks of each of a
+// lane's two rows loaded together: 8 where few warps run (a split partition: the
+// latency of a step counts), 3 where the chip is full (more registers would
+// leave fewer warps: 10 000 queries x 5 partitions of 200 bf16 rows of 96, 660 us
+// with 8, 457 with 4, 381 with 3, 451 with loads two at a time in a rolled loop).
+template <typename T, int kAhead>
 __global__ void __launch_bounds__(32 * kQmWarps) scan_by_query_kernel(
     const T* __restrict__ rows, int kp, const int32_t* __restrict__ row_ids, const int64_t* __restrict__ gstart,
     const float* __restrict__ Qf, int qstride, const int32_t* __restrict__ top, const int32_t* __restrict__ tpq,
-    int64_t nq, int t, int k, Cand* __restrict__ lists) {
+    int64_t nq, int t, int split, int k, Cand* __restrict__ lists) {
   constexpr unsigned kFull = 0xffffffffu;
   constexpr int E = Chunk<T>::E;
   extern __shared__ __align__(16) float q_all[];   // [kQmWarps][kp]
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int64_t e = (int64_t)blockIdx.x * kQmWarps + w;   // pair q * t + j
-  if (e >= nq * t) return;                                // uniform within the warp
+  const int64_t l = (int64_t)blockIdx.x * kQmWarps + w;   // list (q * t + j) * split + slice
+  if (l >= nq * t * split) return;                        // uniform within the warp
+  const int64_t e = l / split;                            // pair q * t + j
+  const int slice = (int)(l - e * split);
   const int64_t q = e / t;
   const int j = (int)(e - q * t);
-  Cand* out = lists + e * k;
+  Cand* out = lists + l * k;
   const int tq = tpq ? min(max(tpq[q], 0), t) : t;
   if (j >= tq) {                                          // probe not taken: an empty list
     if (lane < k) out[lane] = Cand{-INFINITY, -1};
@@ -139,21 +148,29 @@ __global__ void __launch_bounds__(32 * kQmWarps) scan_by_query_kernel(
   const unsigned char* base = reinterpret_cast<const unsigned char*>(rows) + (lane & 7) * 16;
   const int64_t g1 = gstart[p + 1];
   // two 32-row blocks per iteration (lane l: row l of each), so that each
-  // lane has two rows' loads in flight
-  for (int64_t g = gstart[p]; g < g1; g += 8) {
+  // lane has two rows' loads in flight; slices take every split-th iteration
+  for (int64_t g = gstart[p] + 8 * (int64_t)slice; g < g1; g += 8 * (int64_t)split) {
     const int64_t ga = g + (lane >> 3), gb = ga + 4;
     const bool va = ga < g1, vb = gb < g1;
     const int32_t ida = va ? row_ids[ga * 8 + (lane & 7)] : -1;
     const int32_t idb = vb ? row_ids[gb * 8 + (lane & 7)] : -1;
-    const unsigned char* xa = base + (va ? ga : 0) * group_bytes;
-    const unsigned char* xb = base + (vb ? gb : 0) * group_bytes;
+    const unsigned char* xa = base + (va ? ga : g) * group_bytes;
+    const unsigned char* xb = base + (vb ? gb : g) * group_bytes;
     float acc_a = 0.f, acc_b = 0.f;
-#pragma unroll 2
-    for (int c = 0; c < chunks; ++c) {
-      const uint4 wa = __ldg(reinterpret_cast<const uint4*>(xa + c * 128));
-      const uint4 wb = __ldg(reinterpret_cast<const uint4*>(xb + c * 128));
-      acc_a = Chunk<T>::dot(wa, qs + c * E, acc_a);
-      acc_b = Chunk<T>::dot(wb, qs + c * E, acc_b);
+    for (int c0 = 0; c0 < chunks; c0 += kAhead) {
+      uint4 wa[kAhead], wb[kAhead];
+#pragma unroll
+      for (int u = 0; u < kAhead; ++u)
+        if (c0 + u < chunks) {                            // uniform
+          wa[u] = __ldg(reinterpret_cast<const uint4*>(xa + (c0 + u) * 128));
+          wb[u] = __ldg(reinterpret_cast<const uint4*>(xb + (c0 + u) * 128));
+        }
+#pragma unroll
+      for (int u = 0; u < kAhead; ++u)
+        if (c0 + u < chunks) {
+          acc_a = Chunk<T>::dot(wa[u], qs + (c0 + u) * E, acc_a);
+          acc_b = Chunk<T>::dot(wb[u], qs + (c0 + u) * E, acc_b);
+        }
     }
     const uint64_t ka = ida >= 0 ? rank_key(acc_a, (uint32_t)ida) : ~0ull;   // -1: padding row or past the end
     const uint64_t kb = idb >= 0 ? rank_key(acc_b, (uint32_t)idb) : ~0ull;
@@ -167,6 +184,59 @@ __global__ void __launch_bounds__(32 * kQmWarps) scan_by_query_kernel(
   }
 }
 
+// The best k distinct (score, id) of each query's nl lists (k entries, best
+// first, an id of -1 closing a shorter one) by `per` warps: each takes every
+// per-th list, its lanes holding the best k so far; one of them takes the
+// others' k at the end.  Equal keys are a spilled point's copies: one is kept.
+template <int per>
+__global__ void __launch_bounds__(32 * kQmWarps) merge_lists(const Cand* __restrict__ lists, int64_t nq, int nl, int k,
+                                                             int64_t* __restrict__ ids, float* __restrict__ scores) {
+  constexpr unsigned kFull = 0xffffffffu;
+  __shared__ uint64_t keys_s[kQmWarps][32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int64_t q = ((int64_t)blockIdx.x * kQmWarps + w) / per;
+  uint64_t mine = ~0ull, thr = ~0ull;
+  const auto insert = [&](uint64_t key) {
+    unsigned bal = __ballot_sync(kFull, key < thr);
+    while (bal) {
+      const int src = __ffs(bal) - 1;
+      bal &= bal - 1;
+      const uint64_t kk = __shfl_sync(kFull, key, src);
+      if (kk >= thr) continue;
+      if (__ballot_sync(kFull, lane < k && mine == kk)) continue;
+      const int at = __popc(__ballot_sync(kFull, lane < k && mine < kk));
+      const uint64_t up = __shfl_up_sync(kFull, mine, 1);
+      if (lane > at && lane < k) mine = up;
+      if (lane == at) mine = kk;
+      thr = __shfl_sync(kFull, mine, k - 1);
+    }
+  };
+  if (q < nq) {
+    constexpr int kAhead = 4;                       // lists loaded together
+    for (int j0 = w % per; j0 < nl; j0 += per * kAhead) {
+      Cand c[kAhead];
+#pragma unroll
+      for (int u = 0; u < kAhead; ++u) {
+        const int j = j0 + per * u;
+        c[u] = (j < nl && lane < k) ? lists[(q * nl + j) * k + lane] : Cand{0.f, -1};
+      }
+#pragma unroll
+      for (int u = 0; u < kAhead; ++u) insert(c[u].id >= 0 ? rank_key(c[u].s, (uint32_t)c[u].id) : ~0ull);
+    }
+  }
+  if (per > 1) {
+    keys_s[w][lane] = lane < k ? mine : ~0ull;
+    __syncthreads();
+    if (w % per == 0)
+      for (int u = 1; u < per; ++u) insert(keys_s[w + u][lane]);
+  }
+  if (q < nq && w % per == 0 && lane < k) {
+    const bool have = mine != ~0ull;
+    ids[q * k + lane] = have ? (int64_t)(uint32_t)(mine & 0xffffffffu) : -1;
+    scores[q * k + lane] = have ? key_float(~(uint32_t)(mine >> 32)) : -INFINITY;
+  }
+}
+
 }  // namespace
 
 bool scan_by_query_usable(const IndexData& ix, int64_t nq, int t, int k) {
@@ -175,19 +245,39 @@ bool scan_by_query_usable(const IndexData& ix, int64_t nq, int t, int k) {
          nq * (int64_t)t <= 2 * (int64_t)ix.c;
 }
 
+// Warps per (query, probe) pair: one when the pairs alone keep 16 warps on every
+// SM, else as many as that takes, but no more than the largest partition has
+// steps of 64 rows.
+static int scan_split(const IndexData& ix, int64_t pairs) {
+  const int64_t want = 16 * (int64_t)num_sms() / pairs, most = (ix.max_partition + 63) / 64;
+  return (int)std::max<int64_t>(1, std::min<int64_t>({want, most, (int64_t)64}));
+}
+
 void scan_by_query(const IndexData& ix, const float* Qf, int qstride, const int32_t* top, const int32_t* tpq,
-                   int64_t nq, int t, int k, Cand* lists, cudaStream_t s) {
+                   int64_t nq, int t, int k, int64_t* ids_out, float* scores_out, cudaStream_t s, Scratch& scr) {
   const size_t smem = (size_t)kQmWarps * ix.tc_kp * sizeof(float);
-  const unsigned grid = ceil_div(nq * t, kQmWarps);
-  if (ix.dtype == SOAR_F32)
-    scan_by_query_kernel<float><<<grid, 32 * kQmWarps, smem, s>>>(
-        static_cast<const float*>(ix.tc_rows), ix.tc_kp, ix.tc_ids, ix.tc_gstart, Qf, qstride, top, tpq, nq, t, k,
-        lists);
-  else
-    scan_by_query_kernel<__nv_bfloat16><<<grid, 32 * kQmWarps, smem, s>>>(
-        static_cast<const __nv_bfloat16*>(ix.tc_rows), ix.tc_kp, ix.tc_ids, ix.tc_gstart, Qf, qstride, top, tpq,
-        nq, t, k, lists);
+  const int split = scan_split(ix, nq * t);
+  Cand* lists = scr.get<Cand>((size_t)nq * t * split * k);
+  const unsigned grid = ceil_div(nq * t * split, kQmWarps);
+  stage_mark(s, "scan", true);
+  const auto launch = [&](auto elem) {
+    using T = decltype(elem);
+    auto kern = split > 1 ? scan_by_query_kernel<T, 8> : scan_by_query_kernel<T, 3>;
+    kern<<<grid, 32 * kQmWarps, smem, s>>>(static_cast<const T*>(ix.tc_rows), ix.tc_kp, ix.tc_ids, ix.tc_gstart, Qf,
+                                           qstride, top, tpq, nq, t, split, k, lists);
+  };
+  if (ix.dtype == SOAR_F32) launch(float{});
+  else launch(__nv_bfloat16{});
   SOAR_LAUNCHED();
+  stage_mark(s, "scan", false);
+  stage_mark(s, "merge", true);
+  // a warp per query; eight where the batch is small and the lists many
+  if (nq >= 2 * num_sms() * kQmWarps || t * split < 16)
+    merge_lists<1><<<ceil_div(nq, kQmWarps), 32 * kQmWarps, 0, s>>>(lists, nq, t * split, k, ids_out, scores_out);
+  else
+    merge_lists<kQmWarps><<<(unsigned)nq, 32 * kQmWarps, 0, s>>>(lists, nq, t * split, k, ids_out, scores_out);
+  SOAR_LAUNCHED();
+  stage_mark(s, "merge", false);
 }
 
 }  // namespace soar

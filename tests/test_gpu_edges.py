@@ -263,3 +263,15 @@ def test_selection_split_over_the_codebook(soar, nq, c, t):
     assert all(top[q].unique().numel() == t for q in range(nq))
     assert top[0, :3].tolist() == [3, c // 2, c - 1]          # equal scores: the lower id first
     ix.close()
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("nq,k,t", [(1, 10, 14), (1, 32, 30), (3, 1, 20), (9, 32, 7), (70, 5, 3)])
+def test_few_queries_split_partitions_over_warps(soar, dtype, nq, k, t):
+    X, C, A, ix = _index(soar, 9000, 24, 110, 7, dtype, copies=50)
+    g = torch.Generator().manual_seed(nq)
+    Q = torch.nn.functional.normalize(torch.randn(nq, 24, generator=g), dim=1)
+    Q[0] = X[0].float()
+    for counts in (None, torch.randint(0, t + 1, (nq,), generator=g).int()):
+        _check_search(soar, X, C, A, ix, Q, k, t, counts)
+    ix.close()
