@@ -67,26 +67,25 @@ void finish_tc_queries(const IndexData& ix, const Cand* lists, const int2* hdr, 
 // screening on the tensor cores, then exact rescoring; the final top k of
 // every query goes to ids_out / scores_out.  counter: zero; hdr [nq * t]:
 // cleared headers of the grouped pairs; gbound [nq]: the ordered key of -inf;
-// lists: room for scan_tc_list_len(k) candidates a pair.
+// lists: room for kc = scan_tc_list_len(k, nq * t) candidates a pair.
 // k <= scan_tc_max_k(ix) (at most 128).
 void scan_tc_search(const IndexData& ix, const IvfWork& work, int max_items, const float* Qf, const float* qnorm,
                     const int32_t* top, const int32_t* inv, const int32_t* tpq, int64_t nq, int t, int k,
-                    Cand* lists, int* counter, int2* hdr, unsigned* gbound, int* err, int64_t* ids_out,
+                    Cand* lists, int kc, int* counter, int2* hdr, unsigned* gbound, int* err, int64_t* ids_out,
                     float* scores_out, cudaStream_t s, Scratch& scr);
 int scan_tc_max_k(const IndexData& ix);
-// Candidate-list length per pair slot of the group-maxima scan (scan_gm.cu),
-// which takes k <= 16 when its shared memory fits the row width.
-constexpr int kGmList = 128;
+// Group-maxima scan (scan_gm.cu), which takes k <= 16 when its shared memory fits
+// the row width; lists [pairs][kc].  Headers cleared, bounds -inf and the work
+// counter zero before the launch.
 bool scan_gm_usable(const IndexData& ix, int k);
-// Launches it (after the caller cleared the headers, set the bounds to -inf
-// and zeroed the work counter); lists [pairs][kGmList].
 void scan_gm_launch(const IndexData& ix, const IvfWork& work, int grid, const float* Qf, const float* qnorm,
-                    int64_t nq, int k, float dscale, long long wait_limit, int* counter, int* err,
+                    int64_t nq, int k, int kc, float dscale, long long wait_limit, int* counter, int* err,
                     unsigned* gbound, Cand* lists, int2* hdr, cudaStream_t s, Scratch& scr);
 // SM cycles a pipeline wait of the scan may take before its CTA gives up
 // (0: the default of about a second); the teardown's waits keep the default.
 void set_scan_wait_limit(long long cycles);
-int scan_tc_list_len(int k);
+// Candidate-list length per pair slot for a batch of `pairs` (query, probe) pairs.
+int scan_tc_list_len(int k, int64_t pairs);
 
 // Query-major exact scan (scan_query.cu): one or more warps per (query, probe)
 // pair (top [nq][t], tpq per-query counts or null) over the core-matrix rows;

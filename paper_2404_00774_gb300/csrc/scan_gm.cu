@@ -6,10 +6,13 @@
 // Work items are (partition p, up to 128 of the queries probing p), claimed
 // by one persistent CTA per SM.  The item's queries are the A operand (M =
 // 128 rows, K-major core-matrix layout); the partition's rows stream through
-// a ring of 64-row B tiles copied by cp.async.bulk straight from the index;
-// one thread issues the MMAs (kind::tf32 for fp32 rows; kind::f16 with the
-// fp32 query split into bf16 hi + lo parts for bf16 rows) into one of four
-// TMEM accumulators of 64 columns.
+// a ring of B tiles of 64 rows (128 for long partitions) copied by
+// cp.async.bulk straight from the index; one thread issues the MMAs (kind::tf32
+// for fp32 rows; kind::f16 with the fp32 query split into bf16 hi + lo parts for
+// bf16 rows) into one of four TMEM accumulators.  An MMA of 64 columns takes
+// about as long as one of 128 (41 ns), so the wider tile halves the tensor time,
+// which sets the pace of long scans; it leaves no shared memory for parking, so
+// there the surviving groups are picked out of the registers.
 //
 // Pipelining.  The producer publishes the next item's description before it
 // streams the current item's tiles and never waits for an item boundary, so
@@ -60,14 +63,14 @@ namespace soar {
 namespace {
 
 constexpr int kM = 128;        // query slots per item (MMA M)
-constexpr int kN = 64;         // rows per tile (MMA N)
+constexpr int kN = 64;         // rows screened at a time; a tile (MMA N) holds one or two times as many
 constexpr int kThreads = 224;  // producer, MMA issuer, gate, 4 epilogue warps
 constexpr int kMaxStages = 8;
-constexpr int kNB = 4;         // TMEM accumulators (kN columns each)
+constexpr int kNB = 4;         // TMEM accumulators (a tile's columns each)
 constexpr int kRing = 4;       // item descriptions in flight
 constexpr int kGK = 16;        // group maxima kept per query (k <= kGK)
-constexpr int kCap = 32;       // candidate rows held per query slot in shared memory
-constexpr int kStageAt = 2;    // the next item's A buffer is released after this many tiles of the current one
+// candidate rows held per query slot in shared memory
+__host__ __device__ constexpr int cap_for(int nt) { return nt == 1 ? 32 : 16; }
 
 struct GmParams {
   IvfWork work;
@@ -79,12 +82,13 @@ struct GmParams {
   int kp;                  // K, a multiple of 8 (fp32) or 16 (bf16)
   float dscale;            // delta / (||q|| max_p ||x||)
   int k;
+  int kc;                  // candidates per pair in the global list
   int stages;
   long long wait_limit;
   int* counter;            // work-item counter
   int* err;                // set to 1 when a wait expired
   unsigned* gbound;        // [nq] ordered key of the query's best published L_k
-  Cand* cand;              // [pairs][kGmList] (upper bound, row-major row position), written at an item's end
+  Cand* cand;              // [pairs][kc] (upper bound, row-major row position), written at an item's end
   int2* hdr;               // [pairs] (L_k as float bits, count | overflow << 31)
 };
 
@@ -121,8 +125,8 @@ __device__ Item describe(const GmParams& P, int item, int total) {
 
 
 // KX = 10: k fixed at 10 (the k-th of the sorted group maxima is a fixed
-// register); KX = 0: k <= 16 at run time.
-template <typename ET, int KX>
+// register); KX = 0: k <= 16 at run time.  NT: 64-row halves of a tile.
+template <typename ET, int KX, int NT>
 __global__ void __launch_bounds__(kThreads, 1) scan_gm_kernel(GmParams P) {
   constexpr uint32_t es = sizeof(ET);            // bytes per operand element
   constexpr unsigned kFull = 0xffffffffu;
@@ -134,16 +138,21 @@ __global__ void __launch_bounds__(kThreads, 1) scan_gm_kernel(GmParams P) {
   const uint32_t sbo = (uint32_t)kp * 8u * es;         // bytes between 8-row groups
   const uint32_t a_part = (uint32_t)kM * kp * es;      // one A part (bf16: hi or lo)
   const uint32_t a_bytes = (es == 4 ? 1u : 2u) * a_part;   // one A operand buffer
-  const uint32_t b_bytes = (uint32_t)kN * kp * es;
+  constexpr int kCap = cap_for(NT);
+  constexpr int kTile = NT * kN;                       // rows per tile
+  constexpr int kTG = kTile / 8;                       // 8-row groups per tile
+  constexpr int kStageAt = NT == 1 ? 2 : 1;            // the next item's A buffer is released after this many tiles
+  const int kc = P.kc;
+  const uint32_t b_bytes = (uint32_t)kTile * kp * es;
   const char* rows = static_cast<const char*>(P.rows);
   unsigned char* sA = base;                            // two A operand buffers (items alternate)
   unsigned char* sB = base + 2 * a_bytes;
-  // a tile's surviving groups parked per query slot as float4s ([group][kM],
+  // (64-row tiles) a tile's surviving groups parked per query slot as float4s ([group][kM],
   // so that a warp's 32 lanes write 512 consecutive bytes), then the
   // candidates per query slot ([entry][kM]: 32 lanes, 32 distinct banks):
   // scores, then padded row positions
   float4* park_s = reinterpret_cast<float4*>(sB + (size_t)S * b_bytes);
-  float* list_s = reinterpret_cast<float*>(park_s + 16 * kM);
+  float* list_s = reinterpret_cast<float*>(park_s + (NT == 1 ? 16 * kM : 0));
   uint64_t* bars = reinterpret_cast<uint64_t*>(list_s + 2 * kCap * kM);
   // bars: full[S], empty[S], tfull[kNB], tempty[kNB], dfull[kRing], dempty[kRing], aready[2], agone[2]
   __shared__ Item ring_s[kRing];
@@ -185,19 +194,19 @@ __global__ void __launch_bounds__(kThreads, 1) scan_gm_kernel(GmParams P) {
     abort_s = 0;
     issued_s = consumed_s = committed_s = 0;
   }
-  if (warp == 1) tc::tmem_alloc(tc::smem_u32(&tmem_base_s), kNB * kN);
+  if (warp == 1) tc::tmem_alloc(tc::smem_u32(&tmem_base_s), kNB * kTile);
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
   const uint32_t tmem = tmem_base_s;
-  const uint32_t idesc = es == 4 ? tc::idesc_tf32(kM, kN) : tc::idesc_bf16(kM, kN);
+  const uint32_t idesc = es == 4 ? tc::idesc_tf32(kM, kTile) : tc::idesc_bf16(kM, kTile);
   volatile int* abort_v = &abort_s;
   const long long lim = P.wait_limit;
   auto give_up = [&]() {
     if (atomicExch(&abort_s, 1) == 0) atomicExch(P.err, 1);
   };
   const int total = P.work.count();
-  auto tile_bytes = [&](int ngr, int t) { return (uint32_t)min(8, ngr - 8 * t) * 8u * kp * es; };
+  auto tile_bytes = [&](int ngr, int t) { return (uint32_t)min(kTG, ngr - kTG * t) * 8u * kp * es; };
   auto group_ptr = [&](int64_t g) { return rows + g * 8 * kp * es; };
 
   if (warp == 0) {
@@ -214,18 +223,19 @@ __global__ void __launch_bounds__(kThreads, 1) scan_gm_kernel(GmParams P) {
         ring_s[r] = d;
         tc::bar_arrive(dfull(r));                      // release: the description is visible to the waiters
         if (d.p >= 0)
-          for (int j = 0; j < min(S, (d.ng + 7) / 8); ++j) tc::bulk_prefetch_l2(group_ptr(d.g0 + 8 * j), tile_bytes(d.ng, j));
+          for (int j = 0; j < min(S, (d.ng + kTG - 1) / kTG); ++j)
+            tc::bulk_prefetch_l2(group_ptr(d.g0 + kTG * j), tile_bytes(d.ng, j));
         return d;
       };
       uint32_t T = 0;
       Item cur = publish(0);
       for (int i = 0; cur.p >= 0; ++i) {
         const Item nxt = publish(i + 1);
-        const int nt = (cur.ng + 7) / 8;
+        const int nt = (cur.ng + kTG - 1) / kTG;
         bool stop = false;
         for (int j = 0; j < nt; ++j, ++T) {
           const uint32_t s = T % S, ph = (T / S) & 1;
-          if (j + S < nt) tc::bulk_prefetch_l2(group_ptr(cur.g0 + 8 * (j + S)), tile_bytes(cur.ng, j + S));
+          if (j + S < nt) tc::bulk_prefetch_l2(group_ptr(cur.g0 + kTG * (j + S)), tile_bytes(cur.ng, j + S));
           if (!tc::bar_wait(empty(s), ph ^ 1, abort_v, lim)) {
             give_up();
             stop = true;
@@ -233,7 +243,7 @@ __global__ void __launch_bounds__(kThreads, 1) scan_gm_kernel(GmParams P) {
           }
           const uint32_t bytes = tile_bytes(cur.ng, j);
           tc::bar_arrive_expect_tx(full(s), bytes);
-          tc::bulk_copy_g2s(tc::smem_u32(sB) + s * b_bytes, group_ptr(cur.g0 + 8 * j), bytes, full(s));
+          tc::bulk_copy_g2s(tc::smem_u32(sB) + s * b_bytes, group_ptr(cur.g0 + kTG * j), bytes, full(s));
           issued_s = (int)(T + 1);
         }
         if (stop) break;
@@ -255,10 +265,10 @@ __global__ void __launch_bounds__(kThreads, 1) scan_gm_kernel(GmParams P) {
         for (int j = 0; j < steps; ++j) {
           const uint64_t ad = tc::smem_desc(a0 + j * 256, 128, sbo), bd = tc::smem_desc(b0 + j * 256, 128, sbo);
           if constexpr (es == 4) {
-            tc::mma_tf32(tmem + b * kN, ad, bd, idesc, j > 0);
+            tc::mma_tf32(tmem + b * kTile, ad, bd, idesc, j > 0);
           } else {
-            tc::mma_bf16(tmem + b * kN, ad, bd, idesc, j > 0);
-            tc::mma_bf16(tmem + b * kN, tc::smem_desc(a0 + a_part + j * 256, 128, sbo), bd, idesc, 1);
+            tc::mma_bf16(tmem + b * kTile, ad, bd, idesc, j > 0);
+            tc::mma_bf16(tmem + b * kTile, tc::smem_desc(a0 + a_part + j * 256, 128, sbo), bd, idesc, 1);
           }
         }
         tc::mma_commit(empty(s));                      // the stage is free once these MMAs completed
@@ -280,7 +290,7 @@ __global__ void __launch_bounds__(kThreads, 1) scan_gm_kernel(GmParams P) {
         ok = tc::bar_wait(dfull(r), (i / kRing) & 1, abort_v, lim);
         if (ok) {
           const Item d = ring_s[r];
-          nt = d.p < 0 ? -1 : (d.ng + 7) / 8;
+          nt = d.p < 0 ? -1 : (d.ng + kTG - 1) / kTG;
         }
         if (ok && nt >= 0) {
           ok = tc::bar_wait(aready(i & 1), (i >> 1) & 1, abort_v, lim);
@@ -414,7 +424,8 @@ __global__ void __launch_bounds__(kThreads, 1) scan_gm_kernel(GmParams P) {
       float ak = -INFINITY, cut = gq;
       int cnt = 0, wg = 0;                            // candidates in shared memory / in the pair's global list
       bool ovf = false;
-      Cand* out = P.cand + (cur.e0 + (active ? jq : 0)) * (int64_t)kGmList;
+      Cand* out = P.cand + (cur.e0 + (active ? jq : 0)) * (int64_t)kc;
+      float packed = -INFINITY;                       // the cut when the shared list was last cleared (128-row tiles)
       // at the end of the item the shared-memory candidates at or above c_cut
       // move to the pair's global list as (upper bound of the exact score,
       // row); only a full global list overflows (the partition is then
@@ -423,13 +434,14 @@ __global__ void __launch_bounds__(kThreads, 1) scan_gm_kernel(GmParams P) {
         for (int j2 = 0; j2 < cnt; ++j2) {
           const float sv = cub[j2 * kM];
           if (sv >= c_cut) {
-            if (wg < kGmList) out[wg++] = Cand{sv + dlt, cpos[j2 * kM]};
+            if (wg < kc) out[wg++] = Cand{sv + dlt, cpos[j2 * kM]};
             else ovf = true;
           }
         }
         cnt = 0;
       };
-      const int nt = (cur.ng + 7) / 8;
+      const int nt = (cur.ng + kTG - 1) / kTG;
+      if constexpr (NT == 1)                          // 64-row tiles, parked survivors
       for (int j = 0; j < nt; ++j, ++T) {
         const uint32_t b = T % kNB, tph = (T / kNB) & 1;
         const bool ok = tc::bar_wait(tfull(b), tph, abort_v, lim);
@@ -437,7 +449,7 @@ __global__ void __launch_bounds__(kThreads, 1) scan_gm_kernel(GmParams P) {
         tc::fence_after_sync();
         uint32_t ra[32], rb[32];
         float g[16], gu[16];                          // the tile's group maxima (groups of four or eight rows)
-        const uint32_t taddr = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + b * kN;
+        const uint32_t taddr = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + b * kTile;
         const int nvalid = min(kN, cur.nrows - kN * j);
         // After an item's first two tiles the bound has mostly converged: a
         // full tile then takes eight groups of eight rows, half the sorting
@@ -534,7 +546,7 @@ __global__ void __launch_bounds__(kThreads, 1) scan_gm_kernel(GmParams P) {
               for (int u = 0; u < 8; ++u) {
                 const bool take = vv[u] >= cut0;
                 const bool to_s = take && cnt < kCap;
-                const bool to_g = take && !to_s && wg < kGmList;
+                const bool to_g = take && !to_s && wg < kc;
                 if (to_s) {
                   cub[cnt * kM] = vv[u];
                   cpos[cnt * kM] = pr0 + c0 + u;
@@ -631,7 +643,7 @@ __global__ void __launch_bounds__(kThreads, 1) scan_gm_kernel(GmParams P) {
                 // pair's global list (stores only, nothing read back)
                 const bool take = vv[u] >= cut0 && c0 + u < nvalid;
                 const bool to_s = take && cnt < kCap;
-                const bool to_g = take && !to_s && wg < kGmList;
+                const bool to_g = take && !to_s && wg < kc;
                 if (to_s) {
                   cub[cnt * kM] = vv[u];
                   cpos[cnt * kM] = pr0 + c0 + u;
@@ -648,6 +660,183 @@ __global__ void __launch_bounds__(kThreads, 1) scan_gm_kernel(GmParams P) {
           gq = fmaxf(gq, unordered_key(gload) - dlt);
           cut = fmaxf(cut, gq);
         }
+      }
+      else                                            // 128-row tiles, survivors from the registers
+      for (int j = 0, nsub = (cur.ng + 7) / 8; j < nt; ++j, ++T) {
+        const uint32_t b = T % kNB, tph = (T / kNB) & 1;
+        const bool ok = tc::bar_wait(tfull(b), tph, abort_v, lim);
+        if (!ok) give_up();
+        tc::fence_after_sync();
+#pragma unroll 1
+        for (int h = 0; h < NT && ok; ++h) {
+          const int sub = NT * j + h;                 // 64 rows of the item
+          const int nvalid = min(kN, cur.nrows - kN * sub);
+          if (sub >= nsub) break;
+          uint32_t r[64];
+          float g[16];                                // the group maxima (groups of four or eight rows)
+          const uint32_t taddr = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + b * kTile + kN * h;
+          // After an item's first 128 rows the bound has mostly converged: 64 whole
+          // rows then take eight groups of eight, half the sorting and merging
+          // (groups of different sizes are still disjoint sets of distinct rows, so
+          // the bound stays valid).
+          const bool wide = sub >= 2 && nvalid == kN;
+          if (wide) {
+#pragma unroll
+            for (int q8 = 0; q8 < 8; ++q8) tc::tmem_ld8_max(taddr + 8 * q8, r + 8 * q8, g[q8]);
+          } else {
+#pragma unroll
+            for (int q4 = 0; q4 < 16; ++q4) tc::tmem_ld4_max(taddr + 4 * q4, r + 4 * q4, g[q4]);
+          }
+          tc::tmem_ld_wait();
+          if (sub == 0) stage_next();
+          // every 256 rows refresh G_q; the load is issued here and used after
+          // the screening, so its latency overlaps that work
+          const bool refresh = active && (sub & 3) == 3;
+          const unsigned gload = refresh ? __ldcg(P.gbound + qid_c) : 0u;
+          const int32_t pr0 = (int32_t)(cur.row0 + (int64_t)kN * sub);   // row-major position of the first row
+          float g8[8];                                // maxima of the groups of eight
+          if (wide) {
+            float gw[8];
+#pragma unroll
+            for (int q8 = 0; q8 < 8; ++q8) gw[q8] = g8[q8] = g[q8];
+            // bitonic sort of the eight group maxima, descending
+#pragma unroll
+            for (int size = 2; size <= 8; size <<= 1)
+#pragma unroll
+              for (int stride = size >> 1; stride > 0; stride >>= 1)
+#pragma unroll
+                for (int i2 = 0; i2 < 8; ++i2) {
+                  const int j2 = i2 ^ stride;
+                  if (j2 > i2) {
+                    const bool desc = (i2 & size) == 0;
+                    const float x = gw[i2], y = gw[j2];
+                    gw[i2] = desc ? fmaxf(x, y) : fminf(x, y);
+                    gw[j2] = desc ? fminf(x, y) : fmaxf(x, y);
+                  }
+                }
+            // the list's last eight against the reversed eight
+#pragma unroll
+            for (int i2 = 8; i2 < 16; ++i2) gt[i2] = fmaxf(gt[i2], gw[15 - i2]);
+          } else {
+            if (nvalid < kN) {                        // past the partition's end: the missing rows count as -inf
+#pragma unroll
+              for (int c = 0; c < kN; ++c)
+                if (c >= nvalid) r[c] = 0xff800000u;
+#pragma unroll
+              for (int q4 = 0; q4 < 16; ++q4)
+                g[q4] = fmaxf(fmaxf(__uint_as_float(r[4 * q4]), __uint_as_float(r[4 * q4 + 1])),
+                              fmaxf(__uint_as_float(r[4 * q4 + 2]), __uint_as_float(r[4 * q4 + 3])));
+            }
+#pragma unroll
+            for (int q8 = 0; q8 < 8; ++q8) g8[q8] = fmaxf(g[2 * q8], g[2 * q8 + 1]);
+            // bitonic sort of the group maxima, descending
+#pragma unroll
+            for (int size = 2; size <= 16; size <<= 1)
+#pragma unroll
+              for (int stride = size >> 1; stride > 0; stride >>= 1)
+#pragma unroll
+                for (int i2 = 0; i2 < 16; ++i2) {
+                  const int j2 = i2 ^ stride;
+                  if (j2 > i2) {
+                    const bool desc = (i2 & size) == 0;
+                    const float x = g[i2], y = g[j2];
+                    g[i2] = desc ? fmaxf(x, y) : fminf(x, y);
+                    g[j2] = desc ? fminf(x, y) : fmaxf(x, y);
+                  }
+                }
+            // the 16 largest of two descending lists: the pairwise maxima against
+            // the reversed list form a bitonic sequence
+#pragma unroll
+            for (int i2 = 0; i2 < 16; ++i2) gt[i2] = fmaxf(gt[i2], g[15 - i2]);
+          }
+          // half-cleaners sort the bitonic sequence
+#pragma unroll
+          for (int stride = 8; stride > 0; stride >>= 1)
+#pragma unroll
+            for (int i2 = 0; i2 < 16; ++i2)
+              if ((i2 & stride) == 0) {
+                const float x = gt[i2], y = gt[i2 + stride];
+                gt[i2] = fmaxf(x, y);
+                gt[i2 + stride] = fminf(x, y);
+              }
+          if constexpr (KX > 0) {
+            ak = gt[KX - 1];
+          } else {                                    // gt[k - 1] as the smallest of the first k: gt stays in registers
+            ak = INFINITY;
+#pragma unroll
+            for (int j2 = 0; j2 < kGK; ++j2)
+              if (j2 < k) ak = fminf(ak, gt[j2]);
+          }
+          cut = fmaxf(ak - 2.f * dlt, gq);            // s~ + dlt < max(L_k, G_q)  <=>  s~ < cut
+          const float cut0 = active ? cut : INFINITY;
+          // 32 columns at a time, the warp in step: one trip per group of eight that
+          // holds a candidate of the lane with the most such groups, in it one per
+          // row; a full shared list first drops what fell below the cut, once per
+          // rise of it
+#pragma unroll
+          for (int hf = 0; hf < 2; ++hf) {
+            uint32_t gm = 0u;
+#pragma unroll
+            for (int q8 = 0; q8 < 4; ++q8) gm |= (g8[4 * hf + q8] >= cut0 ? 1u : 0u) << q8;
+            while (__any_sync(kFull, gm != 0u)) {
+              const int q8 = __ffs(gm) - 1;         // -1: this lane has none left
+              gm &= gm - 1u;
+              const int c0 = 32 * hf + 8 * q8;
+              float w[8];
+              uint32_t em = 0u;
+#pragma unroll
+              for (int u = 0; u < 8; ++u) {
+                const uint32_t* rh = r + 32 * hf;
+                const uint32_t lo = q8 & 1 ? rh[8 + u] : rh[u], hi = q8 & 1 ? rh[24 + u] : rh[16 + u];
+                w[u] = __uint_as_float(q8 & 2 ? hi : lo);
+                em |= (w[u] >= cut0 && c0 + u < nvalid ? 1u : 0u) << u;
+              }
+              if (q8 < 0) em = 0u;
+              if (em && cnt + 8 > kCap && cut > packed) {
+                packed = cut;
+                int n = 0;
+#pragma unroll 1
+                for (int i = 0; i < cnt; ++i) {
+                  const float o = cub[i * kM];
+                  if (o >= cut) {
+                    cub[n * kM] = o;
+                    cpos[n * kM] = cpos[i * kM];
+                    ++n;
+                  }
+                }
+                cnt = n;
+              }
+              while (__any_sync(kFull, em != 0u)) {
+                const int u = __ffs(em) - 1;
+                em &= em - 1u;
+                const float a0 = u & 1 ? w[1] : w[0], a1 = u & 1 ? w[3] : w[2], a2 = u & 1 ? w[5] : w[4],
+                            a3 = u & 1 ? w[7] : w[6];
+                const float b0 = u & 2 ? a1 : a0, b1 = u & 2 ? a3 : a2;
+                const float sv = u & 4 ? b1 : b0;
+                const bool take = u >= 0;
+                const bool to_s = take && cnt < kCap;
+                const bool to_g = take && !to_s && wg < kc;
+                if (to_s) {
+                  cub[cnt * kM] = sv;
+                  cpos[cnt * kM] = pr0 + c0 + u;
+                }
+                if (to_g) out[wg] = Cand{sv + dlt, pr0 + c0 + u};
+                ovf = ovf || (take && !to_s && !to_g);
+                cnt += to_s ? 1 : 0;
+                wg += to_g ? 1 : 0;
+              }
+            }
+          }
+          if (refresh) {
+            gq = fmaxf(gq, unordered_key(gload) - dlt);
+            cut = fmaxf(cut, gq);
+          }
+        }
+        tc::fence_before_sync();
+        __syncwarp();
+        if (lane == 0) tc::bar_arrive(tempty(b));
+        if (!ok) break;
+        if (j == kStageAt) release_next();
       }
       stage_next();                                   // items with fewer tiles
       release_next();
@@ -683,20 +872,31 @@ __global__ void __launch_bounds__(kThreads, 1) scan_gm_kernel(GmParams P) {
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
-  if (warp == 1) tc::tmem_dealloc(tmem, kNB * kN);
+  if (warp == 1) tc::tmem_dealloc(tmem, kNB * kTile);
 }
 
-size_t gm_smem_bytes(int kp, int stages, int es) {
+size_t gm_smem_bytes(int kp, int nt, int stages, int es) {
   // each of the two A buffers takes kM * kp * 4 bytes (fp32, or bf16 hi and lo); the
-  // parking area kN * kM * 4, the candidate lists 2 * kCap * kM * 4
-  return 1024 + (size_t)2 * kM * kp * 4 + (size_t)stages * kN * kp * es + (size_t)kN * kM * 4 +
-         (size_t)2 * kCap * kM * 4 + (size_t)(2 * stages + 2 * kNB + 2 * kRing + 4) * 8;
+  // parking area kN * kM * 4, the candidate lists 2 * cap * kM * 4
+  return 1024 + (size_t)2 * kM * kp * 4 + (size_t)stages * nt * kN * kp * es + (nt == 1 ? (size_t)kN * kM * 4 : 0) +
+         (size_t)2 * cap_for(nt) * kM * 4 + (size_t)(2 * stages + 2 * kNB + 2 * kRing + 4) * 8;
 }
 
-int gm_pick_stages(int kp, int es) {
-  for (int s = kMaxStages; s >= 2; --s)
-    if (gm_smem_bytes(kp, s, es) <= 227 * 1024 - 1024) return s;   // room for the static shared variables
+int gm_pick_stages(int kp, int nt, int es) {
+  for (int s = kMaxStages / nt; s >= 2; --s)
+    if (gm_smem_bytes(kp, nt, s, es) <= 227 * 1024 - 1024) return s;   // room for the static shared variables
   return 0;
+}
+
+// 64-row halves of a tile.  Long partitions take 128-row tiles, since the MMAs
+// and not the survivors set their pace (brute force of 10 000 queries over chunks
+// of 65 536 fp32 rows of 100: 8.17 ms with 64-row tiles, 6.75 with 128-row ones);
+// short ones keep 64-row tiles and parking (1 200 fp32 rows: 334 us, against 356
+// with 128-row tiles; 2 000 bf16 rows: 1.62 ms against 1.54 to 1.90).
+constexpr int64_t kLongPartition = 8192;   // average rows
+int gm_halves(const IndexData& ix) {
+  const int es = ix.dtype == SOAR_F32 ? 4 : 2;
+  return ix.rows >= kLongPartition * ix.c && gm_pick_stages(ix.tc_kp, 2, es) >= 2 ? 2 : 1;
 }
 
 // the bf16 query operand: per query its hi row bf16(q) and lo row bf16(q - hi)
@@ -711,9 +911,9 @@ __global__ void split_queries_bf16(const float* __restrict__ Qf, int64_t n, int 
   out[q * 2 * kp + kp + c] = __float2bfloat16_rn(v - __bfloat162float(hi));
 }
 
-template <typename ET>
+template <typename ET, int NT>
 void launch_gm(int k, int grid, size_t smem, cudaStream_t s, const GmParams& prm) {
-  auto kern = k == 10 ? scan_gm_kernel<ET, 10> : scan_gm_kernel<ET, 0>;
+  auto kern = k == 10 ? scan_gm_kernel<ET, 10, NT> : scan_gm_kernel<ET, 0, NT>;
   SOAR_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   kern<<<grid, kThreads, smem, s>>>(prm);
   SOAR_LAUNCHED();
@@ -723,14 +923,14 @@ void launch_gm(int k, int grid, size_t smem, cudaStream_t s, const GmParams& prm
 
 bool scan_gm_usable(const IndexData& ix, int k) {
   const int es = ix.dtype == SOAR_F32 ? 4 : 2;
-  return k >= 1 && k <= kGK && gm_pick_stages(ix.tc_kp, es) >= 2;
+  return k >= 1 && k <= kGK && gm_pick_stages(ix.tc_kp, 1, es) >= 2;
 }
 
 void scan_gm_launch(const IndexData& ix, const IvfWork& work, int grid, const float* Qf, const float* qnorm,
-                    int64_t nq, int k, float dscale, long long wait_limit, int* counter, int* err,
+                    int64_t nq, int k, int kc, float dscale, long long wait_limit, int* counter, int* err,
                     unsigned* gbound, Cand* lists, int2* hdr, cudaStream_t s, Scratch& scr) {
   const int es = ix.dtype == SOAR_F32 ? 4 : 2;
-  const int stages = gm_pick_stages(ix.tc_kp, es);
+  const int nt = gm_halves(ix), stages = gm_pick_stages(ix.tc_kp, nt, es);
   if (k < 1 || k > kGK || stages < 2) fail(SOAR_EUNSUPPORTED, "group-maxima scan: unsupported k or row width");
   const void* Qa = Qf;
   if (es == 2) {
@@ -740,11 +940,11 @@ void scan_gm_launch(const IndexData& ix, const IvfWork& work, int grid, const fl
     SOAR_LAUNCHED();
     Qa = qhl;
   }
-  GmParams prm{work, ix.tc_rows, ix.tc_gstart, ix.tc_pmax, Qa, qnorm, ix.tc_kp, dscale, k, stages, wait_limit,
+  GmParams prm{work, ix.tc_rows, ix.tc_gstart, ix.tc_pmax, Qa, qnorm, ix.tc_kp, dscale, k, kc, stages, wait_limit,
                counter, err, gbound, lists, hdr};
-  const size_t smem = gm_smem_bytes(ix.tc_kp, stages, es);
-  if (es == 4) launch_gm<float>(k, grid, smem, s, prm);
-  else launch_gm<__nv_bfloat16>(k, grid, smem, s, prm);
+  const size_t smem = gm_smem_bytes(ix.tc_kp, nt, stages, es);
+  if (es == 4) nt == 2 ? launch_gm<float, 2>(k, grid, smem, s, prm) : launch_gm<float, 1>(k, grid, smem, s, prm);
+  else nt == 2 ? launch_gm<__nv_bfloat16, 2>(k, grid, smem, s, prm) : launch_gm<__nv_bfloat16, 1>(k, grid, smem, s, prm);
 }
 
 }  // namespace soar

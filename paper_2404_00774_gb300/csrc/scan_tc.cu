@@ -43,6 +43,8 @@
 // Every mbarrier wait is bounded (about a second); on expiry the CTA raises
 // *err, stops taking work, waits (bounded) for its copies and MMAs in flight,
 // frees its TMEM and returns.
+#include <algorithm>
+
 #include "scan_common.cuh"
 #include "tc.cuh"
 
@@ -59,14 +61,22 @@ constexpr int kCand = 32;      // candidate rows kept per (query, partition), re
 constexpr int kWideK = kTcWideK;   // largest k of the heap mode
 constexpr int kWideList = kTcWideList;   // largest global candidate list of the heap mode
 
-// Candidate-list length per (query, partition) slot: kGmList for k <= 16
-// (the group-maxima scan of scan_gm.cu appends without a final filter),
-// kCand for k <= 32, else 2k rounded up to a warp multiple (room to append
-// between compactions).
-__host__ __device__ constexpr int list_len_for(int k) {
-  return k <= 16 ? kGmList
-                 : k <= kCand ? kCand
-                              : ((2 * k + 31) / 32 * 32 > kWideList ? kWideList : (2 * k + 31) / 32 * 32);
+// Candidate-list length per (query, partition) slot.  k <= 16 (the group-maxima
+// scan of scan_gm.cu appends without a final filter): 128, and for small batches
+// as many as 16 MB hold, up to 1 024, so that tight clusters whose rows lie within
+// the screening band of each other do not overflow (an overflowed list costs a
+// rescan of its partition: 100 queries over 64 partitions, 89 us of finishing
+// against 25).  kCand for k <= 32, else 2k rounded up to a warp multiple
+// (room to append between compactions).
+constexpr int kGmList = 128, kGmListMost = 1024;
+int list_len_for(int k, int64_t pairs) {
+  if (k <= 16) {
+    int len = kGmList;
+    while (len < kGmListMost && 2 * len * pairs * (int64_t)sizeof(Cand) <= ((int64_t)16 << 20)) len *= 2;
+    return len;
+  }
+  if (k <= kCand) return kCand;
+  return std::min(kWideList, (2 * k + 31) / 32 * 32);
 }
 
 // Shared memory behind the tile scores: register mode keeps kCand candidates
@@ -598,16 +608,15 @@ int scan_tc_max_k(const IndexData& ix) {
   return k;
 }
 
-int scan_tc_list_len(int k) { return list_len_for(k); }
+int scan_tc_list_len(int k, int64_t pairs) { return list_len_for(k, pairs); }
 
 void scan_tc_search(const IndexData& ix, const IvfWork& work, int max_items, const float* Qf, const float* qnorm,
                     const int32_t* top, const int32_t* inv, const int32_t* tpq, int64_t nq, int t, int k,
-                    Cand* lists, int* counter, int2* hdr, unsigned* gbound, int* err, int64_t* ids_out,
+                    Cand* lists, int kc, int* counter, int2* hdr, unsigned* gbound, int* err, int64_t* ids_out,
                     float* scores_out, cudaStream_t s, Scratch& scr) {
   const int es = ix.dtype == SOAR_F32 ? 4 : 2;
   const int stages = pick_stages(ix.tc_kp, k, es);
   if (stages < 2 || k > kWideK) fail(SOAR_EUNSUPPORTED, "tensor-core scan: k too large");
-  const int kc = list_len_for(k);
   const long long lim = g_wait_limit.load();
   const TcParams prm{work, ix.tc_rows, ix.tc_gstart, ix.tc_pmax, Qf, qnorm, ix.tc_kp, delta_scale(ix.tc_kp, es), k,
                      kc, stages, lim > 0 ? lim : tc::kWaitLimit, counter, err, gbound, lists, hdr};
@@ -615,7 +624,7 @@ void scan_tc_search(const IndexData& ix, const IvfWork& work, int max_items, con
   const int grid = std::max(1, std::min(max_items, num_sms()));
   stage_mark(s, "scan", true);
   if (scan_gm_usable(ix, k))
-    scan_gm_launch(ix, work, grid, Qf, qnorm, nq, k, prm.dscale, prm.wait_limit, counter, err, gbound, lists, hdr, s,
+    scan_gm_launch(ix, work, grid, Qf, qnorm, nq, k, kc, prm.dscale, prm.wait_limit, counter, err, gbound, lists, hdr, s,
                    scr);
   else if (es == 4)
     launch_scan_tc<float>(k, grid, smem, s, prm);

@@ -997,11 +997,11 @@ void search(const IndexData& ix, const void* Q, soar_dtype dt, int64_t nq, int32
     }
     const int64_t P = nq * t;
     int32_t* inv = scr.get<int32_t>(P);
-    const int len = scan_tc_list_len(k);
+    const int len = scan_tc_list_len(k, P);
     Cand* lists = scr.get<Cand>((size_t)P * len);
     Grouped g = group_pairs(ix, nq, t, tpq, 128, top, inv, s, scr, true, true);
     IvfWork work{ix.offsets, g.pair_off, g.vals, g.order, g.item_base, ix.c, t, 128};
-    scan_tc_search(ix, work, g.max_items, Qf, qn, top, inv, tpq, nq, t, k, lists, g.counter, g.hdr, g.gbound,
+    scan_tc_search(ix, work, g.max_items, Qf, qn, top, inv, tpq, nq, t, k, lists, len, g.counter, g.hdr, g.gbound,
                    device_error_word(), ids_out, scores_out, s, scr);
     return;
   }
@@ -1099,7 +1099,7 @@ void exact_mips(const void* X, soar_dtype xdt, int64_t n, int32_t d, const void*
     fx.tc_kp = (d + kstep - 1) / kstep * kstep;
     if (k <= scan_tc_max_k(fx)) {
       build_flat_tc(fx, X, pad, kChunkRows, s, scr);
-      const int c = fx.c, len = scan_tc_list_len(k);
+      const int c = fx.c, len = scan_tc_list_len(k, nq * fx.c);
       const size_t qesz = qdt == SOAR_F32 ? 4 : 2;
       // queries in batches whose candidate lists stay within about 1 GB
       const int64_t nb = std::max<int64_t>(128, (int64_t(1) << 30) / ((int64_t)c * len * (int64_t)sizeof(Cand)));
@@ -1116,7 +1116,7 @@ void exact_mips(const void* X, soar_dtype xdt, int64_t n, int32_t d, const void*
         Cand* lists = bs.get<Cand>((size_t)m * c * len);
         Grouped g = group_pairs(fx, m, c, nullptr, 128, top, inv, s, bs, true, false);
         IvfWork work{fx.offsets, g.pair_off, g.vals, g.order, g.item_base, c, c, 128};
-        scan_tc_search(fx, work, g.max_items, Qf, qn, top, inv, nullptr, m, c, k, lists, g.counter, g.hdr, g.gbound,
+        scan_tc_search(fx, work, g.max_items, Qf, qn, top, inv, nullptr, m, c, k, lists, len, g.counter, g.hdr, g.gbound,
                        device_error_word(), ids_out + q0 * k, scores_out + q0 * k, s, bs);
       }
       return;

@@ -275,3 +275,22 @@ def test_few_queries_split_partitions_over_warps(soar, dtype, nq, k, t):
     for counts in (None, torch.randint(0, t + 1, (nq,), generator=g).int()):
         _check_search(soar, X, C, A, ix, Q, k, t, counts)
     ix.close()
+
+
+@pytest.mark.parametrize("dtype,d", [(torch.float32, 100), (torch.float32, 130), (torch.bfloat16, 48)])
+@pytest.mark.parametrize("n,k", [(65_536 + 64, 10), (65_536 * 2 + 65, 16), (70_001, 1)])
+def test_brute_force_over_long_chunks(soar, dtype, d, n, k):
+    """Chunks whose last tile holds 64, 65 or a few rows; tight clusters and equal rows near the top."""
+    g = torch.Generator(device="cuda").manual_seed(n + d)
+    X = torch.randn(n, d, generator=g, device="cuda")
+    X[::3] = X[0] + 0.02 * X[::3]
+    X = torch.nn.functional.normalize(X, dim=1)
+    X[n - 40:] = X[0]
+    X = X.to(dtype)
+    Q = torch.cat([X[:1].float(), torch.nn.functional.normalize(torch.randn(140, d, generator=g, device="cuda"), dim=1)])
+    ids, sc = soar.soar_exact_mips(X, Q, k)
+    full = Q.double() @ X.double().T
+    want = full.topk(k, 1)[0]
+    assert torch.allclose(sc.double(), want, rtol=0, atol=1e-5)
+    assert torch.allclose(full.gather(1, ids), want, rtol=0, atol=1e-5)
+    assert all(ids[q].unique().numel() == k for q in range(0, 141, 20))
