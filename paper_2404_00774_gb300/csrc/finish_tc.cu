@@ -15,6 +15,11 @@ namespace {
 
 // Largest batch finished by a block per query when k <= 32.
 constexpr int64_t kBlockFinishMax = 4096;
+// Queries per SM up to which their blocks are of 512 threads, above that of 128
+// (finishing, us, 128 against 512 threads; 152 SMs: k = 100 of about 270 lists,
+// 70 queries 64 / 32, 300 queries 67 / 42, 600 queries 94 / 69, 1 024 queries
+// 103 / 103; k = 10, 1 200 queries 34 / 51).
+constexpr int64_t kWideBlockMax = 4;
 
 // Exact fp32 <q, x> of row-major row `pos` (row stride rs; k ascending, the
 // same order for every copy of a point).  fp32 rows: rs a multiple of 4.
@@ -69,23 +74,24 @@ __device__ __forceinline__ float exact_dot_rm(const float* __restrict__ q, const
 // a warp (k = 100, 1 024 queries of 272 lists: 870 us with its helper kernels,
 // 99 now), and takes k <= 32 too for batches that do not fill the chip
 // with a warp per query, where one warp rescanning overflowed partitions set
-// the time of a small batch (100 queries: 259 us before, 87 now).
-constexpr int kFbThreads = 128;
-constexpr int kFbKeys = 1024;                  // the best k so far and the pending candidates
-constexpr int kFbPend = kFbKeys - kTcWideK;
-constexpr int kFbUnroll = 4;                   // list entries a thread loads per round
+// the time of a small batch (100 queries: 147 us before, 18 now; most of that
+// since small batches get lists long enough not to overflow).
+constexpr int fb_keys(int threads) { return threads == 128 ? 1024 : 2048; }   // the best k so far and the pending
+constexpr int fb_pend(int threads) { return fb_keys(threads) - kTcWideK; }
+constexpr int fb_unroll(int threads) { return threads == 128 ? 4 : 2; }       // list entries a thread loads per round
 
-template <typename RowT>
-__global__ void __launch_bounds__(kFbThreads) finish_block(
+template <typename RowT, int T>
+__global__ void __launch_bounds__(T) finish_block(
     const Cand* __restrict__ cand, const int2* __restrict__ hdr, const unsigned* __restrict__ gbound,
     const int32_t* __restrict__ inv, int t, const int32_t* __restrict__ tpq, const float* __restrict__ Qf, int kp,
     const RowT* __restrict__ rows, int rs, const int32_t* __restrict__ ids, const int32_t* __restrict__ top,
     const int64_t* __restrict__ part_off, int k, int kc, int64_t* __restrict__ ids_out,
     float* __restrict__ scores_out) {
   constexpr unsigned kFull = 0xffffffffu;
-  constexpr int T = kFbThreads;
-  __shared__ uint64_t buf[kFbKeys];            // [0, best) ascending distinct keys
-  __shared__ int32_t pend[kFbPend];            // row positions
+  constexpr int kPend = fb_pend(T), kUnroll = fb_unroll(T);
+  static_assert(T * kUnroll <= kPend, "a round's entries fit behind an empty list");
+  __shared__ uint64_t buf[fb_keys(T)];         // [0, best) ascending distinct keys
+  __shared__ int32_t pend[kPend];              // row positions
   __shared__ int32_t pre_s[T], e_s[T], warp_s[32];
   __shared__ unsigned ovf_s[T / 32];
   __shared__ int fill_s;
@@ -154,12 +160,12 @@ __global__ void __launch_bounds__(kFbThreads) finish_block(
     const unsigned ob = __ballot_sync(kFull, ovf_l);
     if (lane == 0) ovf_s[w] = ob;
     __syncthreads();
-    for (int base = 0; base < total; base += T * kFbUnroll) {
-      if (fill_s + T * kFbUnroll > kFbPend) flush();     // (fill_s last written before a barrier: uniform)
-      bool keep[kFbUnroll];
-      int32_t pos[kFbUnroll];
+    for (int base = 0; base < total; base += T * kUnroll) {
+      if (fill_s + T * kUnroll > kPend) flush();     // (fill_s last written before a barrier: uniform)
+      bool keep[kUnroll];
+      int32_t pos[kUnroll];
 #pragma unroll
-      for (int u = 0; u < kFbUnroll; ++u) {
+      for (int u = 0; u < kUnroll; ++u) {
         const int f = base + u * T + tid;
         keep[u] = false;
         pos[u] = 0;
@@ -175,7 +181,7 @@ __global__ void __launch_bounds__(kFbThreads) finish_block(
       }
       __syncthreads();                          // every thread has read fill_s
 #pragma unroll
-      for (int u = 0; u < kFbUnroll; ++u) {
+      for (int u = 0; u < kUnroll; ++u) {
         const unsigned kb = __ballot_sync(kFull, keep[u]);
         int at = 0;
         if (lane == 0 && kb) at = atomicAdd(&fill_s, __popc(kb));
@@ -190,7 +196,7 @@ __global__ void __launch_bounds__(kFbThreads) finish_block(
         const int p = top[q * t + j0 + 32 * word + __ffs(bits) - 1];
         const int64_t r1 = part_off[p + 1];
         for (int64_t r0 = part_off[p]; r0 < r1; r0 += T) {
-          if (best < k || fill_s + T > kFbPend) flush();   // early rows fill the best k, then only better ones wait
+          if (best < k || fill_s + T > kPend) flush();   // early rows fill the best k, then only better ones wait
           const uint64_t thr = best == k ? buf[k - 1] : ~0ull;
           __syncthreads();
           const int64_t r = r0 + tid;
@@ -354,10 +360,14 @@ void finish_tc_queries(const IndexData& ix, const Cand* lists, const int2* hdr, 
       finish_queries<RowT><<<ceil_div(nq * 32, 256), 256, 0, s>>>(lists, hdr, gbound, inv, nq, t, tpq, Qf, ix.tc_kp,
                                                                   rows, ix.row_stride, ix.ids, top, ix.offsets, k, kc,
                                                                   ids_out, scores_out);
+    else if (nq > kWideBlockMax * num_sms())
+      finish_block<RowT, 128><<<(unsigned)nq, 128, 0, s>>>(lists, hdr, gbound, inv, t, tpq, Qf, ix.tc_kp, rows,
+                                                           ix.row_stride, ix.ids, top, ix.offsets, k, kc, ids_out,
+                                                           scores_out);
     else
-      finish_block<RowT><<<(unsigned)nq, kFbThreads, 0, s>>>(lists, hdr, gbound, inv, t, tpq, Qf, ix.tc_kp, rows,
-                                                             ix.row_stride, ix.ids, top, ix.offsets, k, kc, ids_out,
-                                                             scores_out);
+      finish_block<RowT, 512><<<(unsigned)nq, 512, 0, s>>>(lists, hdr, gbound, inv, t, tpq, Qf, ix.tc_kp, rows,
+                                                           ix.row_stride, ix.ids, top, ix.offsets, k, kc, ids_out,
+                                                           scores_out);
   };
   if (ix.dtype == SOAR_F32) launch(float{});
   else launch(__nv_bfloat16{});

@@ -94,7 +94,8 @@ struct soar_server {
 namespace {
 
 // Device scratch one request adds to a search: its centroid-score row, query
-// row, probe lists, grouping pairs and per-probe candidate lists.
+// row, probe lists, grouping pairs and per-probe candidate lists (at the length
+// that large batches have; a batch of few pairs takes up to 16 MB for longer ones).
 size_t request_bytes(const soar::IndexData& ix, int k, int t) {
   const size_t list = (size_t)std::max(k <= soar::kTcWideK ? soar::scan_tc_list_len(k, (int64_t)1 << 40) : 32, k) * 8;
   return (size_t)ix.c * 4 + (size_t)(ix.d + 16) * 4 + (size_t)t * (4 + 16 + 4 + 8 + list) + (size_t)k * 12 + 256;

@@ -78,6 +78,7 @@ def _check_search(soar, X, C, A, ix, Q, k, t, tpq=None, sample=40):
     (40, 128, 200, 0),      # more lists than a block has threads, largest k
     (50, 100, 60, 700),     # tied rows overflow the lists: rescans by the block
     (50, 10, 60, 700),
+    (700, 128, 200, 0), (650, 100, 60, 700),            # narrower blocks: batches of several blocks an SM
     (4200, 10, 4, 700),     # rescans by a warp (large batches)
     (4096, 3, 3, 0), (4097, 3, 3, 0),   # both sides of the block / warp line
 ])
@@ -90,6 +91,16 @@ def test_finishing_of_small_and_wide_searches(soar, dtype, nq, k, t, copies):
     tpq = torch.randint(-2, t + 3, (nq,), generator=g).int()     # values outside [0, t] are clamped
     for counts in (None, tpq):
         _check_search(soar, X, C, A, ix, Q, k, t, counts)
+    ix.close()
+
+
+@pytest.mark.parametrize("nq,k", [(20, 20), (20, 128), (620, 40)])
+def test_finishing_of_more_lists_than_block_threads(soar, nq, k):
+    X, C, A, ix = _index(soar, 9000, 24, 800, 7)
+    g = torch.Generator().manual_seed(nq + k)
+    Q = torch.nn.functional.normalize(torch.randn(nq, 24, generator=g), dim=1)
+    _check_search(soar, X, C, A, ix, Q, k, 700)
+    _check_search(soar, X, C, A, ix, Q, k, 700, torch.randint(0, 701, (nq,), generator=g).int())
     ix.close()
 
 
