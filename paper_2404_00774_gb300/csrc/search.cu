@@ -1073,6 +1073,23 @@ void merge_topk(const int64_t* ids, const float* scores, int64_t nq, int m, int 
   SOAR_LAUNCHED();
 }
 
+// Rows per chunk of the flat index: at most 65 536 (a chunk keeps its own top k
+// and bound, so longer ones waste less), at least 512, and as many equal chunks
+// as the same number of waves of (query block, chunk) items takes, so that few
+// queries or few rows still fill the SMs.  Against chunks of 65 536 (us): 10 000
+// queries, 1.18 M rows, k = 10 7 131 / 6 921; 1 024 queries 1 768 / 1 752; 128
+// queries (bf16) 1 573 / 407; one query 846 / 430; 448 queries, 161 000 rows,
+// k = 100 10 644 / 2 640; 16 queries, 12 000 rows, k = 100 1 024 / 360 (479 with
+// at least 1 024 rows a chunk).
+constexpr int64_t kChunkMost = 65536, kChunkLeast = 512;
+int64_t flat_chunk_rows(int64_t n, int64_t nq) {
+  const int64_t blocks = (nq + 127) / 128, sms = num_sms();
+  const int64_t chunks = (n + kChunkMost - 1) / kChunkMost;
+  const int64_t waves = (chunks * blocks + sms - 1) / sms;
+  const int64_t most = std::max(chunks, waves * sms / blocks);
+  return std::min(kChunkMost, std::max(kChunkLeast, ((n + most - 1) / most + 127) / 128 * 128));
+}
+
 void exact_mips(const void* X, soar_dtype xdt, int64_t n, int32_t d, const void* Q, soar_dtype qdt, int64_t nq,
                 int32_t k, int64_t* ids_out, float* scores_out, cudaStream_t s, Scratch& scr) {
   const size_t esz = xdt == SOAR_F32 ? 4 : 2;
@@ -1081,11 +1098,11 @@ void exact_mips(const void* X, soar_dtype xdt, int64_t n, int32_t d, const void*
   // where rows do not start on 16-byte boundaries, a padded copy of them
   void* pad = padded ? scr.get<unsigned char>(esz * (size_t)n * stride) : nullptr;
   const void* rows = padded ? pad : X;
-  // Tensor-core path: the rows become a flat index of 65 536-row chunks that
-  // every query probes, so the partition scan (tensor-core screening with
-  // exact fp32 finishing) returns the exact top k of all rows.
+  // Tensor-core path: the rows become a flat index of equal chunks that every
+  // query probes, so the partition scan (tensor-core screening with exact fp32
+  // finishing) returns the exact top k of all rows.
   {
-    constexpr int64_t kChunkRows = 65536;
+    const int64_t chunk = flat_chunk_rows(n, nq);
     IndexData fx;
     fx.n = n;
     fx.rows = n;
@@ -1094,11 +1111,11 @@ void exact_mips(const void* X, soar_dtype xdt, int64_t n, int32_t d, const void*
     fx.mode = SOAR_SCORE_F32;
     fx.row_stride = stride;
     fx.vectors = const_cast<void*>(rows);
-    fx.c = (int)((n + kChunkRows - 1) / kChunkRows);
+    fx.c = (int)((n + chunk - 1) / chunk);
     const int kstep = xdt == SOAR_F32 ? 8 : 16;
     fx.tc_kp = (d + kstep - 1) / kstep * kstep;
     if (k <= scan_tc_max_k(fx)) {
-      build_flat_tc(fx, X, pad, kChunkRows, s, scr);
+      build_flat_tc(fx, X, pad, chunk, s, scr);
       const int c = fx.c, len = scan_tc_list_len(k, nq * fx.c);
       const size_t qesz = qdt == SOAR_F32 ? 4 : 2;
       // queries in batches whose candidate lists stay within about 1 GB

@@ -305,3 +305,21 @@ def test_brute_force_over_long_chunks(soar, dtype, d, n, k):
     assert torch.allclose(sc.double(), want, rtol=0, atol=1e-5)
     assert torch.allclose(full.gather(1, ids), want, rtol=0, atol=1e-5)
     assert all(ids[q].unique().numel() == k for q in range(0, 141, 20))
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("n,nq,k", [
+    (1, 1, 1), (511, 3, 128), (513, 129, 10),       # one and two chunks of the least size
+    (77_825, 1, 16), (77_825, 128, 33),             # 512 rows a chunk on 152 SMs, and one row past them
+    (65_537, 20_000, 1), (131_072, 2000, 10),       # longest chunks, several waves
+])
+def test_brute_force_chunks_of_every_size(soar, dtype, n, nq, k):
+    g = torch.Generator().manual_seed(n + nq)
+    X = torch.randn(n, 24, generator=g).to(dtype).cuda()
+    Q = torch.randn(nq, 24, generator=g).cuda()
+    ids, sc = soar.soar_exact_mips(X, Q, min(k, n))
+    at = torch.linspace(0, nq - 1, min(nq, 64)).long().cuda()
+    full = Q[at].double() @ X.double().T
+    want = full.topk(min(k, n), 1)[0]
+    assert torch.allclose(sc[at].double(), want, rtol=1e-5, atol=1e-4)
+    assert torch.allclose(full.gather(1, ids[at]), want, rtol=1e-5, atol=1e-4)
