@@ -59,8 +59,7 @@ constexpr int kN = 128;        // centroids of a B tile (MMA N): two operands x 
 constexpr int kEpi = 256;      // epilogue threads (8 warps: 4 lane quarters x 2)
 constexpr int kThr = 96 + kEpi;   // producer, MMA issuer, gate, epilogue
 constexpr int kStagesMax = 8;
-constexpr int kStageBytes = 32768;   // codebook stage: 32 KB keeps bulk copies near full L2 bandwidth
-constexpr int kSteps = kStageBytes / (kN * 32);   // K steps per codebook stage
+constexpr int kStepBytes = kN * 32;   // a K step (8 columns) of a codebook tile
 constexpr int kList = 16;      // candidates handed to the refine per point
 
 // v rounded to the nearest value with 10 explicit mantissa bits (ties away from
@@ -85,7 +84,7 @@ struct AsgParams {
   int astride;
   const float* inv_rn;    // [n][4] 1 / ||x - C[pi(x)]|| (0 for a zero residual)
   float lambda;
-  int stages;
+  int stages, steps;      // codebook stages, K steps in each
   int cap;                // candidates an epilogue thread holds
   int* err;
   int32_t* cand;          // [n][kList] candidate centroids, -1 padded
@@ -110,13 +109,14 @@ __global__ void __launch_bounds__(kThr, 1) assign_tc_kernel(AsgParams<XT> P) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   unsigned char* base = reinterpret_cast<unsigned char*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~uintptr_t(127));
-  const int kp = P.kp, S = P.stages, ksteps = kp / 8;
-  const int nch = (ksteps + kSteps - 1) / kSteps;   // stages per B tile
+  const int kp = P.kp, S = P.stages, ksteps = kp / 8, per = P.steps;
+  const int nch = (ksteps + per - 1) / per;     // stages per B tile
+  const uint32_t stage_bytes = (uint32_t)per * kStepBytes;
   const uint32_t sbo = (uint32_t)kp * 32u;
   const uint32_t a_bytes = (uint32_t)kTM * kp * 4u;
   unsigned char* sA = base;                                                  // OPS operands
   unsigned char* sB = base + (size_t)OPS * a_bytes;
-  float* list_lb = reinterpret_cast<float*>(sB + (size_t)S * kStageBytes);   // [cap][kEpi]
+  float* list_lb = reinterpret_cast<float*>(sB + (size_t)S * stage_bytes);   // [cap][kEpi]
   int* list_id = reinterpret_cast<int*>(list_lb + P.cap * kEpi);             // [cap][kEpi]
   float* nx_s = reinterpret_cast<float*>(list_id + P.cap * kEpi);            // [kEpi] ||x||
   float* mu_s = nx_s + kEpi;                                                // [kTM] U of the second half
@@ -183,10 +183,10 @@ __global__ void __launch_bounds__(kThr, 1) assign_tc_kernel(AsgParams<XT> P) {
           for (int g = 0; g < nch; ++g, ++C) {
             const uint32_t s = C % S, ph = (C / S) & 1;
             if (!tc::bar_wait(empty(s), ph ^ 1, abort_v)) { give_up(); stop = true; break; }
-            const int k0 = g * kSteps, kn = min(kSteps, ksteps - k0);
+            const int k0 = g * per, kn = min(per, ksteps - k0);
             const uint32_t bytes = (uint32_t)kn * kN * 32;
             tc::bar_arrive_expect_tx(full(s), bytes);
-            tc::bulk_copy_g2s(tc::smem_u32(sB) + s * kStageBytes, P.Cc + ((int64_t)ti * ksteps + k0) * kN * 8,
+            tc::bulk_copy_g2s(tc::smem_u32(sB) + s * stage_bytes, P.Cc + ((int64_t)ti * ksteps + k0) * kN * 8,
                               bytes, full(s));
             issued_s = (int)(C + 1);
           }
@@ -285,10 +285,10 @@ __global__ void __launch_bounds__(kThr, 1) assign_tc_kernel(AsgParams<XT> P) {
             if (lane == 0) {
               const uint32_t C = chunk_ctr + i * nch + g, s = C % S;
               tc::fence_after_sync();
-              const int k0 = g * kSteps, kn = min(kSteps, ksteps - k0);
+              const int k0 = g * per, kn = min(per, ksteps - k0);
               for (int jj = 0; jj < kn; ++jj) {
                 const int j = k0 + jj;
-                const uint64_t bd = tc::smem_desc(tc::smem_u32(sB) + s * kStageBytes + jj * kN * 32, 128, 256);
+                const uint64_t bd = tc::smem_desc(tc::smem_u32(sB) + s * stage_bytes + jj * kN * 32, 128, 256);
 #pragma unroll
                 for (int o = 0; o < OPS; ++o)
                   tc::mma_tf32(tmem + b * kW + o * kN,
@@ -646,8 +646,8 @@ __global__ void refine_list(const XT* __restrict__ X, int d, const float* __rest
   }
 }
 
-size_t smem_for(int kp, int ops, int s, int cap) {
-  return 128 + (size_t)ops * kTM * kp * 4 + (size_t)s * kStageBytes + (size_t)cap * kEpi * 8 + (size_t)kEpi * 4 +
+size_t smem_for(int kp, int ops, int s, int steps, int cap) {
+  return 128 + (size_t)ops * kTM * kp * 4 + (size_t)s * steps * kStepBytes + (size_t)cap * kEpi * 8 + (size_t)kEpi * 4 +
          (size_t)6 * kTM * 4 + (size_t)(2 * s + 4) * 8;
 }
 
@@ -655,15 +655,19 @@ size_t smem_for(int kp, int ops, int s, int cap) {
 int kp_for(int d) { return (d + 2 + 7) / 8 * 8; }
 
 // A operands, codebook stages and list length that fit: two operands before one
-// (half the codebook traffic), long lists before deep rings.
+// (half the codebook traffic), lists of 16 before stages of 32 KB (fewer, larger
+// copies), those before deep rings.  Lists of 8 overflow where a point lies in
+// the band of more centroids, and it is then scored against all of them.
 struct Shape {
-  int ops = 0, stages = 0, cap = 0;
+  int ops = 0, stages = 0, steps = 0, cap = 0;
 };
 Shape shape_for(int kp, int ndir) {
   for (int ops = 2; ops >= (ndir ? 2 : 1); --ops)
     for (int cap : {16, 8})
-      for (int s = kStagesMax; s >= 2; --s)
-        if (smem_for(kp, ops, s, cap) <= 227 * 1024 - 256) return Shape{ops, s, cap};   // room for the static shared variables
+      for (int steps : {8, 4})
+        for (int s = kStagesMax; s >= 2; --s)
+          if (smem_for(kp, ops, s, steps, cap) <= 227 * 1024 - 256)   // room for the static shared variables
+            return Shape{ops, s, steps, cap};
   return Shape{};
 }
 
@@ -696,8 +700,8 @@ void assign_tc_pass(const XT* X, int64_t n, int d, const float* C, int c, int nd
   const int vec = std::is_same<XT, float>::value && d % 4 == 0 && reinterpret_cast<uintptr_t>(X) % 16 == 0 &&
                   reinterpret_cast<uintptr_t>(C) % 16 == 0;
   AsgParams<XT> prm{X, n, d, kp, Cc, tmax, C, c, ctiles, assign, astride, inv_rn, lambda, sh.stages,
-                    sh.cap, device_error_word(), cand, ovf, queue, qcount, vec};
-  const size_t smem = smem_for(kp, sh.ops, sh.stages, sh.cap);
+                    sh.steps, sh.cap, device_error_word(), cand, ovf, queue, qcount, vec};
+  const size_t smem = smem_for(kp, sh.ops, sh.stages, sh.steps, sh.cap);
   auto kern = ndir == 0 ? (sh.ops == 2 ? assign_tc_kernel<0, 2, XT> : assign_tc_kernel<0, 1, XT>)
                         : assign_tc_kernel<1, 2, XT>;
   SOAR_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
