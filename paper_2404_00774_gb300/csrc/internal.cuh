@@ -124,6 +124,8 @@ void quantize_fp8(const void* V, soar_dtype dt, int64_t m, int32_t d, uint8_t* c
 bool select_tc_fits(int kp);
 // Fills out [sel_tiles][2][64 * sel_kp] from ix.centroids.
 void pack_select_codebook(const IndexData& ix, float* out, cudaStream_t s);
+// Candidate-list length of a brute-force scan over chunks of `chunk` rows.
+int scan_tc_flat_list_len(int k, int64_t pairs, int64_t chunk);
 // Whether select_tc takes these queries (packed codebook present, t <= 32,
 // rows 16-byte aligned).
 bool select_tc_usable(const IndexData& ix, const float* Qf, int qstride, int t);

@@ -69,6 +69,7 @@ constexpr int kWideList = kTcWideList;   // largest global candidate list of the
 // against 25).  kCand for k <= 32, else 2k rounded up to a warp multiple
 // (room to append between compactions).
 constexpr int kGmList = 128, kGmListMost = 1024;
+int heap_list_len(int k) { return std::min(kWideList, (2 * k + 31) / 32 * 32); }
 int list_len_for(int k, int64_t pairs) {
   if (k <= 16) {
     int len = kGmList;
@@ -76,7 +77,7 @@ int list_len_for(int k, int64_t pairs) {
     return len;
   }
   if (k <= kCand) return kCand;
-  return std::min(kWideList, (2 * k + 31) / 32 * 32);
+  return heap_list_len(k);
 }
 
 // Shared memory behind the tile scores: register mode keeps kCand candidates
@@ -586,10 +587,10 @@ int pick_stages(int kp, int k, int es) {
 }
 
 template <typename ET>
-void launch_scan_tc(int k, int grid, size_t smem, cudaStream_t s, const TcParams& prm) {
+void launch_scan_tc(int k, int kc, int grid, size_t smem, cudaStream_t s, const TcParams& prm) {
   auto kern = k == 10   ? scan_tc_kernel<ET, 10, true>
               : k <= 16 ? scan_tc_kernel<ET, 16, false>
-              : k <= kCand ? scan_tc_kernel<ET, 32, false> : scan_tc_kernel<ET, 0, false>;
+              : kc <= kCand ? scan_tc_kernel<ET, 32, false> : scan_tc_kernel<ET, 0, false>;   // (heap mode: longer lists)
   SOAR_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   kern<<<grid, kThreads, smem, s>>>(prm);
   SOAR_LAUNCHED();
@@ -610,6 +611,20 @@ int scan_tc_max_k(const IndexData& ix) {
 
 int scan_tc_list_len(int k, int64_t pairs) { return list_len_for(k, pairs); }
 
+// Brute force with 16 < k <= 32: heap mode where the register mode's 32 entries
+// are too few.  A chunk holds a fair share of the final k and of the rows within
+// the band of the k-th best, and a list that overflows costs a rescan of the whole
+// chunk (us, register / heap mode: 10 000 queries, chunks of 62 000 rows, k = 17
+// 19 286 / 9 452, k = 32 388 069 / 12 103; 448 queries, chunks of 4 200, k = 17
+// 496 / 650, k = 20 731 / 719, k = 32 5 164 / 1 320; 176 queries, chunks of 512,
+// k = 28 353 / 476, k = 32 837 / 533).  Searches keep the register mode: in tight
+// clusters more rows than a heap's list holds pass the bound (k = 20, 300 queries
+// probing 100 partitions of 800 rows: 2 166 / 10 467).
+int scan_tc_flat_list_len(int k, int64_t pairs, int64_t chunk) {
+  if (k > 16 && k <= kCand && (chunk >= 8192 || k > 28 || (k >= 20 && chunk >= 1024))) return heap_list_len(k);
+  return list_len_for(k, pairs);
+}
+
 void scan_tc_search(const IndexData& ix, const IvfWork& work, int max_items, const float* Qf, const float* qnorm,
                     const int32_t* top, const int32_t* inv, const int32_t* tpq, int64_t nq, int t, int k,
                     Cand* lists, int kc, int* counter, int2* hdr, unsigned* gbound, int* err, int64_t* ids_out,
@@ -627,9 +642,9 @@ void scan_tc_search(const IndexData& ix, const IvfWork& work, int max_items, con
     scan_gm_launch(ix, work, grid, Qf, qnorm, nq, k, kc, prm.dscale, prm.wait_limit, counter, err, gbound, lists, hdr, s,
                    scr);
   else if (es == 4)
-    launch_scan_tc<float>(k, grid, smem, s, prm);
+    launch_scan_tc<float>(k, kc, grid, smem, s, prm);
   else
-    launch_scan_tc<__nv_bfloat16>(k, grid, smem, s, prm);
+    launch_scan_tc<__nv_bfloat16>(k, kc, grid, smem, s, prm);
   stage_mark(s, "scan", false);
   stage_mark(s, "rescore", true);
   finish_tc_queries(ix, lists, hdr, gbound, inv, nq, t, tpq, Qf, top, k, kc, ids_out, scores_out, s);

@@ -1116,7 +1116,7 @@ void exact_mips(const void* X, soar_dtype xdt, int64_t n, int32_t d, const void*
     fx.tc_kp = (d + kstep - 1) / kstep * kstep;
     if (k <= scan_tc_max_k(fx)) {
       build_flat_tc(fx, X, pad, chunk, s, scr);
-      const int c = fx.c, len = scan_tc_list_len(k, nq * fx.c);
+      const int c = fx.c, len = scan_tc_flat_list_len(k, nq * fx.c, chunk);
       const size_t qesz = qdt == SOAR_F32 ? 4 : 2;
       // queries in batches whose candidate lists stay within about 1 GB
       const int64_t nb = std::max<int64_t>(128, (int64_t(1) << 30) / ((int64_t)c * len * (int64_t)sizeof(Cand)));

@@ -231,10 +231,10 @@ def test_shortlists_at_their_limits(soar, mode, d, c, t, R, copies):
 
 
 @pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
-@pytest.mark.parametrize("d,c,n", [(5, 2, 1), (100, 129, 255), (100, 128, 257), (126, 300, 300), (134, 257, 700),
+@pytest.mark.parametrize("d,c,n", [(5, 2, 1), (100, 129, 255), (100, 128, 257), (126, 300, 300), (134, 257, 700), (150, 257, 300), (158, 257, 300),
                                    (142, 257, 300), (278, 130, 200), (64, 3000, 513)])
 def test_assignment_shapes(soar, dtype, d, c, n):
-    """Ragged point blocks and codebook tiles; rows too wide for long lists (126..134) and for two operands (142..278)."""
+    """Ragged point blocks and codebook tiles; rows too wide for long stages (126..150) or lists (158) and for two operands (142..278)."""
     g = torch.Generator().manual_seed(d + c)
     X = torch.randn(n, d, generator=g).to(dtype)
     C = torch.randn(c, d, generator=g)
@@ -312,6 +312,7 @@ def test_brute_force_over_long_chunks(soar, dtype, d, n, k):
     (1, 1, 1), (511, 3, 128), (513, 129, 10),       # one and two chunks of the least size
     (77_825, 1, 16), (77_825, 128, 33),             # 512 rows a chunk on 152 SMs, and one row past them
     (65_537, 20_000, 1), (131_072, 2000, 10),       # longest chunks, several waves
+    (131_072, 2000, 17), (131_072, 5000, 32), (20_000, 200, 20), (20_000, 200, 17), (3000, 50, 29), (700, 20, 32),
 ])
 def test_brute_force_chunks_of_every_size(soar, dtype, n, nq, k):
     g = torch.Generator().manual_seed(n + nq)
