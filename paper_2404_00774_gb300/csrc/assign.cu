@@ -335,32 +335,53 @@ __global__ void gather_rows_f32(const XT* __restrict__ X, int d, const int32_t* 
 //
 // A block per cluster, thread (column, partial sum): the serial chains run side
 // by side, each with sixteen rows' loads in flight.  This GPU's fp64 rate is a
-// sixtieth of its fp32 rate, so sixteen rows are first added in fp32 with their
-// exact rounding errors carried along (Knuth's two-sum): the pair (sum, error)
-// holds their sum to about 2^-48, below the rounding of the fp64 chain it then
-// joins with two additions instead of sixteen.  A batch whose fp32 sum is not
-// finite is added in fp64 directly.  Bound: HBM, the member rows gathered once
-// (1.18 M x 100 fp32 in 2 000 clusters: 849 us with one thread for a column's
-// four fp64 chains, 666 with a thread per chain, now 134).
-constexpr int kUpdCols = 128, kUpdChains = 4, kUpdAhead = 16;
+// sixtieth of its fp32 rate, so 64 rows are first added in fp32 with their
+// rounding errors carried along: Knuth's two-sum gives each addition's error
+// exactly, a second one adds that to the errors so far, and what that addition
+// rounds off goes to a third value.  With M the largest partial sum, the errors
+// stay below 2^-18 M and the third value below 2^-36 M; its own rounding, at
+// most 2^-54 M, is all that is lost (2^-59 M over sixteen rows), and the 64 rows
+// join the fp64 chain with one rounding of 2^-53 of the chain in place of 64.  Sixteen
+// rows that would take the fp32 sum out of range are added in fp64 directly.
+// Bound: HBM, the member rows gathered once (1.18 M x 100 fp32 in 2 000
+// clusters: 849 us with one thread for a column's four fp64 chains, 666 with a
+// thread per chain, now 165; joining after sixteen rows took 208).
+constexpr int kUpdCols = 128, kUpdChains = 4, kUpdAhead = 16, kUpdJoin = 4;
 
-// sum += v[0] + ... + v[kUpdAhead - 1]
-__device__ __forceinline__ void add_batch(const float (&v)[kUpdAhead], double& sum) {
-  float s = v[0], err = 0.f;
-#pragma unroll
-  for (int u = 1; u < kUpdAhead; ++u) {
-    const float t = __fadd_rn(s, v[u]), z = __fsub_rn(t, s);
-    err = __fadd_rn(err, __fadd_rn(__fsub_rn(s, __fsub_rn(t, z)), __fsub_rn(v[u], z)));
-    s = t;
-  }
-  if (fabsf(s) <= 1e37f && fabsf(err) <= 1e37f) {
-    sum += (double)s;
-    sum += (double)err;
-  } else {
-#pragma unroll
-    for (int u = 0; u < kUpdAhead; ++u) sum += (double)v[u];
-  }
+// s = s + v rounded; returns what the rounding left out (exact unless it overflows)
+__device__ __forceinline__ float two_sum(float& s, float v) {
+  const float t = __fadd_rn(s, v), z = __fsub_rn(t, s);
+  const float left = __fadd_rn(__fsub_rn(s, __fsub_rn(t, z)), __fsub_rn(v, z));
+  s = t;
+  return left;
 }
+
+// A partial sum: sum + s + err + rest, the last three over the latest rows.
+struct Chain {
+  double sum = 0;
+  float s = 0.f, err = 0.f, rest = 0.f;
+  int batches = 0;
+  __device__ void join() {
+    sum += (double)s + ((double)err + (double)rest);
+    s = err = rest = 0.f;
+    batches = 0;
+  }
+  __device__ void add(const float (&v)[kUpdAhead]) {
+    float ns = s, ne = err, nr = rest;
+#pragma unroll
+    for (int u = 0; u < kUpdAhead; ++u) nr = __fadd_rn(nr, two_sum(ne, two_sum(ns, v[u])));
+    if (fabsf(ns) <= 1e37f && fabsf(ne) <= 1e37f && fabsf(nr) <= 1e37f) {
+      s = ns;
+      err = ne;
+      rest = nr;
+      if (++batches == kUpdJoin) join();
+    } else {
+      join();
+#pragma unroll
+      for (int u = 0; u < kUpdAhead; ++u) sum += (double)v[u];
+    }
+  }
+};
 
 template <typename XT>
 __global__ void __launch_bounds__(kUpdCols * kUpdChains) kmeans_update(const XT* __restrict__ X, int d,
@@ -374,22 +395,23 @@ __global__ void __launch_bounds__(kUpdCols * kUpdChains) kmeans_update(const XT*
   if (cnt == 0) return;
   for (int k0 = 0; k0 < d; k0 += kUpdCols) {
     const int k = k0 + col;
-    double sum = 0;
     if (k < d) {
+      Chain acc;
       int64_t i = b + chain;
       float v[kUpdAhead];
       for (; i + kUpdChains * (kUpdAhead - 1) < e; i += kUpdChains * kUpdAhead) {
 #pragma unroll
         for (int u = 0; u < kUpdAhead; ++u) v[u] = load_elem(X, (int64_t)members[i + kUpdChains * u] * d + k);
-        add_batch(v, sum);
+        acc.add(v);
       }
 #pragma unroll
       for (int u = 0; u < kUpdAhead; ++u) {
         const int64_t r = i + kUpdChains * u;
         v[u] = r < e ? load_elem(X, (int64_t)members[r] * d + k) : 0.f;
       }
-      add_batch(v, sum);
-      sums[chain][col] = sum;
+      acc.add(v);
+      acc.join();
+      sums[chain][col] = acc.sum;
     }
     __syncthreads();
     if (chain == 0 && k < d)
