@@ -116,7 +116,7 @@ __global__ void __launch_bounds__(kThreads) screen_kernel(
         Xs[kk][m] = xv;
 #pragma unroll
         for (int r = 0; r < NDIR; ++r) {
-          float cv = (p < n && k < d) ? C[(int64_t)prior_s[m][r] * d + k] : 0.f;
+          float cv = (p < n && k < d) ? assigned_row(C, prior_s[m][r], d)[k] : 0.f;
           Rs[r][kk][m] = (xv - cv) * inv_s[m][r];
         }
         int cc = c0 + m;
@@ -191,7 +191,7 @@ __global__ void residual_kernel(const XT* __restrict__ X, int64_t n, int d, cons
   int64_t p = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   int lane = threadIdx.x & 31;
   if (p >= n) return;
-  const float* cr = C + (int64_t)assign[p * astride + dir] * d;
+  const float* cr = assigned_row(C, assign[p * astride + dir], d);
   float ss = 0.f, xd = 0.f;
   for (int k = lane; k < d; k += 32) {
     float xv = load_elem(X, p * d + k);
@@ -222,7 +222,7 @@ __global__ void refine_kernel(const XT* __restrict__ X, int64_t n, int d, const 
   float loss[2] = {0.f, 0.f};
   // squared norms of the earlier residuals
   for (int r = 0; r < col; ++r) {
-    const float* cr = C + (int64_t)assign[p * astride + r] * d;
+    const float* cr = assigned_row(C, assign[p * astride + r], d);
     float s = 0.f;
     for (int k = lane; k < d; k += 32) {
       float v = load_elem(X, p * d + k) - cr[k];
@@ -243,7 +243,7 @@ __global__ void refine_kernel(const XT* __restrict__ X, int64_t n, int d, const 
     float pen = 0.f;
     for (int r = 0; r < col; ++r) {
       if (!(rn2[r] > 0.f)) continue;
-      const float* cr = C + (int64_t)assign[p * astride + r] * d;
+      const float* cr = assigned_row(C, assign[p * astride + r], d);
       float pr = 0.f;
       for (int k = lane; k < d; k += 32) {
         float xv = load_elem(X, p * d + k);

@@ -213,7 +213,7 @@ __global__ void __launch_bounds__(kThr, 1) assign_tc_kernel(AsgParams<XT> P) {
         if (resid && active) {
           prior = P.assign[p * P.astride];
           inv = P.inv_rn[p * 4];
-          cr = P.C + (int64_t)prior * P.d;
+          cr = assigned_row(P.C, prior, P.d);
         }
         float ss = 0.f, xd = 0.f;
         const bool vec = std::is_same<XT, float>::value && P.vec;
@@ -585,7 +585,7 @@ __global__ void refine_list(const XT* __restrict__ X, int d, const float* __rest
     const int64_t p = queue[qi];
     const XT* x = X + p * d;
     const int prior = col > 0 ? assign[p * astride] : -1;
-    const float* cr = C + (int64_t)(col > 0 ? prior : 0) * d;
+    const float* cr = assigned_row(C, prior, d);
     float rn2 = 0.f;
     if (col > 0) {
       float s = 0.f;

@@ -30,6 +30,12 @@ int bits_for(int64_t num_keys);
 
 // ----------------------------------------------------------- assign.cu
 
+// The centroid a point is assigned to.  A point none of whose losses is a number
+// is assigned to -1; its reads go to row 0 (the residual is NaN either way).
+__device__ __forceinline__ const float* assigned_row(const float* C, int32_t a, int d) {
+  return C + (int64_t)(a < 0 ? 0 : a) * d;
+}
+
 // pi(x) for every row (nearest centroid, lower index on ties), optionally the
 // SOAR spills, written to assign[n][1+spills].
 void assign_points(const void* X, soar_dtype dt, int64_t n, int32_t d, const float* C, int32_t c,

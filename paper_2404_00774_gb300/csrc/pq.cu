@@ -39,7 +39,7 @@ __global__ void pq_residuals_kernel(const T* __restrict__ X, int64_t n, int d, c
   if (e >= n * d) return;
   const int64_t i = e / d;
   const int k = (int)(e - i * d);
-  R[e] = load_elem(X, e) - C[(int64_t)part[i] * d + k];
+  R[e] = load_elem(X, e) - assigned_row(C, part[i], d)[k];
 }
 
 // B[s][j] = R[init[j]][2s .. 2s+1].
