@@ -88,9 +88,9 @@ struct AsgParams {
   int cap;                // candidates an epilogue thread holds
   int* err;
   int32_t* cand;          // [n][kList] candidate centroids, -1 padded
-  int32_t* ovf;           // [n] 1 when the candidates are not conclusive
-  int32_t* queue;         // [n] points left to the refine
-  int* qcount;
+  int32_t* queue;         // [n] points left to the refine: with candidates from the front, flagged ones from the back
+  uint64_t* best;         // [n] the flagged points' best keys so far (set to none here)
+  int* qcount;            // [2] how many of each
   int vec;                // fp32 rows, d % 4 == 0, X and C 16-byte aligned: 16-byte copies
 };
 
@@ -474,21 +474,29 @@ __global__ void __launch_bounds__(kThr, 1) assign_tc_kernel(AsgParams<XT> P) {
               ++ncand;
             }
           }
-          const bool over = ev <= U || ncand > kList;
+          // (no candidate at all: no finite loss)
+          const bool over = ev <= U || ncand > kList || ncand == 0;
           if (ncand == 1 && !over) {
             P.assign[p * P.astride + NDIR] = only;     // the bounds leave one centroid: decided
-          } else {
+          } else if (!over) {
             for (int q = ncand; q < kList; ++q) cand[q] = -1;
-            P.ovf[p] = over ? 1 : 0;
           }
-          // queue the undecided points for the direct-form refine (one atomic per warp)
+          // queue the undecided points for the direct-form refine (an atomic per warp and queue)
           const unsigned am = __activemask();
-          const unsigned need = __ballot_sync(am, ncand != 1 || over);
+          const unsigned listed = __ballot_sync(am, ncand != 1 && !over), flagged = __ballot_sync(am, over);
           const int leader = __ffs(am) - 1;
-          int qbase = 0;
-          if (lane == leader && need) qbase = atomicAdd(P.qcount, __popc(need));
-          qbase = __shfl_sync(am, qbase, leader);
-          if (need & (1u << lane)) P.queue[qbase + __popc(need & ((1u << lane) - 1))] = (int32_t)p;
+          int lbase = 0, fbase = 0;
+          if (lane == leader && listed) lbase = atomicAdd(P.qcount, __popc(listed));
+          if (lane == leader && flagged) fbase = atomicAdd(P.qcount + 1, __popc(flagged));
+          lbase = __shfl_sync(am, lbase, leader);
+          fbase = __shfl_sync(am, fbase, leader);
+          const unsigned before = (1u << lane) - 1;
+          if (listed & (1u << lane)) P.queue[lbase + __popc(listed & before)] = (int32_t)p;
+          if (flagged & (1u << lane)) {
+            const int f = fbase + __popc(flagged & before);
+            P.queue[P.n - 1 - f] = (int32_t)p;
+            P.best[f] = ~0ull;
+          }
         }
       }
       tile_ctr += P.ctiles;
@@ -568,73 +576,165 @@ __global__ void tile_max_norms(const float* __restrict__ n1, int c, int ctiles, 
   if (lane == 0) tmax[w] = v;
 }
 
-// Direct-form decision among the candidates of each queued point (warp per
-// point, persistent over the queue): two lanes per listed candidate, or,
-// for a point the screen flagged, the lanes split every centroid not yet
-// assigned to it.  Lower index on equal losses.
+// ||r||^2, r = x - c_prior, by a warp.
 template <typename XT>
-__global__ void refine_list(const XT* __restrict__ X, int d, const float* __restrict__ C, int c,
-                            int32_t* __restrict__ assign, int astride, int col, float lambda,
-                            const int32_t* __restrict__ cand, const int32_t* __restrict__ ovf,
-                            const int32_t* __restrict__ queue, const int* __restrict__ qcount) {
-  constexpr unsigned kFull = 0xffffffffu;
-  const int lane = threadIdx.x & 31;
-  const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  const int total = *qcount;
-  for (int64_t qi = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; qi < total; qi += nwarps) {
-    const int64_t p = queue[qi];
-    const XT* x = X + p * d;
-    const int prior = col > 0 ? assign[p * astride] : -1;
-    const float* cr = assigned_row(C, prior, d);
-    float rn2 = 0.f;
-    if (col > 0) {
-      float s = 0.f;
-      for (int k = lane; k < d; k += 32) {
-        const float v = load_elem(x, k) - cr[k];
-        s = fmaf(v, v, s);
-      }
-      rn2 = warp_sum(s);
+__device__ __forceinline__ float residual_norm2(const XT* x, const float* cr, int d, int lane) {
+  float s = 0.f;
+  for (int k = lane; k < d; k += 32) {
+    const float v = load_elem(x, k) - cr[k];
+    s = fmaf(v, v, s);
+  }
+  return warp_sum(s);
+}
+
+// Direct-form losses of the flagged points (the last qcount[1] of the queue)
+// against every centroid not yet assigned to them, as keys (loss, centroid)
+// that order like losses, lower index first, the least kept in best[f].  A
+// block takes 64 points and a share of the codebook in tiles of 64 centroids, 4 x
+// 4 pairs a thread, staged 16 columns at a time; every sum runs over k in
+// ascending order in one fp32 accumulator, the order of the listed decision's
+// two halves apart.  Few flagged points split the codebook over more blocks.
+// Bound: the FMA pipe, two (primary) or three operations a pair and column.  In
+// clusters tighter than the screening band every point is flagged, and a warp
+// per point with a centroid per lane, whose loads touch 32 rows at once, took
+// 72 ms for 200 000 x 150 against 2 000 (the pass now 5.8; the spill 77, now 9.3)
+// and 454 at 320 columns (13.4); the general kernels of assign.cu take 13.5 for
+// that spill and 14.9 at 320 columns.
+constexpr int kFt = 64, kFk = 16, kFlagThreads = 256;
+template <int NDIR, typename XT>
+__global__ void __launch_bounds__(kFlagThreads) refine_flagged(const XT* __restrict__ X, int64_t n, int d,
+                                                               const float* __restrict__ C, int c,
+                                                               const int32_t* __restrict__ assign, int astride,
+                                                               float lambda, const int32_t* __restrict__ queue,
+                                                               const int* __restrict__ qcount,
+                                                               uint64_t* __restrict__ best) {
+  __shared__ __align__(16) float xs[kFk][kFt + 4], cs[kFk][kFt + 4], rs[NDIR > 0 ? kFk : 1][kFt + 4];
+  __shared__ int32_t pt_s[kFt], prior_s[kFt];
+  __shared__ float rn2_s[kFt];
+  const int total = qcount[1], tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  const int pblocks = (total + kFt - 1) / kFt, ctiles = (c + kFt - 1) / kFt;
+  if (pblocks == 0) return;
+  const int slices = max(1, min(ctiles, (int)gridDim.x / pblocks)), per = (ctiles + slices - 1) / slices;
+  const int tx = tid % 16, ty = tid / 16;        // centroids 4 tx .., points 4 ty ..
+  for (int64_t item = blockIdx.x; item < (int64_t)pblocks * slices; item += gridDim.x) {
+    const int f0 = (int)(item % pblocks) * kFt, t0 = (int)(item / pblocks) * per, t1 = min(ctiles, t0 + per);
+    __syncthreads();
+    if (tid < kFt) {
+      const int32_t p = f0 + tid < total ? queue[n - 1 - f0 - tid] : -1;
+      pt_s[tid] = p;
+      prior_s[tid] = NDIR > 0 && p >= 0 ? assign[(int64_t)p * astride] : -1;
     }
-    float best = INFINITY;
-    int bi = -1;
-    const bool listed = !ovf[p] && cand[p * kList] >= 0;
-    if (listed) {
-      static_assert(kList * 2 == 32, "two lanes per candidate");
-      const int g = lane >> 1, part = lane & 1;
-      const int cq = cand[p * kList + g];
-      float dist = 0.f, pr = 0.f;
-      if (cq >= 0) {
-        const float* cv = C + (int64_t)cq * d;
-        for (int k = part; k < d; k += 2) {
-          const float xv = load_elem(x, k);
-          const float v = xv - cv[k];
-          dist = fmaf(v, v, dist);
-          if (col > 0) pr = fmaf(v, xv - cr[k], pr);
+    __syncthreads();
+    if constexpr (NDIR > 0)
+      for (int i = w; i < kFt; i += kFlagThreads / 32) {
+        const int64_t p = pt_s[i];
+        const float r = p >= 0 ? residual_norm2(X + p * d, assigned_row(C, prior_s[i], d), d, lane) : 0.f;
+        if (lane == 0) rn2_s[i] = r;
+      }
+    uint64_t key[4] = {~0ull, ~0ull, ~0ull, ~0ull};
+    for (int t = t0; t < t1; ++t) {
+      float dist[4][4], pr[4][4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) dist[i][j] = pr[i][j] = 0.f;
+      for (int k0 = 0; k0 < d; k0 += kFk) {
+        __syncthreads();
+#pragma unroll
+        for (int i = tid; i < kFt * kFk; i += kFlagThreads) {
+          const int r = i / kFk, kk = i % kFk, k = k0 + kk;
+          const int64_t p = pt_s[r];
+          const int cq = t * kFt + r;
+          const float xv = p >= 0 && k < d ? load_elem(X, p * d + k) : 0.f;
+          xs[kk][r] = xv;
+          cs[kk][r] = cq < c && k < d ? C[(int64_t)cq * d + k] : 0.f;
+          if constexpr (NDIR > 0) rs[kk][r] = p >= 0 && k < d ? xv - assigned_row(C, prior_s[r], d)[k] : 0.f;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int kk = 0; kk < kFk; ++kk) {           // (zeros past d add nothing)
+          const float4 xq = *reinterpret_cast<const float4*>(&xs[kk][4 * ty]);
+          const float4 cq = *reinterpret_cast<const float4*>(&cs[kk][4 * tx]);
+          const float xv[4] = {xq.x, xq.y, xq.z, xq.w}, cv[4] = {cq.x, cq.y, cq.z, cq.w};
+          float rv[4] = {0.f, 0.f, 0.f, 0.f};
+          if constexpr (NDIR > 0) {
+            const float4 rq = *reinterpret_cast<const float4*>(&rs[kk][4 * ty]);
+            rv[0] = rq.x; rv[1] = rq.y; rv[2] = rq.z; rv[3] = rq.w;
+          }
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              const float v = xv[i] - cv[j];
+              dist[i][j] = fmaf(v, v, dist[i][j]);
+              if constexpr (NDIR > 0) pr[i][j] = fmaf(v, rv[i], pr[i][j]);
+            }
         }
       }
 #pragma unroll
-      for (int o = 1; o < 2; o <<= 1) {
-        dist += __shfl_xor_sync(kFull, dist, o);
-        pr += __shfl_xor_sync(kFull, pr, o);
-      }
-      if (cq >= 0) {
-        best = (col > 0 && rn2 > 0.f) ? fmaf(lambda, pr * pr / rn2, dist) : dist;
-        bi = cq;
-      }
-    } else {
-      for (int cq = lane; cq < c; cq += 32) {
-        if (cq == prior) continue;
-        const float* cv = C + (int64_t)cq * d;
-        float dist = 0.f, pr = 0.f;
-        for (int k = 0; k < d; ++k) {
-          const float xv = load_elem(x, k);
-          const float v = xv - cv[k];
-          dist = fmaf(v, v, dist);
-          if (col > 0) pr = fmaf(v, xv - cr[k], pr);
+      for (int i = 0; i < 4; ++i) {
+        const int prior = prior_s[4 * ty + i];
+        const float rn2 = NDIR > 0 ? rn2_s[4 * ty + i] : 0.f;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const int cq = t * kFt + 4 * tx + j;
+          const float l = NDIR > 0 && rn2 > 0.f ? fmaf(lambda, pr[i][j] * pr[i][j] / rn2, dist[i][j]) : dist[i][j];
+          if (cq < c && cq != prior && l == l)       // losses are not negative: ordered like their bits
+            key[i] = min(key[i], ((uint64_t)__float_as_uint(l) << 32) | (uint32_t)cq);
         }
-        const float l = (col > 0 && rn2 > 0.f) ? fmaf(lambda, pr * pr / rn2, dist) : dist;
-        if (l < best || (l == best && (unsigned)cq < (unsigned)bi)) { best = l; bi = cq; }
       }
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+#pragma unroll
+      for (int o = 8; o > 0; o >>= 1) key[i] = min(key[i], (uint64_t)__shfl_xor_sync(0xffffffffu, key[i], o));
+      const int f = f0 + 4 * ty + i;
+      if (tx == 0 && f < total)
+        atomicMin(reinterpret_cast<unsigned long long*>(best + f), (unsigned long long)key[i]);
+    }
+  }
+}
+
+// Direct-form decision among the candidates of each listed point (warp per
+// point, persistent over the queue, two lanes per candidate), lower index on
+// equal losses; the flagged points' best centroids (-1 where no loss is a
+// number) are written out.
+template <typename XT>
+__global__ void refine_list(const XT* __restrict__ X, int64_t n, int d, const float* __restrict__ C,
+                            int32_t* __restrict__ assign, int astride, int col, float lambda,
+                            const int32_t* __restrict__ cand, const int32_t* __restrict__ queue,
+                            const uint64_t* __restrict__ best_flagged, const int* __restrict__ qcount) {
+  constexpr unsigned kFull = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  const int64_t nthreads = (int64_t)gridDim.x * blockDim.x, thread = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int total = qcount[0], flagged = qcount[1];
+  for (int64_t f = thread; f < flagged; f += nthreads)
+    assign[(int64_t)queue[n - 1 - f] * astride + col] = (int32_t)(uint32_t)best_flagged[f];
+  for (int64_t qi = thread >> 5; qi < total; qi += nthreads >> 5) {
+    const int64_t p = queue[qi];
+    const XT* x = X + p * d;
+    const float* cr = assigned_row(C, col > 0 ? assign[p * astride] : 0, d);
+    const float rn2 = col > 0 ? residual_norm2(x, cr, d, lane) : 0.f;
+    static_assert(kList * 2 == 32, "two lanes per candidate");
+    const int g = lane >> 1, part = lane & 1;
+    const int cq = cand[p * kList + g];
+    float dist = 0.f, pr = 0.f;
+    if (cq >= 0) {
+      const float* cv = C + (int64_t)cq * d;
+      for (int k = part; k < d; k += 2) {
+        const float xv = load_elem(x, k);
+        const float v = xv - cv[k];
+        dist = fmaf(v, v, dist);
+        if (col > 0) pr = fmaf(v, xv - cr[k], pr);
+      }
+    }
+    dist += __shfl_xor_sync(kFull, dist, 1);
+    pr += __shfl_xor_sync(kFull, pr, 1);
+    float best = INFINITY;
+    int bi = -1;
+    if (cq >= 0) {
+      best = (col > 0 && rn2 > 0.f) ? fmaf(lambda, pr * pr / rn2, dist) : dist;
+      bi = cq;
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -656,8 +756,12 @@ int kp_for(int d) { return (d + 2 + 7) / 8 * 8; }
 
 // A operands, codebook stages and list length that fit: two operands before one
 // (half the codebook traffic), lists of 16 before stages of 32 KB (fewer, larger
-// copies), those before deep rings.  Lists of 8 overflow where a point lies in
-// the band of more centroids, and it is then scored against all of them.
+// copies), those before deep rings.  A point in the band of more centroids than
+// its list holds is scored against all of them.  Where two operands leave room
+// for lists of 8 only (151 to 166 columns), they still pay: 200 000 x 152 against
+// 2 000 centroids 0.49 ms, with one operand and lists of 16 0.55; against 20 000,
+// forty to a cluster, 3.30 and 3.49; twenty tight ones to a cluster, every list
+// full either way, 7.8 and 5.7.
 struct Shape {
   int ops = 0, stages = 0, steps = 0, cap = 0;
 };
@@ -693,14 +797,14 @@ void assign_tc_pass(const XT* X, int64_t n, int d, const float* C, int c, int nd
   tile_max_norms<<<ceil_div((int64_t)ctiles * 32, 256), 256, 0, s>>>(n1, c, ctiles, tmax);
   SOAR_LAUNCHED();
   int32_t* cand = scr.get<int32_t>((size_t)n * kList);
-  int32_t* ovf = scr.get<int32_t>(n);
   int32_t* queue = scr.get<int32_t>(n);
-  int* qcount = scr.get<int>(1);             // queued points
-  SOAR_CUDA(cudaMemsetAsync(qcount, 0, sizeof(int), s));
+  uint64_t* best = scr.get<uint64_t>(n);
+  int* qcount = scr.get<int>(2);             // queued points
+  SOAR_CUDA(cudaMemsetAsync(qcount, 0, 2 * sizeof(int), s));
   const int vec = std::is_same<XT, float>::value && d % 4 == 0 && reinterpret_cast<uintptr_t>(X) % 16 == 0 &&
                   reinterpret_cast<uintptr_t>(C) % 16 == 0;
   AsgParams<XT> prm{X, n, d, kp, Cc, tmax, C, c, ctiles, assign, astride, inv_rn, lambda, sh.stages,
-                    sh.steps, sh.cap, device_error_word(), cand, ovf, queue, qcount, vec};
+                    sh.steps, sh.cap, device_error_word(), cand, queue, best, qcount, vec};
   const size_t smem = smem_for(kp, sh.ops, sh.stages, sh.steps, sh.cap);
   auto kern = ndir == 0 ? (sh.ops == 2 ? assign_tc_kernel<0, 2, XT> : assign_tc_kernel<0, 1, XT>)
                         : assign_tc_kernel<1, 2, XT>;
@@ -709,7 +813,10 @@ void assign_tc_pass(const XT* X, int64_t n, int d, const float* C, int c, int nd
   const int grid = (int)std::min<int64_t>((n + pts - 1) / pts, num_sms());
   kern<<<grid, kThr, smem, s>>>(prm);
   SOAR_LAUNCHED();
-  refine_list<XT><<<num_sms() * 8, 256, 0, s>>>(X, d, C, c, assign, astride, ndir, lambda, cand, ovf, queue, qcount);
+  auto flagged = ndir == 0 ? refine_flagged<0, XT> : refine_flagged<1, XT>;
+  flagged<<<num_sms() * 4, kFlagThreads, 0, s>>>(X, n, d, C, c, assign, astride, lambda, queue, qcount, best);
+  SOAR_LAUNCHED();
+  refine_list<XT><<<num_sms() * 8, 256, 0, s>>>(X, n, d, C, assign, astride, ndir, lambda, cand, queue, best, qcount);
   SOAR_LAUNCHED();
 }
 

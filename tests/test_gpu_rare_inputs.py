@@ -21,3 +21,38 @@ def test_points_without_a_number_are_assigned_nowhere(soar, dtype, d, spills):
     rest[bad] = False
     assert torch.equal(got[rest.cuda()], want[rest.cuda()])
     assert (got[bad.cuda()] == -1).all()
+
+
+@pytest.mark.parametrize("d", [150, 160, 320])       # widths whose lists hold 16 and 8 candidates; a single operand
+@pytest.mark.parametrize("spills", [0, 1])
+def test_assignment_in_clusters_tighter_than_the_screening_band(soar, d, spills):
+    """Twenty centroids to a cluster and all of them within the band: every point is scored against the whole
+    codebook.  Two operations a pair and column (three for the spill) on the FMA pipe; a pass may take eight times
+    what they need there at 1.5 GHz, which a lane per centroid, reading its row alone, does not reach."""
+    n, c = 200_000, 2000
+    g = torch.Generator(device="cuda").manual_seed(d)
+    mu = torch.randn(c // 20, d, generator=g, device="cuda")
+    X = mu[torch.randint(0, c // 20, (n,), generator=g, device="cuda")]
+    X = torch.nn.functional.normalize(X + 0.05 * torch.randn(n, d, generator=g, device="cuda"), dim=1)
+    C = X[torch.randperm(n, generator=g, device="cuda")[:c]].contiguous()
+    A = soar.soar_assign(X, C, 1.0, spills)
+    best = float("inf")
+    for _ in range(3):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        soar.soar_assign(X, C, 1.0, spills)
+        b.record()
+        torch.cuda.synchronize()
+        best = min(best, a.elapsed_time(b))
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    assert best <= 1e3 * 8 * n * c * d * (2 + 3 * spills) / (sms * 128 * 1.5e9)
+    at = torch.randint(0, n, (4000,), generator=g, device="cuda")
+    x, cc, own = X[at].double(), C.double(), A[at].long()
+    dist = torch.cdist(x, cc, compute_mode="donot_use_mm_for_euclid_dist") ** 2
+    assert (dist.gather(1, own[:, :1])[:, 0] <= dist.min(1)[0] * (1 + 1e-5)).all()
+    if spills:
+        r = x - cc[own[:, 0]]
+        r = r / r.norm(dim=1, keepdim=True).clamp(min=1e-30)
+        loss = dist + ((x * r).sum(1, keepdim=True) - r @ cc.T) ** 2
+        loss.scatter_(1, own[:, :1], float("inf"))
+        assert (loss.gather(1, own[:, 1:])[:, 0] <= loss.min(1)[0] * (1 + 1e-5)).all()
