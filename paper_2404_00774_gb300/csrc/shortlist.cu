@@ -18,7 +18,7 @@
 // a fixed order (`Rows::exact`).  The tensor cores add in another order, so a
 // key holds such a score within delta only (`Rows::delta`).  With T the R-th
 // largest key of a slice, a row above T + 2 delta is in the shortlist and one
-// below T - 2 delta is not; the few between are scored again in the defined
+// below T - 2 delta is not; those between are scored again in the defined
 // order and ranked by it (score descending, lower id first), so the shortlist
 // is the defined one.
 //
@@ -42,9 +42,10 @@ namespace {
 constexpr int kWarps = 8;
 constexpr int kThreads = 32 * kWarps;
 
-__device__ __forceinline__ float fp8_code_value(uint32_t b) {
-  __half_raw h = __nv_cvt_fp8_to_halfraw((__nv_fp8_storage_t)b, __NV_E4M3);
-  return __half2float(__half(h));
+// the values of two e4m3 codes, the low byte's first
+__device__ __forceinline__ float2 fp8_pair_values(uint32_t two) {
+  const __half2_raw h = __nv_cvt_fp8x2_to_halfraw2((__nv_fp8x2_storage_t)two, __NV_E4M3);
+  return __half22float2(__half2(h));
 }
 
 // D (16 x 8, fp32) += A (16 x 32 e4m3) B (32 x 8 e4m3)
@@ -160,6 +161,8 @@ struct Fp8Rows {
   __device__ float delta(float3 v, int64_t q, float smax) const {
     return ldexpf((float)code_stride, -22) * sqrtf(v.x) * 448.f * sqrtf((float)code_stride) * qscale[q] * smax;
   }
+  __device__ bool tabulate(const float*, float*, int) const { return false; }
+  __device__ float exact_tabulated(const float*, int64_t, float) const { return 0.f; }
   __device__ float exact(const float* qs, int64_t q, int64_t r, float) const {
     const uint4* x = reinterpret_cast<const uint4*>(codes + r * (int64_t)code_stride);
     float acc = 0.f;
@@ -169,7 +172,11 @@ struct Fp8Rows {
 #pragma unroll
       for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int b = 0; b < 4; ++b) acc = fmaf(qs[16 * c + 4 * i + b], fp8_code_value((wv[i] >> (8 * b)) & 0xffu), acc);
+        for (int b = 0; b < 4; b += 2) {
+          const float2 w = fp8_pair_values((wv[i] >> (8 * b)) & 0xffffu);
+          acc = fmaf(qs[16 * c + 4 * i + b], w.x, acc);
+          acc = fmaf(qs[16 * c + 4 * i + b + 1], w.y, acc);
+        }
     }
     return acc * qscale[q] * row_scales[r];
   }
@@ -286,6 +293,27 @@ struct Pq4Rows {
   __device__ float delta(float3 v, int64_t, float) const {
     const float qb = sqrtf(v.x) * sqrtf(v.y);
     return qb * (ldexpf(1.f, -14) + ldexpf((float)d, -20)) + ldexpf(v.z + qb, -21);
+  }
+  // the query's products with every centre, for many rows (all threads), where they fit `room` floats
+  __device__ bool tabulate(const float* qs, float* table, int room) const {
+    if (16 * m > room) return false;
+    for (int e = threadIdx.x; e < 16 * m; e += kThreads) {
+      const float2 c = reinterpret_cast<const float2*>(B)[e];
+      table[e] = fmaf(qs[2 * (e / 16) + 1], c.y, qs[2 * (e / 16)] * c.x);
+    }
+    return true;
+  }
+  __device__ float exact_tabulated(const float* table, int64_t r, float pair_base) const {
+    const uint32_t* x = reinterpret_cast<const uint32_t*>(codes + r * (int64_t)code_stride);
+    float acc = 0.f;
+#pragma unroll 4
+    for (int w = 0; w < m / 8; ++w) {
+      const uint32_t v = __ldg(x + w);
+#pragma unroll
+      for (int b = 0; b < 8; ++b) acc += table[16 * (8 * w + b) + ((v >> (4 * b)) & 15u)];
+    }
+    for (int s = m / 8 * 8; s < m; ++s) acc += table[16 * s + ((__ldg(x + s / 8) >> (4 * (s % 8))) & 15u)];
+    return pair_base + acc;
   }
   __device__ float exact(const float* qs, int64_t, int64_t r, float pair_base) const {
     const uint32_t* x = reinterpret_cast<const uint32_t*>(codes + r * (int64_t)code_stride);
@@ -620,15 +648,22 @@ __device__ void block_sort(uint64_t* buf, int N) {
 //            R-th best lies in one bin, and the bins within 2 delta of that
 //            one are the band
 //   list     every row above the band, then the band's best in the defined
-//            order.  A band that does not fit (thousands of near-equal scores,
-//            or infinities) is resolved by a radix select over all rows'
-//            defined keys instead.
+//            order.  Where linear bins cannot tell (rows of very uneven length, a
+//            misleading sample, infinities), the R-th largest key of the slice is
+//            found byte by byte and the band is taken around it; a band that does
+//            not fit (thousands of near-equal scores, or a delta as wide as the
+//            scores' spread) has its defined scores computed once, in place of its
+//            keys.  (A radix select that computed every row's defined score nine
+//            times took its place before: 10 000 queries, 10^6 x 96 in 1 000
+//            partitions, t = 6, one row in a thousand 1 000 times longer, FP8 with
+//            R = 1 000 42.0 ms, now 7.8; PQ4 with R = 100 34.6, now 6.1; 1.6 and
+//            1.3 with rows of equal length)
 //   rescore  a thread per row; the best k by per-warp sorted lists (k <= 32) or
 //            a sort
 // Bound: the latency of one pass over the slice and of the scattered rows.
 template <typename Rows, typename OT>
 __global__ void __launch_bounds__(kThreads) finish_slices(
-    Rows rows, const uint32_t* __restrict__ keys, const int64_t* __restrict__ counts, int64_t slice,
+    Rows rows, uint32_t* keys, const int64_t* __restrict__ counts, int64_t slice,
     const int64_t* __restrict__ pos, const int32_t* __restrict__ top, const int32_t* __restrict__ tpq, int64_t q0,
     int t, const int64_t* __restrict__ off, const int32_t* __restrict__ ids, const float* __restrict__ base,
     const float* __restrict__ smax, const void* __restrict__ Q, int qdt, int d, const OT* __restrict__ orig,
@@ -643,7 +678,7 @@ __global__ void __launch_bounds__(kThreads) finish_slices(
   __shared__ int64_t row_s[kProbeTable];        // and the index row of the slice's position 0 in that probe
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   const int64_t ql = blockIdx.x, q = q0 + ql;
-  const uint32_t* K = keys + ql * slice;
+  uint32_t* K = keys + ql * slice;             // (rewritten in place by the rarest branch)
   const int n = (int)counts[ql];
   const int tq = tpq ? min(max(tpq[q], 0), t) : t;
   const int64_t* qpos = pos + ql * t;
@@ -723,17 +758,17 @@ __global__ void __launch_bounds__(kThreads) finish_slices(
   hi = hi_s;
   const float delta = delta_s;
   // position i of the slice: its probe, its row
-  const bool table = tq <= kProbeTable;
+  const bool in_table = tq <= kProbeTable;
   const auto probe_of = [&](int i) {
     int a = 0, b = tq - 1;
     while (a < b) {
       const int mid = (a + b + 1) >> 1;
-      if ((table ? at_s[mid] : (int)qpos[mid]) <= i) a = mid;
+      if ((in_table ? at_s[mid] : (int)qpos[mid]) <= i) a = mid;
       else b = mid - 1;
     }
     return a;
   };
-  const auto row_of = [&](int i, int j) { return table ? row_s[j] + i : off[probes[j]] - qpos[j] + i; };
+  const auto row_of = [&](int i, int j) { return in_table ? row_s[j] + i : off[probes[j]] - qpos[j] + i; };
   const auto defined_key = [&](int i) {
     const int j = probe_of(i);
     const int64_t r = row_of(i, j);
@@ -778,16 +813,26 @@ __global__ void __launch_bounds__(kThreads) finish_slices(
     __syncthreads();
     return all;
   };
-  // The list from `count` rows (key_at, pos_at), all rows of the slice that
-  // count or (open) all at or above lo; false where it cannot tell.
-  const auto choose = [&](int count, auto key_at, auto pos_at, bool open) {
+  // n_list rows of the list so far, as positions, and m <= kBand rows of the band:
+  // the rows as ids, then the band's best in the defined order
+  const auto finish_band = [&](int m) {
+    int N = 2;
+    while (N < m) N <<= 1;
+    for (int i = tid; i < N; i += kThreads) band_key[i] = i < m ? defined_key(band[i]) : ~0ull;   // (bins: no longer read)
+    __syncthreads();
+    block_sort(band_key, N);
+    const int have = n_list;
+    for (int i = tid; i < have; i += kThreads) list[i] = ids[row_of(list[i], probe_of(list[i]))];
+    for (int i = tid; i < R - have; i += kThreads) list[have + i] = (int32_t)(band_key[i] & 0xffffffffu);
+    __syncthreads();
+    if (tid == 0) n_list = R;
+  };
+  // The list from the kept rows, all rows of the slice that count or (open) all
+  // at or above lo; false where linear bins cannot tell.
+  const auto choose = [&](int count, bool open) {
     if (!set_bins()) return false;
-    for (int i = tid; i < count; i += kThreads) {
-      const uint32_t key = key_at(i);
-      if (key) atomicAdd(&hist[bin_of(key)], 1);
-    }
-    const int all = find_bin(R);
-    if (all <= R) return false;
+    for (int i = tid; i < count; i += kThreads) atomicAdd(&hist[bin_of(kept[i])], 1);
+    if (find_bin(R) <= R) return false;
     const float wide = ceilf(2.f * delta * scale) + 1.f;
     const int mb = wide < (float)kBins ? (int)wide : kBins;
     if (open && bin_s < mb) return false;                                // rows below lo might be in the band
@@ -798,27 +843,49 @@ __global__ void __launch_bounds__(kThreads) finish_slices(
     if (m > kBand) return false;
     for (int i0 = 0; i0 < count; i0 += kThreads) {
       const int i = i0 + tid;
-      const uint32_t key = i < count ? key_at(i) : 0u;
-      const int b = key ? bin_of(key) : -1;
+      const int b = i < count ? bin_of(kept[i]) : -1;
       if (!__any_sync(kFull, b >= b_lo)) continue;
-      append(b > b_hi, &n_list, list, R, b > b_hi ? pos_at(i) : 0);
-      append(b >= b_lo && b <= b_hi, &n_band, band, kBand, b >= b_lo ? pos_at(i) : 0);
+      append(b > b_hi, &n_list, list, R, b > b_hi ? kept_at[i] : 0);
+      append(b >= b_lo && b <= b_hi, &n_band, band, kBand, b >= b_lo ? kept_at[i] : 0);
     }
     __syncthreads();
-    int N = 2;
-    while (N < m) N <<= 1;
-    for (int i = tid; i < N; i += kThreads) band_key[i] = i < m ? defined_key(band[i]) : ~0ull;   // (bins: no longer read)
-    __syncthreads();
-    block_sort(band_key, N);
-    // the list's rows as ids, then the band's best
-    const int have = n_list;
-    for (int i = tid; i < have; i += kThreads) {
-      list[i] = ids[row_of(list[i], probe_of(list[i]))];
-    }
-    for (int i = tid; i < R - have; i += kThreads) list[have + i] = (int32_t)(band_key[i] & 0xffffffffu);
-    __syncthreads();
-    if (tid == 0) n_list = R;
+    finish_band(m);
     return true;
+  };
+  // The need-th largest of the values value(i) > 0, i in [0, n), and (in need) how
+  // many of its equals count; at least `need` values are positive.
+  const auto nth_largest = [&](int& need, auto value) {
+    uint32_t prefix = 0u, mask = 0u;
+    for (int shift = 24; shift >= 0; shift -= 8) {
+      __syncthreads();
+      hist[tid] = 0;
+      __syncthreads();
+      int last = 0, run = 0;                            // (a thread's keys mostly share their leading bytes)
+      for (int i = tid; i < n; i += kThreads) {
+        const uint32_t v = value(i);
+        if (!v || (v & mask) != prefix) continue;
+        const int b = (v >> shift) & 0xffu;
+        if (b != last) {
+          if (run) atomicAdd(&hist[last], run);
+          last = b;
+          run = 0;
+        }
+        ++run;
+      }
+      if (run) atomicAdd(&hist[last], run);
+      __syncthreads();
+      int all;
+      const int mine = hist[255 - tid], c = block_exclusive_scan<int>(mine, warp_s, all);
+      if (c < need && c + mine >= need) {
+        bin_s = 255 - tid;
+        above_s = c;
+      }
+      __syncthreads();
+      need -= above_s;
+      prefix |= (uint32_t)bin_s << shift;
+      mask |= 0xffu << shift;
+    }
+    return prefix;
   };
 
   uint32_t floor_key = 1u;                              // every row that counts
@@ -831,43 +898,50 @@ __global__ void __launch_bounds__(kThreads) finish_slices(
     const int want = (int)(1.25f * expect + 4.f * sqrtf(expect) + 8.f);
     if (find_bin(want) > want) floor_key = max(1u, float_key(lo + (float)(bin_s - 1) / scale));
   }
-  // one pass: four keys a load (slices start on 16 bytes), one counter step a warp and load
+  // one pass: four keys a load (slices start on 16 bytes), two loads in flight, one counter step a warp and load
   if (finite) {
+    constexpr int kPass = 2;
     const int n4 = n / 4;
-#pragma unroll 2
-    for (int i0 = 32 * w; i0 <= n4; i0 += kThreads) {
-      const int i = i0 + lane;
-      uint4 v = make_uint4(0u, 0u, 0u, 0u);
-      if (i < n4) {
-        v = __ldg(reinterpret_cast<const uint4*>(K) + i);
-      } else if (i == n4) {                             // the last one to three keys
-        if (n % 4 > 0) v.x = K[4 * i];
-        if (n % 4 > 1) v.y = K[4 * i + 1];
-        if (n % 4 > 2) v.z = K[4 * i + 2];
-      }
-      const uint32_t key[4] = {v.x, v.y, v.z, v.w};
-      int mine = 0;
+    for (int i0 = 32 * w; i0 <= n4; i0 += kPass * kThreads) {
+      uint4 v[kPass];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) mine += key[u] >= floor_key ? 1 : 0;
-      if (!__any_sync(kFull, mine)) continue;
-      int incl = mine;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(kFull, incl, o);
-        if (lane >= o) incl += y;
-      }
-      int at = 0;
-      if (lane == 31) at = atomicAdd(&n_kept, incl);
-      at = __shfl_sync(kFull, at, 31) + incl - mine;
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-        if (key[u] >= floor_key) {
-          if (at < cap) {
-            kept[at] = key[u];
-            kept_at[at] = 4 * i + u;
-          }
-          ++at;
+      for (int u = 0; u < kPass; ++u) {
+        const int i = i0 + u * kThreads + lane;
+        v[u] = make_uint4(0u, 0u, 0u, 0u);
+        if (i < n4) {
+          v[u] = reinterpret_cast<const uint4*>(K)[i];
+        } else if (i == n4) {                           // the last one to three keys
+          if (n % 4 > 0) v[u].x = K[4 * i];
+          if (n % 4 > 1) v[u].y = K[4 * i + 1];
+          if (n % 4 > 2) v[u].z = K[4 * i + 2];
         }
+      }
+#pragma unroll
+      for (int u = 0; u < kPass; ++u) {
+        const uint32_t key[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
+        int mine = 0;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) mine += key[e] >= floor_key ? 1 : 0;
+        if (!__any_sync(kFull, mine)) continue;
+        int incl = mine;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const int y = __shfl_up_sync(kFull, incl, o);
+          if (lane >= o) incl += y;
+        }
+        int at = 0;
+        if (lane == 31) at = atomicAdd(&n_kept, incl);
+        at = __shfl_sync(kFull, at, 31) + incl - mine;
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+          if (key[e] >= floor_key) {
+            if (at < cap) {
+              kept[at] = key[e];
+              kept_at[at] = 4 * (i0 + u * kThreads + lane) + e;
+            }
+            ++at;
+          }
+      }
     }
   }
   __syncthreads();
@@ -878,59 +952,69 @@ __global__ void __launch_bounds__(kThreads) finish_slices(
       few = true;
     } else if (m_kept > R) {
       if (floor_key > 1u) lo = key_float(floor_key);
-      done = choose(m_kept, [&](int i) { return kept[i]; }, [&](int i) { return kept_at[i]; }, floor_key > 1u);
+      done = choose(m_kept, floor_key > 1u);
     }
-  }
-  if (!done && !few) {
-    __syncthreads();
-    if (tid == 0) n_list = n_band = 0;
-    lo = lo_s;
-    done = choose(n, [&](int i) { return K[i]; }, [&](int i) { return i; }, false);
   }
   __syncthreads();
   if (!done) {
-    // every row that counts, or (more than R of them) those up to the R-th
-    // smallest defined key, found byte by byte
-    uint64_t limit = ~0ull;
+    if (tid == 0) n_list = n_band = 0;
     int cnt = 0, total;
     for (int i = tid; i < n; i += kThreads) cnt += K[i] != 0u;
     block_exclusive_scan<int>(cnt, warp_s, total);
-    if (total > R) {
-      uint64_t prefix = 0, mask = 0;
-      int need = R;
-      for (int shift = 56; shift >= 0; shift -= 8) {
-        __syncthreads();
-        for (int i = tid; i < 256; i += kThreads) hist[i] = 0;
-        __syncthreads();
-        for (int i = tid; i < n; i += kThreads) {
-          if (!K[i]) continue;
-          const uint64_t kk = defined_key(i);
-          if ((kk & mask) == prefix) atomicAdd(&hist[(kk >> shift) & 0xff], 1);
-        }
-        __syncthreads();
-        if (tid == 0) {
-          int b = 0, c = 0;
-          while (b < 255 && c + hist[b] < need) c += hist[b++];
-          bin_s = b;
-          above_s = c;
-        }
-        __syncthreads();
-        need -= above_s;
-        prefix |= (uint64_t)bin_s << shift;
-        mask |= (uint64_t)0xff << shift;
+    if (few || total <= R) {
+      for (int i0 = 0; i0 < n; i0 += kThreads) {
+        const int i = i0 + tid;
+        const bool in = i < n && K[i] != 0u;
+        append(in, &n_list, list, R, in ? ids[row_of(i, probe_of(i))] : -1);
       }
-      limit = prefix;
-    }
-    __syncthreads();
-    if (tid == 0) n_list = 0;
-    __syncthreads();
-    for (int i0 = 0; i0 < n; i0 += kThreads) {
-      const int i = i0 + tid;
-      const bool counts_ = i < n && K[i] != 0u;
-      const bool in = counts_ && (limit == ~0ull || defined_key(i) <= limit);
-      int32_t id = -1;
-      if (in) id = ids[row_of(i, probe_of(i))];
-      append(in, &n_list, list, R, id);
+    } else {
+      // the band around the R-th largest key itself; all rows where that or delta is not finite
+      int need = R;
+      const float f = key_float(nth_largest(need, [&](int i) { return K[i]; }));
+      uint32_t lo_key = 1u, hi_key = ~0u;
+      if (fabsf(f) < INFINITY && delta < INFINITY) {
+        lo_key = max(1u, float_key(__fsub_rd(f, 2.f * delta)));
+        hi_key = float_key(__fadd_ru(f, 2.f * delta));
+      }
+      int in_band = 0, m;
+      for (int i = tid; i < n; i += kThreads) in_band += K[i] >= lo_key && K[i] <= hi_key ? 1 : 0;
+      block_exclusive_scan<int>(in_band, warp_s, m);
+      const bool fits = m <= kBand;
+      float* table = reinterpret_cast<float*>(kept);      // (the kept rows: no longer read)
+      const bool tabulated = !fits && rows.tabulate(qs, table, 2 * cap);
+      __syncthreads();
+      const auto defined = [&](int i) {
+        const int j = probe_of(i);
+        const int64_t r = row_of(i, j);
+        const float b = base ? base[ql * t + j] : 0.f;
+        return max(1u, float_key(tabulated ? rows.exact_tabulated(table, r, b) : rows.exact(qs, q, r, b)));
+      };
+      // a band too large for shared memory: its keys become those of the defined
+      // scores, in place, and the other rows' zero
+      for (int i0 = 0; i0 < n; i0 += kThreads) {
+        const int i = i0 + tid;
+        const uint32_t key = i < n ? K[i] : 0u;
+        const bool in = key >= lo_key && key <= hi_key;
+        append(key > hi_key, &n_list, list, R, i);
+        if (fits) append(in, &n_band, band, kBand, i);
+        else if (i < n) K[i] = in ? defined(i) : 0u;
+      }
+      __syncthreads();
+      if (fits) {
+        finish_band(m);
+      } else {
+        need = R - n_list;
+        const uint32_t least = nth_largest(need, [&](int i) { return K[i]; });
+        // of the rows that score as the last one does, those of the lowest ids
+        const auto tie = [&](int i) { return K[i] == least ? ~(uint32_t)ids[row_of(i, probe_of(i))] : 0u; };
+        const uint32_t last = nth_largest(need, tie);
+        for (int i0 = 0; i0 < n; i0 += kThreads) {
+          const int i = i0 + tid;
+          append(i < n && (K[i] > least || tie(i) >= last), &n_list, list, R, i);
+        }
+        __syncthreads();
+        for (int i = tid; i < R; i += kThreads) list[i] = ids[row_of(list[i], probe_of(list[i]))];
+      }
     }
     __syncthreads();
   }

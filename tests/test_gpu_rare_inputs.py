@@ -6,6 +6,19 @@ import torch
 pytestmark = pytest.mark.gpu
 
 
+def _milliseconds(f):
+    f()
+    best = float("inf")
+    for _ in range(3):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        f()
+        b.record()
+        torch.cuda.synchronize()
+        best = min(best, a.elapsed_time(b))
+    return best
+
+
 @pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
 @pytest.mark.parametrize("d", [24, 160, 400])        # both tensor-core shapes and the general kernels
 @pytest.mark.parametrize("spills", [0, 1, 2])
@@ -36,14 +49,7 @@ def test_assignment_in_clusters_tighter_than_the_screening_band(soar, d, spills)
     X = torch.nn.functional.normalize(X + 0.05 * torch.randn(n, d, generator=g, device="cuda"), dim=1)
     C = X[torch.randperm(n, generator=g, device="cuda")[:c]].contiguous()
     A = soar.soar_assign(X, C, 1.0, spills)
-    best = float("inf")
-    for _ in range(3):
-        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
-        a.record()
-        soar.soar_assign(X, C, 1.0, spills)
-        b.record()
-        torch.cuda.synchronize()
-        best = min(best, a.elapsed_time(b))
+    best = _milliseconds(lambda: soar.soar_assign(X, C, 1.0, spills))
     sms = torch.cuda.get_device_properties(0).multi_processor_count
     assert best <= 1e3 * 8 * n * c * d * (2 + 3 * spills) / (sms * 128 * 1.5e9)
     at = torch.randint(0, n, (4000,), generator=g, device="cuda")
@@ -56,3 +62,34 @@ def test_assignment_in_clusters_tighter_than_the_screening_band(soar, d, spills)
         loss = dist + ((x * r).sum(1, keepdim=True) - r @ cc.T) ** 2
         loss.scatter_(1, own[:, :1], float("inf"))
         assert (loss.gather(1, own[:, 1:])[:, 0] <= loss.min(1)[0] * (1 + 1e-5)).all()
+
+
+@pytest.mark.parametrize("mode,R,every,most", [("fp8", 1000, 1000, 12), ("pq4", 100, 1000, 12)])
+def test_compressed_search_over_rows_of_very_uneven_length(soar, mode, R, every, most):
+    """One row in a thousand is 1 000 times longer, so that the rounding bound spans the other rows' scores and each of
+    those is scored again in the defined order: once, on the FMA pipe, which is within twelve times the usual search
+    (nine times over is not)."""
+    n, d, c, nq = 400_000, 96, 400, 10_000
+    g = torch.Generator(device="cuda").manual_seed(3)
+    mu = torch.randn(c // 10, d, generator=g, device="cuda")
+
+    def draw(rows):
+        at = torch.randint(0, c // 10, (rows,), generator=g, device="cuda")
+        return torch.nn.functional.normalize(mu[at] + 0.3 * torch.randn(rows, d, generator=g, device="cuda"), dim=1)
+
+    X, Q = draw(n), draw(nq)
+    C = X[torch.randperm(n, generator=g, device="cuda")[:c]].contiguous()
+    A = soar.soar_assign(X, C, 1.0, 1)
+    times = []
+    for long_rows in (False, True):
+        if long_rows:
+            X[::every] *= 1000
+        if mode == "fp8":
+            ix = soar.soar_index_build(X, C, A, mode=soar.SOAR_SCORE_FP8)
+        else:
+            B = soar.soar_pq_train(X[:20_000], C, A[:20_000, 0].contiguous(), 3,
+                                   torch.arange(16, dtype=torch.int32, device="cuda"))
+            ix = soar.soar_index_build_pq(X, C, A, B)
+        times.append(_milliseconds(lambda: soar.soar_search(ix, Q, 10, 6, rescore=R)))
+        ix.close()
+    assert times[1] <= most * times[0], times
