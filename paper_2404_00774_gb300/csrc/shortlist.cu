@@ -92,6 +92,7 @@ struct Frag {
 // Per-row scaled E4M3 codes.
 struct Fp8Rows {
   static constexpr int kTiles = 4;      // most 8-query tiles per item
+  static constexpr bool kScaled = true;
   const uint8_t* codes;
   int code_stride;
   const float* row_scales;
@@ -157,7 +158,7 @@ struct Fp8Rows {
   // code_stride fp32 additions, off by 2^-24 (defined order) and at most 2^-23
   // (tensor cores; measured 2^-23 over a whole sum) of a partial sum that stays
   // below ||q8|| ||x8||, and ||x8|| <= 448 sqrt(d); the rest covers the scaling.
-  // The scale of a row is at most smax.
+  // The scale of a row that the query meets is at most smax.
   __device__ float delta(float3 v, int64_t q, float smax) const {
     return ldexpf((float)code_stride, -22) * sqrtf(v.x) * 448.f * sqrtf((float)code_stride) * qscale[q] * smax;
   }
@@ -187,6 +188,7 @@ struct Fp8Rows {
 // a code is one shared-memory read of its centre (hi and lo parts); centres and
 // queries enter as hi + lo and the lo lo product is dropped.
 struct Pq4Rows {
+  static constexpr bool kScaled = false;
   static constexpr int kTiles = 4;      // (eight took 122 registers: two blocks an SM, 1 346 us)
   const uint8_t* codes;
   int code_stride, m, d;
@@ -406,8 +408,8 @@ struct ProbeMasks {
 // Work items (partition, up to 32 of its queries; blockIdx.y takes every
 // gridDim.y-th step of 128 rows): keys of every (query, row).  A key is the
 // order-preserving image of the score, 0 for a copy that does not count.  smax
-// (FP8, zero before the launch): the largest scale of the rows met, which are
-// positive and so ordered like their bits.
+// (FP8, [queries of the pass], zero before the launch): the largest scale of the
+// rows each query met, which are positive and so ordered like their bits.
 template <typename Rows>
 __global__ void __launch_bounds__(kThreads, 3) score_items(Rows rows, IvfWork work, const int32_t* __restrict__ ids,
                                                         const int32_t* __restrict__ assign, int a,
@@ -424,7 +426,7 @@ __global__ void __launch_bounds__(kThreads, 3) score_items(Rows rows, IvfWork wo
   __shared__ float qf_s[QB];
   __shared__ int64_t q_s[QB];
   __shared__ ProbeMasks masks;
-  __shared__ int earlier_s;
+  __shared__ int earlier_s, most_s;
   const int item = blockIdx.x;
   if (item >= work.count()) return;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -448,7 +450,7 @@ __global__ void __launch_bounds__(kThreads, 3) score_items(Rows rows, IvfWork wo
       masks.key[i] = -1;
       masks.mask[i] = 0u;
     }
-  if (threadIdx.x == 0) earlier_s = 0;
+  if (threadIdx.x == 0) earlier_s = most_s = 0;
   __syncthreads();
   if (threadIdx.x < QB) {                       // a thread per query slot
     const int i = threadIdx.x;
@@ -558,7 +560,9 @@ __global__ void __launch_bounds__(kThreads, 3) score_items(Rows rows, IvfWork wo
   if (smax) {
 #pragma unroll
     for (int o = 8; o > 0; o >>= 1) most = fmaxf(most, __shfl_xor_sync(kFull, most, o));
-    if (lane == 0 && __float_as_int(most) > __ldcg(smax)) atomicMax(smax, __float_as_int(most));
+    if (lane == 0) atomicMax(&most_s, __float_as_int(most));
+    __syncthreads();
+    if ((int)threadIdx.x < nqi) atomicMax(smax + (q_s[threadIdx.x] - q0), most_s);
   }
 }
 
@@ -751,7 +755,7 @@ __global__ void __launch_bounds__(kThreads) finish_slices(
     }
     lo_s = lo;
     hi_s = hi;
-    delta_s = rows.delta(norms, q, smax ? *smax : 0.f);
+    delta_s = rows.delta(norms, q, smax ? smax[ql] : 0.f);
   }
   __syncthreads();
   lo = lo_s;
@@ -1097,7 +1101,7 @@ uint32_t* key_room(int64_t slice, int64_t nq, int64_t& cq, Scratch& scr) {
 }
 
 template <typename Rows>
-void run(const IndexData& ix, Rows rws, float* base, int* smax, const float* Qf, int qstride, const void* Q,
+void run(const IndexData& ix, Rows rws, float* base, const float* Qf, int qstride, const void* Q,
          soar_dtype dt, const int32_t* top, const int32_t* tpq, int64_t nq, int t, int R, int k, int64_t* ids_out,
          float* scores_out, cudaStream_t s, Scratch& scr) {
   rws.tiles = Rows::kTiles;
@@ -1107,6 +1111,7 @@ void run(const IndexData& ix, Rows rws, float* base, int* smax, const float* Qf,
   int64_t cq;
   uint32_t* keys = key_room(slice, nq, cq, scr);
   int64_t* counts = scr.get<int64_t>(cq);
+  int* smax = Rows::kScaled ? scr.get<int>(cq) : nullptr;
   int64_t* pos = scr.get<int64_t>((size_t)cq * t);
   int32_t* inv = scr.get<int32_t>((size_t)cq * t);
   const int a = 1 + ix.spills;
@@ -1147,6 +1152,7 @@ void run(const IndexData& ix, Rows rws, float* base, int* smax, const float* Qf,
     const int64_t items = std::min<int64_t>(m * t, g.max_items);
     const unsigned split = (unsigned)std::max<int64_t>(1, std::min<int64_t>(16, 8 * num_sms() / std::max<int64_t>(1, items)));
     const IvfWork work{ix.offsets, g.pair_off, g.vals, g.order, g.item_base, ix.c, t, QB};
+    if (smax) SOAR_CUDA(cudaMemsetAsync(smax, 0, sizeof(int) * m, s));
     score_items<Rows><<<dim3((unsigned)items, split), kThreads, item_smem, s>>>(rws, work, ix.ids, ix.assign, a, top,
                                                                                q0, slice, pos, keys, smax);
     SOAR_LAUNCHED();
@@ -1163,12 +1169,9 @@ void run(const IndexData& ix, Rows rws, float* base, int* smax, const float* Qf,
 void fp8_search(const IndexData& ix, const float* Qf, const float* qscale, const void* Q, soar_dtype dt,
                 const int32_t* top, const int32_t* tpq, int64_t nq, int t, int R, int k, int64_t* ids_out,
                 float* scores_out, cudaStream_t s, Scratch& scr) {
-  int* smax = scr.get<int>(1);
-  SOAR_CUDA(cudaMemsetAsync(smax, 0, sizeof(int), s));
   const Fp8Rows rws{static_cast<const uint8_t*>(ix.vectors), ix.code_stride, ix.row_scales, Qf, qscale,
                     (ix.code_stride + 63) / 64, 0};
-  run(ix, rws, nullptr, smax, Qf, ix.code_stride, Q, dt, top, tpq, nq, t, R, k,
-      ids_out, scores_out, s, scr);
+  run(ix, rws, nullptr, Qf, ix.code_stride, Q, dt, top, tpq, nq, t, R, k, ids_out, scores_out, s, scr);
 }
 
 void pq_search(const IndexData& ix, const float* Qf, int qstride, const void* Q, soar_dtype dt, const int32_t* top,
@@ -1178,7 +1181,7 @@ void pq_search(const IndexData& ix, const float* Qf, int qstride, const void* Q,
   float* base = scr.get<float>((size_t)key_chunk(slice, nq, (int64_t)1 << 30) * t);
   const Pq4Rows rws{static_cast<const uint8_t*>(ix.vectors), ix.code_stride, ix.pq_m, ix.d, ix.pq_cb, Qf, qstride,
                     base, (ix.pq_m + 7) / 8, 0};
-  run(ix, rws, base, nullptr, Qf, qstride, Q, dt, top, tpq, nq, t, R, k, ids_out, scores_out, s, scr);
+  run(ix, rws, base, Qf, qstride, Q, dt, top, tpq, nq, t, R, k, ids_out, scores_out, s, scr);
 }
 
 }  // namespace soar

@@ -64,11 +64,12 @@ def test_assignment_in_clusters_tighter_than_the_screening_band(soar, d, spills)
         assert (loss.gather(1, own[:, 1:])[:, 0] <= loss.min(1)[0] * (1 + 1e-5)).all()
 
 
-@pytest.mark.parametrize("mode,R,every,most", [("fp8", 1000, 1000, 12), ("pq4", 100, 1000, 12)])
+@pytest.mark.parametrize("mode,R,every,most", [("fp8", 1000, 1000, 12), ("pq4", 100, 1000, 12),
+                                                ("fp8", 1000, 400_000, 2)])    # a single long row
 def test_compressed_search_over_rows_of_very_uneven_length(soar, mode, R, every, most):
     """One row in a thousand is 1 000 times longer, so that the rounding bound spans the other rows' scores and each of
     those is scored again in the defined order: once, on the FMA pipe, which is within twelve times the usual search
-    (nine times over is not)."""
+    (nine times over is not).  A single long row widens the bound of the few queries that probe its partitions."""
     n, d, c, nq = 400_000, 96, 400, 10_000
     g = torch.Generator(device="cuda").manual_seed(3)
     mu = torch.randn(c // 10, d, generator=g, device="cuda")
