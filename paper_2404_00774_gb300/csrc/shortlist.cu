@@ -346,12 +346,23 @@ __global__ void pair_bases(const float* __restrict__ Qf, int qstride, const floa
   if (lane == 0) base[e] = v;
 }
 
+// Where the queries' keys lie.  Slices of the longest possible length where those
+// fit (start null); else one behind the other, each on 16 bytes, a pass taking
+// those that start in [from, to).
+struct Slices {
+  uint32_t* keys;
+  const int64_t* start;     // [queries + 1]
+  int64_t stride, from, to;
+  __device__ int64_t at(int64_t ql) const { return (start ? start[ql] : ql * stride) - from; }
+  __device__ bool in_pass(int64_t ql) const { return !start || (start[ql] >= from && start[ql] < to); }
+};
+
 // Each probed pair's first position in its query's slice (the sizes of the
-// query's earlier probed partitions added up) and the slice's length; a warp
-// per query.
+// query's earlier probed partitions added up) and the slice's length, in packed
+// (unless null, [nq + 1]) rounded up to four; a warp per query.
 __global__ void pair_offsets(const int64_t* __restrict__ off, const int32_t* __restrict__ top,
                              const int32_t* __restrict__ tpq, int64_t q0, int64_t nq, int t,
-                             int64_t* __restrict__ pos, int64_t* __restrict__ counts) {
+                             int64_t* __restrict__ pos, int64_t* __restrict__ counts, int64_t* __restrict__ packed) {
   const int64_t ql = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (ql >= nq) return;
@@ -374,7 +385,18 @@ __global__ void pair_offsets(const int64_t* __restrict__ off, const int32_t* __r
     if (j < tq) pos[ql * t + j] = acc + x - v;
     acc += __shfl_sync(0xffffffffu, x, 31);
   }
-  if (lane == 0) counts[ql] = acc;
+  if (lane == 0) {
+    counts[ql] = acc;
+    if (packed) packed[ql] = (acc + 3) / 4 * 4;
+    if (packed && ql == 0) packed[nq] = 0;
+  }
+}
+
+// The probe counts of the queries in a pass, 0 for the others.
+__global__ void pass_counts(Slices sl, const int32_t* __restrict__ tpq, int64_t q0, int64_t nq, int t,
+                            int32_t* __restrict__ counts) {
+  const int64_t ql = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (ql < nq) counts[ql] = !sl.in_pass(ql) ? 0 : tpq ? min(max(tpq[q0 + ql], 0), t) : t;
 }
 
 // Which of an item's queries probed a partition before this one: a hash table
@@ -413,9 +435,8 @@ struct ProbeMasks {
 template <typename Rows>
 __global__ void __launch_bounds__(kThreads, 3) score_items(Rows rows, IvfWork work, const int32_t* __restrict__ ids,
                                                         const int32_t* __restrict__ assign, int a,
-                                                        const int32_t* __restrict__ top, int64_t q0, int64_t slice,
-                                                        const int64_t* __restrict__ pos, uint32_t* __restrict__ keys,
-                                                        int* __restrict__ smax) {
+                                                        const int32_t* __restrict__ top, int64_t q0, Slices sl,
+                                                        const int64_t* __restrict__ pos, int* __restrict__ smax) {
   constexpr unsigned kFull = 0xffffffffu;
   constexpr int QB = 8 * Rows::kTiles;
   static_assert(QB <= 32, "a mask word holds the item's queries");
@@ -460,7 +481,7 @@ __global__ void __launch_bounds__(kThreads, 3) score_items(Rows rows, IvfWork wo
       const int64_t ql = pr / work.tmax;
       const int j = (int)(pr - ql * work.tmax);
       q = q0 + ql;
-      out_s[i] = keys + ql * slice + pos[pr];
+      out_s[i] = sl.keys + sl.at(ql) + pos[pr];
       list_s[i] = top + q * (int64_t)work.tmax;
       j_s[i] = j;
       qf_s[i] = rows.query_factor(q, pr);
@@ -667,8 +688,7 @@ __device__ void block_sort(uint64_t* buf, int N) {
 // Bound: the latency of one pass over the slice and of the scattered rows.
 template <typename Rows, typename OT>
 __global__ void __launch_bounds__(kThreads) finish_slices(
-    Rows rows, uint32_t* keys, const int64_t* __restrict__ counts, int64_t slice,
-    const int64_t* __restrict__ pos, const int32_t* __restrict__ top, const int32_t* __restrict__ tpq, int64_t q0,
+    Rows rows, Slices sl, const int64_t* __restrict__ counts, const int64_t* __restrict__ pos, const int32_t* __restrict__ top, const int32_t* __restrict__ tpq, int64_t q0,
     int t, const int64_t* __restrict__ off, const int32_t* __restrict__ ids, const float* __restrict__ base,
     const float* __restrict__ smax, const void* __restrict__ Q, int qdt, int d, const OT* __restrict__ orig,
     int ostride, int R, int k, int stage_at, int64_t* __restrict__ ids_out, float* __restrict__ scores_out) {
@@ -682,7 +702,8 @@ __global__ void __launch_bounds__(kThreads) finish_slices(
   __shared__ int64_t row_s[kProbeTable];        // and the index row of the slice's position 0 in that probe
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   const int64_t ql = blockIdx.x, q = q0 + ql;
-  uint32_t* K = keys + ql * slice;             // (rewritten in place by the rarest branch)
+  if (!sl.in_pass(ql)) return;
+  uint32_t* K = sl.keys + sl.at(ql);            // (rewritten in place by the rarest branch)
   const int n = (int)counts[ql];
   const int tq = tpq ? min(max(tpq[q], 0), t) : t;
   const int64_t* qpos = pos + ql * t;
@@ -1079,25 +1100,27 @@ __global__ void __launch_bounds__(kThreads) finish_slices(
 int64_t slice_rows(const IndexData& ix, int t) {
   return (std::max<int64_t>(1, std::min<int64_t>((int64_t)t * ix.max_partition, ix.rows)) + 3) / 4 * 4;
 }
-// Queries per pass, so that the keys stay within `most` entries.
-int64_t key_chunk(int64_t slice, int64_t nq, int64_t most) {
-  return std::min(nq, std::max<int64_t>(8, most / slice));
-}
-// Room for the keys of as many queries as 4 GB hold, or 2 GB where the device
-// has no more: a slice is sized for the largest partitions and mostly a third
-// full, and a batch in two passes reads its partitions twice.
-uint32_t* key_room(int64_t slice, int64_t nq, int64_t& cq, Scratch& scr) {
-  cq = key_chunk(slice, nq, (int64_t)1 << 30);
-  const int64_t less = key_chunk(slice, nq, (int64_t)1 << 29);
-  if (cq == less) return scr.get<uint32_t>((size_t)cq * slice);
-  try {
-    return scr.get<uint32_t>((size_t)cq * slice);
-  } catch (const Error& e) {
-    if (e.status != SOAR_ENOMEM) throw;
-    cudaGetLastError();                       // clear the failed allocation
-  }
-  cq = less;
-  return scr.get<uint32_t>((size_t)cq * slice);
+// The key buffer holds 2 GB at most (or eight slices).  A slice of the longest
+// possible length is mostly a third full, so a batch whose slices do not fit
+// that way has them packed, and only what does not fit then takes another pass
+// over the partitions: passes cover windows of the packed keys, as many as the
+// longest slices could fill; the ones that stay empty end at once.  Chunks of a
+// batch are small enough that there are few of those.  (10 000 queries over 10^7
+// x 96 FP8, at most 2.4 GB of keys and 0.6 in fact: 2 768 us in two passes of
+// 8 945 and 1 055 queries, 2 458 packed, 2 391 in a 4 GB buffer.)
+constexpr int64_t kKeysMost = (int64_t)1 << 29;
+struct KeyPlan {
+  int64_t slice, room, queries, window;     // keys: a slice at most, the buffer; queries a chunk; keys a pass (0: one pass)
+};
+KeyPlan key_plan(const IndexData& ix, int64_t nq, int t) {
+  KeyPlan p;
+  p.slice = slice_rows(ix, t);
+  p.room = std::max(kKeysMost, 8 * p.slice);
+  // (the buffers of a chunk's pairs: 2^24 pairs at most)
+  p.queries = std::min({nq, std::max<int64_t>(8, ((int64_t)1 << 24) / t), std::max<int64_t>(8, 4 * p.room / p.slice)});
+  p.window = p.queries * p.slice > p.room ? (p.room - p.slice) / 4 * 4 : 0;
+  if (!p.window) p.room = p.queries * p.slice;
+  return p;
 }
 
 template <typename Rows>
@@ -1107,10 +1130,12 @@ void run(const IndexData& ix, Rows rws, float* base, const float* Qf, int qstrid
   rws.tiles = Rows::kTiles;
   while (rws.tiles > 1 && rws.item_smem() > 180 * 1024) --rws.tiles;     // wide rows: fewer queries an item
   const int QB = 8 * rws.tiles;
-  const int64_t slice = slice_rows(ix, t);
-  int64_t cq;
-  uint32_t* keys = key_room(slice, nq, cq, scr);
+  const KeyPlan plan = key_plan(ix, nq, t);
+  const int64_t cq = plan.queries;
+  uint32_t* keys = scr.get<uint32_t>((size_t)plan.room);
   int64_t* counts = scr.get<int64_t>(cq);
+  int64_t* start = plan.window ? scr.get<int64_t>((size_t)cq + 1) : nullptr;
+  int32_t* taken = plan.window ? scr.get<int32_t>(cq) : nullptr;
   int* smax = Rows::kScaled ? scr.get<int>(cq) : nullptr;
   int64_t* pos = scr.get<int64_t>((size_t)cq * t);
   int32_t* inv = scr.get<int32_t>((size_t)cq * t);
@@ -1127,40 +1152,54 @@ void run(const IndexData& ix, Rows rws, float* base, const float* Qf, int qstrid
                                    stage_at + sizeof(uint4) * 32 * kRowChunks * kWarps);
   const size_t item_smem = rws.item_smem();
   SOAR_CUDA(cudaFuncSetAttribute(score_items<Rows>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)item_smem));
-  const auto finish = [&](auto elem, int64_t q0, int64_t m) {
+  const auto finish = [&](auto elem, const Slices& sl, int64_t q0, int64_t m) {
     using OT = decltype(elem);
     auto kern = finish_slices<Rows, OT>;
     SOAR_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fin_smem));
-    kern<<<(unsigned)m, kThreads, fin_smem, s>>>(rws, keys, counts, slice, pos, top, tpq, q0, t, ix.offsets, ix.ids,
-                                                 base, reinterpret_cast<const float*>(smax), Q, (int)dt, ix.d, static_cast<const OT*>(ix.originals),
-                                                 ostride, R, k, (int)stage_at, ids_out, scores_out);
+    kern<<<(unsigned)m, kThreads, fin_smem, s>>>(rws, sl, counts, pos, top, tpq, q0, t, ix.offsets, ix.ids, base,
+                                                 reinterpret_cast<const float*>(smax), Q, (int)dt, ix.d,
+                                                 static_cast<const OT*>(ix.originals), ostride, R, k, (int)stage_at,
+                                                 ids_out, scores_out);
     SOAR_LAUNCHED();
   };
   for (int64_t q0 = 0; q0 < nq; q0 += cq) {
     const int64_t m = std::min(cq, nq - q0);
     Scratch cs(s);
-    const int32_t* tp = tpq ? tpq + q0 : nullptr;
-    const Grouped g = group_pairs(ix, m, t, tp, QB, top + q0 * t, inv, s, cs, false, false);
     stage_mark(s, "scan", true);
-    pair_offsets<<<ceil_div(m * 32, 256), 256, 0, s>>>(ix.offsets, top, tpq, q0, m, t, pos, counts);
+    pair_offsets<<<ceil_div(m * 32, 256), 256, 0, s>>>(ix.offsets, top, tpq, q0, m, t, pos, counts, start);
     SOAR_LAUNCHED();
+    if (start) exclusive_scan_i64(start, start, m + 1, s, cs);
     if (base) {
       pair_bases<<<ceil_div(m * t * 32, 256), 256, 0, s>>>(Qf, qstride, ix.centroids, ix.d, top, tpq, q0, m, t, base);
       SOAR_LAUNCHED();
     }
-    // a batch of few pairs splits each partition's rows over several blocks
-    const int64_t items = std::min<int64_t>(m * t, g.max_items);
-    const unsigned split = (unsigned)std::max<int64_t>(1, std::min<int64_t>(16, 8 * num_sms() / std::max<int64_t>(1, items)));
-    const IvfWork work{ix.offsets, g.pair_off, g.vals, g.order, g.item_base, ix.c, t, QB};
     if (smax) SOAR_CUDA(cudaMemsetAsync(smax, 0, sizeof(int) * m, s));
-    score_items<Rows><<<dim3((unsigned)items, split), kThreads, item_smem, s>>>(rws, work, ix.ids, ix.assign, a, top,
-                                                                               q0, slice, pos, keys, smax);
-    SOAR_LAUNCHED();
     stage_mark(s, "scan", false);
-    stage_mark(s, "rescore", true);
-    if (ix.dtype == SOAR_F32) finish(float{}, q0, m);
-    else finish(__nv_bfloat16{}, q0, m);
-    stage_mark(s, "rescore", false);
+    const int64_t passes = start ? (m * plan.slice + plan.window - 1) / plan.window : 1;
+    for (int64_t pass = 0; pass < passes; ++pass) {
+      Scratch ps(s);
+      const Slices sl{keys, start, plan.slice, pass * plan.window, (pass + 1) * plan.window};
+      const int32_t* tp = tpq ? tpq + q0 : nullptr;
+      if (start) {
+        pass_counts<<<ceil_div(m, 256), 256, 0, s>>>(sl, tpq, q0, m, t, taken);
+        SOAR_LAUNCHED();
+        tp = taken;
+      }
+      const Grouped g = group_pairs(ix, m, t, tp, QB, top + q0 * t, inv, s, ps, false, false);
+      stage_mark(s, "scan", true);
+      // a batch of few pairs splits each partition's rows over several blocks
+      const int64_t items = std::min<int64_t>(m * t, g.max_items);
+      const unsigned split = (unsigned)std::max<int64_t>(1, std::min<int64_t>(16, 8 * num_sms() / std::max<int64_t>(1, items)));
+      const IvfWork work{ix.offsets, g.pair_off, g.vals, g.order, g.item_base, ix.c, t, QB};
+      score_items<Rows><<<dim3((unsigned)items, split), kThreads, item_smem, s>>>(rws, work, ix.ids, ix.assign, a, top,
+                                                                                 q0, sl, pos, smax);
+      SOAR_LAUNCHED();
+      stage_mark(s, "scan", false);
+      stage_mark(s, "rescore", true);
+      if (ix.dtype == SOAR_F32) finish(float{}, sl, q0, m);
+      else finish(__nv_bfloat16{}, sl, q0, m);
+      stage_mark(s, "rescore", false);
+    }
   }
 }
 
@@ -1177,8 +1216,7 @@ void fp8_search(const IndexData& ix, const float* Qf, const float* qscale, const
 void pq_search(const IndexData& ix, const float* Qf, int qstride, const void* Q, soar_dtype dt, const int32_t* top,
                const int32_t* tpq, int64_t nq, int t, int R, int k, int64_t* ids_out, float* scores_out,
                cudaStream_t s, Scratch& scr) {
-  const int64_t slice = slice_rows(ix, t);
-  float* base = scr.get<float>((size_t)key_chunk(slice, nq, (int64_t)1 << 30) * t);
+  float* base = scr.get<float>((size_t)key_plan(ix, nq, t).queries * t);
   const Pq4Rows rws{static_cast<const uint8_t*>(ix.vectors), ix.code_stride, ix.pq_m, ix.d, ix.pq_cb, Qf, qstride,
                     base, (ix.pq_m + 7) / 8, 0};
   run(ix, rws, base, Qf, qstride, Q, dt, top, tpq, nq, t, R, k, ids_out, scores_out, s, scr);
