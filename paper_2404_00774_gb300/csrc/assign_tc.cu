@@ -808,7 +808,7 @@ void assign_tc_pass(const XT* X, int64_t n, int d, const float* C, int c, int nd
   const size_t smem = smem_for(kp, sh.ops, sh.stages, sh.steps, sh.cap);
   auto kern = ndir == 0 ? (sh.ops == 2 ? assign_tc_kernel<0, 2, XT> : assign_tc_kernel<0, 1, XT>)
                         : assign_tc_kernel<1, 2, XT>;
-  SOAR_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  allow_smem(kern, smem);
   const int pts = ndir == 0 && sh.ops == 2 ? 2 * kTM : kTM;
   const int grid = (int)std::min<int64_t>((n + pts - 1) / pts, num_sms());
   kern<<<grid, kThr, smem, s>>>(prm);

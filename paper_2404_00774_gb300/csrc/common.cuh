@@ -51,6 +51,23 @@ struct Error : std::runtime_error {
     ::soar::g_launches.fetch_add(1, std::memory_order_relaxed); \
   } while (0)
 
+// Allows `kern` launches with `need` bytes of dynamic shared memory.  The limit
+// belongs to the process and is never lowered: it goes to all that the kernel's
+// static arrays leave at once, so that host threads launching one kernel with
+// different sizes cannot undercut each other between this call and the launch.
+template <typename Kernel>
+void allow_smem(Kernel kern, size_t need) {
+  cudaFuncAttributes a;
+  SOAR_CUDA(cudaFuncGetAttributes(&a, kern));
+  if (need <= (size_t)a.maxDynamicSharedSizeBytes) return;
+  int dev = 0, most = 0;
+  SOAR_CUDA(cudaGetDevice(&dev));
+  SOAR_CUDA(cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+  most -= (int)a.sharedSizeBytes;
+  // (more than there is: the call fails and says so)
+  SOAR_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, need <= (size_t)most ? most : (int)need));
+}
+
 // ------------------------------------------------------ stream-ordered scratch
 
 // Device scratch taken from the stream-ordered pool and returned on `stream`

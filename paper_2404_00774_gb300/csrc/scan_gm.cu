@@ -914,7 +914,7 @@ __global__ void split_queries_bf16(const float* __restrict__ Qf, int64_t n, int 
 template <typename ET, int NT>
 void launch_gm(int k, int grid, size_t smem, cudaStream_t s, const GmParams& prm) {
   auto kern = k == 10 ? scan_gm_kernel<ET, 10, NT> : scan_gm_kernel<ET, 0, NT>;
-  SOAR_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  allow_smem(kern, smem);
   kern<<<grid, kThreads, smem, s>>>(prm);
   SOAR_LAUNCHED();
 }

@@ -591,7 +591,7 @@ void launch_scan_tc(int k, int kc, int grid, size_t smem, cudaStream_t s, const 
   auto kern = k == 10   ? scan_tc_kernel<ET, 10, true>
               : k <= 16 ? scan_tc_kernel<ET, 16, false>
               : kc <= kCand ? scan_tc_kernel<ET, 32, false> : scan_tc_kernel<ET, 0, false>;   // (heap mode: longer lists)
-  SOAR_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  allow_smem(kern, smem);
   kern<<<grid, kThreads, smem, s>>>(prm);
   SOAR_LAUNCHED();
 }

@@ -755,7 +755,7 @@ void launch_scan(const Work& work, int step_nrc, int max_items, const RowT* rows
   const int xs = scan_xs<RowT>(row_stride);
   const int smem = scan_smem_bytes(xs, k, qb);
   auto kern = scan_kernel<RowT, Work>;
-  SOAR_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  allow_smem(kern, smem);
   int per_sm = 0;
   SOAR_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kThreads, smem));
   if (per_sm < 1) fail(SOAR_EUNSUPPORTED, "scan: shared memory for k too large");
@@ -822,7 +822,7 @@ void select_prepared(const IndexData& ix, const float* Qf, const float* qscale, 
   }
   const int t2 = pow2_at_least(t);
   const int smem = t2 * 8 + (ix.c <= kToptSmemRow ? ix.c * 4 : 0);
-  SOAR_CUDA(cudaFuncSetAttribute(topt_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  allow_smem(topt_kernel, smem);
   topt_kernel<<<(unsigned)nq, 256, smem, s>>>(S, ix.c, t, t2, top, top_s);
   SOAR_LAUNCHED();
 }
@@ -925,7 +925,7 @@ void select_partitions_in(const IndexData& ix, const void* Q, soar_dtype dt, int
   score_centroids(ix, Qf, qscale, nq, qstride, S, s);
   const int t2 = pow2_at_least(t);
   const int smem = t2 * 8 + (ix.c <= kToptSmemRow ? ix.c * 4 : 0);
-  SOAR_CUDA(cudaFuncSetAttribute(topt_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  allow_smem(topt_kernel, smem);
   topt_kernel<<<(unsigned)nq, 256, smem, s>>>(S, ix.c, t, t2, top, top_scores);
   SOAR_LAUNCHED();
 }
@@ -1036,7 +1036,7 @@ void search(const IndexData& ix, const void* Q, soar_dtype dt, int64_t nq, int32
     else
       ivf_scan_typed<__nv_bfloat16>(ix, Qf, qscale, nq, t, tpq, k, partials, inv, top, s, scr);
     const int smem = 4 * t * (int)sizeof(uint16_t);
-    SOAR_CUDA(cudaFuncSetAttribute(merge_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    allow_smem(merge_kernel<true>, smem);
     stage_mark(s, "merge", true);
     merge_kernel<true><<<ceil_div(nq, 4), 128, smem, s>>>(partials, k, nq, t, tpq, inv, 0, k, ids_out, nullptr,
                                                           scores_out);
@@ -1067,7 +1067,7 @@ void merge_topk(const int64_t* ids, const float* scores, int64_t nq, int m, int 
   pack_lists<<<ceil_div(count, 256), 256, 0, s>>>(ids, scores, count, m, len, id_offsets, c);
   SOAR_LAUNCHED();
   const int smem = 4 * m * (int)sizeof(uint16_t);
-  SOAR_CUDA(cudaFuncSetAttribute(merge_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  allow_smem(merge_kernel<false>, smem);
   merge_kernel<false><<<ceil_div(nq, 4), 128, smem, s>>>(c, len, nq, 0, nullptr, nullptr, m, k, ids_out, nullptr,
                                                          scores_out);
   SOAR_LAUNCHED();
@@ -1163,7 +1163,7 @@ void exact_mips(const void* X, soar_dtype xdt, int64_t n, int32_t d, const void*
     launch_scan<__nv_bfloat16, BruteWork>(work, nrc, max_items, static_cast<const __nv_bfloat16*>(rows), stride,
                                           nullptr, nullptr, Qf, nullptr, k, qb, partials, counter, s);
   const int smem = 4 * nrc * (int)sizeof(uint16_t);
-  SOAR_CUDA(cudaFuncSetAttribute(merge_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  allow_smem(merge_kernel<false>, smem);
   merge_kernel<false><<<ceil_div(nq, 4), 128, smem, s>>>(partials, k, nq, 0, nullptr, nullptr, nrc, k, ids_out,
                                                          nullptr, scores_out);
   SOAR_LAUNCHED();

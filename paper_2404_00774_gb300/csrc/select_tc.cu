@@ -441,7 +441,7 @@ void select_tc(const IndexData& ix, const float* Qf, int64_t nq, int qstride, in
   }
   const size_t smem = select_smem_bytes(ix.sel_kp);
   auto kern = t <= 16 ? select_tc_kernel<16> : select_tc_kernel<32>;
-  SOAR_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  allow_smem(kern, smem);
   kern<<<(unsigned)((units + per - 1) / per), kThreads, smem, s>>>(P);
   SOAR_LAUNCHED();
   if (parts > 1) {

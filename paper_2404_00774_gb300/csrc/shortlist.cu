@@ -1151,11 +1151,11 @@ void run(const IndexData& ix, Rows rws, float* base, const float* Qf, int qstrid
   const size_t fin_smem = std::max(kept_at + sizeof(uint64_t) * (size_t)std::max(kept_rows(R), sorted),
                                    stage_at + sizeof(uint4) * 32 * kRowChunks * kWarps);
   const size_t item_smem = rws.item_smem();
-  SOAR_CUDA(cudaFuncSetAttribute(score_items<Rows>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)item_smem));
+  allow_smem(score_items<Rows>, item_smem);
   const auto finish = [&](auto elem, const Slices& sl, int64_t q0, int64_t m) {
     using OT = decltype(elem);
     auto kern = finish_slices<Rows, OT>;
-    SOAR_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fin_smem));
+    allow_smem(kern, fin_smem);
     kern<<<(unsigned)m, kThreads, fin_smem, s>>>(rws, sl, counts, pos, top, tpq, q0, t, ix.offsets, ix.ids, base,
                                                  reinterpret_cast<const float*>(smax), Q, (int)dt, ix.d,
                                                  static_cast<const OT*>(ix.originals), ostride, R, k, (int)stage_at,
