@@ -27,9 +27,10 @@
 // lane.  Each epilogue thread keeps its query's t best (score, id) in
 // registers; a tile's 64 scores are screened 16 at a time against the
 // current t-th best, the survivors parked in shared memory and inserted.
-// Columns arrive in ascending id order and only a strictly larger score is
-// inserted, so equal scores keep the lower centroid id first (the order of
-// the other selection kernels: score descending, id ascending).
+// Columns arrive in ascending id order, a score goes behind its equals and the
+// smaller ones move down in their order, so equal scores keep the lower centroid
+// id first (the order of the other selection kernels: score descending, id
+// ascending).
 // Every mbarrier wait is bounded (about a second); on expiry the CTA raises
 // *err, stops, waits (bounded) for its copies and MMAs in flight, frees its
 // TMEM and returns.
@@ -294,18 +295,16 @@ __global__ void __launch_bounds__(kThreads, 1) select_tc_kernel(SelParams P) {
         if (nvalid < kN) mask &= ch * kChunk >= nvalid ? 0u : nvalid - ch * kChunk >= 32 ? ~0u : (1u << (nvalid - ch * kChunk)) - 1;
         for (; mask; mask &= mask - 1) {
           const int cc = __ffs(mask) - 1;
-          float v = park[cc * kM + m];
+          const float v = park[cc * kM + m];
           if (!(v > cut)) continue;
-          int id = col0 + ch * kChunk + cc;
+          const int id = col0 + ch * kChunk + cc;
+          // v goes in front of the first smaller score and the rest moves down one
+          // place (from the last on, so that each reads its neighbour's old entry)
 #pragma unroll
-          for (int j = 0; j < TMAX; ++j) {
-            const bool gt = v > ts[j];
-            const float tv = ts[j];
-            const int tid = ti[j];
-            ts[j] = gt ? v : tv;
-            ti[j] = gt ? id : tid;
-            v = gt ? tv : v;
-            id = gt ? tid : id;
+          for (int j = TMAX - 1; j >= 0; --j) {
+            const bool gt = v > ts[j], up = j > 0 && v > ts[j > 0 ? j - 1 : 0];
+            ts[j] = up ? ts[j > 0 ? j - 1 : 0] : gt ? v : ts[j];
+            ti[j] = up ? ti[j > 0 ? j - 1 : 0] : gt ? id : ti[j];
           }
           cut = ts[TMAX - 1];
         }
@@ -369,7 +368,7 @@ __global__ void __launch_bounds__(256) merge_parts(const int32_t* __restrict__ i
     for (int u = 0; u < kAhead; ++u) {
       const int64_t at = (q * parts + r0 + u) * t + lane;
       const int32_t id = r0 + u < n && lane < t ? ids[at] : -1;
-      key[u] = id >= 0 ? rank_key(scores[at], (uint32_t)id) : ~0ull;
+      key[u] = id >= 0 ? rank_key(scores[at] + 0.f, (uint32_t)id) : ~0ull;   // (-0 + 0 is 0: equal scores, the lower id first)
     }
 #pragma unroll
     for (int u = 0; u < kAhead; ++u) {

@@ -94,3 +94,26 @@ def test_compressed_search_over_rows_of_very_uneven_length(soar, mode, R, every,
         times.append(_milliseconds(lambda: soar.soar_search(ix, Q, 10, 6, rescore=R)))
         ix.close()
     assert times[1] <= most * times[0], times
+
+
+@pytest.mark.parametrize("c,t", [(350, 1), (350, 7), (2000, 32)])
+def test_selection_of_scores_that_are_zeros_of_either_sign(soar, c, t):
+    """A batch split over the codebook orders equal scores as a whole one does: the lower id first."""
+    g = torch.Generator().manual_seed(c)
+    d = 40
+    C = -torch.rand(c, d, generator=g)                       # products with the query's zeros are negative zeros
+    C[:, 0] = torch.where(torch.rand(c, generator=g) < 0.5, 0.0, -0.0)
+    C[1::2] *= torch.where(torch.rand(c // 2, d, generator=g) < 0.5, 1.0, -1.0)
+    C[5, 0], C[c - 3, 0] = -1.0, 1.0
+    A = torch.arange(c).int()[:, None].contiguous()
+    ix = soar.soar_index_build(C.cuda(), C.cuda(), A.cuda())
+    one = torch.zeros(1, d)
+    one[0, 0] = 1.0
+    want = torch.cat([torch.tensor([c - 3]), torch.tensor([i for i in range(c) if i not in (5, c - 3)])])[:t]
+    for q in (one, -one):
+        if q is not one:
+            want = torch.cat([torch.tensor([5]), torch.tensor([i for i in range(c) if i not in (5, c - 3)])])[:t]
+        for nq in (1, 200, 6000):
+            top = soar.soar_select_partitions(ix, q.expand(nq, d).contiguous().cuda(), t).cpu()
+            assert (top == want.int()).all(), nq
+    ix.close()
