@@ -129,6 +129,12 @@ __device__ __forceinline__ uint64_t rank_key(float score, uint32_t id) {
   return ((uint64_t)(~float_key(score)) << 32) | (uint64_t)id;
 }
 
+// The same, after every real key for a score that is not a number: such a row is
+// never a result.
+__device__ __forceinline__ uint64_t rank_key_of_number(float score, uint32_t id) {
+  return score == score ? rank_key(score, id) : ~0ull;
+}
+
 // Exclusive scan of one value per thread across the block (all threads of
 // the block call it; blockDim.x a multiple of 32); `total` gets the sum.
 template <typename T>

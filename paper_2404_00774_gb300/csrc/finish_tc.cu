@@ -109,7 +109,7 @@ __global__ void __launch_bounds__(T) finish_block(
     if (n == 0) return;
     for (int i = tid; i < n; i += T) {
       const int32_t pos = pend[i];
-      buf[best + i] = rank_key(exact_dot_rm(qv, rows, rs, pos), (uint32_t)ids[pos]);
+      buf[best + i] = rank_key_of_number(exact_dot_rm(qv, rows, rs, pos), (uint32_t)ids[pos]);
     }
     int N = 2;
     while (N < best + n) N <<= 1;
@@ -200,7 +200,7 @@ __global__ void __launch_bounds__(T) finish_block(
           const uint64_t thr = best == k ? buf[k - 1] : ~0ull;
           __syncthreads();
           const int64_t r = r0 + tid;
-          const bool in = r < r1 && rank_key(exact_dot_rm(qv, rows, rs, r), (uint32_t)ids[r]) < thr;
+          const bool in = r < r1 && rank_key_of_number(exact_dot_rm(qv, rows, rs, r), (uint32_t)ids[r]) < thr;
           const unsigned kb = __ballot_sync(kFull, in);
           int at = 0;
           if (lane == 0 && kb) at = atomicAdd(&fill_s, __popc(kb));
@@ -334,7 +334,8 @@ __global__ void __launch_bounds__(256) finish_queries(
       const int64_t nrows = part_off[p + 1] - part_off[p];
       for (int64_t rb = 0; rb < nrows; rb += 32) {
         const int64_t r = rb + lane;
-        const uint64_t key = r < nrows ? rank_key(exact_dot_rm(qv, rows, rs, r0 + r), (uint32_t)ids[r0 + r]) : ~0ull;
+        const uint64_t key =
+            r < nrows ? rank_key_of_number(exact_dot_rm(qv, rows, rs, r0 + r), (uint32_t)ids[r0 + r]) : ~0ull;
         insert_round(key);
       }
     }

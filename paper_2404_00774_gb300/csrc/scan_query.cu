@@ -172,8 +172,8 @@ __global__ void __launch_bounds__(32 * kQmWarps) scan_by_query_kernel(
           acc_b = Chunk<T>::dot(wb[u], qs + (c0 + u) * E, acc_b);
         }
     }
-    const uint64_t ka = ida >= 0 ? rank_key(acc_a, (uint32_t)ida) : ~0ull;   // -1: padding row or past the end
-    const uint64_t kb = idb >= 0 ? rank_key(acc_b, (uint32_t)idb) : ~0ull;
+    const uint64_t ka = ida >= 0 ? rank_key_of_number(acc_a, (uint32_t)ida) : ~0ull;   // -1: padding row or past the end
+    const uint64_t kb = idb >= 0 ? rank_key_of_number(acc_b, (uint32_t)idb) : ~0ull;
     mine = merge_block(mine, ka, __shfl_sync(kFull, mine, 31), lane);
     mine = merge_block(mine, kb, __shfl_sync(kFull, mine, 31), lane);
   }

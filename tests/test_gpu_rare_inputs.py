@@ -117,3 +117,41 @@ def test_selection_of_scores_that_are_zeros_of_either_sign(soar, c, t):
             top = soar.soar_select_partitions(ix, q.expand(nq, d).contiguous().cuda(), t).cpu()
             assert (top == want.int()).all(), nq
     ix.close()
+
+
+@pytest.mark.parametrize("layout,nq,k,t", [
+    ("full", 6, 10, 12), ("full", 300, 10, 12), ("full", 4200, 10, 12), ("full", 300, 100, 12),
+    ("full", 4200, 30, 4), ("tied", 300, 10, 12), ("tied", 4200, 10, 12), ("tied", 300, 100, 12),
+    ("fp8", 300, 10, 12), ("fp8", 300, 100, 12), ("pq4", 300, 10, 12),
+])
+def test_rows_that_are_not_numbers_are_no_results(soar, layout, nq, k, t):
+    """Every tenth row has a NaN: the query-major scan, the tensor-core scans with both finishing kernels (with full
+    candidate lists too) and the compressed layouts return the best of the other rows."""
+    g = torch.Generator().manual_seed(nq + k)
+    n, d, c = 16_000, 24, 40
+    X = torch.nn.functional.normalize(torch.randn(n, d, generator=g), dim=1)
+    Q = torch.nn.functional.normalize(torch.randn(nq, d, generator=g), dim=1)
+    if layout == "tied":
+        X[100:1500] = X[0]
+        Q[::2] = X[0] + 0.05 * Q[::2]
+    C = torch.nn.functional.normalize(torch.randn(c, d, generator=g), dim=1)
+    A = soar.soar_assign(X.cuda(), C.cuda(), 1.0, 1)
+    X[7::10, 3] = float("nan")
+    if layout == "pq4":
+        B = 0.2 * torch.randn(d // 2, 16, 2, generator=g)
+        ix = soar.soar_index_build_pq(X.cuda(), C.cuda(), A, B.cuda())
+    else:
+        ix = soar.soar_index_build(X.cuda(), C.cuda(), A,
+                                   mode=soar.SOAR_SCORE_FP8 if layout == "fp8" else soar.SOAR_SCORE_F32)
+    rescore = 0 if layout in ("full", "tied") else 2000
+    ids, sc = (v.cpu() for v in soar.soar_search(ix, Q.cuda(), k, t, rescore=rescore))
+    top = soar.soar_select_partitions(ix, Q.cuda(), t).cpu()
+    A = A.cpu()
+    for q in torch.linspace(0, nq - 1, 40).long().tolist():
+        inside = torch.isin(A, top[q]).any(1)
+        full = torch.nan_to_num(X.double() @ Q[q].double(), nan=-float("inf"))
+        full = torch.where(inside, full, torch.tensor(-float("inf"), dtype=torch.float64))
+        want = full.topk(k)[0]
+        assert torch.allclose(full[ids[q]], want, rtol=0, atol=1e-5) and ids[q].unique().numel() == k
+        assert torch.allclose(sc[q].double(), want, rtol=0, atol=1e-5)
+    ix.close()
