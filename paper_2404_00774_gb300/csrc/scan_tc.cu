@@ -356,6 +356,7 @@ __global__ void __launch_bounds__(kThreads, 1) scan_tc_kernel(TcParams P) {
       float cut = gq;                                  // rows below cut cannot reach the top k
       int cnt = 0;
       bool ovf = false;
+      float packed = -INFINITY;                        // the cut when the list was last cleared
       // register mode (KMAX > 0): the k best screened scores in the last k
       // of KMAX registers (the first KMAX - k hold +inf, which no insertion
       // passes, so the k-th best is always the last register) and up to
@@ -492,9 +493,10 @@ __global__ void __launch_bounds__(kThreads, 1) scan_tc_kernel(TcParams P) {
             }
           }
           cut = fmaxf(fmaxf(ak, floor_) - 2.f * dlt, gq);   // s~ + dlt < max(L_k, G_q)  <=>  s~ < cut
-          if (a < cut) return;
+          if (ovf || a < cut) return;                // (an overflowed list is not read: its partition is rescanned)
           if constexpr (KMAX > 0) {
-            if (cnt == kCand) {                      // drop candidates that fell below the cut
+            if (cnt == kCand && cut > packed) {      // drop candidates that fell below the cut, once per rise of it
+              packed = cut;
               int w = 0;
               for (int j = 0; j < kCand; ++j)
                 if (cub[j * kM] >= cut) { cub[w * kM] = cub[j * kM]; cpos[w * kM] = cpos[j * kM]; ++w; }
@@ -508,7 +510,8 @@ __global__ void __launch_bounds__(kThreads, 1) scan_tc_kernel(TcParams P) {
               ovf = true;
             }
           } else {
-            if (cnt == P.kc) {                       // drop candidates that fell below the cut
+            if (cnt == P.kc && cut > packed) {
+              packed = cut;
               int w = 0;
               for (int j = 0; j < P.kc; ++j) {
                 const Cand v = glist[j];
@@ -532,6 +535,7 @@ __global__ void __launch_bounds__(kThreads, 1) scan_tc_kernel(TcParams P) {
       if (active && !abort_s) {
         const int64_t e = e0 + jq;
         int w = 0;
+        if (ovf) cnt = 0;
         if constexpr (KMAX > 0) {
           Cand* out = P.cand + e * (int64_t)P.kc;
           for (int j = 0; j < cnt; ++j)

@@ -155,3 +155,28 @@ def test_rows_that_are_not_numbers_are_no_results(soar, layout, nq, k, t):
         assert torch.allclose(full[ids[q]], want, rtol=0, atol=1e-5) and ids[q].unique().numel() == k
         assert torch.allclose(sc[q].double(), want, rtol=0, atol=1e-5)
     ix.close()
+
+
+def _clusters(n, nq, d, comps, sigma):
+    g = torch.Generator(device="cuda").manual_seed(n + d)
+    mu = torch.randn(comps, d, generator=g, device="cuda")
+
+    def draw(rows):
+        at = torch.randint(0, comps, (rows,), generator=g, device="cuda")
+        return torch.nn.functional.normalize(mu[at] + sigma * torch.randn(rows, d, generator=g, device="cuda"), dim=1)
+
+    return draw(n), draw(nq)
+
+
+def test_brute_force_in_clusters_tighter_than_the_screening_band(soar):
+    """Every list overflows, and the rows are rescored whatever k is: k = 17 and k = 100 (other kernels than k = 16) cost
+    a few times as much, and not what clearing a full list at every row does (20 and 70 times)."""
+    X, Q = _clusters(400_000, 700, 16, 5, 0.01)
+    ms = {k: _milliseconds(lambda: soar.soar_exact_mips(X, Q, k)) for k in (16, 17, 100)}
+    assert ms[17] <= 5 * ms[16] and ms[100] <= 10 * ms[16], ms
+    for k in (17, 100):
+        ids, sc = soar.soar_exact_mips(X, Q, k)
+        full = Q[:50].double() @ X.double().T
+        want = full.topk(k, 1)[0]
+        assert torch.allclose(sc[:50].double(), want, rtol=0, atol=1e-5)
+        assert torch.allclose(full.gather(1, ids[:50]), want, rtol=0, atol=1e-5)

@@ -38,8 +38,8 @@ def test_searches_of_different_sizes_from_two_threads(soar):
     fp8 = soar.soar_index_build(X, C, A, mode=soar.SOAR_SCORE_FP8)
     full = soar.soar_index_build(X, C, A)
     assert not _run([lambda: soar.soar_search(fp8, Q, 10, 8, rescore=10),
-                     lambda: soar.soar_search(fp8, Q, 40, 8, rescore=4096)], 500)
-    assert not _run([lambda: soar.soar_search(full, Q, 17, 8), lambda: soar.soar_search(full, Q, 128, 8)], 500)
-    assert not _run([lambda: soar.soar_search(full, Q, 129, 8), lambda: soar.soar_search(full, Q, 700, 8)], 300)
+                     lambda: soar.soar_search(fp8, Q, 40, 8, rescore=4096)], 400)
+    assert not _run([lambda: soar.soar_search(full, Q, 17, 8), lambda: soar.soar_search(full, Q, 128, 8)], 200)
+    assert not _run([lambda: soar.soar_search(full, Q, 129, 8), lambda: soar.soar_search(full, Q, 700, 8)], 60)
     fp8.close()
     full.close()
