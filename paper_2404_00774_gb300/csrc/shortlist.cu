@@ -359,10 +359,11 @@ struct Slices {
 
 // Each probed pair's first position in its query's slice (the sizes of the
 // query's earlier probed partitions added up) and the slice's length, in packed
-// (unless null, [nq + 1]) rounded up to four; a warp per query.
+// (unless null, [nq + 1]) rounded up to four; smax cleared; a warp per query.
 __global__ void pair_offsets(const int64_t* __restrict__ off, const int32_t* __restrict__ top,
                              const int32_t* __restrict__ tpq, int64_t q0, int64_t nq, int t,
-                             int64_t* __restrict__ pos, int64_t* __restrict__ counts, int64_t* __restrict__ packed) {
+                             int64_t* __restrict__ pos, int64_t* __restrict__ counts, int64_t* __restrict__ packed,
+                             int* __restrict__ smax) {
   const int64_t ql = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (ql >= nq) return;
@@ -387,6 +388,7 @@ __global__ void pair_offsets(const int64_t* __restrict__ off, const int32_t* __r
   }
   if (lane == 0) {
     counts[ql] = acc;
+    if (smax) smax[ql] = 0;
     if (packed) packed[ql] = (acc + 3) / 4 * 4;
     if (packed && ql == 0) packed[nq] = 0;
   }
@@ -403,14 +405,23 @@ __global__ void pass_counts(Slices sl, const int32_t* __restrict__ tpq, int64_t 
 // in shared memory from partition to a mask of the item's query slots, so that a
 // row looks its point's other partitions up once for all queries (comparing each
 // query's earlier probes row by row was two thirds of the scoring's
-// instructions).  kHashMost entries at most; an item with more (large t) compares.
-constexpr int kHashSize = 2048, kHashMost = 1024;
+// instructions).  The table is as large as the item's earlier probes or the
+// partitions need, whichever are fewer; an item with more of both compares
+// (50 queries of 200 probes over 400 partitions, two spills: 1 111 us compared, 152
+// hashed).
+constexpr int kHashSize = 4096, kHashMost = 3072;
 struct ProbeMasks {
   int32_t key[kHashSize];
   uint32_t mask[kHashSize];
-  __device__ static int at(int32_t p) { return (int)(((uint32_t)p * 2654435769u) >> 21); }   // 11 bits
-  __device__ void add(int32_t p, uint32_t bit) {
-    for (int h = at(p);; h = (h + 1) & (kHashSize - 1)) {
+  __device__ static int at(int32_t p, int bits) { return (int)(((uint32_t)p * 2654435769u) >> (32 - bits)); }
+  __device__ void clear(int bits) {
+    for (int i = threadIdx.x; i < 1 << bits; i += blockDim.x) {
+      key[i] = -1;
+      mask[i] = 0u;
+    }
+  }
+  __device__ void add(int32_t p, uint32_t bit, int bits) {
+    for (int h = at(p, bits);; h = (h + 1) & ((1 << bits) - 1)) {
       const int32_t old = atomicCAS(&key[h], -1, p);
       if (old == -1 || old == p) {
         atomicOr(&mask[h], bit);
@@ -418,8 +429,8 @@ struct ProbeMasks {
       }
     }
   }
-  __device__ uint32_t find(int32_t p) const {
-    for (int h = at(p);; h = (h + 1) & (kHashSize - 1)) {
+  __device__ uint32_t find(int32_t p, int bits) const {
+    for (int h = at(p, bits);; h = (h + 1) & ((1 << bits) - 1)) {
       const int32_t k = key[h];
       if (k == p) return mask[h];
       if (k == -1) return 0u;
@@ -466,43 +477,46 @@ __global__ void __launch_bounds__(kThreads, 3) score_items(Rows rows, IvfWork wo
   const int64_t r0 = work.part_off[p], r1 = work.part_off[p + 1];
   const int nrows = (int)(r1 - r0);
   rows.stage_shared(sl_smem);
-  if (a > 1)
-    for (int i = threadIdx.x; i < kHashSize; i += kThreads) {
-      masks.key[i] = -1;
-      masks.mask[i] = 0u;
-    }
-  if (threadIdx.x == 0) earlier_s = most_s = 0;
-  __syncthreads();
-  if (threadIdx.x < QB) {                       // a thread per query slot
+  static_assert(QB <= 32, "a warp fills the slots");
+  if (threadIdx.x < 32) {                       // a thread per query slot
     const int i = threadIdx.x;
     int64_t q = -1;
+    int j = 0;
     if (i < nqi) {
       const int pr = work.pair_vals[e0 + i];    // ql * t + j
       const int64_t ql = pr / work.tmax;
-      const int j = (int)(pr - ql * work.tmax);
+      j = (int)(pr - ql * work.tmax);
       q = q0 + ql;
       out_s[i] = sl.keys + sl.at(ql) + pos[pr];
       list_s[i] = top + q * (int64_t)work.tmax;
       j_s[i] = j;
       qf_s[i] = rows.query_factor(q, pr);
-      atomicAdd(&earlier_s, min(j, kHashMost + 1));
     }
-    q_s[i] = q;
+    if (i < QB) q_s[i] = q;
+    j = warp_sum(j);
+    if (i == 0) {
+      earlier_s = j;
+      most_s = 0;
+    }
   }
   __syncthreads();
 #pragma unroll 4
   for (int i = w; i < 8 * rows.tiles; i += kWarps) rows.stage_query(sl_smem, i, q_s[i], lane);
+  const int probed = min(earlier_s, work.c);    // distinct partitions among the earlier probes, at most
+  const bool hashed = probed <= kHashMost;
+  int bits = 6;
+  while (hashed && (1 << bits) < kHashSize && (1 << bits) < 2 * probed) ++bits;
+  if (a > 1 && hashed) masks.clear(bits);
   __syncthreads();
-  const bool hashed = earlier_s <= kHashMost;
   if (a > 1 && hashed) {
     for (int i = w; i < nqi; i += kWarps)
-      for (int jj = lane; jj < j_s[i]; jj += 32) masks.add(list_s[i][jj], 1u << i);
+      for (int jj = lane; jj < j_s[i]; jj += 32) masks.add(list_s[i][jj], 1u << i, bits);
     __syncthreads();
   }
   const int nt = (nqi + 7) / 8, g = lane >> 2, tig = lane & 3;
   // the item's queries whose earlier probes hold the row's point
   const auto dropped = [&](int32_t o) -> uint32_t {
-    if (hashed) return masks.find(o);
+    if (hashed) return masks.find(o, bits);
     uint32_t m = 0u;
     for (int i = 0; i < nqi; ++i)
       for (int jj = 0; jj < j_s[i]; ++jj)
@@ -729,59 +743,62 @@ __global__ void __launch_bounds__(kThreads) finish_slices(
     qrow[i] = i >= d ? 0.f
               : qdt == SOAR_F32 ? static_cast<const float*>(Q)[q * d + i]
                                 : __bfloat162float(static_cast<const __nv_bfloat16*>(Q)[q * d + i]);
-  float3 norms = rows.stage_finish(qs, q, base ? base + ql * t : nullptr, tq);
-  norms.x = warp_sum(norms.x);
-  norms.y = warp_sum(norms.y);
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) norms.z = fmaxf(norms.z, __shfl_xor_sync(kFull, norms.z, o));
   if (tid == 0) n_list = n_band = n_kept = 0;
   if (tid < tq && tid < kProbeTable) {
     at_s[tid] = (int)qpos[tid];
     row_s[tid] = off[probes[tid]] - qpos[tid];
   }
-  // a sample and its range
+  const bool short_slice = n <= R;              // every row that counts is listed
   uint32_t sample[kSample];
-  float lo = INFINITY, hi = -INFINITY;
+  float lo = INFINITY, hi = -INFINITY, delta = 0.f;
+  if (!short_slice) {
+    float3 norms = rows.stage_finish(qs, q, base ? base + ql * t : nullptr, tq);
+    norms.x = warp_sum(norms.x);
+    norms.y = warp_sum(norms.y);
 #pragma unroll
-  for (int u = 0; u < kSample; ++u) {
-    const int64_t i = (int64_t)(u * kThreads + tid) * n / (kSample * kThreads);
-    sample[u] = i < n ? K[i] : 0u;
-  }
+    for (int o = 16; o > 0; o >>= 1) norms.z = fmaxf(norms.z, __shfl_xor_sync(kFull, norms.z, o));
+    // a sample and its range
 #pragma unroll
-  for (int u = 0; u < kSample; ++u)
-    if (sample[u]) {
-      lo = fminf(lo, key_float(sample[u]));
-      hi = fmaxf(hi, key_float(sample[u]));
+    for (int u = 0; u < kSample; ++u) {
+      const int64_t i = (int64_t)(u * kThreads + tid) * n / (kSample * kThreads);
+      sample[u] = i < n ? K[i] : 0u;
     }
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    lo = fminf(lo, __shfl_xor_sync(kFull, lo, o));
-    hi = fmaxf(hi, __shfl_xor_sync(kFull, hi, o));
-  }
-  if (lane == 0) {
-    red_s[0][w] = lo;
-    red_s[1][w] = hi;
-    red_s[2][w] = norms.x;
-    red_s[3][w] = norms.y;
-    red_s[4][w] = norms.z;
-  }
-  __syncthreads();
-  if (tid == 0) {
-    for (int u = 1; u < kWarps; ++u) {
-      lo = fminf(lo, red_s[0][u]);
-      hi = fmaxf(hi, red_s[1][u]);
-      norms.x += red_s[2][u];
-      norms.y += red_s[3][u];
-      norms.z = fmaxf(norms.z, red_s[4][u]);
+    for (int u = 0; u < kSample; ++u)
+      if (sample[u]) {
+        lo = fminf(lo, key_float(sample[u]));
+        hi = fmaxf(hi, key_float(sample[u]));
+      }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      lo = fminf(lo, __shfl_xor_sync(kFull, lo, o));
+      hi = fmaxf(hi, __shfl_xor_sync(kFull, hi, o));
     }
-    lo_s = lo;
-    hi_s = hi;
-    delta_s = rows.delta(norms, q, smax ? smax[ql] : 0.f);
+    if (lane == 0) {
+      red_s[0][w] = lo;
+      red_s[1][w] = hi;
+      red_s[2][w] = norms.x;
+      red_s[3][w] = norms.y;
+      red_s[4][w] = norms.z;
+    }
+    __syncthreads();
+    if (tid == 0) {
+      for (int u = 1; u < kWarps; ++u) {
+        lo = fminf(lo, red_s[0][u]);
+        hi = fmaxf(hi, red_s[1][u]);
+        norms.x += red_s[2][u];
+        norms.y += red_s[3][u];
+        norms.z = fmaxf(norms.z, red_s[4][u]);
+      }
+      lo_s = lo;
+      hi_s = hi;
+      delta_s = rows.delta(norms, q, smax ? smax[ql] : 0.f);
+    }
+    __syncthreads();
+    lo = lo_s;
+    hi = hi_s;
+    delta = delta_s;
   }
-  __syncthreads();
-  lo = lo_s;
-  hi = hi_s;
-  const float delta = delta_s;
   // position i of the slice: its probe, its row
   const bool in_table = tq <= kProbeTable;
   const auto probe_of = [&](int i) {
@@ -914,7 +931,7 @@ __global__ void __launch_bounds__(kThreads) finish_slices(
   };
 
   uint32_t floor_key = 1u;                              // every row that counts
-  bool finite = n <= cap || set_bins();
+  const bool finite = !short_slice && (n <= cap || set_bins());
   if (n > cap && finite) {
 #pragma unroll
     for (int u = 0; u < kSample; ++u)
@@ -971,7 +988,7 @@ __global__ void __launch_bounds__(kThreads) finish_slices(
   }
   __syncthreads();
   const int m_kept = n_kept;
-  bool done = false, few = false;                       // few: every row that counts is kept, and at most R are
+  bool done = false, few = short_slice;                 // few: at most R rows count
   if (finite && m_kept <= cap) {
     if (floor_key == 1u && m_kept <= R) {
       few = true;
@@ -1166,14 +1183,13 @@ void run(const IndexData& ix, Rows rws, float* base, const float* Qf, int qstrid
     const int64_t m = std::min(cq, nq - q0);
     Scratch cs(s);
     stage_mark(s, "scan", true);
-    pair_offsets<<<ceil_div(m * 32, 256), 256, 0, s>>>(ix.offsets, top, tpq, q0, m, t, pos, counts, start);
+    pair_offsets<<<ceil_div(m * 32, 256), 256, 0, s>>>(ix.offsets, top, tpq, q0, m, t, pos, counts, start, smax);
     SOAR_LAUNCHED();
     if (start) exclusive_scan_i64(start, start, m + 1, s, cs);
     if (base) {
       pair_bases<<<ceil_div(m * t * 32, 256), 256, 0, s>>>(Qf, qstride, ix.centroids, ix.d, top, tpq, q0, m, t, base);
       SOAR_LAUNCHED();
     }
-    if (smax) SOAR_CUDA(cudaMemsetAsync(smax, 0, sizeof(int) * m, s));
     stage_mark(s, "scan", false);
     const int64_t passes = start ? (m * plan.slice + plan.window - 1) / plan.window : 1;
     for (int64_t pass = 0; pass < passes; ++pass) {

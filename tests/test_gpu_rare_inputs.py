@@ -180,3 +180,20 @@ def test_brute_force_in_clusters_tighter_than_the_screening_band(soar):
         want = full.topk(k, 1)[0]
         assert torch.allclose(sc[:50].double(), want, rtol=0, atol=1e-5)
         assert torch.allclose(full.gather(1, ids[:50]), want, rtol=0, atol=1e-5)
+
+
+@pytest.mark.parametrize("spills", [1, 2])
+def test_compressed_search_of_many_probes(soar, spills):
+    """200 probes a query for 50 queries score as many rows as 20 for 500: which earlier probes hold a row's point is
+    looked up in both, and not compared probe by probe (nine times the time with two spills)."""
+    n, d, c = 20_000, 64, 400
+    g = torch.Generator(device="cuda").manual_seed(1)
+    X = torch.nn.functional.normalize(torch.randn(n, d, generator=g, device="cuda"), dim=1)
+    Q = torch.nn.functional.normalize(torch.randn(500, d, generator=g, device="cuda"), dim=1)
+    C = X[:c].contiguous()
+    A = soar.soar_assign(X, C, 1.0, spills)
+    ix = soar.soar_index_build(X, C, A, mode=soar.SOAR_SCORE_FP8)
+    few = _milliseconds(lambda: soar.soar_search(ix, Q, 10, 20, rescore=100))
+    many = _milliseconds(lambda: soar.soar_search(ix, Q[:50].contiguous(), 10, 200, rescore=100))
+    assert many <= (2.5 if spills == 1 else 4) * few, (few, many)
+    ix.close()

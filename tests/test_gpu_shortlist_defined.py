@@ -134,3 +134,21 @@ def test_pq4_shortlist_is_the_defined_one(soar, pattern, d, R, k):
         scores[:, :, col] = lanes[:, :, 0][:, A[:, col]] + acc
     _check(soar, ix, c, A, X, Q, scores, t, R, k)
     ix.close()
+
+
+@pytest.mark.parametrize("n,c,t,spills", [
+    (3000, 300, 250, 1), (3000, 300, 250, 2),       # more earlier probes than the largest table, fewer partitions
+    (9000, 4000, 900, 2),                           # more of both than the largest table: compared
+    (700, 100, 3, 1),                               # fewer rows than the shortlist
+])
+def test_fp8_shortlist_of_many_probes(soar, n, c, t, spills):
+    g = torch.Generator().manual_seed(n)
+    d, nq = 24, 12
+    X = _rows("even", n, d, g)
+    Q = torch.nn.functional.normalize(torch.randn(nq, d, generator=g), dim=1)
+    C = X[torch.randperm(n, generator=g)[:c]].contiguous()
+    A = soar.soar_assign(X.cuda(), C.cuda(), 1.0, spills)
+    ix = soar.soar_index_build(X.cuda(), C.cuda(), A, mode=soar.SOAR_SCORE_FP8)
+    s = _fp8_scores(soar, Q, X)
+    _check(soar, ix, c, A.cpu().long(), X, Q, s[:, :, None].expand(-1, -1, 1 + spills), t, 200, 200)
+    ix.close()
