@@ -69,8 +69,12 @@ constexpr int kMaxStages = 8;
 constexpr int kNB = 4;         // TMEM accumulators (a tile's columns each)
 constexpr int kRing = 4;       // item descriptions in flight
 constexpr int kGK = 16;        // group maxima kept per query (k <= kGK)
-// candidate rows held per query slot in shared memory
-__host__ __device__ constexpr int cap_for(int nt) { return nt == 1 ? 32 : 16; }
+// Candidate rows held per query slot in shared memory; 128-row tiles leave room for
+// fewer on wide rows.  The list always holds the k best so far and is cleared of
+// stale rows only when it is full: cleared with eight places left, lists of 16
+// were cleared at nearly every candidate from k = 9 on (brute force of 1 000
+// queries over 1.18 M x 96, k = 10, the scan: 1 458 us, now 967).
+constexpr int kCapMost = 32, kCapLeast = 16;
 
 struct GmParams {
   IvfWork work;
@@ -83,6 +87,7 @@ struct GmParams {
   float dscale;            // delta / (||q|| max_p ||x||)
   int k;
   int kc;                  // candidates per pair in the global list
+  int cap;                 // candidates per query slot in shared memory
   int stages;
   long long wait_limit;
   int* counter;            // work-item counter
@@ -138,7 +143,7 @@ __global__ void __launch_bounds__(kThreads, 1) scan_gm_kernel(GmParams P) {
   const uint32_t sbo = (uint32_t)kp * 8u * es;         // bytes between 8-row groups
   const uint32_t a_part = (uint32_t)kM * kp * es;      // one A part (bf16: hi or lo)
   const uint32_t a_bytes = (es == 4 ? 1u : 2u) * a_part;   // one A operand buffer
-  constexpr int kCap = cap_for(NT);
+  const int kCap = NT == 1 ? kCapMost : P.cap;
   constexpr int kTile = NT * kN;                       // rows per tile
   constexpr int kTG = kTile / 8;                       // 8-row groups per tile
   constexpr int kStageAt = NT == 1 ? 2 : 1;            // the next item's A buffer is released after this many tiles
@@ -523,7 +528,7 @@ __global__ void __launch_bounds__(kThreads, 1) scan_gm_kernel(GmParams P) {
               if (j2 < k) ak = fminf(ak, gt[j2]);
           }
           cut = fmaxf(ak - 2.f * dlt, gq);
-          const float cut0 = active ? cut : INFINITY;
+          const float cut0 = active && !ovf ? cut : INFINITY;
           uint32_t gm = 0u;                           // eight-row groups holding a row at or above the cut
 #pragma unroll
           for (int q8 = 0; q8 < 8; ++q8) gm |= (g[q8] >= cut0 ? 1u : 0u) << q8;
@@ -612,7 +617,7 @@ __global__ void __launch_bounds__(kThreads, 1) scan_gm_kernel(GmParams P) {
               if (j2 < k) ak = fminf(ak, gt[j2]);
           }
           cut = fmaxf(ak - 2.f * dlt, gq);              // s~ + dlt < max(L_k, G_q)  <=>  s~ < cut
-          const float cut0 = active ? cut : INFINITY;
+          const float cut0 = active && !ovf ? cut : INFINITY;
           uint32_t gm = 0u;                             // groups holding a row at or above the cut
 #pragma unroll
           for (int q4 = 0; q4 < 16; ++q4) gm |= (gu[q4] >= cut0 ? 1u : 0u) << q4;
@@ -768,7 +773,7 @@ __global__ void __launch_bounds__(kThreads, 1) scan_gm_kernel(GmParams P) {
               if (j2 < k) ak = fminf(ak, gt[j2]);
           }
           cut = fmaxf(ak - 2.f * dlt, gq);            // s~ + dlt < max(L_k, G_q)  <=>  s~ < cut
-          const float cut0 = active ? cut : INFINITY;
+          const float cut0 = active && !ovf ? cut : INFINITY;
           // 32 columns at a time, the warp in step: one trip per group of eight that
           // holds a candidate of the lane with the most such groups, in it one per
           // row; a full shared list first drops what fell below the cut, once per
@@ -792,7 +797,7 @@ __global__ void __launch_bounds__(kThreads, 1) scan_gm_kernel(GmParams P) {
                 em |= (w[u] >= cut0 && c0 + u < nvalid ? 1u : 0u) << u;
               }
               if (q8 < 0) em = 0u;
-              if (em && cnt + 8 > kCap && cut > packed) {
+              if (cnt + __popc(em) > kCap && cut > packed) {
                 packed = cut;
                 int n = 0;
 #pragma unroll 1
@@ -875,28 +880,44 @@ __global__ void __launch_bounds__(kThreads, 1) scan_gm_kernel(GmParams P) {
   if (warp == 1) tc::tmem_dealloc(tmem, kNB * kTile);
 }
 
-size_t gm_smem_bytes(int kp, int nt, int stages, int es) {
+size_t gm_smem_bytes(int kp, int nt, int stages, int es, int cap) {
   // each of the two A buffers takes kM * kp * 4 bytes (fp32, or bf16 hi and lo); the
   // parking area kN * kM * 4, the candidate lists 2 * cap * kM * 4
   return 1024 + (size_t)2 * kM * kp * 4 + (size_t)stages * nt * kN * kp * es + (nt == 1 ? (size_t)kN * kM * 4 : 0) +
-         (size_t)2 * cap_for(nt) * kM * 4 + (size_t)(2 * stages + 2 * kNB + 2 * kRing + 4) * 8;
+         (size_t)2 * cap * kM * 4 + (size_t)(2 * stages + 2 * kNB + 2 * kRing + 4) * 8;
 }
 
+constexpr size_t kGmSmem = 227 * 1024 - 1024;   // room for the static shared variables
 int gm_pick_stages(int kp, int nt, int es) {
   for (int s = kMaxStages / nt; s >= 2; --s)
-    if (gm_smem_bytes(kp, nt, s, es) <= 227 * 1024 - 1024) return s;   // room for the static shared variables
+    if (gm_smem_bytes(kp, nt, s, es, nt == 1 ? kCapMost : kCapLeast) <= kGmSmem) return s;
   return 0;
 }
+int gm_pick_cap(int kp, int nt, int stages, int es) {
+  int cap = kCapMost;
+  while (cap > kCapLeast && gm_smem_bytes(kp, nt, stages, es, cap) > kGmSmem) --cap;
+  return cap;
+}
 
-// 64-row halves of a tile.  Long partitions take 128-row tiles, since the MMAs
-// and not the survivors set their pace (brute force of 10 000 queries over chunks
-// of 65 536 fp32 rows of 100: 8.17 ms with 64-row tiles, 6.75 with 128-row ones);
-// short ones keep 64-row tiles and parking (1 200 fp32 rows: 334 us, against 356
+// 64-row halves of a tile.  Long partitions of wide rows take 128-row tiles, since
+// the MMAs and not the survivors set their pace, and so do k > 10, whose survivors
+// overflow the 64-row kernel's lists, which are cleared only at an item's end.
+// Measured, us, 64-row / 128-row tiles:
+//   brute force, 4 000 queries over 600 000 broad rows, fp32, k = 10: 64 columns
+//     1 469 / 1 838, 80 1 605 / 1 925, 96 1 844 / 1 921; 10 000 over 1.18 M x 100
+//     8 213 / 6 614; k = 16: 64 columns 29 257 / 2 488, 96 51 817 / 2 625
+//   the same in bf16, k = 10: 64 columns 1 402 / 1 678, 96 1 631 / 1 706, 128 1 912
+//     / 1 736; k = 16: 64 columns 4 330 / 2 198
+//   700 queries probing 4 of 8 partitions, k = 10: 64 columns 1 942 / 2 230, 96
+//     2 628 / 2 337
+// Short ones keep 64-row tiles and parking (1 200 fp32 rows: 334 us, against 356
 // with 128-row tiles; 2 000 bf16 rows: 1.62 ms against 1.54 to 1.90).
 constexpr int64_t kLongPartition = 8192;   // average rows
-int gm_halves(const IndexData& ix) {
+constexpr int kWideRow = 88;               // columns
+int gm_halves(const IndexData& ix, int k) {
   const int es = ix.dtype == SOAR_F32 ? 4 : 2;
-  return ix.rows >= kLongPartition * ix.c && gm_pick_stages(ix.tc_kp, 2, es) >= 2 ? 2 : 1;
+  return ix.rows >= kLongPartition * ix.c && (k > 10 || ix.tc_kp >= kWideRow) && gm_pick_stages(ix.tc_kp, 2, es) >= 2
+             ? 2 : 1;
 }
 
 // the bf16 query operand: per query its hi row bf16(q) and lo row bf16(q - hi)
@@ -930,8 +951,9 @@ void scan_gm_launch(const IndexData& ix, const IvfWork& work, int grid, const fl
                     int64_t nq, int k, int kc, float dscale, long long wait_limit, int* counter, int* err,
                     unsigned* gbound, Cand* lists, int2* hdr, cudaStream_t s, Scratch& scr) {
   const int es = ix.dtype == SOAR_F32 ? 4 : 2;
-  const int nt = gm_halves(ix), stages = gm_pick_stages(ix.tc_kp, nt, es);
+  const int nt = gm_halves(ix, k), stages = gm_pick_stages(ix.tc_kp, nt, es);
   if (k < 1 || k > kGK || stages < 2) fail(SOAR_EUNSUPPORTED, "group-maxima scan: unsupported k or row width");
+  const int cap = gm_pick_cap(ix.tc_kp, nt, stages, es);
   const void* Qa = Qf;
   if (es == 2) {
     __nv_bfloat16* qhl = scr.get<__nv_bfloat16>((size_t)nq * 2 * ix.tc_kp);
@@ -940,9 +962,9 @@ void scan_gm_launch(const IndexData& ix, const IvfWork& work, int grid, const fl
     SOAR_LAUNCHED();
     Qa = qhl;
   }
-  GmParams prm{work, ix.tc_rows, ix.tc_gstart, ix.tc_pmax, Qa, qnorm, ix.tc_kp, dscale, k, kc, stages, wait_limit,
+  GmParams prm{work, ix.tc_rows, ix.tc_gstart, ix.tc_pmax, Qa, qnorm, ix.tc_kp, dscale, k, kc, cap, stages, wait_limit,
                counter, err, gbound, lists, hdr};
-  const size_t smem = gm_smem_bytes(ix.tc_kp, nt, stages, es);
+  const size_t smem = gm_smem_bytes(ix.tc_kp, nt, stages, es, cap);
   if (es == 4) nt == 2 ? launch_gm<float, 2>(k, grid, smem, s, prm) : launch_gm<float, 1>(k, grid, smem, s, prm);
   else nt == 2 ? launch_gm<__nv_bfloat16, 2>(k, grid, smem, s, prm) : launch_gm<__nv_bfloat16, 1>(k, grid, smem, s, prm);
 }
