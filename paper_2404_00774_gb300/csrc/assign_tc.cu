@@ -91,7 +91,7 @@ struct AsgParams {
   int32_t* queue;         // [n] points left to the refine: with candidates from the front, flagged ones from the back
   uint64_t* best;         // [n] the flagged points' best keys so far (set to none here)
   int* qcount;            // [2] how many of each
-  int vec;                // fp32 rows, d % 4 == 0, X and C 16-byte aligned: 16-byte copies
+  int vec;                // rows of whole 16-byte pieces, X and C 16-byte aligned: 16-byte copies (fp32) or loads
 };
 
 __device__ __forceinline__ float ld(const float* p) { return __ldg(p); }
@@ -118,7 +118,7 @@ __global__ void __launch_bounds__(kThr, 1) assign_tc_kernel(AsgParams<XT> P) {
   unsigned char* sB = base + (size_t)OPS * a_bytes;
   float* list_lb = reinterpret_cast<float*>(sB + (size_t)S * stage_bytes);   // [cap][kEpi]
   int* list_id = reinterpret_cast<int*>(list_lb + P.cap * kEpi);             // [cap][kEpi]
-  float* nx_s = reinterpret_cast<float*>(list_id + P.cap * kEpi);            // [kEpi] ||x||
+  float* nx_s = reinterpret_cast<float*>(list_id + P.cap * kEpi);            // [kEpi] ||x||^2 (one operand: of either half of the columns)
   float* mu_s = nx_s + kEpi;                                                // [kTM] U of the second half
   float* mev_s = mu_s + kTM;                                                // [kTM]
   int* mcnt_s = reinterpret_cast<int*>(mev_s + kTM);                        // [kTM]
@@ -203,8 +203,9 @@ __global__ void __launch_bounds__(kThr, 1) assign_tc_kernel(AsgParams<XT> P) {
 
       // ---- A operands: a thread stages one row, rounded to tf32 and closed by
       // (-1/2, -1/2) in columns d, d + 1 against the codebook's (hi, lo) split of
-      // ||c||^2; with residuals, the second half of the threads stages those
-      if (warp >= 3 && (OPS == 2 || hh == 0)) {
+      // ||c||^2; with residuals, the second half of the threads stages those, with a
+      // single operand the second half of its columns
+      if (warp >= 3) {
         const bool resid = NDIR > 0 && hh == 1;
         float* row = reinterpret_cast<float*>(sA + (size_t)(OPS == 2 ? hh : 0) * a_bytes) + (m >> 3) * (kp * 8) + (m & 7) * 4;
         float inv = 0.f;
@@ -217,19 +218,32 @@ __global__ void __launch_bounds__(kThr, 1) assign_tc_kernel(AsgParams<XT> P) {
         }
         float ss = 0.f, xd = 0.f;
         const bool vec = std::is_same<XT, float>::value && P.vec;
-        const int d4 = vec ? P.d / 4 : 0;               // 16-byte chunks staged by cp.async
+        const bool vec8 = !std::is_same<XT, float>::value && P.vec;   // bf16: 8 columns a load
+        const int d4 = P.vec ? P.d / 4 : 0;             // 4-column chunks in 16-byte loads
+        const int mid = OPS == 1 ? kp / 16 * 2 : 0;
+        const int c0 = OPS == 1 && hh == 1 ? mid : 0, c1 = OPS == 1 && hh == 0 ? mid : kp / 4;   // this thread's chunks
         if (vec && active) {
           const float* xsrc = reinterpret_cast<const float*>(P.X) + p * P.d;
-          for (int k4 = 0; k4 < d4; ++k4) tc::cp_async16(tc::smem_u32(row + k4 * 32), xsrc + 4 * k4);
+          for (int k4 = c0; k4 < min(c1, d4); ++k4) tc::cp_async16(tc::smem_u32(row + k4 * 32), xsrc + 4 * k4);
         }
         tc::cp_async_wait_all();
+        uint4 eight = make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll 4
-        for (int k4 = 0; k4 < kp / 4; ++k4) {
+        for (int k4 = c0; k4 < c1; ++k4) {
           float xv[4], cv[4] = {0.f, 0.f, 0.f, 0.f};
           if (k4 < d4) {
             if (active) {
-              const float4 a = *reinterpret_cast<const float4*>(row + k4 * 32);
-              xv[0] = a.x; xv[1] = a.y; xv[2] = a.z; xv[3] = a.w;
+              if (vec8) {                               // (c0 is even, and so is d4)
+                if (k4 % 2 == 0) eight = __ldg(reinterpret_cast<const uint4*>(P.X + p * P.d + 4 * k4));
+                const uint32_t lo = k4 % 2 ? eight.z : eight.x, hi = k4 % 2 ? eight.w : eight.y;
+                xv[0] = __uint_as_float(lo << 16);
+                xv[1] = __uint_as_float(lo & 0xffff0000u);
+                xv[2] = __uint_as_float(hi << 16);
+                xv[3] = __uint_as_float(hi & 0xffff0000u);
+              } else {
+                const float4 a = *reinterpret_cast<const float4*>(row + k4 * 32);
+                xv[0] = a.x; xv[1] = a.y; xv[2] = a.z; xv[3] = a.w;
+              }
               if (resid) {
                 const float4 b = __ldg(reinterpret_cast<const float4*>(cr + 4 * k4));
                 cv[0] = b.x; cv[1] = b.y; cv[2] = b.z; cv[3] = b.w;
@@ -265,7 +279,7 @@ __global__ void __launch_bounds__(kThr, 1) assign_tc_kernel(AsgParams<XT> P) {
           rn_s[m] = inv > 0.f ? 1.f : 0.f;
           prior_s[m] = prior;
         } else {
-          nx_s[mp] = sqrtf(ss);
+          nx_s[OPS == 1 ? m + kTM * hh : mp] = ss;
         }
         tc::fence_async_smem();
       }
@@ -329,7 +343,7 @@ __global__ void __launch_bounds__(kThr, 1) assign_tc_kernel(AsgParams<XT> P) {
         int cnt = 0;
         float U = INFINITY, packed = INFINITY;         // packed: U when the list was last cleared of stale entries
         float ev = INFINITY;                           // the smallest lower bound the list had no room for
-        const float nx = nx_s[mp], nx2 = nx * nx;
+        const float nx = sqrtf(OPS == 1 ? nx_s[m] + nx_s[m + kTM] : nx_s[mp]), nx2 = nx * nx;
         const float xr = NDIR > 0 ? xr_s[m] : 0.f, er0 = NDIR > 0 ? ldexpf(rn_s[m], -10) * 1.0625f : 0.f;
         const int prior = NDIR > 0 ? prior_s[m] : -1;
         const float lam = P.lambda;
@@ -652,7 +666,8 @@ __global__ void __launch_bounds__(kFlagThreads) refine_flagged(const XT* __restr
         }
         __syncthreads();
 #pragma unroll
-        for (int kk = 0; kk < kFk; ++kk) {           // (zeros past d add nothing)
+        for (int kk = 0; kk < kFk; ++kk) {
+          if (kk >= d - k0) break;                   // uniform
           const float4 xq = *reinterpret_cast<const float4*>(&xs[kk][4 * ty]);
           const float4 cq = *reinterpret_cast<const float4*>(&cs[kk][4 * tx]);
           const float xv[4] = {xq.x, xq.y, xq.z, xq.w}, cv[4] = {cq.x, cq.y, cq.z, cq.w};
@@ -765,8 +780,8 @@ int kp_for(int d) { return (d + 2 + 7) / 8 * 8; }
 struct Shape {
   int ops = 0, stages = 0, steps = 0, cap = 0;
 };
-Shape shape_for(int kp, int ndir) {
-  for (int ops = 2; ops >= (ndir ? 2 : 1); --ops)
+Shape shape_for(int kp, int ndir, int most_ops = 2) {
+  for (int ops = most_ops; ops >= (ndir ? 2 : 1); --ops)
     for (int cap : {16, 8})
       for (int steps : {8, 4})
         for (int s = kStagesMax; s >= 2; --s)
@@ -777,13 +792,23 @@ Shape shape_for(int kp, int ndir) {
 
 }  // namespace
 
-bool assign_tc_supported(int d, int ndir) { return ndir <= 1 && shape_for(kp_for(d), ndir).ops > 0; }
+// Wide rows (a primary past 278 columns, a spill past 134) of few points against a
+// small codebook go to the general kernels, which take fewer launches (us, here /
+// there: primary of 300 columns, 2 000 x 64 81 / 57, 10 000 x 64 82 / 76, 10 000 x
+// 128 74 / 116, 100 000 x 2 225 / 342; spill of 150, 2 000 x 64 66 / 38, 10 000 x 64
+// 70 / 64, 10 000 x 128 71 / 101, 100 000 x 2 227 / 312).
+bool assign_tc_usable(int64_t n, int d, int c, int ndir) {
+  if (ndir > 1 || shape_for(kp_for(d), ndir).ops == 0) return false;
+  return d <= (ndir ? 134 : 278) || n > 16384 || c > 64;
+}
 
 template <typename XT>
 void assign_tc_pass(const XT* X, int64_t n, int d, const float* C, int c, int ndir, int32_t* assign, int astride,
                     const float* inv_rn, float lambda, cudaStream_t s, Scratch& scr) {
   const int kp = kp_for(d);
-  const Shape sh = shape_for(kp, ndir);
+  // few points: 128 of them a block, so that twice as many SMs work (1 000 to 19 000
+  // x 100 against 500 centroids: 72 -> 65 us)
+  const Shape sh = shape_for(kp, ndir, ndir == 0 && n <= (int64_t)kTM * num_sms() ? 1 : 2);
   if (ndir > 1 || sh.ops == 0) fail(SOAR_EUNSUPPORTED, "tensor-core assignment: unsupported shape");
   const int ctiles = (c + kN - 1) / kN;
   float* Cc = scr.get<float>((size_t)ctiles * kN * kp);
@@ -801,7 +826,7 @@ void assign_tc_pass(const XT* X, int64_t n, int d, const float* C, int c, int nd
   uint64_t* best = scr.get<uint64_t>(n);
   int* qcount = scr.get<int>(2);             // queued points
   SOAR_CUDA(cudaMemsetAsync(qcount, 0, 2 * sizeof(int), s));
-  const int vec = std::is_same<XT, float>::value && d % 4 == 0 && reinterpret_cast<uintptr_t>(X) % 16 == 0 &&
+  const int vec = d * sizeof(XT) % 16 == 0 && reinterpret_cast<uintptr_t>(X) % 16 == 0 &&
                   reinterpret_cast<uintptr_t>(C) % 16 == 0;
   AsgParams<XT> prm{X, n, d, kp, Cc, tmax, C, c, ctiles, assign, astride, inv_rn, lambda, sh.stages,
                     sh.steps, sh.cap, device_error_word(), cand, queue, best, qcount, vec};
