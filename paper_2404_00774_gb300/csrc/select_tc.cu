@@ -416,14 +416,16 @@ bool select_tc_usable(const IndexData& ix, const float* Qf, int qstride, int t) 
 // afresh, which pays from about forty tiles a CTA on (10 000 queries, t = 5,
 // against 10 000 centroids, 82 tiles a CTA: 289 -> 186 us with the merge; against
 // 2 000, 17 tiles: 80 + 18 against 87), or where most SMs have nothing else to do
-// (one query against 2 000: 67 -> 17 us), with at least two tiles a CTA.
+// (one query against 2 000: 67 -> 17 us), with at least two tiles a CTA.  Fewer than
+// eight tiles take less than the merge (d = 32, us, whole / split: 320 centroids, one
+// query 20 / 23, 700 31 / 38; 512, 23 / 23 and 36 / 29; 2 000, 42 / 30 and 68 / 40).
 void select_tc(const IndexData& ix, const float* Qf, int64_t nq, int qstride, int t, int32_t* top, float* top_s,
                cudaStream_t s, Scratch* scr) {
   SOAR_REQUIRE(select_tc_usable(ix, Qf, qstride, t), "tensor-core selection not applicable");
   if (nq == 0) return;
   const int64_t blocks = (nq + kM - 1) / kM, units = blocks * ix.sel_tiles;
   int64_t per = ix.sel_tiles;
-  if (scr && blocks < 2 * num_sms()) {
+  if (scr && ix.sel_tiles >= 8 && blocks < 2 * num_sms()) {
     const int64_t even = std::max<int64_t>(std::min(2, ix.sel_tiles), (units + num_sms() - 1) / num_sms());
     if (even >= 40 || blocks <= num_sms() / 4) per = std::min<int64_t>(per, even);
   }
