@@ -37,8 +37,8 @@
 // L2 (tf32 floor 0.51 ms for 1.18 M x 100 against 2 000 centroids).  Keeping the
 // sixteen smallest lower bounds sorted cost 37 of 47 instructions a pair (5.9 ms
 // a pass, the spill 6.8); most pairs are now dismissed eight at a time by a
-// maximum that the TMEM load computes: 1.45 ms, the spill 3.46 (of which copies and
-// MMAs 0.88 and 1.73, staging the operands 0.27 and 0.63, the survivors 0.26 and
+// maximum that the TMEM load computes: 1.36 ms, the spill 3.50 (of which copies and
+// MMAs 0.88 and 1.73, staging the operands 0.27 and 0.63, the survivors 0.2 and
 // 0.57).
 //
 // Warp roles: 0 = bulk-copy producer, 1 = TMEM owner and MMA issuer,
@@ -770,20 +770,22 @@ size_t smem_for(int kp, int ops, int s, int steps, int cap) {
 int kp_for(int d) { return (d + 2 + 7) / 8 * 8; }
 
 // A operands, codebook stages and list length that fit: two operands before one
-// (half the codebook traffic), lists of 16 before stages of 32 KB (fewer, larger
-// copies), those before deep rings.  A point in the band of more centroids than
-// its list holds is scored against all of them.  Where two operands leave room
-// for lists of 8 only (151 to 166 columns), they still pay: 200 000 x 152 against
-// 2 000 centroids 0.49 ms, with one operand and lists of 16 0.55; against 20 000,
-// forty to a cluster, 3.30 and 3.49; twenty tight ones to a cluster, every list
-// full either way, 7.8 and 5.7.
+// (half the codebook traffic), stages of 32 KB before 16 KB (fewer, larger copies),
+// lists of 16 before 8, those before deep rings.  A point in the band of more
+// centroids than its list holds is scored against all of them, which costs less
+// than shorter stages or a second codebook stream (lists of 8 in 32 KB stages
+// against lists of 16 in 16 KB ones, 4 M x 128 bf16 points: 40 000 centroids 90.5
+// / 97.0 ms, with the spill 298 / 327; 4 000 centroids 10.0 / 11.2; two operands and
+// lists of 8 against one and lists of 16, 200 000 x 152 points: 2 000 centroids
+// 0.49 / 0.55 ms, 20 000, forty to a cluster, 3.30 / 3.49; 2 000, twenty tight ones to
+// a cluster, every list full either way, 7.8 / 5.7).
 struct Shape {
   int ops = 0, stages = 0, steps = 0, cap = 0;
 };
 Shape shape_for(int kp, int ndir, int most_ops = 2) {
   for (int ops = most_ops; ops >= (ndir ? 2 : 1); --ops)
-    for (int cap : {16, 8})
-      for (int steps : {8, 4})
+    for (int steps : {8, 4})
+      for (int cap : {16, 8})
         for (int s = kStagesMax; s >= 2; --s)
           if (smem_for(kp, ops, s, steps, cap) <= 227 * 1024 - 256)   // room for the static shared variables
             return Shape{ops, s, steps, cap};
