@@ -217,48 +217,11 @@ __global__ void __launch_bounds__(kThr, 1) assign_tc_kernel(AsgParams<XT> P) {
           cr = assigned_row(P.C, prior, P.d);
         }
         float ss = 0.f, xd = 0.f;
-        const bool vec = std::is_same<XT, float>::value && P.vec;
-        const bool vec8 = !std::is_same<XT, float>::value && P.vec;   // bf16: 8 columns a load
-        const int d4 = P.vec ? P.d / 4 : 0;             // 4-column chunks in 16-byte loads
+        const int d4 = P.vec ? P.d / 4 : 0;             // 4-column chunks in 16-byte copies or loads
         const int mid = OPS == 1 ? kp / 16 * 2 : 0;
         const int c0 = OPS == 1 && hh == 1 ? mid : 0, c1 = OPS == 1 && hh == 0 ? mid : kp / 4;   // this thread's chunks
-        if (vec && active) {
-          const float* xsrc = reinterpret_cast<const float*>(P.X) + p * P.d;
-          for (int k4 = c0; k4 < min(c1, d4); ++k4) tc::cp_async16(tc::smem_u32(row + k4 * 32), xsrc + 4 * k4);
-        }
-        tc::cp_async_wait_all();
-        uint4 eight = make_uint4(0u, 0u, 0u, 0u);
-#pragma unroll 4
-        for (int k4 = c0; k4 < c1; ++k4) {
-          float xv[4], cv[4] = {0.f, 0.f, 0.f, 0.f};
-          if (k4 < d4) {
-            if (active) {
-              if (vec8) {                               // (c0 is even, and so is d4)
-                if (k4 % 2 == 0) eight = __ldg(reinterpret_cast<const uint4*>(P.X + p * P.d + 4 * k4));
-                const uint32_t lo = k4 % 2 ? eight.z : eight.x, hi = k4 % 2 ? eight.w : eight.y;
-                xv[0] = __uint_as_float(lo << 16);
-                xv[1] = __uint_as_float(lo & 0xffff0000u);
-                xv[2] = __uint_as_float(hi << 16);
-                xv[3] = __uint_as_float(hi & 0xffff0000u);
-              } else {
-                const float4 a = *reinterpret_cast<const float4*>(row + k4 * 32);
-                xv[0] = a.x; xv[1] = a.y; xv[2] = a.z; xv[3] = a.w;
-              }
-              if (resid) {
-                const float4 b = __ldg(reinterpret_cast<const float4*>(cr + 4 * k4));
-                cv[0] = b.x; cv[1] = b.y; cv[2] = b.z; cv[3] = b.w;
-              }
-            } else {
-              xv[0] = xv[1] = xv[2] = xv[3] = 0.f;
-            }
-          } else {
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-              const int k = 4 * k4 + u;
-              xv[u] = (active && k < P.d) ? ld(P.X + p * P.d + k) : 0.f;
-              if (resid) cv[u] = (active && k < P.d) ? __ldg(cr + k) : 0.f;
-            }
-          }
+        const int cv1 = min(c1, d4);
+        const auto put = [&](int k4, const float (&xv)[4], const float (&cv)[4]) {
           float av[4];
 #pragma unroll
           for (int u = 0; u < 4; ++u) {
@@ -273,6 +236,42 @@ __global__ void __launch_bounds__(kThr, 1) assign_tc_kernel(AsgParams<XT> P) {
             }
           }
           *reinterpret_cast<float4*>(row + k4 * 32) = make_float4(av[0], av[1], av[2], av[3]);
+        };
+        const auto centroid4 = [&](int k4) {
+          return resid && active ? __ldg(reinterpret_cast<const float4*>(cr + 4 * k4)) : make_float4(0.f, 0.f, 0.f, 0.f);
+        };
+        if constexpr (std::is_same<XT, float>::value) {
+          const float* xsrc = P.X + p * P.d;
+          if (active)
+            for (int k4 = c0; k4 < cv1; ++k4) tc::cp_async16(tc::smem_u32(row + k4 * 32), xsrc + 4 * k4);
+          tc::cp_async_wait_all();
+#pragma unroll 4
+          for (int k4 = c0; k4 < cv1; ++k4) {
+            const float4 x = active ? *reinterpret_cast<const float4*>(row + k4 * 32) : make_float4(0.f, 0.f, 0.f, 0.f);
+            const float4 cc = centroid4(k4);
+            put(k4, {x.x, x.y, x.z, x.w}, {cc.x, cc.y, cc.z, cc.w});
+          }
+        } else {
+#pragma unroll 4
+          for (int k4 = c0; k4 < cv1; k4 += 2) {        // 8 columns a load (c0 and cv1 are even)
+            const uint4 x = active ? __ldg(reinterpret_cast<const uint4*>(P.X + p * P.d + 4 * k4)) : make_uint4(0u, 0u, 0u, 0u);
+            const float4 ca = centroid4(k4), cb = centroid4(k4 + 1);
+            put(k4, {__uint_as_float(x.x << 16), __uint_as_float(x.x & 0xffff0000u), __uint_as_float(x.y << 16),
+                     __uint_as_float(x.y & 0xffff0000u)}, {ca.x, ca.y, ca.z, ca.w});
+            put(k4 + 1, {__uint_as_float(x.z << 16), __uint_as_float(x.z & 0xffff0000u), __uint_as_float(x.w << 16),
+                         __uint_as_float(x.w & 0xffff0000u)}, {cb.x, cb.y, cb.z, cb.w});
+          }
+        }
+#pragma unroll 4
+        for (int k4 = max(c0, cv1); k4 < c1; ++k4) {    // rows of other widths, and the padding
+          float xv[4], cv[4];
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            const int k = 4 * k4 + u;
+            xv[u] = (active && k < P.d) ? ld(P.X + p * P.d + k) : 0.f;
+            cv[u] = (resid && active && k < P.d) ? __ldg(cr + k) : 0.f;
+          }
+          put(k4, xv, cv);
         }
         if (resid) {
           xr_s[m] = xd;                                  // <x, r_hat> of the fp32 r_hat
@@ -534,10 +533,12 @@ __global__ void __launch_bounds__(kThr, 1) assign_tc_kernel(AsgParams<XT> P) {
   if (warp == 1) tc::tmem_dealloc(tmem, 2 * kW);
 }
 
+// ||c||^2 and ||c|| of every centroid (a warp each); clears the pass's queue counters.
 __global__ void codebook_norms(const float* __restrict__ C, int c, int d, float* __restrict__ n2,
-                               float* __restrict__ n1) {
+                               float* __restrict__ n1, int* __restrict__ qcount) {
   const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (w >= c) return;
+  if (w == 0 && lane < 2) qcount[lane] = 0;
   float s = 0.f;
   for (int k = lane; k < d; k += 32) {
     const float v = C[(int64_t)w * d + k];
@@ -817,7 +818,8 @@ void assign_tc_pass(const XT* X, int64_t n, int d, const float* C, int c, int nd
   float* n2 = scr.get<float>(c);
   float* n1 = scr.get<float>(c);
   float* tmax = scr.get<float>(ctiles);
-  codebook_norms<<<ceil_div((int64_t)c * 32, 256), 256, 0, s>>>(C, c, d, n2, n1);
+  int* qcount = scr.get<int>(2);             // queued points
+  codebook_norms<<<ceil_div((int64_t)c * 32, 256), 256, 0, s>>>(C, c, d, n2, n1, qcount);
   SOAR_LAUNCHED();
   pack_codebook<<<ceil_div((int64_t)ctiles * kN * kp, 256), 256, 0, s>>>(C, n2, c, d, kp, ctiles * kN, Cc);
   SOAR_LAUNCHED();
@@ -826,8 +828,6 @@ void assign_tc_pass(const XT* X, int64_t n, int d, const float* C, int c, int nd
   int32_t* cand = scr.get<int32_t>((size_t)n * kList);
   int32_t* queue = scr.get<int32_t>(n);
   uint64_t* best = scr.get<uint64_t>(n);
-  int* qcount = scr.get<int>(2);             // queued points
-  SOAR_CUDA(cudaMemsetAsync(qcount, 0, 2 * sizeof(int), s));
   const int vec = d * sizeof(XT) % 16 == 0 && reinterpret_cast<uintptr_t>(X) % 16 == 0 &&
                   reinterpret_cast<uintptr_t>(C) % 16 == 0;
   AsgParams<XT> prm{X, n, d, kp, Cc, tmax, C, c, ctiles, assign, astride, inv_rn, lambda, sh.stages,
