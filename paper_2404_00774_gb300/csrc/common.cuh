@@ -55,17 +55,26 @@ struct Error : std::runtime_error {
 // belongs to the process and is never lowered: it goes to all that the kernel's
 // static arrays leave at once, so that host threads launching one kernel with
 // different sizes cannot undercut each other between this call and the launch.
+// Each thread remembers the kernels it raised (asking the driver took some 5 us).
 template <typename Kernel>
 void allow_smem(Kernel kern, size_t need) {
+  struct Raised {
+    const void* kern;
+    int dev, limit;
+  };
+  thread_local std::vector<Raised> raised;
+  int dev = 0;
+  SOAR_CUDA(cudaGetDevice(&dev));
+  for (const Raised& r : raised)
+    if (r.kern == (const void*)kern && r.dev == dev && need <= (size_t)r.limit) return;
+  int most = 0;
   cudaFuncAttributes a;
   SOAR_CUDA(cudaFuncGetAttributes(&a, kern));
-  if (need <= (size_t)a.maxDynamicSharedSizeBytes) return;
-  int dev = 0, most = 0;
-  SOAR_CUDA(cudaGetDevice(&dev));
   SOAR_CUDA(cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
   most -= (int)a.sharedSizeBytes;
   // (more than there is: the call fails and says so)
   SOAR_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, need <= (size_t)most ? most : (int)need));
+  raised.push_back({(const void*)kern, dev, most});
 }
 
 // ------------------------------------------------------ stream-ordered scratch
