@@ -7,7 +7,7 @@
 // (approximate score <q, C_p> + sum_s <q_s, B[s][code_s]>).  A point counts by
 // its copy in the partition the query probed earliest.
 //
-//   score_items    (partition, up to 32 / 64 of its queries): the partition's
+//   score_items    (partition, up to 32 of its queries): the partition's
 //                  rows times the queries on the tensor cores, one 4-byte key
 //                  per (query, row) written at the pair's place in the
 //                  query's slice; 0 for a copy that does not count
@@ -26,8 +26,8 @@
 // once per query and spent one table look-up or one fp8 conversion a term
 // (10 000 queries, 10^7 x 96 fp8, t = 6, R = 1 000: scoring 6 230, selecting
 // 2 990, rescoring 2 810 us; 1.18 M x 100 PQ4, t = 14, R = 100: 4 076, 1 884
-// and 398 us).  Here the codes are read and decoded once for up to 64 queries:
-// 763 and 988 us, 756 and 567 us.  The product is a few
+// and 398 us).  Here the codes are read and decoded once for up to 32 queries:
+// 768 and 954 us, 769 and 549 us.  The product is a few
 // percent of the work, so warp-level MMAs fed from registers are used: a key
 // leaves the registers it was computed in, with no TMEM round trip.
 #include <algorithm>
@@ -156,8 +156,10 @@ struct Fp8Rows {
   }
   // |key's score - defined score|: both sums of exact products have at most
   // code_stride fp32 additions, off by 2^-24 (defined order) and at most 2^-23
-  // (tensor cores; measured 2^-23 over a whole sum) of a partial sum that stays
-  // below ||q8|| ||x8||, and ||x8|| <= 448 sqrt(d); the rest covers the scaling.
+  // (tensor cores: their width is not documented; whole shortlists of rows that one
+  // large product and many small ones make up are compared with the defined ones in
+  // tests/test_gpu_shortlist_defined.py) of a partial sum that stays below ||q8||
+  // ||x8||, and ||x8|| <= 448 sqrt(d); the rest covers the scaling.
   // The scale of a row that the query meets is at most smax.
   __device__ float delta(float3 v, int64_t q, float smax) const {
     return ldexpf((float)code_stride, -22) * sqrtf(v.x) * 448.f * sqrtf((float)code_stride) * qscale[q] * smax;
@@ -409,7 +411,7 @@ __global__ void pass_counts(Slices sl, const int32_t* __restrict__ tpq, int64_t 
 // partitions need, whichever are fewer; an item with more of both compares
 // (50 queries of 200 probes over 400 partitions, two spills: 1 111 us compared, 152
 // hashed).
-constexpr int kHashSize = 4096, kHashMost = 3072;
+constexpr int kHashSize = 2048, kHashMost = 1536;
 struct ProbeMasks {
   int32_t key[kHashSize];
   uint32_t mask[kHashSize];
@@ -505,7 +507,7 @@ __global__ void __launch_bounds__(kThreads, 3) score_items(Rows rows, IvfWork wo
   const int probed = min(earlier_s, work.c);    // distinct partitions among the earlier probes, at most
   const bool hashed = probed <= kHashMost;
   int bits = 6;
-  while (hashed && (1 << bits) < kHashSize && (1 << bits) < 2 * probed) ++bits;
+  while (hashed && (1 << bits) < kHashSize && (1 << bits) < 8 * probed) ++bits;
   if (a > 1 && hashed) masks.clear(bits);
   __syncthreads();
   if (a > 1 && hashed) {
@@ -869,11 +871,14 @@ __global__ void __launch_bounds__(kThreads) finish_slices(
     __syncthreads();
     if (tid == 0) n_list = R;
   };
-  // The list from the kept rows, all rows of the slice that count or (open) all
-  // at or above lo; false where linear bins cannot tell.
-  const auto choose = [&](int count, bool open) {
+  // The list from `count` rows (key_at, pos_at), all rows of the slice that count
+  // or (open) all at or above lo; false where linear bins cannot tell.
+  const auto choose = [&](int count, auto key_at, auto pos_at, bool open) {
     if (!set_bins()) return false;
-    for (int i = tid; i < count; i += kThreads) atomicAdd(&hist[bin_of(kept[i])], 1);
+    for (int i = tid; i < count; i += kThreads) {
+      const uint32_t key = key_at(i);
+      if (key) atomicAdd(&hist[bin_of(key)], 1);
+    }
     if (find_bin(R) <= R) return false;
     const float wide = ceilf(2.f * delta * scale) + 1.f;
     const int mb = wide < (float)kBins ? (int)wide : kBins;
@@ -885,10 +890,11 @@ __global__ void __launch_bounds__(kThreads) finish_slices(
     if (m > kBand) return false;
     for (int i0 = 0; i0 < count; i0 += kThreads) {
       const int i = i0 + tid;
-      const int b = i < count ? bin_of(kept[i]) : -1;
+      const uint32_t key = i < count ? key_at(i) : 0u;
+      const int b = key ? bin_of(key) : -1;
       if (!__any_sync(kFull, b >= b_lo)) continue;
-      append(b > b_hi, &n_list, list, R, b > b_hi ? kept_at[i] : 0);
-      append(b >= b_lo && b <= b_hi, &n_band, band, kBand, b >= b_lo ? kept_at[i] : 0);
+      append(b > b_hi, &n_list, list, R, b > b_hi ? pos_at(i) : 0);
+      append(b >= b_lo && b <= b_hi, &n_band, band, kBand, b >= b_lo ? pos_at(i) : 0);
     }
     __syncthreads();
     finish_band(m);
@@ -994,8 +1000,12 @@ __global__ void __launch_bounds__(kThreads) finish_slices(
       few = true;
     } else if (m_kept > R) {
       if (floor_key > 1u) lo = key_float(floor_key);
-      done = choose(m_kept, floor_key > 1u);
+      done = choose(m_kept, [&](int i) { return kept[i]; }, [&](int i) { return kept_at[i]; }, floor_key > 1u);
     }
+  }
+  if (!done && !few) {                                  // (a long slice has more rows above the floor than are kept)
+    lo = lo_s;
+    done = choose(n, [&](int i) { return K[i]; }, [&](int i) { return i; }, false);
   }
   __syncthreads();
   if (!done) {
