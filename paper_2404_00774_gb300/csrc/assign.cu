@@ -343,7 +343,7 @@ __global__ void gather_rows_f32(const XT* __restrict__ X, int d, const int32_t* 
 // most 2^-54 M, is all that is lost (2^-59 M over sixteen rows), and the 64 rows
 // join the fp64 chain with one rounding of 2^-53 of the chain in place of 64.  Sixteen
 // rows that would take the fp32 sum out of range are added in fp64 directly.
-// Bound: HBM, the member rows gathered once (1.18 M x 100 fp32 in 2 000
+// Bound: issue slots and the latency of the gathers (0.42 of HBM; 1.18 M x 100 fp32 in 2 000
 // clusters: 849 us with one thread for a column's four fp64 chains, 666 with a
 // thread per chain, now 165; joining after sixteen rows took 208).
 constexpr int kUpdCols = 128, kUpdChains = 4, kUpdAhead = 16, kUpdJoin = 4;

@@ -13,12 +13,19 @@ namespace soar {
 
 namespace {
 
-// Largest batch finished by a block per query when k <= 32.
+// Largest batch finished by a block per query when k <= 32.  Finishing, us, a warp /
+// a block per query (Glove-shaped, t = 14): k = 10 2 048 queries 33 / 34, 3 000 36 /
+// 36, 4 096 44 / 49, 6 000 56 / 63, 10 000 70 / 102; k = 32, where lists overflow and
+// partitions are rescanned, 1 216 1 721 / 1 115, 2 048 1 856 / 1 618, 4 096 2 707 /
+// 2 849, 10 000 4 986 / 6 314; in tight clusters (bf16) k = 10 2 048 28 / 27, 4 096 35
+// / 39, 10 000 67 / 79, k = 32 2 048 3 166 / 1 752, 4 096 4 019 / 3 081, 10 000 7 458 /
+// 6 751.  The line gives up 5 us without overflow below it for what it saves with.
 constexpr int64_t kBlockFinishMax = 4096;
 // Queries per SM up to which their blocks are of 512 threads, above that of 128
 // (finishing, us, 128 against 512 threads; 152 SMs: k = 100 of about 270 lists,
 // 70 queries 64 / 32, 300 queries 67 / 42, 600 queries 94 / 69, 1 024 queries
-// 103 / 103; k = 10, 1 200 queries 34 / 51).
+// 103 / 103; k = 10 of 14 lists, 300 queries 20 / 19, 608 21 / 32, 1 216 22 / 57;
+// k = 32 with overflows, 300 761 / 325, 608 821 / 470, 1 216 1 115 / 810).
 constexpr int64_t kWideBlockMax = 4;
 
 // Exact fp32 <q, x> of row-major row `pos` (row stride rs; k ascending, the

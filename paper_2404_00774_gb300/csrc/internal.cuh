@@ -74,7 +74,7 @@ struct IndexData {
   void* tc_rows = nullptr;        // [tc_groups * 8 * tc_kp] elements of dtype
   int64_t* tc_gstart = nullptr;   // [c + 1] first group of each partition
   int32_t* tc_ids = nullptr;      // [tc_groups * 8] point id (-1 on padding)
-  float* tc_norms = nullptr;      // [tc_groups * 8] ||x|| (0 on padding)
+  float* tc_norms = nullptr;      // [tc_groups * 8] ||x|| (0 on padding); a section of the index file, read by no kernel
   float* tc_pmax = nullptr;       // [c] largest ||x|| of each partition
   int32_t tc_kp = 0;
   int64_t tc_groups = 0;

@@ -14,11 +14,10 @@
 // the query in shared memory), two rows per lane in flight, and the warp
 // keeps the pair's 32 best (score, id) rank keys, lane j the j-th: a block
 // with many newcomers is sorted across the warp and merged (bitonic), a
-// block with few is inserted key by key.  Each pair's list is written best first;
-// the caller's k-way merge over a query's lists drops the second copy of a
-// spilled point (its exact score and id are identical).  Every probed pair
-// reads its rows once; a warp per pair keeps the whole GPU busy even for a
-// batch of a few queries.
+// block with few is inserted key by key.  Each list is written best first;
+// merge_lists takes a query's lists and drops the second copy of a spilled point
+// (its exact score and id are identical).  Every probed pair reads its rows once;
+// a batch of a few queries splits each partition over several warps.
 #include <algorithm>
 
 #include "internal.cuh"

@@ -618,12 +618,22 @@ int scan_tc_list_len(int k, int64_t pairs) { return list_len_for(k, pairs); }
 // Brute force with 16 < k <= 32: heap mode where the register mode's 32 entries
 // are too few.  A chunk holds a fair share of the final k and of the rows within
 // the band of the k-th best, and a list that overflows costs a rescan of the whole
-// chunk (us, register / heap mode: 10 000 queries, chunks of 62 000 rows, k = 17
-// 19 286 / 9 452, k = 32 388 069 / 12 103; 448 queries, chunks of 4 200, k = 17
-// 496 / 650, k = 20 731 / 719, k = 32 5 164 / 1 320; 176 queries, chunks of 512,
-// k = 28 353 / 476, k = 32 837 / 533).  Searches keep the register mode: in tight
-// clusters more rows than a heap's list holds pass the bound (k = 20, 300 queries
-// probing 100 partitions of 800 rows: 2 166 / 10 467).
+// chunk.  Measured at the lines, us, register / heap mode, 128 queries over rows of
+// 96 (broad fp32, then tight bf16 clusters):
+//   chunks of 512     k = 20 333 / 400, 266 / 351   28 1 468 / 601, 373 / 514
+//                     29 1 434 / 617, 399 / 528     32 1 359 / 730, 839 / 578
+//   chunks of 1 024   k = 17 347 / 428, 268 / 366   20 462 / 532, 308 / 400
+//                     24 1 731 / 630, 373 / 531     29 2 646 / 811, 516 / 632
+//   chunks of 4 096   k = 17 590 / 749, 414 / 568   20 1 496 / 832, 472 / 677
+//   chunks of 8 192   k = 17 978 / 974, 549 / 794   20 3 499 / 1 144, 621 / 843
+//   chunks of 16 000  k = 17 2 009 / 1 377, 766 / 1 039   32 36 565 / 2 615, 17 629 / 1 840
+//   1 024 queries, chunks of 65 536   k = 17 9 864 / 2 086, 1 303 / 1 666
+//                     32 116 078 / 4 040, 56 826 / 2 921
+// so the lines take up to 1.4 times the register mode's time where it would have
+// been enough, against many times where it is not.  Searches keep the register mode
+// (us: 300 queries probing 100 partitions of 800 rows, k = 20 971 / 1 047; 1 000
+// probing 200 638 / 778; where its lists overflow it is the slower one: Glove-shaped,
+// 10 000 queries, k = 24 3 726 / 1 841).
 int scan_tc_flat_list_len(int k, int64_t pairs, int64_t chunk) {
   if (k > 16 && k <= kCand && (chunk >= 8192 || k > 28 || (k >= 20 && chunk >= 1024))) return heap_list_len(k);
   return list_len_for(k, pairs);

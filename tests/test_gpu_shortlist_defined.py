@@ -152,3 +152,18 @@ def test_fp8_shortlist_of_many_probes(soar, n, c, t, spills):
     s = _fp8_scores(soar, Q, X)
     _check(soar, ix, c, A.cpu().long(), X, Q, s[:, :, None].expand(-1, -1, 1 + spills), t, 200, 200)
     ix.close()
+
+
+@pytest.mark.parametrize("R", [10, 100])
+def test_fp8_shortlist_of_a_long_slice(soar, R):
+    """More rows above the sampled floor than are kept: the bins run over the whole slice."""
+    g = torch.Generator().manual_seed(R)
+    n, d, c, nq = 300_000, 16, 3, 3
+    X = torch.nn.functional.normalize(torch.randn(n, d, generator=g), dim=1)
+    Q = torch.nn.functional.normalize(torch.randn(nq, d, generator=g), dim=1)
+    C = X[:c].contiguous()
+    A = soar.soar_assign(X.cuda(), C.cuda(), 1.0, 1)
+    ix = soar.soar_index_build(X.cuda(), C.cuda(), A, mode=soar.SOAR_SCORE_FP8)
+    s = _fp8_scores(soar, Q, X)
+    _check(soar, ix, c, A.cpu().long(), X, Q, s[:, :, None].expand(-1, -1, 2), c, R, R)
+    ix.close()
